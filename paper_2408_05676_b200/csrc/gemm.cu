@@ -84,7 +84,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles = (raw + 1023u) & ~1023u;          // swizzled tiles need 1024-byte alignment
   const uint32_t w_bytes = kBM * 128, a_bytes = uint32_t(NT) * 128, stage_bytes = MT * w_bytes + a_bytes;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (uniform)
   const int krank = blockIdx.x % splits, ttile = blockIdx.x / splits;   // cluster rank = K range
   const int wtile = blockIdx.y;
   const int r0 = ttile * NT, n0 = wtile * kBM * MT;           // wtile counts groups of MT weight tiles
@@ -96,11 +96,15 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   const int slice = (NT + splits - 1) / splits;            // token columns finished by one CTA of the cluster
   const int own = max(0, min(slice, NT - krank * slice));
 
-  if (threadIdx.x == 0) {
-    abort_flag = 0;
-    for (int s = 0; s < stages; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), 1); }
-    mbar_init(smem_u32(&acc_bar), 1);
-    mbar_fence_init();
+  const uint32_t elected = elect_one();
+  if (warp == 0) {
+    if (elected) {
+      abort_flag = 0;
+      for (int s = 0; s < stages; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), 1); }
+      mbar_init(smem_u32(&acc_bar), 1);
+      mbar_fence_init();
+    }
+    __syncwarp();
     // The first weight stages are requested here, before tensor memory is allocated and the CTA's
     // threads meet: they depend on nothing, and a CTA that starts late (once an earlier kernel's CTA
     // has left its slot) has its first bytes on the way that much sooner.
@@ -108,19 +112,19 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     for (int kb = 0; kb < min(stages, nkb); ++kb) {
       const uint32_t bar = smem_u32(&full_bar[kb]), dst = tiles + uint32_t(kb) * stage_bytes;
       const int wk = ((kb0 + kb) >> wshift) * kBK;
-      mbar_expect_tx(bar, stage_bytes);
+      if (elected) mbar_expect_tx(bar, stage_bytes);
 #pragma unroll
       for (int t = 0; t < MT; ++t) {
         const int T = wtile * MT + t;
         if (EPI == EPI_SWIGLU) {   // 64 gate rows and the 64 up rows of the same features (the map's box is 64 rows)
-          tma_load_2d_hint(dst + t * w_bytes, &tmW, wk, T * 64, bar, w_policy0);
-          tma_load_2d_hint(dst + t * w_bytes + w_bytes / 2, &tmW, wk, e.f + T * 64, bar, w_policy0);
+          tma_load_2d_elect(dst + t * w_bytes, &tmW, wk, T * 64, bar, w_policy0, elected);
+          tma_load_2d_elect(dst + t * w_bytes + w_bytes / 2, &tmW, wk, e.f + T * 64, bar, w_policy0, elected);
         } else {                   // 128 consecutive rows: one copy (the map's box is 128 rows)
-          tma_load_2d_hint(dst + t * w_bytes, &tmW, wk, T * kBM, bar, w_policy0);
+          tma_load_2d_elect(dst + t * w_bytes, &tmW, wk, T * kBM, bar, w_policy0, elected);
         }
       }
     }
-    tma_prefetch_map(&tmA);
+    if (elected) tma_prefetch_map(&tmA);
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_u32(&tmem_slot)), "r"(tmem_cols) : "memory");
@@ -129,7 +133,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-  const uint32_t tmem_acc = tmem_slot;
+  const uint32_t tmem_acc = __shfl_sync(0xffffffffu, tmem_slot, 0);
   // floats between consecutive token rows of the staged accumulator; the verdict epilogue reads one row per lane
   // and pads the rows so that those reads spread over the banks
   constexpr int kRow = EPI == EPI_VERDICT ? kVerdictRow : kBM;
@@ -167,13 +171,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   };
 
   if (warp == 0) {
-    if (lane == 0) {  // ---- TMA producer ----
+    {  // ---- TMA producer (the whole warp runs the loop, one lane issues) ----
       const uint32_t full0 = smem_u32(&full_bar[0]);
       // weights are read once per step: they must not push the activations, the residual stream and the
       // cache pages of this step out of L2; every CTA of the launch reads the activations
       const uint64_t w_policy = make_policy_evict_first(), a_policy = make_policy_evict_last();
-      auto load = [&](uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t bar, uint64_t pol) { tma_load_2d_hint(dst, tm, x, y, bar, pol); };
-      auto expect = [&](int s) { mbar_expect_tx(smem_u32(&full_bar[s]), stage_bytes); };
+      auto load = [&](uint32_t dst, const CUtensorMap* tm, int x, int y, uint32_t bar, uint64_t pol) { tma_load_2d_elect(dst, tm, x, y, bar, pol, elected); };
+      auto expect = [&](int s) { if (elected) mbar_expect_tx(smem_u32(&full_bar[s]), stage_bytes); };
       auto load_w = [&](int kb, int s) {
         const int k = ((kb0 + kb) >> wshift) * kBK;
         const uint32_t dst = tiles + uint32_t(s) * stage_bytes, bar = full0 + uint32_t(s) * 8;
@@ -213,27 +217,23 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         for (int j = max(0, kb - stages); j < kb; ++j) mbar_drain(smem_u32(&full_bar[j % stages]), (j / stages) & 1);
     }
   } else if (warp == 1) {
-    if (lane == 0) {  // ---- MMA issuer ----
+    {  // ---- MMA issuer (likewise) ----
       const uint32_t idesc = (1u << 4) | (1u << 7) | (1u << 10) | (uint32_t(NT >> 3) << 17) | (uint32_t(kBM >> 4) << 24);
+      const uint64_t wdesc0 = umma_desc(tiles);
       bool ok = true;
       for (int kb = 0, s = 0, par = 0; kb < nkb && ok; ++kb) {
         ok = mbar_wait_hot(smem_u32(&full_bar[s]), par, &abort_flag);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint32_t w_addr = tiles + uint32_t(s) * stage_bytes;
-        const uint64_t adesc = umma_desc(w_addr + MT * w_bytes);
+        const uint64_t stage = wdesc0 + uint64_t(uint32_t(s) * (stage_bytes >> 4)), adesc = stage + uint64_t(MT * (w_bytes >> 4));
 #pragma unroll
-        for (int t = 0; t < MT; ++t) {
-          const uint64_t wdesc = umma_desc(w_addr + t * w_bytes);
-#pragma unroll
-          for (int k = 0; k < kBK / 16; ++k)  // 16 bf16 = 32 bytes further along K inside the swizzle span
-            umma_bf16(tmem_acc + uint32_t(t) * kAccCols, wdesc + uint64_t(k * 2), adesc + uint64_t(k * 2), idesc, (kb | k) != 0);
-        }
-        umma_commit(smem_u32(&empty_bar[s]));
+        for (int t = 0; t < MT; ++t)
+          umma_kblock(tmem_acc + uint32_t(t) * kAccCols, stage + uint64_t(t * (w_bytes >> 4)), adesc, idesc, uint32_t(kb != 0), elected);
+        umma_commit(smem_u32(&empty_bar[s]), elected);
         if (++s == stages) { s = 0; par ^= 1; }
       }
       // arrives when every MMA issued so far has finished
-      umma_commit(smem_u32(&acc_bar));
+      umma_commit(smem_u32(&acc_bar), elected);
     }
   } else {
     // ---- epilogue warps, part 1: everything that can be done before the accumulator is ready ----
