@@ -20,11 +20,9 @@
 //              cluster barrier, all six warps sum the partial tiles of the cluster through
 //              distributed shared memory in rank order (run-to-run identical, no partial sums
 //              in global memory) for the token columns this CTA owns and apply the fused epilogue.
-// Variants chosen by the host per launch: two weight tiles per CTA (MT = 2, one CTA per SM, token
-// tiles of up to 256 rows) where several token tiles make the launch L2->SM-bound; activations as
-// hi + lo bf16 pairs (the model's precise mode: every weight block is multiplied with both parts
-// into the same accumulator); and, for the LM head, an epilogue that leaves what the acceptance
-// rule needs per (row, vocabulary tile) instead of the logits.
+// Variants: activations as hi + lo bf16 pairs (the model's precise mode: every weight block is multiplied with
+// both parts into the same accumulator); and, for the LM head, an epilogue that leaves what the acceptance rule
+// needs per (row, vocabulary tile) instead of the logits.  Steps of many token rows run in gemm_pair.cu.
 // Every mbarrier wait is bounded: on expiry the CTA records LASER_ERR_TIMEOUT, drains its
 // copies, still joins the cluster barriers, frees its tensor memory and exits.
 #include <map>
@@ -32,6 +30,7 @@
 #include <type_traits>
 
 #include "epilogue.cuh"
+#include "gemm_pair.cuh"
 #include "tma.cuh"
 #include "umma.cuh"
 
@@ -41,13 +40,7 @@ namespace {
 constexpr int kTcThreads = 192;
 constexpr int kMaxStages = 6;
 constexpr int kMaxNT = 192;       // token rows per tile: accumulator staging must fit shared memory
-#ifndef LASER_WIDE_NT
-#define LASER_WIDE_NT 256
-#endif
-constexpr int kMaxNTWide = LASER_WIDE_NT;   // ... with two weight tiles per CTA (one CTA per SM); 256 = the largest MMA N
 constexpr int kSmemBudget = 110 * 1024;  // shared memory of one CTA: two CTAs per SM
-constexpr int kSmemBudgetWide = 200 * 1024;  // with two weight tiles per CTA: one CTA per SM
-constexpr int kAccCols = 256;     // tensor-memory columns between the accumulators of a CTA's weight tiles
 
 __device__ __forceinline__ void cluster_sync_all() {
   asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -65,12 +58,8 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t cluster_addr) {
 __device__ __forceinline__ void st_shared_f32(uint32_t addr, float v) {
   asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v));
 }
-// MT = weight tiles per CTA.  1: the form for few token rows (the step is bound by the weight stream;
-// two CTAs per SM).  2: for several token tiles, where the launches are bound by L2->SM traffic: a CTA
-// multiplies two 128-row weight tiles with the same staged activation tile (two accumulators), so the
-// activation bytes per flop halve; one CTA per SM, no K split.
-template <int EPI, int MT>
-__global__ void __launch_bounds__(kTcThreads, MT == 1 ? 2 : 1)
+template <int EPI>
+__global__ void __launch_bounds__(kTcThreads, 2)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmA, const GemmEpilogue e,
                int N, int NT, int total_kb, int kb_per_split, int splits, int stages, int tmem_cols,
                int32_t* __restrict__ status) {
@@ -78,16 +67,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   __shared__ uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], acc_bar;
   __shared__ uint32_t tmem_slot;
   __shared__ int abort_flag;
-  __shared__ float s_rstd[MT == 1 ? kMaxNT : kMaxNTWide];
-  __shared__ int s_pos[MT == 1 ? kMaxNT : kMaxNTWide], s_page[MT == 1 ? kMaxNT : kMaxNTWide];
+  __shared__ float s_rstd[kMaxNT];
+  __shared__ int s_pos[kMaxNT], s_page[kMaxNT];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");   // the next kernel may start its prologue
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles = (raw + 1023u) & ~1023u;          // swizzled tiles need 1024-byte alignment
-  const uint32_t w_bytes = kBM * 128, a_bytes = uint32_t(NT) * 128, stage_bytes = MT * w_bytes + a_bytes;
+  const uint32_t w_bytes = kBM * 128, a_bytes = uint32_t(NT) * 128, stage_bytes = w_bytes + a_bytes;
   const int warp = __shfl_sync(0xffffffffu, int(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (uniform)
   const int krank = blockIdx.x % splits, ttile = blockIdx.x / splits;   // cluster rank = K range
   const int wtile = blockIdx.y;
-  const int r0 = ttile * NT, n0 = wtile * kBM * MT;           // wtile counts groups of MT weight tiles
+  const int r0 = ttile * NT, n0 = wtile * kBM;
   const int kb0 = krank * kb_per_split;
   const int nkb = max(0, min(kb_per_split, total_kb - kb0));
   // Activations given as hi + lo bf16 pairs ([hi | lo] side by side in a row, lo starting at column a_lo_off): K
@@ -113,15 +102,11 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       const uint32_t bar = smem_u32(&full_bar[kb]), dst = tiles + uint32_t(kb) * stage_bytes;
       const int wk = ((kb0 + kb) >> wshift) * kBK;
       if (elected) mbar_expect_tx(bar, stage_bytes);
-#pragma unroll
-      for (int t = 0; t < MT; ++t) {
-        const int T = wtile * MT + t;
-        if (EPI == EPI_SWIGLU) {   // 64 gate rows and the 64 up rows of the same features (the map's box is 64 rows)
-          tma_load_2d_elect(dst + t * w_bytes, &tmW, wk, T * 64, bar, w_policy0, elected);
-          tma_load_2d_elect(dst + t * w_bytes + w_bytes / 2, &tmW, wk, e.f + T * 64, bar, w_policy0, elected);
-        } else {                   // 128 consecutive rows: one copy (the map's box is 128 rows)
-          tma_load_2d_elect(dst + t * w_bytes, &tmW, wk, T * kBM, bar, w_policy0, elected);
-        }
+      if (EPI == EPI_SWIGLU) {   // 64 gate rows and the 64 up rows of the same features (the map's box is 64 rows)
+        tma_load_2d_elect(dst, &tmW, wk, wtile * 64, bar, w_policy0, elected);
+        tma_load_2d_elect(dst + w_bytes / 2, &tmW, wk, e.f + wtile * 64, bar, w_policy0, elected);
+      } else {                   // 128 consecutive rows: one copy (the map's box is 128 rows)
+        tma_load_2d_elect(dst, &tmW, wk, n0, bar, w_policy0, elected);
       }
     }
     if (elected) tma_prefetch_map(&tmA);
@@ -138,16 +123,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   // and pads the rows so that those reads spread over the banks
   constexpr int kRow = EPI == EPI_VERDICT ? kVerdictRow : kBM;
 
-  // gains of the next norm for the first weight tile: a weight, not a result of the kernel before, so
+  // gains of the next norm: a weight, not a result of the kernel before, so
   // requested now, long before the epilogue uses it
-  uint2 gain4_first = make_uint2(0u, 0u);
-  if (EPI == EPI_RESID && n0 + 4 * lane < N) gain4_first = *reinterpret_cast<const uint2*>(e.gain_next + n0 + 4 * lane);
+  uint2 gain4 = make_uint2(0u, 0u);
+  if (EPI == EPI_RESID && n0 + 4 * lane < N) gain4 = *reinterpret_cast<const uint2*>(e.gain_next + n0 + 4 * lane);
   bool acc_ok = true;
-  // accumulator t from tensor memory to shared memory, token-major [NT][128] (epilogue warps; a warp may
+  // the accumulator from tensor memory to shared memory, token-major [NT][128] (epilogue warps; a warp may
   // only touch its own 32 TMEM lanes)
-  auto drain = [&](int t) {
+  auto drain = [&]() {
     const int quarter = warp & 3;
-    const uint32_t src = tmem_acc + uint32_t(t) * kAccCols + (uint32_t(quarter * 32) << 16);
+    const uint32_t src = tmem_acc + (uint32_t(quarter * 32) << 16);
     const uint32_t dst0 = tiles + uint32_t((quarter * 32 + lane) * 4);
     for (int c = 0; c < NT; c += 48) {   // three loads in flight, one wait; reads past NT stay inside the allocation
       uint32_t v0[16], v1[16], v2[16];
@@ -181,20 +166,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       auto load_w = [&](int kb, int s) {
         const int k = ((kb0 + kb) >> wshift) * kBK;
         const uint32_t dst = tiles + uint32_t(s) * stage_bytes, bar = full0 + uint32_t(s) * 8;
-#pragma unroll
-        for (int t = 0; t < MT; ++t) {
-          const int T = wtile * MT + t;
-          if (EPI == EPI_SWIGLU) {
-            load(dst + t * w_bytes, &tmW, k, T * 64, bar, w_policy);
-            load(dst + t * w_bytes + w_bytes / 2, &tmW, k, e.f + T * 64, bar, w_policy);
-          } else {
-            load(dst + t * w_bytes, &tmW, k, T * kBM, bar, w_policy);
-          }
+        if (EPI == EPI_SWIGLU) {
+          load(dst, &tmW, k, wtile * 64, bar, w_policy);
+          load(dst + w_bytes / 2, &tmW, k, e.f + wtile * 64, bar, w_policy);
+        } else {
+          load(dst, &tmW, k, n0, bar, w_policy);
         }
       };
       auto load_a = [&](int kb, int s) {
         const int g = kb0 + kb;
-        load(tiles + uint32_t(s) * stage_bytes + MT * w_bytes, &tmA, (g & wshift) * e.a_lo_off + (g >> wshift) * kBK, r0,
+        load(tiles + uint32_t(s) * stage_bytes + w_bytes, &tmA, (g & wshift) * e.a_lo_off + (g >> wshift) * kBK, r0,
              full0 + uint32_t(s) * 8, a_policy);
       };
       // The ring was filled with weight tiles at the start of the kernel (they do not depend on the
@@ -225,10 +206,8 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         ok = mbar_wait_hot(smem_u32(&full_bar[s]), par, &abort_flag);
         if (!ok) break;
         asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-        const uint64_t stage = wdesc0 + uint64_t(uint32_t(s) * (stage_bytes >> 4)), adesc = stage + uint64_t(MT * (w_bytes >> 4));
-#pragma unroll
-        for (int t = 0; t < MT; ++t)
-          umma_kblock(tmem_acc + uint32_t(t) * kAccCols, stage + uint64_t(t * (w_bytes >> 4)), adesc, idesc, uint32_t(kb != 0), elected);
+        const uint64_t stage = wdesc0 + uint64_t(uint32_t(s) * (stage_bytes >> 4)), adesc = stage + uint64_t(w_bytes >> 4);
+        umma_kblock(tmem_acc, stage, adesc, idesc, uint32_t(kb != 0), elected);
         umma_commit(smem_u32(&empty_bar[s]), elected);
         if (++s == stages) { s = 0; par ^= 1; }
       }
@@ -256,25 +235,16 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       }
       s_rstd[j] = rstd; s_pos[j] = pos; s_page[j] = page;
     }
-    // part 2: the first accumulator to shared memory
+    // part 2: the accumulator to shared memory
     acc_ok = mbar_wait(smem_u32(&acc_bar), 0, &abort_flag);
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
-    drain(0);
-  }
-#pragma unroll
-  for (int t = 0; t < MT; ++t) {   // the CTA's weight tiles, one after the other through the same staging buffer
-  if (t > 0) {
-    __syncthreads();               // the staged tile before this one has been finished
-    if (warp >= 2) drain(t);
+    drain();
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
   __syncthreads();
   if (splits > 1) cluster_sync_all();  // every partial tile of the cluster is staged
-  const int wt = wtile * MT + t, n0t = wt * kBM;
-  const int nfeat = n0t + 4 * lane;
-  const LaneCtx lc = make_lane_ctx<EPI>(e, n0t, lane, N);
-  uint2 gain4 = gain4_first;
-  if (EPI == EPI_RESID && t > 0 && nfeat < N) gain4 = *reinterpret_cast<const uint2*>(e.gain_next + nfeat);
+  const int nfeat = n0 + 4 * lane;
+  const LaneCtx lc = make_lane_ctx<EPI>(e, n0, lane, N);
   auto fetch_operands = [&](int jj, float4& g0, float4& g1) {
     g0 = make_float4(0.f, 0.f, 0.f, 0.f); g1 = g0;
     const int r = r0 + krank * slice + jj;
@@ -289,10 +259,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   };
 
   __syncwarp();
-  // (an odd tile count leaves the last group's second tile beyond the matrix: nothing to finish)
-  const bool tile_valid = EPI == EPI_SWIGLU ? wt * 64 < e.f : n0t < N;
-  if (!tile_valid) {
-  } else if (EPI == EPI_VERDICT && splits == 1) {
+  if (EPI == EPI_VERDICT && splits == 1) {
     // part 3, acceptance fused into the LM head: one lane per token row scans the row's 128 staged logits
     if (e.out) {   // on request the logits are stored as well (the plain epilogue's stores)
       for (int j = warp; j < NT; j += kTcThreads / 32) {
@@ -302,9 +269,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
       }
     }
     const bool ok = !abort_flag;
-    if (e.top_n <= 1) verdict_rows<1>(e, tiles, NT, r0, n0t, wt, N, warp, lane, s_rstd, s_pos, ok);
-    else if (e.top_n == 2) verdict_rows<2>(e, tiles, NT, r0, n0t, wt, N, warp, lane, s_rstd, s_pos, ok);
-    else verdict_rows<4>(e, tiles, NT, r0, n0t, wt, N, warp, lane, s_rstd, s_pos, ok);
+    if (e.top_n <= 1) verdict_rows<1>(e, tiles, NT, r0, n0, wtile, N, warp, lane, s_rstd, s_pos, ok);
+    else if (e.top_n == 2) verdict_rows<2>(e, tiles, NT, r0, n0, wtile, N, warp, lane, s_rstd, s_pos, ok);
+    else verdict_rows<4>(e, tiles, NT, r0, n0, wtile, N, warp, lane, s_rstd, s_pos, ok);
   } else if ((EPI == EPI_SWIGLU || EPI == EPI_PLAIN) && splits == 1) {
     // part 3 without partial tiles to sum or operands to prefetch: all six warps finish rows,
     // in wide groups whose loads are issued first.
@@ -323,7 +290,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
         const bool live = jb + b < NT && r < e.R_rows && !(abort_flag);
         const float rstd = s_rstd[j];
         if (EPI == EPI_PLAIN) epi_plain(e, lc, r, live, acc[b], rstd, N);
-        else epi_swiglu(e, r, live, wt * 64, lane, acc[b], rstd);
+        else epi_swiglu(e, r, live, wtile * 64, lane, acc[b], rstd);
       }
     }
   } else {
@@ -358,9 +325,9 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           const bool live = jj < own && r < e.R_rows && !abort_flag;   // the last token tile may overhang the buffers
           const float rstd = s_rstd[j];
           if (EPI == EPI_PLAIN) epi_plain(e, lc, r, live, acc, rstd, N);
-          else if (EPI == EPI_VERDICT) epi_verdict(e, lc, r, live, lane, acc, rstd, N, wt, s_pos[j]);
-          else if (EPI == EPI_RESID) epi_resid(e, lc, r, live, lane, acc, N, wt, g0[b], gain4);
-          else if (EPI == EPI_SWIGLU) epi_swiglu(e, r, live, wt * 64, lane, acc, rstd);
+          else if (EPI == EPI_VERDICT) epi_verdict(e, lc, r, live, lane, acc, rstd, N, wtile, s_pos[j]);
+          else if (EPI == EPI_RESID) epi_resid(e, lc, r, live, lane, acc, N, wtile, g0[b], gain4);
+          else if (EPI == EPI_SWIGLU) epi_swiglu(e, r, live, wtile * 64, lane, acc, rstd);
           else epi_qkv(e, lc, r, live, acc, rstd, s_pos[j], s_page[j], g0[b], g1[b]);
         }
       }
@@ -378,7 +345,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     }
   }
   __syncwarp();
-  }  // weight tiles of the CTA
   if (splits > 1) cluster_sync_all();  // peers may still be reading this CTA's staged tile or tensor memory
   __syncthreads();
   if (warp == 1) {
@@ -391,7 +357,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 struct GemmState {
   // (pointer, rows, cols, box rows) -> tensor map
   std::map<std::tuple<const void*, int, int, int>, CUtensorMap> maps;
-  bool ready = false;
+  bool ready = false, pair_fits = false;
 };
 
 GemmState* get_state(laser_model* m) {
@@ -413,21 +379,19 @@ laser_status tensor_map(GemmState* st, const void* ptr, int rows, int cols, int 
 
 struct TcShape { int n_ttiles, NT, stages, tmem_cols; size_t smem; };
 
-// mt = weight tiles per CTA (1 or 2); max_nt = most token rows per tile
-TcShape tc_shape(int R_pad, int mt = 1, int max_nt = kMaxNT) {
+TcShape tc_shape(int R_pad) {
   TcShape s;
-  s.n_ttiles = ceil_div(R_pad, max_nt);
+  s.n_ttiles = ceil_div(R_pad, kMaxNT);
   s.NT = ceil_div(ceil_div(R_pad, s.n_ttiles), 16) * 16;
-  const int stage_bytes = mt * kBM * 128 + s.NT * 128;
-  s.stages = std::max(2, std::min(kMaxStages, (mt == 1 ? kSmemBudget : kSmemBudgetWide) / stage_bytes));
+  const int stage_bytes = kBM * 128 + s.NT * 128;
+  s.stages = std::max(2, std::min(kMaxStages, kSmemBudget / stage_bytes));
   s.tmem_cols = 32;
   while (s.tmem_cols < s.NT) s.tmem_cols <<= 1;
-  if (mt == 2) s.tmem_cols = 2 * kAccCols;
   s.smem = std::max(size_t(s.stages) * stage_bytes, size_t(s.NT) * kVerdictRow * 4) + 1024;
   return s;
 }
 
-template <int EPI, int MT>
+template <int EPI>
 laser_status launch_epi(const CUtensorMap& tw, const CUtensorMap& ta, const GemmEpilogue& e, int N, const TcShape& sh,
                         int n_wtiles, int total_kb, int kbps, int splits, int32_t* status, cudaStream_t stream) {
   cudaLaunchConfig_t cfg = {};
@@ -446,24 +410,20 @@ laser_status launch_epi(const CUtensorMap& tw, const CUtensorMap& ta, const Gemm
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  LASER_CUDA(cudaLaunchKernelEx(&cfg, gemm_tc_kernel<EPI, MT>, tw, ta, e, N, sh.NT, total_kb, kbps, splits, sh.stages,
+  LASER_CUDA(cudaLaunchKernelEx(&cfg, gemm_tc_kernel<EPI>, tw, ta, e, N, sh.NT, total_kb, kbps, splits, sh.stages,
                                 sh.tmem_cols, status));
   return LASER_OK;
 }
 
 laser_status prepare(GemmState* st) {
   if (st->ready) return LASER_OK;
-  const int bytes = kSmemBudget + 2048, wide = kSmemBudgetWide + 2048;
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_PLAIN, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_PLAIN, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide));
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide));
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide));
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide));
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_VERDICT, 1>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_VERDICT, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize, wide));
+  const int bytes = kSmemBudget + 2048;
+  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_VERDICT>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
+  st->pair_fits = gemm_pair_fits();
   st->ready = true;
   return LASER_OK;
 }
@@ -491,39 +451,29 @@ laser_status gemm_fused(laser_model* m, const __nv_bfloat16* A, const __nv_bfloa
   }
   GemmState* st = get_state(m);
   LASER_TRY(prepare(st));
-  const int n_wtiles = epi == EPI_SWIGLU ? ceil_div(N / 2, 64) : ceil_div(N, kBM);
-  const int splits = pick_splits(R_pad, N, K, epi);
-  // several token tiles and no K split: two weight tiles per CTA share every staged activation tile
-  // (where the halved CTA count still gives every SM one)
-  const int n_tt = tc_shape(R_pad).n_ttiles;
-  const int mt = (n_tt > 1 && splits == 1 && ceil_div(n_wtiles, 2) * n_tt >= 148) ? 2 : 1;
-  TcShape sh = tc_shape(R_pad, mt);
-  if (mt == 2) {
-    // Token tiles of up to 256 rows (the largest MMA N) re-read the weights from L2 fewer times, but make fewer,
-    // longer CTAs: taken where they do not cost more in whole waves of CTAs over the SMs (a CTA's time goes with
-    // the bytes it stages per K block: 256 weight rows + NT token rows).
-    const TcShape wide = tc_shape(R_pad, 2, kMaxNTWide);
-    auto cost = [&](const TcShape& t) { return ceil_div(ceil_div(n_wtiles, 2) * t.n_ttiles, 148) * (256 + t.NT); };
-    if (cost(wide) < cost(sh)) sh = wide;
-  }
   const CUtensorMap *tw = nullptr, *ta = nullptr;
   LASER_TRY(tensor_map(st, W, N, K, epi == EPI_SWIGLU ? 64 : 128, &tw));
+  if (st->pair_fits && R_pad > gemm_pair_rows(e.a_lo_off != 0)) {   // many token rows: two SMs per tile (gemm_pair.cu)
+    const GemmPairShape sh = gemm_pair_shape(R_pad, N, K, epi, e.a_lo_off != 0);
+    LASER_TRY(tensor_map(st, A, m->R_pad, e.a_lo_off ? 2 * K : K, sh.NT / 2, &ta));
+    LASER_TRY(gemm_pair_launch(m, sh, *tw, *ta, N, K, epi, e, stream));
+    count_launch();
+    return LASER_OK;
+  }
+  const int n_wtiles = epi == EPI_SWIGLU ? ceil_div(N / 2, 64) : ceil_div(N, kBM);
+  const int splits = pick_splits(R_pad, N, K, epi);
+  const TcShape sh = tc_shape(R_pad);
   LASER_TRY(tensor_map(st, A, m->R_pad, e.a_lo_off ? 2 * K : K, sh.NT, &ta));
   const int total_kb = ceil_div(K, kBK) * (e.a_lo_off ? 2 : 1), kbps = ceil_div(total_kb, splits);
-  const int n_groups = ceil_div(n_wtiles, mt);     // grid rows: groups of mt weight tiles
-#define LASER_GEMM_LAUNCH(E)                                                                                            \
-  do {                                                                                                                  \
-    if (mt == 1) LASER_TRY((launch_epi<E, 1>(*tw, *ta, e, N, sh, n_groups, total_kb, kbps, splits, m->status, stream))); \
-    else LASER_TRY((launch_epi<E, 2>(*tw, *ta, e, N, sh, n_groups, total_kb, kbps, splits, m->status, stream)));         \
-  } while (0);
+  auto launch = [&](auto tag) { return launch_epi<decltype(tag)::value>(*tw, *ta, e, N, sh, n_wtiles, total_kb, kbps, splits, m->status, stream); };
+  using std::integral_constant;
   switch (epi) {
-    case EPI_PLAIN: LASER_GEMM_LAUNCH(EPI_PLAIN) break;
-    case EPI_RESID: LASER_GEMM_LAUNCH(EPI_RESID) break;
-    case EPI_SWIGLU: LASER_GEMM_LAUNCH(EPI_SWIGLU) break;
-    case EPI_VERDICT: LASER_GEMM_LAUNCH(EPI_VERDICT) break;
-    default: LASER_GEMM_LAUNCH(EPI_QKV) break;
+    case EPI_PLAIN: LASER_TRY(launch(integral_constant<int, EPI_PLAIN>{})); break;
+    case EPI_RESID: LASER_TRY(launch(integral_constant<int, EPI_RESID>{})); break;
+    case EPI_SWIGLU: LASER_TRY(launch(integral_constant<int, EPI_SWIGLU>{})); break;
+    case EPI_VERDICT: LASER_TRY(launch(integral_constant<int, EPI_VERDICT>{})); break;
+    default: LASER_TRY(launch(integral_constant<int, EPI_QKV>{})); break;
   }
-#undef LASER_GEMM_LAUNCH
   count_launch();
   return LASER_OK;
 }

@@ -7,6 +7,7 @@
 // are written to the pages before attention, so attention reads cache and new rows alike.
 #include <cmath>
 
+#include "gemm_pair.cuh"
 #include "model.cuh"
 #include "tma.cuh"
 
@@ -352,6 +353,10 @@ LASER_API laser_status laser_model_create(const laser_model_cfg* cfg, const lase
   LASER_TRY(model_alloc(m, &m->top_idx, Rp * v_tiles));
   LASER_TRY(model_alloc(m, &m->tile_sum, Rp * v_tiles));
   LASER_TRY(model_alloc(m, &m->status, size_t(1)));
+  if (m->R_pad > gemm_pair_rows(m->precise)) {
+    LASER_TRY(model_alloc(m, &m->pair_scratch, gemm_pair_scratch_floats(m->R_pad)));
+    LASER_TRY(model_alloc(m, &m->pair_state, size_t(kPairStateInts)));
+  }
   guard.p = nullptr;
   *out = m;
   return LASER_OK;
@@ -473,6 +478,8 @@ LASER_API laser_status laser_check(laser_model* m, void* stream) {
   LASER_CUDA(cudaStreamSynchronize(as_stream(stream)));
   if (st != 0) {
     LASER_CUDA(cudaMemsetAsync(m->status, 0, 4, as_stream(stream)));
+    if (m->pair_state)   // a launch that gave up may have left it
+      LASER_CUDA(cudaMemsetAsync(m->pair_state, 0, kPairStateInts * sizeof(int32_t), as_stream(stream)));
     set_error(st == LASER_ERR_CAPACITY ? "a sequence outgrew its KV pages"
               : st == LASER_ERR_TIMEOUT ? "a device-side wait ran out" : "a step was given a bad sequence id");
     return st;

@@ -36,6 +36,8 @@ struct laser_model {
   int4* top_idx = nullptr;         // [R_pad][vocab tiles] their token ids
   float* tile_sum = nullptr;       // [R_pad][vocab tiles] sum over the tile of exp(l - tile max)
   int32_t* status = nullptr;       // first device-side error of the stream, 0 = none
+  float* pair_scratch = nullptr;   // partial sums of the contractions for many rows (gemm_pair.cu), and the cut tiles' state
+  int32_t* pair_state = nullptr;
   void* gemm_state = nullptr;      // tensor-map cache of the tensor-core GEMM
   void* gen_buf = nullptr;         // work buffers of laser_generate, kept between calls (in `owned`)
   size_t gen_bytes = 0;

@@ -92,6 +92,15 @@ __device__ __forceinline__ void tma_load_2d_elect(uint32_t dst, const CUtensorMa
       "@q cp.async.bulk.tensor.2d.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;\n}"
       ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(bar), "l"(policy), "r"(elected) : "memory");
 }
+// The same load in a CTA pair: the destination is this CTA's, the completion bytes count on a barrier of the pair's
+// first CTA (a cluster address).
+__device__ __forceinline__ void tma_load_2d_pair(uint32_t dst, const CUtensorMap* map, int x, int y, uint32_t leader_bar, uint64_t policy,
+                                                 uint32_t elected) {
+  asm volatile(
+      "{\n.reg .pred q;\nsetp.ne.b32 q, %6, 0;\n"
+      "@q cp.async.bulk.tensor.2d.cta_group::2.shared::cluster.global.mbarrier::complete_tx::bytes.L2::cache_hint [%0], [%1, {%2, %3}], [%4], %5;\n}"
+      ::"r"(dst), "l"(map), "r"(x), "r"(y), "r"(leader_bar), "l"(policy), "r"(elected) : "memory");
+}
 __device__ __forceinline__ uint64_t make_policy_evict_first() {
   uint64_t p;
   asm volatile("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(p));

@@ -39,6 +39,25 @@ __device__ __forceinline__ void umma_kblock(uint32_t tmem_d, uint64_t wdesc, uin
       "@q tcgen05.mma.cta_group::1.kind::f16 [%0], w3, a3, %3, 1;\n}"
       ::"r"(tmem_d), "l"(wdesc), "l"(adesc), "r"(idesc), "r"(accumulate), "r"(elected) : "memory");
 }
+// The same in a CTA pair (cluster ranks 0 and 1): one 256-row MMA over both, each CTA holding half of both operands in its
+// shared memory; issued by rank 0.
+__device__ __forceinline__ void umma_kblock_pair(uint32_t tmem_d, uint64_t wdesc, uint64_t adesc, uint32_t idesc, uint32_t accumulate, uint32_t elected) {
+  asm volatile(
+      "{\n.reg .pred p, q;\n.reg .b64 w1, w2, w3, a1, a2, a3;\nsetp.ne.b32 q, %5, 0;\nsetp.ne.b32 p, %4, 0;\n"
+      "add.s64 w1, %1, 2;\nadd.s64 a1, %2, 2;\nadd.s64 w2, %1, 4;\nadd.s64 a2, %2, 4;\nadd.s64 w3, %1, 6;\nadd.s64 a3, %2, 6;\n"
+      "@q tcgen05.mma.cta_group::2.kind::f16 [%0], %1, %2, %3, p;\n"
+      "@q tcgen05.mma.cta_group::2.kind::f16 [%0], w1, a1, %3, 1;\n"
+      "@q tcgen05.mma.cta_group::2.kind::f16 [%0], w2, a2, %3, 1;\n"
+      "@q tcgen05.mma.cta_group::2.kind::f16 [%0], w3, a3, %3, 1;\n}"
+      ::"r"(tmem_d), "l"(wdesc), "l"(adesc), "r"(idesc), "r"(accumulate), "r"(elected) : "memory");
+}
+// arrives on the barrier at the same shared-memory offset in every CTA named by the rank mask
+__device__ __forceinline__ void umma_commit_pair(uint32_t bar, uint32_t rank_mask, uint32_t elected) {
+  asm volatile(
+      "{\n.reg .pred q;\n.reg .b16 m;\ncvt.u16.u32 m, %1;\nsetp.ne.b32 q, %2, 0;\n"
+      "@q tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], m;\n}"
+      ::"r"(bar), "r"(rank_mask), "r"(elected) : "memory");
+}
 // 16 consecutive fp32 columns of this thread's TMEM lane (no wait: pair with tmem_ld_wait)
 __device__ __forceinline__ void tmem_ld16(uint32_t taddr, uint32_t (&v)[16]) {
   asm volatile(
