@@ -49,7 +49,7 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
                   const int32_t* __restrict__ row_n, int Rs, int H, int Hkv,
                   const int32_t* __restrict__ page_table, int pages_per_seq, int layer_row0,
                   bf16* __restrict__ out, int32_t* __restrict__ status,
-                  const unsigned long long* __restrict__ row_mask) {
+                  const unsigned long long* __restrict__ row_mask, int fresh) {
   constexpr int HALVES = DH / 64;                 // 64-element (128-byte) column blocks per row
   constexpr int SUB = 16 * 128;                   // bytes of one 16-token x 64-element sub-tile
   constexpr int STAGE = 2 * HALVES * SUB;         // K then V
@@ -90,7 +90,7 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
   uint8_t* tiles_ptr = smem_raw + (tiles - raw);
   const uint32_t q_smem = tiles + kStages * STAGE;
   bf16* q_ptr = reinterpret_cast<bf16*>(tiles_ptr + kStages * STAGE);
-  const int n_keys = ctx + nr;
+  const int n_keys = ctx + (row_mask ? nr : min(nr, cta_row0 + 16 * TPC));   // chain: no row here sees a later one
   const int n_pg = (n_keys + 15) >> 4;
 
   if (tid == 0) {
@@ -104,7 +104,8 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
   if (warp == kConsumers) {  // producer
     if (lane == 0) {
       const int32_t* pt = page_table + size_t(seq_ids[b]) * pages_per_seq;
-      const int n_early = min(min(ctx >> 4, n_pg), kStages);   // whole pages of older tokens that fit the ring
+      // whole pages of older tokens that fit the ring (none where the kernel before may have written them)
+      const int n_early = fresh ? 0 : min(min(ctx >> 4, n_pg), kStages);
       bool ok = true;
       int issued = 0;
       const uint64_t kv_policy = make_policy_evict_first();   // a page is read once per step
@@ -329,7 +330,7 @@ bool attention_tma_supported(const laser_model* m, const laser_kv* kv) {
   return kv->has_pages_map && (m->cfg.head_dim == 64 || m->cfg.head_dim == 128);
 }
 
-laser_status attention_tma_launch(laser_model* m, laser_kv* kv, int layer, const int32_t* seq_ids, int B, int Rs, bool tree,
+laser_status attention_tma_launch(laser_model* m, laser_kv* kv, int layer, const int32_t* seq_ids, int B, int Rs, bool tree, bool fresh,
                                   cudaStream_t stream) {
   const int dh = m->cfg.head_dim, H = m->cfg.n_heads, Hkv = m->cfg.n_kv_heads;
   const int64_t rows_per_layer = int64_t(kv->n_pages) * 2 * Hkv * 16;
@@ -355,7 +356,7 @@ laser_status attention_tma_launch(laser_model* m, laser_kv* kv, int layer, const
   do {                                                                                                                   \
     LASER_CUDA(cudaFuncSetAttribute(attn_paged_kernel<DH_, TPC_, PR_>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))); \
     LASER_CUDA(cudaLaunchKernelEx(&cfg, attn_paged_kernel<DH_, TPC_, PR_>, kv->pages_map, q, qf, seq_ids, rc, rn, Rs, H, Hkv, pt, \
-                                  kv->pages_per_seq, layer_row0, m->attn, m->status, mask));                              \
+                                  kv->pages_per_seq, layer_row0, m->attn, m->status, mask, fresh ? 1 : 0));                              \
   } while (0)
   if (pr) {
     if (dh == 128 && tpc == 1) LASER_ATTN_LAUNCH(128, 1, true);

@@ -455,7 +455,7 @@ laser_status gemm_fused(laser_model* m, const __nv_bfloat16* A, const __nv_bfloa
   LASER_TRY(tensor_map(st, W, N, K, epi == EPI_SWIGLU ? 64 : 128, &tw));
   if (st->pair_fits && R_pad > gemm_pair_rows(e.a_lo_off != 0)) {   // many token rows: two SMs per tile (gemm_pair.cu)
     const GemmPairShape sh = gemm_pair_shape(R_pad, N, K, epi, e.a_lo_off != 0);
-    LASER_TRY(tensor_map(st, A, m->R_pad, e.a_lo_off ? 2 * K : K, sh.NT / 2, &ta));
+    LASER_TRY(tensor_map(st, A, m->R_cap, e.a_lo_off ? 2 * K : K, sh.NT / 2, &ta));
     LASER_TRY(gemm_pair_launch(m, sh, *tw, *ta, N, K, epi, e, stream));
     count_launch();
     return LASER_OK;
@@ -463,7 +463,7 @@ laser_status gemm_fused(laser_model* m, const __nv_bfloat16* A, const __nv_bfloa
   const int n_wtiles = epi == EPI_SWIGLU ? ceil_div(N / 2, 64) : ceil_div(N, kBM);
   const int splits = pick_splits(R_pad, N, K, epi);
   const TcShape sh = tc_shape(R_pad);
-  LASER_TRY(tensor_map(st, A, m->R_pad, e.a_lo_off ? 2 * K : K, sh.NT, &ta));
+  LASER_TRY(tensor_map(st, A, m->R_cap, e.a_lo_off ? 2 * K : K, sh.NT, &ta));
   const int total_kb = ceil_div(K, kBK) * (e.a_lo_off ? 2 : 1), kbps = ceil_div(total_kb, splits);
   auto launch = [&](auto tag) { return launch_epi<decltype(tag)::value>(*tw, *ta, e, N, sh, n_wtiles, total_kb, kbps, splits, m->status, stream); };
   using std::integral_constant;

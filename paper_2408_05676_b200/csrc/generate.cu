@@ -12,32 +12,12 @@ namespace {
 struct GenState {
   int32_t* seq_tok;      // [B, max_total] prompt followed by generated tokens
   int32_t* seq_len;      // [B] tokens in seq_tok
-  int32_t* prompt_len;   // [B]
   int32_t* out_len;      // [B] generated so far
   int32_t* done;         // [B]
-  int32_t* cursor;       // [B] prompt tokens already cached
   unsigned long long* counters;  // steps, drafted, accepted, emitted
   int32_t* n_active;     // [1]
   int max_total;
 };
-
-// Prompt chunk for the prefill of sequences b0 .. b0 + nb - 1: up to Rs of the not yet cached prompt
-// tokens (all but the last) of each.
-__global__ void prefill_rows_kernel(GenState g, int b0, int Rs, int32_t* __restrict__ tokens, int32_t* __restrict__ n_rows) {
-  const int i = blockIdx.x, b = b0 + i;
-  const int remaining = g.prompt_len[b] - 1 - g.cursor[b];
-  const int n = max(0, min(Rs, remaining));
-  for (int j = threadIdx.x; j < Rs; j += blockDim.x)
-    tokens[i * Rs + j] = j < n ? g.seq_tok[size_t(b) * g.max_total + g.cursor[b] + j] : -1;
-  if (threadIdx.x == 0) n_rows[i] = n;
-}
-
-__global__ void prefill_advance_kernel(GenState g, int b0, int nb, const int32_t* __restrict__ n_rows, int32_t* __restrict__ kv_len) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= nb) return;
-  g.cursor[b0 + i] += n_rows[i];
-  kv_len[b0 + i] += n_rows[i];
-}
 
 // Tail (last n_max tokens, right-aligned) and pending token of every active sequence.
 __global__ void step_prep_kernel(GenState g, int B, int n_max, int32_t* __restrict__ tails, int32_t* __restrict__ tail_len,
@@ -160,13 +140,11 @@ LASER_API laser_status laser_generate(laser_model* m, laser_kv* kv, const laser_
   float* logits;
   LASER_TRY(buf.get(&g.seq_tok, size_t(B) * g.max_total));
   LASER_TRY(buf.get(&g.seq_len, size_t(B)));
-  LASER_TRY(buf.get(&g.prompt_len, size_t(B)));
   LASER_TRY(buf.get(&g.out_len, size_t(B)));
   LASER_TRY(buf.get(&g.done, size_t(B)));
-  LASER_TRY(buf.get(&g.cursor, size_t(B)));
   LASER_TRY(buf.get(&g.counters, size_t(4)));
   LASER_TRY(buf.get(&g.n_active, size_t(1)));
-  LASER_TRY(buf.get(&tokens, std::max(size_t(B) * Rs, size_t(m->R_pad))));
+  LASER_TRY(buf.get(&tokens, size_t(B) * Rs));
   LASER_TRY(buf.get(&n_rows, size_t(B)));
   LASER_TRY(buf.get(&tails, size_t(B) * n_max));
   LASER_TRY(buf.get(&tail_len, size_t(B)));
@@ -185,21 +163,38 @@ LASER_API laser_status laser_generate(laser_model* m, laser_kv* kv, const laser_
   LASER_TRY(buf.get(&d_out, size_t(B) * p->max_new));
   const bool fused = p->fused_accept && !(pool && p->tree);   // chain steps without stored logits
   LASER_TRY(buf.get(&logits, fused ? size_t(4) : size_t(B) * Rs * m->cfg.vocab));
+  // prefill: every prompt token but the last, cut into chunks; [chunks][kPrefillChunk] tokens, then per chunk its slot, its
+  // first position and its rows
+  std::vector<int32_t> h_pre, h_slot, h_start, h_rows;
+  for (int b = 0; b < B; ++b) {
+    const int32_t* prompt = prompts + prompt_offsets[b];
+    const int n = int(prompt_offsets[b + 1] - prompt_offsets[b]) - 1;
+    for (int p0 = 0; p0 < n; p0 += kPrefillChunk) {
+      const int rows = std::min(kPrefillChunk, n - p0);
+      h_pre.insert(h_pre.end(), prompt + p0, prompt + p0 + rows);
+      h_pre.insert(h_pre.end(), kPrefillChunk - rows, -1);
+      h_slot.push_back(b); h_start.push_back(p0); h_rows.push_back(rows);
+    }
+  }
+  const int n_chunks = int(h_slot.size());
+  for (const auto* v : {&h_slot, &h_start, &h_rows}) h_pre.insert(h_pre.end(), v->begin(), v->end());
+  int32_t* pre = nullptr;
+  LASER_TRY(buf.get(&pre, h_pre.size()));
   LASER_TRY(buf.commit(m, stream));
 
   // host -> device: prompts, lengths, ids
-  std::vector<int32_t> h_len(B), h_ids(B);
+  std::vector<int32_t> h_len(B), h_ids(B), h_cached(B);
   for (int b = 0; b < B; ++b) {
     h_len[b] = int32_t(prompt_offsets[b + 1] - prompt_offsets[b]);
     h_ids[b] = b;
+    h_cached[b] = h_len[b] - 1;
     LASER_CUDA(cudaMemcpyAsync(g.seq_tok + size_t(b) * g.max_total, prompts + prompt_offsets[b], size_t(h_len[b]) * 4,
                                cudaMemcpyHostToDevice, stream));
   }
   LASER_CUDA(cudaMemcpyAsync(g.seq_len, h_len.data(), size_t(B) * 4, cudaMemcpyHostToDevice, stream));
-  LASER_CUDA(cudaMemcpyAsync(g.prompt_len, h_len.data(), size_t(B) * 4, cudaMemcpyHostToDevice, stream));
   LASER_CUDA(cudaMemcpyAsync(seq_ids, h_ids.data(), size_t(B) * 4, cudaMemcpyHostToDevice, stream));
   if (pool) LASER_CUDA(cudaMemcpyAsync(gid, group_id, size_t(B) * 4, cudaMemcpyHostToDevice, stream));
-  LASER_CUDA(cudaMemsetAsync(kv->seq_len, 0, size_t(B) * 4, stream));
+  if (n_chunks) LASER_CUDA(cudaMemcpyAsync(pre, h_pre.data(), h_pre.size() * 4, cudaMemcpyHostToDevice, stream));
   LASER_CUDA(cudaMemsetAsync(d_out, 0xff, size_t(B) * p->max_new * 4, stream));
   int32_t h_active = B;
   LASER_CUDA(cudaMemcpyAsync(g.n_active, &h_active, 4, cudaMemcpyHostToDevice, stream));
@@ -209,24 +204,14 @@ LASER_API laser_status laser_generate(laser_model* m, laser_kv* kv, const laser_
   float ms_prefill = 0, ms_draft = 0, ms_verify = 0, ms_accept = 0, ms;
   LASER_CUDA(cudaEventRecord(ev.e[0], stream));
 
-  // prefill: every prompt token but the last.  A pass of Rs rows per sequence would read a sequence's
-  // whole cached prefix once per Rs prompt tokens; instead the model's row workspace is given to few
-  // sequences at a time, up to 128 rows each, and the LM head is left out.
-  const int chunk = std::max(Rs, std::min(128, m->R_pad / 16 * 16));
-  const int group = std::max(1, std::min(B, m->R_pad / chunk));
-  int n_pass = 0;
-  for (int b0 = 0; b0 < B; b0 += group) {
-    const int nb = std::min(group, B - b0);
-    int longest = 0;
-    for (int b = b0; b < b0 + nb; ++b) longest = std::max(longest, h_len[b] - 1);
-    for (int it = 0; it < ceil_div(longest, chunk); ++it, ++n_pass) {
-      prefill_rows_kernel<<<nb, 32, 0, stream>>>(g, b0, chunk, tokens, n_rows);
-      LASER_TRY(prefill_rows(m, kv, seq_ids + b0, tokens, n_rows, nb, chunk, stream));
-      prefill_advance_kernel<<<ceil_div(nb, 128), 128, 0, stream>>>(g, b0, nb, n_rows, kv->seq_len);
-      count_launch(2);
-      if ((n_pass & 15) == 15) LASER_TRY(laser_check(m, stream));   // do not keep launching after a device-side error
-    }
+  // As many chunks a pass as the workspace holds, of whatever prompts; a prompt's chunks come in order, in one pass or several.
+  int32_t *slot = pre + size_t(n_chunks) * kPrefillChunk, *start = slot + n_chunks, *rows = start + n_chunks;
+  const int pass = m->R_cap / kPrefillChunk;
+  for (int c0 = 0, n_pass = 0; c0 < n_chunks; c0 += pass, ++n_pass) {
+    LASER_TRY(prefill_chunks(m, kv, slot + c0, start + c0, pre + size_t(c0) * kPrefillChunk, rows + c0, std::min(pass, n_chunks - c0), stream));
+    if ((n_pass & 15) == 15) LASER_TRY(laser_check(m, stream));   // do not keep launching after a device-side error
   }
+  LASER_CUDA(cudaMemcpyAsync(kv->seq_len, h_cached.data(), size_t(B) * 4, cudaMemcpyHostToDevice, stream));
   LASER_CUDA(cudaEventRecord(ev.e[1], stream));
   LASER_CUDA(cudaStreamSynchronize(stream));
   LASER_CUDA(cudaEventElapsedTime(&ms_prefill, ev.e[0], ev.e[1]));

@@ -21,9 +21,10 @@ using bf16 = __nv_bfloat16;
 // One block per row: position, cache slot, capacity check, rotary angles (fp64 -> fp32).
 // With `parents` (token tree, Section 3.3) a row's position is ctx + its depth, its cache slot
 // stays ctx + row index, and row_mask gets the rows it attends to (its ancestors and itself).
+// With `start` (prompt chunks) row group b begins there instead of at its slot's committed length.
 __global__ void prep_rows_kernel(const int32_t* __restrict__ seq_ids, const int32_t* __restrict__ n_rows,
-                                 const int32_t* __restrict__ parents, unsigned long long* __restrict__ row_mask,
-                                 int B, int Rs, int R_pad, const int32_t* __restrict__ seq_len,
+                                 const int32_t* __restrict__ parents, const int32_t* __restrict__ start,
+                                 unsigned long long* __restrict__ row_mask, int B, int Rs, const int32_t* __restrict__ seq_len,
                                  int max_seqs, int capacity, int half, double theta, int head_dim,
                                  int32_t* __restrict__ row_pos, int32_t* __restrict__ row_seq,
                                  int32_t* __restrict__ row_ctx, int32_t* __restrict__ row_n,
@@ -42,7 +43,7 @@ __global__ void prep_rows_kernel(const int32_t* __restrict__ seq_ids, const int3
       nr = 0; seq = 0;
       if (threadIdx.x == 0) atomicCAS(status, 0, LASER_ERR_INVALID_ARG);
     } else {
-      ctx = seq_len[seq];
+      ctx = start ? start[b] : seq_len[seq];
       if (ctx + nr > capacity) {
         nr = 0;
         if (threadIdx.x == 0) atomicCAS(status, 0, LASER_ERR_CAPACITY);
@@ -330,33 +331,42 @@ LASER_API laser_status laser_model_create(const laser_model_cfg* cfg, const lase
     m->attn_norm.push_back(static_cast<const bf16*>(w->attn_norm[l]));
     m->ffn_norm.push_back(static_cast<const bf16*>(w->ffn_norm[l]));
   }
-  const size_t Rp = size_t(m->R_pad);
-  LASER_TRY(model_alloc(m, &m->resid, Rp * d));
+  m->R_cap = std::max(m->R_pad, kPrefillRows);
   m->precise = cfg->precise != 0;
-  const size_t pair = m->precise ? 2 : 1;     // hi + lo parts side by side in a row
-  LASER_TRY(model_alloc(m, &m->xn, Rp * d * pair));
-  LASER_TRY(model_alloc(m, &m->q, Rp * m->dq));
-  if (m->precise) LASER_TRY(model_alloc(m, &m->qf, Rp * m->dq));
-  LASER_TRY(model_alloc(m, &m->attn, Rp * m->dq * pair));
-  LASER_TRY(model_alloc(m, &m->act, Rp * f * pair));
-  LASER_TRY(model_alloc(m, &m->sumsq, size_t(ceil_div(d, 128)) * Rp));
-  LASER_TRY(model_alloc(m, &m->rope, Rp * (cfg->head_dim / 2) * 2));
-  LASER_TRY(model_alloc(m, &m->row_pos, Rp));
-  LASER_TRY(model_alloc(m, &m->row_seq, Rp));
-  LASER_TRY(model_alloc(m, &m->row_ctx, size_t(cfg->max_batch)));
-  LASER_TRY(model_alloc(m, &m->row_n, size_t(cfg->max_batch)));
-  LASER_TRY(model_alloc(m, &m->row_mask, size_t(m->R_pad)));
-  const size_t v_tiles = size_t(ceil_div(cfg->vocab, 128));
-  LASER_TRY(model_alloc(m, &m->row_draft, Rp));
-  LASER_TRY(model_alloc(m, &m->draft_logit, Rp));
-  LASER_TRY(model_alloc(m, &m->top_val, Rp * v_tiles));
-  LASER_TRY(model_alloc(m, &m->top_idx, Rp * v_tiles));
-  LASER_TRY(model_alloc(m, &m->tile_sum, Rp * v_tiles));
-  LASER_TRY(model_alloc(m, &m->status, size_t(1)));
-  if (m->R_pad > gemm_pair_rows(m->precise)) {
-    LASER_TRY(model_alloc(m, &m->pair_scratch, gemm_pair_scratch_floats(m->R_pad)));
-    LASER_TRY(model_alloc(m, &m->pair_state, size_t(kPairStateInts)));
-  }
+  const size_t Rp = size_t(m->R_cap), pair = m->precise ? 2 : 1;     // pair: hi + lo parts side by side in a row
+  const size_t groups = std::max<size_t>(cfg->max_batch, Rp / kPrefillChunk);
+  // the workspace: one zeroed allocation, its parts 256-byte aligned
+  struct Part { void** p; size_t bytes; };
+  std::vector<Part> parts;
+  auto part = [&](auto** p, size_t count) { parts.push_back(Part{reinterpret_cast<void**>(p), count * sizeof(**p)}); };
+  part(&m->resid, Rp * d);
+  part(&m->xn, Rp * d * pair);
+  if (m->precise) part(&m->qf, Rp * m->dq);
+  else part(&m->q, Rp * m->dq);
+  part(&m->attn, Rp * m->dq * pair);
+  part(&m->act, Rp * f * pair);
+  part(&m->sumsq, size_t(ceil_div(d, 128)) * Rp);
+  part(&m->rope, Rp * (cfg->head_dim / 2) * 2);
+  part(&m->row_pos, Rp);
+  part(&m->row_seq, Rp);
+  part(&m->row_ctx, groups);
+  part(&m->row_n, groups);
+  const size_t Rv = size_t(m->R_pad), v_tiles = size_t(ceil_div(cfg->vocab, 128));   // verify rows alone have these
+  part(&m->row_mask, Rv);
+  part(&m->row_draft, Rv);
+  part(&m->draft_logit, Rv);
+  part(&m->top_val, Rv * v_tiles);
+  part(&m->top_idx, Rv * v_tiles);
+  part(&m->tile_sum, Rv * v_tiles);
+  part(&m->status, 1);
+  part(&m->pair_scratch, gemm_pair_scratch_floats(m->R_cap));
+  part(&m->pair_state, kPairStateInts);
+  size_t total = 0;
+  for (const Part& x : parts) total += (x.bytes + 255) & ~size_t(255);
+  uint8_t* slab = nullptr;
+  LASER_TRY(model_alloc(m, &slab, total));
+  size_t off = 0;
+  for (const Part& x : parts) { *x.p = slab + off; off += (x.bytes + 255) & ~size_t(255); }
   guard.p = nullptr;
   *out = m;
   return LASER_OK;
@@ -478,8 +488,8 @@ LASER_API laser_status laser_check(laser_model* m, void* stream) {
   LASER_CUDA(cudaStreamSynchronize(as_stream(stream)));
   if (st != 0) {
     LASER_CUDA(cudaMemsetAsync(m->status, 0, 4, as_stream(stream)));
-    if (m->pair_state)   // a launch that gave up may have left it
-      LASER_CUDA(cudaMemsetAsync(m->pair_state, 0, kPairStateInts * sizeof(int32_t), as_stream(stream)));
+    // (a contraction that gave up may have left its tiles' state)
+    LASER_CUDA(cudaMemsetAsync(m->pair_state, 0, kPairStateInts * sizeof(int32_t), as_stream(stream)));
     set_error(st == LASER_ERR_CAPACITY ? "a sequence outgrew its KV pages"
               : st == LASER_ERR_TIMEOUT ? "a device-side wait ran out" : "a step was given a bad sequence id");
     return st;
@@ -491,7 +501,7 @@ LASER_API laser_status laser_check(laser_model* m, void* stream) {
 // the number of largest logits kept per vocabulary tile (1..4), negative when the tile sums of exp are wanted too
 static laser_status verify_impl(laser_model* m, laser_kv* kv, const int32_t* seq_ids, const int32_t* tokens,
                                 const int32_t* parents, const int32_t* n_rows, int32_t B, int32_t Rs, float* logits, void* stream_,
-                                int fused = 0);
+                                int fused = 0, const int32_t* start = nullptr);
 
 LASER_API laser_status laser_verify_step(laser_model* m, laser_kv* kv, const int32_t* seq_ids, const int32_t* tokens,
                                          const int32_t* n_rows, int32_t B, float* logits, void* stream) {
@@ -509,11 +519,12 @@ LASER_API laser_status laser_verify_step_tree(laser_model* m, laser_kv* kv, cons
 }
 
 namespace laser {
-// Prompt processing (the x_<=t of Eq. 3): the same forward over B sequences with Rs rows each, any Rs
-// with B * Rs inside the model's row workspace; only K and V are wanted, so the LM head is left out.
-laser_status prefill_rows(laser_model* m, laser_kv* kv, const int32_t* seq_ids, const int32_t* tokens,
-                          const int32_t* n_rows, int32_t B, int32_t Rs, cudaStream_t stream) {
-  return verify_impl(m, kv, seq_ids, tokens, nullptr, n_rows, B, Rs, nullptr, stream);
+// Prompt processing (the x_<=t of Eq. 3): the same forward over chunks of the prompts, each a row group of its own that
+// starts inside its prompt; only K and V are wanted, so the LM head is left out.
+laser_status prefill_chunks(laser_model* m, laser_kv* kv, const int32_t* seq_ids, const int32_t* start, const int32_t* tokens,
+                            const int32_t* n_rows, int32_t n_chunks, cudaStream_t stream) {
+  LASER_REQUIRE(start, "null argument");
+  return verify_impl(m, kv, seq_ids, tokens, nullptr, n_rows, n_chunks, kPrefillChunk, nullptr, stream, 0, start);
 }
 // The verify forward whose LM head leaves, per (row, vocabulary tile), what the acceptance rule needs
 // (see GemmEpilogue) in the model's buffers; logits may be null.
@@ -526,10 +537,11 @@ laser_status verify_fused(laser_model* m, laser_kv* kv, const int32_t* seq_ids, 
 // The forward over B sequences of Rs rows each; logits == nullptr: no LM head (prompt processing).
 static laser_status verify_impl(laser_model* m, laser_kv* kv, const int32_t* seq_ids, const int32_t* tokens,
                                 const int32_t* parents, const int32_t* n_rows, int32_t B, int32_t Rs, float* logits, void* stream_,
-                                int fused) {
+                                int fused, const int32_t* start) {
   LASER_REQUIRE(m && kv && seq_ids && tokens && n_rows, "null argument");
-  LASER_REQUIRE(B >= 1 && Rs >= 1 && B <= m->cfg.max_batch && int64_t(B) * Rs <= m->R_pad,
-                "B = %d sequences of %d rows outside the model's %d rows (max_batch = %d)", B, Rs, m->R_pad, m->cfg.max_batch);
+  const int max_rows = start ? m->R_cap : m->R_pad;
+  LASER_REQUIRE(B >= 1 && Rs >= 1 && (start || B <= m->cfg.max_batch) && int64_t(B) * Rs <= max_rows,
+                "B = %d sequences of %d rows outside the model's %d rows (max_batch = %d)", B, Rs, max_rows, m->cfg.max_batch);
   LASER_REQUIRE(kv->n_layers == m->cfg.n_layers && kv->n_kv_heads == m->cfg.n_kv_heads && kv->head_dim == m->cfg.head_dim,
                 "cache was created for another model shape");
   // the LM head stores four logits at a time
@@ -540,14 +552,13 @@ static laser_status verify_impl(laser_model* m, laser_kv* kv, const int32_t* seq
   const int d = c.d_model, f = c.d_ffn, dh = c.head_dim, H = c.n_heads, Hkv = c.n_kv_heads;
   const int capacity = int(std::min<int64_t>(kv->capacity_tokens(), INT32_MAX));
 
-  // Every row of the workspace is (re)marked: a GEMM's last token tile may reach past this call's
-  // rows, and whatever it finds there must be inactive (no cache write) and finite.
+  // (rows are independent columns of every product: what a token tile finds beyond these is multiplied and dropped)
   const bool tree = parents != nullptr;
-  prep_rows_kernel<<<m->R_pad, 64, 0, stream>>>(seq_ids, n_rows, parents, tree ? m->row_mask : nullptr, B, Rs, Rp, kv->seq_len, kv->max_seqs, capacity, dh / 2,
+  prep_rows_kernel<<<Rp, 64, 0, stream>>>(seq_ids, n_rows, parents, start, tree ? m->row_mask : nullptr, B, Rs, kv->seq_len, kv->max_seqs, capacity, dh / 2,
                                           double(c.rope_theta), dh, m->row_pos, m->row_seq, m->row_ctx, m->row_n,
                                           m->rope, m->status);
   const __nv_bfloat16* first_gain = c.n_layers > 0 ? m->attn_norm[0] : m->final_norm;
-  embed_kernel<<<m->R_pad, 256, 0, stream>>>(tokens, R, d, c.vocab, m->tok_emb, first_gain, m->resid, m->xn, m->sumsq, n_rows, Rs,
+  embed_kernel<<<Rp, 256, 0, stream>>>(tokens, R, d, c.vocab, m->tok_emb, first_gain, m->resid, m->xn, m->sumsq, n_rows, Rs,
                                              fused ? m->row_draft : nullptr, m->precise ? 1 : 0);
   count_launch(2);
   const bool use_tma_attn = attention_tma_supported(m, kv);
@@ -558,8 +569,8 @@ static laser_status verify_impl(laser_model* m, laser_kv* kv, const int32_t* seq
   }
   const int d_tiles = ceil_div(d, 128);
   GemmEpilogue base;
-  base.R_rows = m->R_pad;
-  base.sumsq_ld = m->R_pad;
+  base.R_rows = Rp;
+  base.sumsq_ld = m->R_cap;
   base.inv_d = 1.f / float(d);
   base.eps = c.rms_eps;
   base.out_split = m->precise ? 1 : 0;
@@ -579,7 +590,7 @@ static laser_status verify_impl(laser_model* m, laser_kv* kv, const int32_t* seq
     {
       ProfScope ps(m, 1, stream);
       if (use_tma_attn) {
-        LASER_TRY(attention_tma_launch(m, kv, l, seq_ids, B, Rs, tree, stream));
+        LASER_TRY(attention_tma_launch(m, kv, l, seq_ids, B, Rs, tree, start != nullptr, stream));
       } else {
         attention_kernel<<<dim3(B, H), 128, attn_smem, stream>>>(m->q, m->qf, m->precise ? 1 : 0, seq_ids, m->row_ctx, m->row_n, Rs, H, Hkv, dh,
                                                                 kv->page_table, kv->pages_per_seq, pages_l,

@@ -9,25 +9,26 @@ struct laser_model {
   int rows_per_seq = 0;  // max_draft + 1
   int R = 0;             // max_batch * rows_per_seq
   int R_pad = 0;         // R rounded up to a multiple of 16
+  int R_cap = 0;         // rows of the workspace: R_pad, or kPrefillRows where that is more
   int dq = 0, dkv = 0, dqkv = 0;
   const __nv_bfloat16 *tok_emb = nullptr, *lm_head = nullptr, *final_norm = nullptr;
   std::vector<const __nv_bfloat16*> wqkv, wo, wgu, wdown, attn_norm, ffn_norm;
   std::vector<void*> owned;  // device allocations released with the model
-  // workspace (all device)
-  float* resid = nullptr;          // [R_pad, d] residual stream, fp32
-  __nv_bfloat16* xn = nullptr;     // [R_pad, d] normalised activations (GEMM operand)
-  __nv_bfloat16* q = nullptr;      // [R_pad, dq] rotated queries
-  float* qf = nullptr;             // [R_pad, dq] the same in fp32 (precise mode only)
+  // workspace (all device, one allocation)
+  float* resid = nullptr;          // [R_cap, d] residual stream, fp32
+  __nv_bfloat16* xn = nullptr;     // [R_cap, d] normalised activations (GEMM operand)
+  __nv_bfloat16* q = nullptr;      // [R_cap, dq] rotated queries
+  float* qf = nullptr;             // [R_cap, dq] the same in fp32 (precise mode only)
   bool precise = false;            // activations handed to the contractions as hi + lo bf16 pairs: xn, attn, act are
-                                   // [R_pad, 2 x width] with the lo parts in the second half of a row
-  __nv_bfloat16* attn = nullptr;   // [R_pad, dq] attention output
-  __nv_bfloat16* act = nullptr;    // [R_pad, f] SwiGLU output
-  float* sumsq = nullptr;          // [ceil(d/128)][R_pad] per-tile sums of squares of the residual
-  float* rope = nullptr;           // [R_pad, head_dim/2, 2] cos, sin of each row's position
-  int32_t* row_pos = nullptr;      // [R_pad] position of the row, -1 = inactive
-  int32_t* row_seq = nullptr;      // [R_pad] cache slot of the row
-  int32_t* row_ctx = nullptr;      // [max_batch] committed length of each sequence of the step
-  int32_t* row_n = nullptr;        // [max_batch] effective rows of each sequence
+                                   // [R_cap, 2 x width] with the lo parts in the second half of a row
+  __nv_bfloat16* attn = nullptr;   // [R_cap, dq] attention output
+  __nv_bfloat16* act = nullptr;    // [R_cap, f] SwiGLU output
+  float* sumsq = nullptr;          // [ceil(d/128)][R_cap] per-tile sums of squares of the residual
+  float* rope = nullptr;           // [R_cap, head_dim/2, 2] cos, sin of each row's position
+  int32_t* row_pos = nullptr;      // [R_cap] position of the row, -1 = inactive
+  int32_t* row_seq = nullptr;      // [R_cap] cache slot of the row
+  int32_t* row_ctx = nullptr;      // [row groups] cached tokens before each sequence of the step (a prompt chunk's start in a prefill)
+  int32_t* row_n = nullptr;        // [row groups] effective rows of each
   unsigned long long* row_mask = nullptr;  // [R_pad] token tree: rows of its sequence a row attends to (bit j = row j)
   // acceptance fused into the LM head: what its epilogue leaves per (row, 128-token vocabulary tile)
   int32_t* row_draft = nullptr;    // [R_pad] token whose verdict the row gives, -1 = none
@@ -49,11 +50,17 @@ struct laser_model {
 
 namespace laser {
 
+// A prefill pass runs the contractions over up to this many prompt tokens: enough rows for the tensor pipe to be the bound
+// (7B, 4 layers: 3.6 us a row at 144 rows, 1.6 us at 1024).  16 prompts of 256 .. 1024 tokens and 32 new tokens each, 7B: 456 -> 233
+// ms against passes of 128 rows of one prompt.
+constexpr int kPrefillRows = 1024;
+constexpr int kPrefillChunk = 32;   // rows that share each staged K/V page in the attention kernel
+
 // What the GEMM does with a finished 128-feature x NT-row accumulator tile.
 enum { EPI_PLAIN = 0, EPI_RESID = 1, EPI_SWIGLU = 2, EPI_QKV = 3, EPI_VERDICT = 4 };
 
 struct GemmEpilogue {
-  int R_rows = 0;                    // rows the activation / output buffers really have
+  int R_rows = 0;                    // rows of the step: a token tile may overhang them, and what lies beyond is not finished
   // Operands as hi + lo bf16 pairs (the precise mode): the A operand's rows are [hi | lo] with lo starting at column
   // a_lo_off (0 = plain bf16 operand); out_split = the bf16 activations this epilogue writes (xb, act) are pairs too
   int a_lo_off = 0, out_split = 0;
@@ -119,14 +126,16 @@ struct ProfScope {
 // TMA-fed paged attention (head_dim 64 or 128 and a cache small enough for 32-bit row
 // coordinates); the verify forward falls back to a plain kernel otherwise.
 bool attention_tma_supported(const laser_model* m, const laser_kv* kv);
-laser_status attention_tma_launch(laser_model* m, laser_kv* kv, int layer, const int32_t* seq_ids, int B, int Rs, bool tree,
+// fresh: pages below a sequence's row_ctx may be written by the kernel right before (prompt chunks of one prefill pass).
+laser_status attention_tma_launch(laser_model* m, laser_kv* kv, int layer, const int32_t* seq_ids, int B, int Rs, bool tree, bool fresh,
                                   cudaStream_t stream);
 
-// Prompt processing: the verify forward without the LM head over B sequences of Rs rows each (any Rs with
-// B * Rs inside the model's row workspace); K and V of the rows go to the cache, lengths are not changed.
-laser_status prefill_rows(laser_model* m, laser_kv* kv, const int32_t* seq_ids, const int32_t* tokens,
-                          const int32_t* n_rows, int32_t B, int32_t Rs, cudaStream_t stream);
-
+// Prompt processing: the verify forward without the LM head over chunks of up to kPrefillChunk prompt tokens.  Chunk i is
+// n_rows[i] tokens of cache slot seq_ids[i] from position start[i] on; chunks of one prompt may share a call, in any order:
+// every layer caches the K and V of all of them before its attention.  K and V of the rows go to the cache, lengths are not
+// changed.  n_chunks * kPrefillChunk rows at most m->R_cap.
+laser_status prefill_chunks(laser_model* m, laser_kv* kv, const int32_t* seq_ids, const int32_t* start, const int32_t* tokens,
+                            const int32_t* n_rows, int32_t n_chunks, cudaStream_t stream);
 
 // The verify forward with acceptance fused into the LM head: per (row, 128-token vocabulary tile) the tile's
 // top_n (1..4) largest logits and ids, with `sums` the tile's sum of exp(l - tile max), and per row the logit of
