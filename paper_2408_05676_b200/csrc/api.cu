@@ -23,7 +23,68 @@ constexpr int kMaxDevices = 64;
 struct Scratch { void* ptr = nullptr; size_t bytes = 0; };
 Scratch g_scratch[kMaxDevices][SCRATCH_SLOTS];
 std::mutex g_scratch_mu;
+cudaMemPool_t g_pool[kMaxDevices] = {};
+std::mutex g_pool_mu;
+constexpr uint64_t kPoolKeeps = uint64_t(2) << 30;
+
+// The current device's memory pool (null when `make` is false and there is none).
+laser_status current_pool(bool make, cudaMemPool_t* out) {
+  int dev = 0;
+  LASER_CUDA(cudaGetDevice(&dev));
+  if (dev < 0 || dev >= kMaxDevices) { set_error("device index %d out of range", dev); return LASER_ERR_UNSUPPORTED; }
+  std::lock_guard<std::mutex> lock(g_pool_mu);
+  if (!g_pool[dev] && make) {
+    cudaMemPoolProps props = {};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = dev;
+    cudaMemPool_t pool = nullptr;
+    LASER_CUDA(cudaMemPoolCreate(&pool, &props));
+    uint64_t keep = kPoolKeeps;
+    cudaError_t e = cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+    if (e != cudaSuccess) { cudaMemPoolDestroy(pool); LASER_CUDA(e); }
+    g_pool[dev] = pool;
+  }
+  *out = g_pool[dev];
+  return LASER_OK;
+}
+
+// Gives the pool's unused memory back to the device.
+void trim_pool() {
+  cudaMemPool_t pool = nullptr;
+  if (current_pool(false, &pool) != LASER_OK || !pool) return;
+  cudaDeviceSynchronize();
+  cudaMemPoolTrimTo(pool, 0);
+}
 }  // namespace
+
+laser_status pooled_alloc(void** p, size_t bytes, cudaStream_t stream) {
+  cudaMemPool_t pool = nullptr;
+  LASER_TRY(current_pool(true, &pool));
+  cudaError_t e = cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, stream);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();
+    trim_pool();
+    e = cudaMallocFromPoolAsync(p, bytes ? bytes : 1, pool, stream);
+    if (e != cudaSuccess) cudaGetLastError();
+  }
+  LASER_CUDA(e);
+  return LASER_OK;
+}
+
+void pooled_free(void* p, cudaStream_t stream) {
+  if (p) cudaFreeAsync(p, stream);
+}
+
+cudaError_t device_malloc(void** p, size_t bytes) {
+  cudaError_t e = cudaMalloc(p, bytes);
+  if (e != cudaErrorMemoryAllocation) return e;
+  cudaGetLastError();
+  trim_pool();
+  e = cudaMalloc(p, bytes);
+  if (e != cudaSuccess) cudaGetLastError();
+  return e;
+}
 
 laser_status scratch_get(int slot, size_t bytes, void** out) {
   int dev = 0;
@@ -36,7 +97,7 @@ laser_status scratch_get(int slot, size_t bytes, void** out) {
     if (s.ptr) LASER_CUDA(cudaFree(s.ptr));
     s.ptr = nullptr; s.bytes = 0;
     size_t want = (bytes + 255) & ~size_t(255);
-    LASER_CUDA(cudaMalloc(&s.ptr, want));
+    LASER_CUDA(device_malloc(&s.ptr, want));
     LASER_CUDA(cudaMemset(s.ptr, 0, want));
     s.bytes = want;
   }

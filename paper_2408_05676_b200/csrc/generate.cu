@@ -87,7 +87,7 @@ struct DevBuf {
         m->owned.erase(std::remove(m->owned.begin(), m->owned.end(), m->gen_buf), m->owned.end());
       }
       m->gen_buf = nullptr; m->gen_bytes = 0;
-      LASER_CUDA(cudaMalloc(&m->gen_buf, total));
+      LASER_CUDA(device_malloc(&m->gen_buf, total));
       m->owned.push_back(m->gen_buf);
       m->gen_bytes = total;
     }

@@ -223,7 +223,7 @@ __global__ void set_len_kernel(int32_t* __restrict__ seq_len, const int32_t* __r
 
 template <typename T>
 laser_status model_alloc(laser_model* m, T** p, size_t count) {
-  LASER_CUDA(cudaMalloc(reinterpret_cast<void**>(p), std::max<size_t>(count, 1) * sizeof(T)));
+  LASER_CUDA(device_malloc(reinterpret_cast<void**>(p), std::max<size_t>(count, 1) * sizeof(T)));
   LASER_CUDA(cudaMemset(*p, 0, std::max<size_t>(count, 1) * sizeof(T)));
   m->owned.push_back(*p);
   return LASER_OK;
@@ -388,11 +388,11 @@ LASER_API laser_status laser_kv_create(const laser_model* m, int32_t max_seqs, i
   kv->max_seqs = max_seqs; kv->n_pages = n_pages;
   kv->pages_per_seq = int32_t(std::min<int64_t>(n_pages / max_seqs, 1 << 20));
   const size_t elems = std::max<size_t>(1, size_t(kv->n_layers) * kv->layer_elems());
-  LASER_CUDA(cudaMalloc(reinterpret_cast<void**>(&kv->pages), elems * sizeof(__nv_bfloat16)));
+  LASER_CUDA(device_malloc(reinterpret_cast<void**>(&kv->pages), elems * sizeof(__nv_bfloat16)));
   // masked keys still enter P*V with weight 0, so the pages must never hold NaN/Inf patterns
   LASER_CUDA(cudaMemset(kv->pages, 0, elems * sizeof(__nv_bfloat16)));
-  LASER_CUDA(cudaMalloc(reinterpret_cast<void**>(&kv->page_table), size_t(max_seqs) * kv->pages_per_seq * 4));
-  LASER_CUDA(cudaMalloc(reinterpret_cast<void**>(&kv->seq_len), size_t(max_seqs) * 4));
+  LASER_CUDA(device_malloc(reinterpret_cast<void**>(&kv->page_table), size_t(max_seqs) * kv->pages_per_seq * 4));
+  LASER_CUDA(device_malloc(reinterpret_cast<void**>(&kv->seq_len), size_t(max_seqs) * 4));
   LASER_CUDA(cudaMemset(kv->seq_len, 0, size_t(max_seqs) * 4));
   std::vector<int32_t> table(size_t(max_seqs) * kv->pages_per_seq);
   for (int s = 0; s < max_seqs; ++s)

@@ -2,14 +2,16 @@
 // (Section 3.3).
 //
 // Index: for every n in [n_min, n_max] one open-addressing hash table keyed by a 64-bit
-// hash of (group, n-gram) whose entries point at a run of a position array sorted by
-// (hash, position).  A run lists, ascending, every position where that n-gram ends inside
-// that group - exactly the nodes a per-group trie reaches with the n-gram as prefix, with
-// multiplicity.  A hash collision only merges runs; every position read at lookup time is
-// checked against the actual pool tokens and the group bounds, so results never depend on
-// the hash.
+// hash of (group, n-gram) whose 8-byte entries {low half of the key, start} point at a run of a
+// position array sorted by (hash, position); the last position of a run carries a mark.  A run
+// lists, ascending, every position where that n-gram ends inside that group - exactly the nodes a
+// per-group trie reaches with the n-gram as prefix, with multiplicity.  A key's home slot is its
+// high half scaled to the table, so the sorted keys fill the table from end to end and an insert
+// touches the lines of its neighbours' inserts.  Equal halves of different keys only cost a look at
+// the wrong run, a collision of whole keys only merges runs: every position read at lookup time is
+// checked against the actual pool tokens and the group bounds, so results never depend on the hash.
 //
-// Lookup: one warp per query.  All 32 lanes probe 32 consecutive slots (512 B, coalesced);
+// Lookup: one warp per query.  All 32 lanes probe 32 consecutive slots (256 B, coalesced);
 // the run is read 32 positions at a time, verified, and compacted; the greedy
 // highest-frequency walk votes over at most 64 occurrences held two per lane.  Queries that
 // need more than 64 occurrences (max_occ = 0 or > 64) go to a work list served by one CTA
@@ -20,6 +22,7 @@
 #include <cub/device/device_radix_sort.cuh>
 
 #include <algorithm>
+#include <type_traits>
 
 #include "common.cuh"
 
@@ -27,14 +30,16 @@ struct laser_pool {
   int64_t n_tokens = 0;
   int32_t n_groups = 0, n_min = 0, n_max = 0;
   int32_t vocab_bound = 0;  // largest token id + 1
+  int device = 0;
+  void* memory = nullptr;            // the one device allocation that holds all of the below
   int32_t* tokens = nullptr;         // dev [n_tokens]
   int64_t* group_offsets = nullptr;  // dev [n_groups + 1]
   struct Level {
-    uint4* table = nullptr;    // {key.lo, key.hi, start, count}
-    uint64_t mask = 0;         // slots - 1
-    uint32_t* positions = nullptr;
-    int64_t n_positions = 0, n_keys = 0;
-  } level[9];                  // indexed by n
+    uint2* table = nullptr;          // {key's low half, start of its run}, all ones = empty
+    uint32_t slots = 0;
+    uint32_t* positions = nullptr;   // [n_tokens + 32], runs end with a marked position
+    int64_t n_keys = 0;
+  } level[9];                        // indexed by n
   int64_t device_bytes = 0;
 };
 
@@ -44,6 +49,7 @@ namespace {
 constexpr int kMaxN = 8;
 constexpr int kMaxK = 64;
 constexpr uint64_t kEmpty = ~0ULL;
+constexpr uint32_t kRunEnd = 0x80000000u;   // mark of a run's last position (positions are below 2^31)
 
 __host__ __device__ __forceinline__ uint64_t mix64(uint64_t x) {
   x ^= x >> 30; x *= 0xbf58476d1ce4e5b9ULL;
@@ -58,9 +64,12 @@ __host__ __device__ __forceinline__ uint64_t key_push(uint64_t h, int32_t tok) {
   return mix64(h ^ (uint64_t(uint32_t(tok)) * 0x9E3779B97F4A7C15ULL));
 }
 __host__ __device__ __forceinline__ uint64_t key_end(uint64_t h) { return h == kEmpty ? 0 : h; }
+__device__ __forceinline__ uint32_t home_slot(uint64_t key, uint32_t slots) { return uint32_t(__umul64hi(key, slots)); }
 
-__device__ __forceinline__ int group_of(const int64_t* __restrict__ goff, int G, int64_t p) {
-  int lo = 0, hi = G;  // largest g with goff[g] <= p (skips empty groups)
+constexpr int kKeyThreads = 256;
+
+// Largest g in [lo, hi) with goff[g] <= p (skips empty groups)
+__device__ __forceinline__ int group_of(const int64_t* __restrict__ goff, int lo, int hi, int64_t p) {
   while (hi - lo > 1) {
     int mid = (lo + hi) >> 1;
     if (goff[mid] <= p) lo = mid; else hi = mid;
@@ -68,68 +77,65 @@ __device__ __forceinline__ int group_of(const int64_t* __restrict__ goff, int G,
   return lo;
 }
 
-__global__ void make_keys_kernel(const int32_t* __restrict__ tok, int64_t N,
-                                 const int64_t* __restrict__ goff, int G, int n,
-                                 uint64_t* __restrict__ keys, uint32_t* __restrict__ pos,
-                                 unsigned long long* __restrict__ n_valid, int* __restrict__ max_tok) {
-  int64_t p = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  bool valid = false;
-  uint64_t h = kEmpty;
+// Bound by its 16 bytes a position in and out (10 M positions: 396 -> 40 us; before, every warp added to two counters and every
+// thread searched all groups).  A block's positions are consecutive: two searches bound those of its threads.
+__global__ void __launch_bounds__(kKeyThreads)
+make_keys_kernel(const int32_t* __restrict__ tok, int64_t N, const int64_t* __restrict__ goff, int G, int n,
+                 uint64_t* __restrict__ keys, uint32_t* __restrict__ pos, int* __restrict__ max_tok) {
+  __shared__ int s_g[2], s_max[kKeyThreads / 32];
+  const int64_t p0 = int64_t(blockIdx.x) * kKeyThreads, p = p0 + threadIdx.x;
+  if (threadIdx.x < 2) s_g[threadIdx.x] = group_of(goff, 0, G, min(N - 1, p0 + threadIdx.x * (kKeyThreads - 1)));
+  __syncthreads();
   int mt = -1;
   if (p < N) {
-    const int g = group_of(goff, G, p);
-    valid = (p - n + 1 >= goff[g]);
-    if (valid) {
-      h = key_begin(g, n);
+    const int g = s_g[0] == s_g[1] ? s_g[0] : group_of(goff, s_g[0], s_g[1] + 1, p);
+    bool valid = p - n + 1 >= goff[g];
+    uint64_t h = key_begin(g, n);
+    if (valid)
       for (int j = 0; j < n; ++j) {
         const int32_t t = tok[p - n + 1 + j];
         if (t < 0) { valid = false; break; }
         h = key_push(h, t);
       }
-      h = valid ? key_end(h) : kEmpty;
-    }
-    mt = tok[p];
-    keys[p] = h;
+    keys[p] = valid ? key_end(h) : kEmpty;
     pos[p] = uint32_t(p);
+    mt = max_tok ? tok[p] : -1;
   }
-  const unsigned ball = __ballot_sync(0xffffffffu, valid);
-  for (int o = 16; o; o >>= 1) mt = max(mt, __shfl_xor_sync(0xffffffffu, mt, o));
-  if ((threadIdx.x & 31) == 0) {
-    if (ball) atomicAdd(n_valid, (unsigned long long)__popc(ball));
-    atomicMax(max_tok, mt);
-  }
-}
-
-__global__ void count_heads_kernel(const uint64_t* __restrict__ keys, int64_t n,
-                                   unsigned long long* __restrict__ n_heads) {
-  int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  const bool head = i < n && (i == 0 || keys[i] != keys[i - 1]);
-  const unsigned ball = __ballot_sync(0xffffffffu, head);
-  if ((threadIdx.x & 31) == 0 && ball) atomicAdd(n_heads, (unsigned long long)__popc(ball));
-}
-
-__global__ void insert_heads_kernel(const uint64_t* __restrict__ keys, int64_t n,
-                                    uint4* __restrict__ table, uint64_t mask) {
-  int64_t i = int64_t(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i >= n) return;
-  const uint64_t k = keys[i];
-  if (i != 0 && keys[i - 1] == k) return;
-  int64_t lo = i, hi = n;  // hi -> first index with a different key
-  while (hi - lo > 1) {
-    int64_t mid = (lo + hi) >> 1;
-    if (keys[mid] == k) lo = mid; else hi = mid;
-  }
-  const uint32_t count = uint32_t(hi - i);
-  unsigned long long* slots = reinterpret_cast<unsigned long long*>(table);
-  uint64_t s = k & mask;
-  for (uint64_t tries = 0; tries <= mask; ++tries, s = (s + 1) & mask) {
-    const unsigned long long old = atomicCAS(&slots[2 * s], (unsigned long long)kEmpty, (unsigned long long)k);
-    if (old == kEmpty) {
-      reinterpret_cast<uint32_t*>(table)[4 * s + 2] = uint32_t(i);
-      reinterpret_cast<uint32_t*>(table)[4 * s + 3] = count;
-      return;
+  if (max_tok) {
+    for (int o = 16; o; o >>= 1) mt = max(mt, __shfl_xor_sync(0xffffffffu, mt, o));
+    if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = mt;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      for (int w = 1; w < kKeyThreads / 32; ++w) mt = max(mt, s_max[w]);
+      if (mt > *max_tok) atomicMax(max_tok, mt);
     }
   }
+}
+
+// Sorted (key, position) pairs to the position array with its run marks, and the first of every run to the table.  Bound by
+// its streams: 16 bytes a position and 8 a distinct key, whose slots ascend with the keys (10 M positions, mean of four levels:
+// count and insert 611 -> 150 us against random 16-byte slots, a search for every run's end and a counter update per warp).
+__global__ void __launch_bounds__(kKeyThreads)
+index_runs_kernel(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ pos, int64_t N, uint32_t* __restrict__ positions,
+                  unsigned long long* __restrict__ table, uint32_t slots, unsigned long long* __restrict__ n_heads) {
+  const int64_t i = int64_t(blockIdx.x) * kKeyThreads + threadIdx.x;
+  bool head = false;
+  if (i < N) {
+    const uint64_t k = keys[i];
+    const bool end = i + 1 == N || keys[i + 1] != k;
+    positions[i] = pos[i] | (end ? kRunEnd : 0u);
+    head = k != kEmpty && (i == 0 || keys[i - 1] != k);
+    if (head) {
+      const unsigned long long entry = (uint64_t(uint32_t(i)) << 32) | uint32_t(k);
+      uint32_t s = home_slot(k, slots);
+      for (uint32_t tries = 0; tries < slots; ++tries) {   // there are more slots than keys
+        if (atomicCAS(&table[s], (unsigned long long)kEmpty, entry) == kEmpty) break;
+        if (++s == slots) s = 0;
+      }
+    }
+  }
+  const int heads = __syncthreads_count(head);
+  if (threadIdx.x == 0 && heads) atomicAdd(n_heads, (unsigned long long)heads);
 }
 
 // ---------------------------------------------------------------------------------------
@@ -137,31 +143,46 @@ struct PoolView {
   const int32_t* tok;
   const int64_t* goff;
   int G;
-  const uint4* table[kMaxN + 1];
-  uint64_t mask[kMaxN + 1];
+  const uint2* table[kMaxN + 1];
+  uint32_t slots[kMaxN + 1];
   const uint32_t* positions[kMaxN + 1];
 };
+
+PoolView view_of(const laser_pool* pool) {
+  PoolView pv{};
+  pv.tok = pool->tokens; pv.goff = pool->group_offsets; pv.G = pool->n_groups;
+  for (int n = pool->n_min; n <= pool->n_max; ++n) {
+    pv.table[n] = pool->level[n].table; pv.slots[n] = pool->level[n].slots;
+    pv.positions[n] = pool->level[n].positions;
+  }
+  return pv;
+}
 
 struct DraftArgs {
   const int32_t* tails; const int32_t* tail_len; const int32_t* group_id;
   int B, K, n_min, n_max, min_draft, max_occ;
   int32_t* draft; int32_t* draft_len; int32_t* match_n;
-  int32_t* work;  // [0] = count, [1..] = query ids for the large-run path
+  int32_t* work;       // large-run path: kWorkHead counters (zero between calls), then (query, suffix length) pairs
+  int64_t n_positions;
 };
 
-// Warp-cooperative probe: returns true and (start, count) if the key is present.
-__device__ __forceinline__ bool probe(const uint4* __restrict__ table, uint64_t mask, uint64_t key,
-                                      int lane, uint32_t& start, uint32_t& count) {
-  uint64_t s = key & mask;
-  for (uint64_t tries = 0; tries <= mask; tries += 32, s = (s + 32) & mask) {
-    const uint4 e = __ldg(&table[(s + lane) & mask]);
-    const uint64_t k = (uint64_t(e.y) << 32) | e.x;
-    const unsigned hit = __ballot_sync(0xffffffffu, k == key);
-    const unsigned empty = __ballot_sync(0xffffffffu, k == kEmpty);
-    if (hit) {  // linear probing without deletions: no empty slot lies before the hit
+// Warp-cooperative probe: the next slot, `off` or more past the key's home, whose entry carries the key's low half.  Returns
+// false when an empty slot comes first (linear probing without deletions: the key is not behind it); else `off` is that slot's.
+__device__ __forceinline__ bool probe(const uint2* __restrict__ table, uint32_t slots, uint64_t key, int lane, uint32_t& off,
+                                      uint32_t& start) {
+  const uint32_t home = home_slot(key, slots);
+  for (; off < slots; off += 32) {
+    uint64_t s = uint64_t(home) + off + lane;
+    if (s >= slots) s -= slots;
+    if (s >= slots) s -= slots;            // (a table has at least 64 slots)
+    const uint2 e = __ldg(&table[s]);
+    const unsigned empty = __ballot_sync(0xffffffffu, e.x == 0xffffffffu && e.y == 0xffffffffu);
+    unsigned hit = __ballot_sync(0xffffffffu, e.x == uint32_t(key) && e.y != 0xffffffffu);
+    if (empty) hit &= (empty & -empty) - 1u;
+    if (hit) {
       const int src = __ffs(hit) - 1;
-      start = __shfl_sync(0xffffffffu, e.z, src);
-      count = __shfl_sync(0xffffffffu, e.w, src);
+      start = __shfl_sync(0xffffffffu, e.y, src);
+      off += src;
       return true;
     }
     if (empty) return false;
@@ -177,12 +198,99 @@ __device__ __forceinline__ bool is_occurrence(const int32_t* __restrict__ tok, i
   return true;
 }
 
+// The group's occurrences of the n tail tokens, ascending, behind the n_occ that s_occ[64] already holds, until there are
+// `cap` (more may be counted, 64 are kept).  All lanes of a warp.
+__device__ __forceinline__ int gather_occurrences(const PoolView& pv, int64_t lo, int64_t hi, const int32_t* tail, int n, uint64_t key,
+                                                  int lane, uint32_t* s_occ, int n_occ, int cap) {
+  const int before = n_occ;
+  uint32_t start;
+  for (uint32_t off = 0; n_occ < cap && n_occ == before && probe(pv.table[n], pv.slots[n], key, lane, off, start); ++off) {
+    for (uint32_t base = start; n_occ < cap; base += 32) {   // (the array is padded: lanes past its end read marked padding)
+      const uint32_t v = pv.positions[n][base + lane];
+      const unsigned ends = __ballot_sync(0xffffffffu, (v & kRunEnd) != 0);
+      const int64_t p = int64_t(v & ~kRunEnd);
+      const bool ok = (!ends || lane < __ffs(ends)) && is_occurrence(pv.tok, lo, hi, p, tail, n);
+      const unsigned ball = __ballot_sync(0xffffffffu, ok);
+      const int slot = n_occ + __popc(ball & ((1u << lane) - 1));
+      if (ok && slot < 64) s_occ[slot] = uint32_t(p);
+      n_occ += __popc(ball);
+      if (ends) break;
+    }
+  }
+  return n_occ;
+}
+
+// The greedy highest-frequency walk over up to 64 occurrences, two a lane (e0, e1; alive a0, a1), from depth `len` on (their
+// tokens up to there agree): at every depth the most frequent next token, ties to the smallest, and the occurrences that
+// continue with it.  An occurrence is a pool position, or with bit 31 an index into the history h[0 .. hl).  Writes the
+// tokens to s_cur and returns the depth reached, at most K.  All lanes of a warp.
+// The tokens of eight depths are requested together, so the walk costs a memory round trip per eight tokens; a vote takes one
+// step per distinct token (the first of those left names it, ballots count it) and stops at a majority, and a lone
+// occurrence is copied.  Each lane comparing its token with all 64 in shared memory cost 400 instructions a depth; 4096 queries
+// on 50 M tokens, max_occ 64: 34.8 -> 17.1 us with this and the 8-byte table entries.
+__device__ __forceinline__ int walk_occurrences(const int32_t* __restrict__ tok, int64_t hi, const int32_t* __restrict__ h, int hl,
+                                                uint32_t e0, uint32_t e1, bool a0, bool a1, int len, int K, int lane, int32_t* s_cur) {
+  auto next = [&](uint32_t e, int j) -> int32_t {
+    if (e & 0x80000000u) {
+      const int idx = int(e & 0x7fffffffu) + j;
+      return idx < hl ? h[idx] : -1;
+    }
+    const int64_t p = int64_t(e) + j;
+    return p < hi ? tok[p] : -1;
+  };
+  unsigned m0 = __ballot_sync(0xffffffffu, a0), m1 = __ballot_sync(0xffffffffu, a1);
+  while (len < K && (m0 | m1)) {
+    if (__popc(m0) + __popc(m1) == 1) {   // lane l copies depths len + 1 + l, ..
+      const uint32_t e = __shfl_sync(0xffffffffu, m0 ? e0 : e1, __ffs(m0 | m1) - 1);
+      for (; len < K; len += 32) {
+        const int32_t t = len + 1 + lane <= K ? next(e, len + 1 + lane) : -1;
+        const unsigned stop = __ballot_sync(0xffffffffu, t < 0);
+        const int n = stop ? __ffs(stop) - 1 : 32;
+        if (lane < n) s_cur[len + lane] = t;
+        if (n < 32) { len += n; break; }
+      }
+      break;
+    }
+    int32_t r0[8], r1[8];
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      r0[u] = a0 && len + 1 + u <= K ? next(e0, len + 1 + u) : -1;
+      r1[u] = a1 && len + 1 + u <= K ? next(e1, len + 1 + u) : -1;
+    }
+    const int base = len;
+#pragma unroll
+    for (int u = 0; u < 8; ++u) {
+      if (len != base + u) continue;      // (stopped)
+      a0 = a0 && r0[u] >= 0; a1 = a1 && r1[u] >= 0;
+      m0 = __ballot_sync(0xffffffffu, a0); m1 = __ballot_sync(0xffffffffu, a1);
+      if (!(m0 | m1) || (u > 0 && __popc(m0) + __popc(m1) == 1)) continue;
+      unsigned l0 = m0, l1 = m1;          // those not counted yet
+      int best = 0, left = __popc(l0) + __popc(l1);
+      int32_t pick = 0;
+      while (left >= best && left > 0) {  // (an equal count may still belong to a smaller token)
+        const int32_t v = __shfl_sync(0xffffffffu, l0 ? r0[u] : r1[u], __ffs(l0 ? l0 : l1) - 1);
+        const unsigned q0 = __ballot_sync(0xffffffffu, a0 && r0[u] == v), q1 = __ballot_sync(0xffffffffu, a1 && r1[u] == v);
+        const int c = __popc(q0) + __popc(q1);
+        if (c > best || (c == best && v < pick)) { best = c; pick = v; }
+        l0 &= ~q0; l1 &= ~q1;
+        left -= c;
+      }
+      if (lane == 0) s_cur[len] = pick;
+      a0 = a0 && r0[u] == pick; a1 = a1 && r1[u] == pick;
+      m0 = __ballot_sync(0xffffffffu, a0); m1 = __ballot_sync(0xffffffffu, a1);
+      ++len;
+    }
+  }
+  __syncwarp();
+  return len;
+}
+
 constexpr int kDraftWarps = 4;
+constexpr int kWorkHead = 3;   // work list: items, next item, CTAs done; then (query, suffix length) pairs
 
 __global__ void __launch_bounds__(kDraftWarps * 32)
 draft_warp_kernel(PoolView pv, DraftArgs a) {
   __shared__ uint32_t s_occ[kDraftWarps][64];
-  __shared__ int32_t s_tok[kDraftWarps][64];
   __shared__ int32_t s_cur[kDraftWarps][kMaxK];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = blockIdx.x * kDraftWarps + warp;
@@ -190,7 +298,7 @@ draft_warp_kernel(PoolView pv, DraftArgs a) {
   int32_t* out = a.draft + size_t(q) * a.K;
   const int g = a.group_id[q];
   int best_len = 0, best_n = 0;
-  bool overflow = false;
+  int overflow = 0;                  // suffix length from which the large-run kernel takes over
   if (g >= 0 && g < pv.G) {
     const int64_t lo = pv.goff[g], hi = pv.goff[g + 1];
     const int tl = min(max(a.tail_len[q], 0), a.n_max);
@@ -204,67 +312,14 @@ draft_warp_kernel(PoolView pv, DraftArgs a) {
         h = key_push(h, tn[j]);
       }
       if (bad) continue;
-      uint32_t start, count;
-      if (!probe(pv.table[n], pv.mask[n], key_end(h), lane, start, count)) continue;
-      const uint32_t* plist = pv.positions[n] + start;
-      // gather verified occurrences, ascending, into s_occ
       const int want = (a.max_occ > 0 && a.max_occ <= 64) ? a.max_occ : 65;
-      int n_occ = 0;
-      for (uint32_t base = 0; base < count && n_occ < want; base += 32) {
-        const uint32_t idx = base + lane;
-        const int64_t p = idx < count ? int64_t(plist[idx]) : -1;
-        const bool ok = idx < count && is_occurrence(pv.tok, lo, hi, p, tn, n);
-        const unsigned ball = __ballot_sync(0xffffffffu, ok);
-        const int slot = n_occ + __popc(ball & ((1u << lane) - 1));
-        if (ok && slot < 64) s_occ[warp][slot] = uint32_t(p);
-        n_occ += __popc(ball);
-      }
-      if (want == 65 && n_occ > 64) { overflow = true; break; }
+      int n_occ = gather_occurrences(pv, lo, hi, tn, n, key_end(h), lane, s_occ[warp], 0, want);
+      if (want == 65 && n_occ > 64) { overflow = n; break; }
       n_occ = min(n_occ, min(want, 64));
       if (n_occ == 0) continue;
       __syncwarp();
-      // greedy highest-frequency walk
-      const int64_t p0 = lane < n_occ ? int64_t(s_occ[warp][lane]) : -1;
-      const int64_t p1 = lane + 32 < n_occ ? int64_t(s_occ[warp][lane + 32]) : -1;
-      bool al0 = p0 >= 0, al1 = p1 >= 0;
-      int len = 0;
-      bool go = true;
-      // The continuation of every occurrence is fetched eight depths at a time, all loads issued before
-      // the first vote: the walk then costs one memory round trip per eight tokens, not one per token.
-      for (int jb = 1; jb <= a.K && go; jb += 8) {
-        int32_t r0[8], r1[8];
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int j = jb + u;
-          r0[u] = (al0 && j <= a.K && p0 + j < hi) ? pv.tok[p0 + j] : -1;
-          r1[u] = (al1 && j <= a.K && p1 + j < hi) ? pv.tok[p1 + j] : -1;
-        }
-#pragma unroll
-        for (int u = 0; u < 8; ++u) {
-          const int j = jb + u;
-          if (j > a.K) { go = false; break; }
-          const int32_t t0 = al0 ? r0[u] : -1, t1 = al1 ? r1[u] : -1;
-          al0 = t0 >= 0; al1 = t1 >= 0;
-          if (!__any_sync(0xffffffffu, al0 || al1)) { go = false; break; }
-          s_tok[warp][lane] = t0;
-          s_tok[warp][lane + 32] = t1;
-          __syncwarp();
-          uint32_t c0 = 0, c1 = 0;
-          for (int e = 0; e < n_occ; ++e) {
-            const int32_t x = s_tok[warp][e];
-            c0 += (x == t0); c1 += (x == t1);
-          }
-          unsigned long long cand = 0;
-          if (al0) cand = (uint64_t(c0) << 32) | uint32_t(0x7fffffff - t0);
-          if (al1) cand = max(cand, (unsigned long long)((uint64_t(c1) << 32) | uint32_t(0x7fffffff - t1)));
-          for (int o = 16; o; o >>= 1) cand = max(cand, __shfl_xor_sync(0xffffffffu, cand, o));
-          const int32_t pick = 0x7fffffff - int32_t(uint32_t(cand));
-          if (lane == 0) s_cur[warp][j - 1] = pick;
-          al0 = al0 && t0 == pick; al1 = al1 && t1 == pick;
-          len = j;
-          __syncwarp();
-        }
-      }
+      const int len = walk_occurrences(pv.tok, hi, nullptr, 0, lane < n_occ ? s_occ[warp][lane] : 0u,
+                                       lane + 32 < n_occ ? s_occ[warp][lane + 32] : 0u, lane < n_occ, lane + 32 < n_occ, 0, a.K, lane, s_cur[warp]);
       if (len > best_len) {
         for (int j = lane; j < len; j += 32) out[j] = s_cur[warp][j];
         best_len = len; best_n = n;
@@ -273,8 +328,12 @@ draft_warp_kernel(PoolView pv, DraftArgs a) {
       if (best_len >= max(a.min_draft, 1)) break;
     }
   }
-  if (overflow) {  // hand the whole query to the large-run kernel
-    if (lane == 0) { const int w = atomicAdd(&a.work[0], 1); a.work[1 + w] = q; }
+  if (overflow) {  // the rest of the query, and the best draft so far, to the large-run kernel
+    if (lane == 0) {
+      const int w = kWorkHead + 2 * atomicAdd(&a.work[0], 1);
+      a.work[w] = q; a.work[w + 1] = overflow;
+      a.draft_len[q] = best_len; a.match_n[q] = best_n;
+    }
     return;
   }
   for (int j = best_len + lane; j < a.K; j += 32) out[j] = -1;
@@ -292,7 +351,6 @@ struct TempArgs {
 __global__ void __launch_bounds__(kDraftWarps * 32)
 draft_temp_kernel(PoolView pv, DraftArgs a, TempArgs t) {
   __shared__ uint32_t s_occ[kDraftWarps][64];
-  __shared__ int32_t s_tok[kDraftWarps][64];
   __shared__ int32_t s_cur[kDraftWarps][kMaxK];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = blockIdx.x * kDraftWarps + warp;
@@ -327,57 +385,12 @@ draft_temp_kernel(PoolView pv, DraftArgs a, TempArgs t) {
       n_occ += __popc(ball);
     }
     n_occ = min(n_occ, cap);
-    uint32_t start = 0, count = 0;
-    if (has_group && n_occ < cap && probe(pv.table[n], pv.mask[n], key_end(key), lane, start, count)) {
-      const uint32_t* plist = pv.positions[n] + start;
-      for (uint32_t base = 0; base < count && n_occ < cap; base += 32) {   // the group, ascending
-        const uint32_t idx = base + lane;
-        const int64_t p = idx < count ? int64_t(plist[idx]) : -1;
-        const bool ok = idx < count && is_occurrence(pv.tok, lo, hi, p, tn, n);
-        const unsigned ball = __ballot_sync(0xffffffffu, ok);
-        const int slot = n_occ + __popc(ball & ((1u << lane) - 1));
-        if (ok && slot < 64) s_occ[warp][slot] = uint32_t(p);
-        n_occ += __popc(ball);
-      }
-      n_occ = min(n_occ, cap);
-    }
+    if (has_group && n_occ < cap)   // the group, ascending
+      n_occ = min(cap, gather_occurrences(pv, lo, hi, tn, n, key_end(key), lane, s_occ[warp], n_occ, cap));
     if (n_occ == 0) continue;
     __syncwarp();
-    // greedy highest-frequency walk over both sources
-    const uint32_t e0 = lane < n_occ ? s_occ[warp][lane] : 0u, e1 = lane + 32 < n_occ ? s_occ[warp][lane + 32] : 0u;
-    bool al0 = lane < n_occ, al1 = lane + 32 < n_occ;
-    auto next_token = [&](uint32_t e, int j) -> int32_t {
-      if (e & 0x80000000u) {
-        const int idx = int(e & 0x7fffffffu) + j;
-        return idx < hl ? h[idx] : -1;
-      }
-      const int64_t p = int64_t(e) + j;
-      return p < hi ? pv.tok[p] : -1;
-    };
-    int len = 0;
-    for (int j = 1; j <= a.K; ++j) {
-      const int32_t t0 = al0 ? next_token(e0, j) : -1;
-      const int32_t t1 = al1 ? next_token(e1, j) : -1;
-      al0 = t0 >= 0; al1 = t1 >= 0;
-      if (!__any_sync(0xffffffffu, al0 || al1)) break;
-      s_tok[warp][lane] = t0;
-      s_tok[warp][lane + 32] = t1;
-      __syncwarp();
-      uint32_t c0 = 0, c1 = 0;
-      for (int e = 0; e < n_occ; ++e) {
-        const int32_t x = s_tok[warp][e];
-        c0 += (x == t0); c1 += (x == t1);
-      }
-      unsigned long long cand = 0;
-      if (al0) cand = (uint64_t(c0) << 32) | uint32_t(0x7fffffff - t0);
-      if (al1) cand = max(cand, (unsigned long long)((uint64_t(c1) << 32) | uint32_t(0x7fffffff - t1)));
-      for (int o = 16; o; o >>= 1) cand = max(cand, __shfl_xor_sync(0xffffffffu, cand, o));
-      const int32_t pick = 0x7fffffff - int32_t(uint32_t(cand));
-      if (lane == 0) s_cur[warp][j - 1] = pick;
-      al0 = al0 && t0 == pick; al1 = al1 && t1 == pick;
-      len = j;
-      __syncwarp();
-    }
+    const int len = walk_occurrences(pv.tok, hi, h, hl, lane < n_occ ? s_occ[warp][lane] : 0u, lane + 32 < n_occ ? s_occ[warp][lane + 32] : 0u,
+                                     lane < n_occ, lane + 32 < n_occ, 0, a.K, lane, s_cur[warp]);
     if (len > best_len) {
       for (int j = lane; j < len; j += 32) out[j] = s_cur[warp][j];
       best_len = len; best_n = n;
@@ -443,20 +456,7 @@ draft_tree_kernel(PoolView pv, DraftArgs a, TempArgs t, int32_t* __restrict__ dr
       n_occ += __popc(ball);
     }
     n_occ = min(n_occ, cap);
-    uint32_t start = 0, count = 0;
-    if (has_group && n_occ < cap && probe(pv.table[n], pv.mask[n], key_end(key), lane, start, count)) {
-      const uint32_t* plist = pv.positions[n] + start;
-      for (uint32_t base = 0; base < count && n_occ < cap; base += 32) {
-        const uint32_t idx = base + lane;
-        const int64_t p = idx < count ? int64_t(plist[idx]) : -1;
-        const bool ok = idx < count && is_occurrence(pv.tok, lo, hi, p, tn, n);
-        const unsigned ball = __ballot_sync(0xffffffffu, ok);
-        const int slot = n_occ + __popc(ball & ((1u << lane) - 1));
-        if (ok && slot < 64) s_occ[slot] = uint32_t(p);
-        n_occ += __popc(ball);
-      }
-      n_occ = min(n_occ, cap);
-    }
+    if (has_group && n_occ < cap) n_occ = min(cap, gather_occurrences(pv, lo, hi, tn, n, key_end(key), lane, s_occ, n_occ, cap));
     if (n_occ == 0) continue;
     __syncwarp();
     // ---- continuations ----
@@ -584,31 +584,39 @@ __global__ void make_tree_rows_kernel(const int32_t* __restrict__ last, const in
   if (j == 0) n_rows[b] = lt < 0 ? 0 : 1 + m;
 }
 
-// Large-run path: one CTA per query, votes through a shared-memory histogram over the
-// vocabulary.  Occurrences are streamed from the run at every depth; one is alive at depth
-// j if its tokens match the tail and its continuation agrees with the draft so far.
-constexpr int kBigThreads = 256;
+// Large-run path: one CTA per query, votes through a shared-memory histogram over the vocabulary.  The run is read once: its
+// occurrences (those whose tokens match the tail) vote on the first token while their positions go to a list in shared
+// memory; from then on only the list is walked, cut after every vote to the occurrences that continue with the winner - a
+// small share of them, as token frequencies fall fast.  A run that overflows the list is read again at every depth, with the
+// draft so far compared, until what is left fits.  Up to 64 survivors are walked by one warp in registers.
+// Bound by the latency of the longest run's passes; 4096 queries on 50 M tokens in 10,000 groups, the warp kernel included:
+// 1350 .. 2650 us (by the box) with three passes over the run at every depth and 256 threads -> 73 us.
+constexpr int kBigThreads = 1024;
+constexpr int kBigUnroll = 4;
+constexpr int kBigList = 4096;      // positions: four a thread
 
 __global__ void __launch_bounds__(kBigThreads)
 draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound) {
-  extern __shared__ uint32_t s_hist[];
+  extern __shared__ uint32_t s_hist[];            // [vocab_bound] votes, all zero between depths; then the list
+  uint32_t* s_list = s_hist + vocab_bound;
   __shared__ int32_t s_cur[kMaxK];
-  __shared__ uint32_t s_start, s_count, s_cut;
-  __shared__ int s_found;
-  __shared__ unsigned long long s_red[kBigThreads / 32];
-  __shared__ uint8_t s_flag[kBigThreads];
+  __shared__ uint32_t s_start, s_off, s_end, s_cut, s_count;
+  __shared__ int s_found, s_item, s_warp_n[kBigThreads / 32];
+  __shared__ unsigned long long s_best;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   for (int v = tid; v < vocab_bound; v += kBigThreads) s_hist[v] = 0;
-  __syncthreads();
   const int n_work = a.work[0];
-  for (int w = blockIdx.x; w < n_work; w += gridDim.x) {
-    const int q = a.work[1 + w];
+  for (;;) {
+    __syncthreads();
+    if (tid == 0) s_item = atomicAdd(&a.work[1], 1);
+    __syncthreads();
+    if (s_item >= n_work) break;
+    const int q = a.work[kWorkHead + 2 * s_item], n_first = a.work[kWorkHead + 2 * s_item + 1];
     int32_t* out = a.draft + size_t(q) * a.K;
     const int g = a.group_id[q];
     const int64_t lo = pv.goff[g], hi = pv.goff[g + 1];
-    const int tl = min(max(a.tail_len[q], 0), a.n_max);
-    int best_len = 0, best_n = 0;
-    for (int n = tl; n >= a.n_min; --n) {
+    int best_len = a.draft_len[q], best_n = a.match_n[q];      // of the longer suffixes, with their draft in `out`
+    for (int n = n_first; n >= a.n_min; --n) {
       int32_t tn[kMaxN];
       bool bad = false;
       uint64_t h = key_begin(g, n);
@@ -618,65 +626,156 @@ draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound) {
         h = key_push(h, tn[j]);
       }
       if (bad) continue;
-      if (warp == 0) {
-        uint32_t st = 0, ct = 0;
-        const bool f = probe(pv.table[n], pv.mask[n], key_end(h), lane, st, ct);
-        if (lane == 0) { s_found = f; s_start = st; s_count = ct; s_cut = ct; }
-      }
-      __syncthreads();
-      const bool found = s_found;
-      const uint32_t count = s_count;
-      const uint32_t* plist = pv.positions[n] + s_start;
-      __syncthreads();
-      if (!found) continue;
-      if (a.max_occ > 0) {  // cut the run after the max_occ-th verified occurrence
-        uint32_t total = 0;
-        for (uint32_t base = 0; base < count; base += kBigThreads) {
-          const uint32_t idx = base + tid;
-          const bool ok = idx < count && is_occurrence(pv.tok, lo, hi, int64_t(plist[idx]), tn, n);
-          s_flag[tid] = ok;
-          const uint32_t c = __syncthreads_count(ok);
-          if (total + c >= uint32_t(a.max_occ)) {
-            if (tid == 0) {
-              uint32_t run = total, i = 0;
-              for (; i < kBigThreads; ++i) { run += s_flag[i]; if (run == uint32_t(a.max_occ)) break; }
-              s_cut = min(count, base + i + 1);
-            }
-            break;
-          }
-          total += c;
-          __syncthreads();
-        }
-        __syncthreads();
-      }
-      const uint32_t cut = s_cut;
       int len = 0;
-      for (int j = 1; j <= a.K; ++j) {
-        unsigned long long cand = 0;
-        for (int phase = 0; phase < 3; ++phase) {
-          for (uint32_t idx = tid; idx < cut; idx += kBigThreads) {
-            const int64_t p = plist[idx];
-            if (!is_occurrence(pv.tok, lo, hi, p, tn, n) || p + j >= hi) continue;
-            bool alive = true;
-            for (int c = 1; c < j; ++c) alive = alive && pv.tok[p + c] == s_cur[c - 1];
-            const int32_t t = pv.tok[p + j];
-            if (!alive || t < 0) continue;
-            if (phase == 0) atomicAdd(&s_hist[t], 1u);
-            else if (phase == 1) cand = max(cand, (unsigned long long)((uint64_t(s_hist[t]) << 32) | uint32_t(0x7fffffff - t)));
-            else s_hist[t] = 0;
+      uint32_t total = 0;                          // verified occurrences of the run
+      for (uint32_t off = 0; total == 0; ++off) {  // (a run of another key with the same low half has none)
+        if (warp == 0) {
+          uint32_t st = 0;
+          const bool f = probe(pv.table[n], pv.slots[n], key_end(h), lane, off, st);
+          if (lane == 0) { s_found = f; s_start = st; s_off = off; s_end = s_cut = 0xffffffffu; }
+        }
+        __syncthreads();
+        if (!s_found) break;
+        off = s_off;
+        const uint32_t* plist = pv.positions[n] + s_start;
+        if (a.max_occ > 0) {                       // the run counts up to its max_occ-th verified occurrence
+          uint32_t seen = 0;
+          for (uint32_t base = 0;; base += kBigThreads) {
+            const uint32_t idx = base + tid;
+            const int64_t left = a.n_positions - int64_t(s_start);
+            const uint32_t v = int64_t(idx) < left ? plist[idx] : kRunEnd;
+            if (v & kRunEnd) atomicMin(&s_end, idx);
+            __syncthreads();
+            const bool ok = idx <= s_end && int64_t(idx) < left && is_occurrence(pv.tok, lo, hi, int64_t(v & ~kRunEnd), tn, n);
+            const unsigned ball = __ballot_sync(0xffffffffu, ok);
+            if (lane == 0) s_warp_n[warp] = __popc(ball);
+            __syncthreads();
+            uint32_t rank = seen + __popc(ball & ((1u << lane) - 1)), all = seen;
+            for (int w = 0; w < kBigThreads / 32; ++w) { if (w < warp) rank += s_warp_n[w]; all += s_warp_n[w]; }
+            if (ok && rank + 1 == uint32_t(a.max_occ)) s_cut = idx;
+            seen = all;
+            const bool more = s_end == 0xffffffffu && seen < uint32_t(a.max_occ);
+            __syncthreads();
+            if (!more) break;
           }
+          if (tid == 0) s_end = 0xffffffffu;
           __syncthreads();
         }
-        for (int o = 16; o; o >>= 1) cand = max(cand, __shfl_xor_sync(0xffffffffu, cand, o));
-        if (lane == 0) s_red[warp] = cand;
-        __syncthreads();
-        cand = 0;
-        for (int x = 0; x < kBigThreads / 32; ++x) cand = max(cand, s_red[x]);
-        __syncthreads();
-        if (cand == 0) break;
-        if (tid == 0) s_cur[j - 1] = 0x7fffffff - int32_t(uint32_t(cand));
-        len = j;
-        __syncthreads();
+        const uint32_t cut = s_cut;
+        // depth j = len + 1 by passes over the run, until the alive occurrences fit the list
+        bool listed = false;
+        for (;;) {
+          const int j = len + 1;
+          if (tid == 0) { s_count = 0; s_best = 0; s_end = 0xffffffffu; }
+          __syncthreads();
+          unsigned long long cand = 0;
+          uint32_t n_ok = 0;
+          for (uint32_t base = 0;; base += kBigThreads * kBigUnroll) {
+            uint32_t v[kBigUnroll];
+#pragma unroll
+            for (int u = 0; u < kBigUnroll; ++u) {
+              const uint32_t idx = base + u * kBigThreads + tid;
+              v[u] = int64_t(s_start) + idx < a.n_positions ? plist[idx] : kRunEnd;
+              if (v[u] & kRunEnd) atomicMin(&s_end, idx);
+            }
+            __syncthreads();
+            const uint32_t end = s_end;
+            int32_t t[kBigUnroll];
+            bool alive[kBigUnroll];
+#pragma unroll
+            for (int u = 0; u < kBigUnroll; ++u) {
+              const uint32_t idx = base + u * kBigThreads + tid;
+              const int64_t p = int64_t(v[u] & ~kRunEnd);
+              alive[u] = idx <= end && idx <= cut && int64_t(s_start) + idx < a.n_positions;
+              t[u] = alive[u] && p + j < hi && p >= lo ? pv.tok[p + j] : -1;
+              if (alive[u]) alive[u] = is_occurrence(pv.tok, lo, hi, p, tn, n);
+              n_ok += alive[u];
+              alive[u] = alive[u] && t[u] >= 0;
+              for (int x = 1; x < j && alive[u]; ++x) alive[u] = pv.tok[p + x] == s_cur[x - 1];
+            }
+#pragma unroll
+            for (int u = 0; u < kBigUnroll; ++u) {
+              if (alive[u]) {
+                const uint32_t votes = atomicAdd(&s_hist[t[u]], 1u) + 1;   // whoever votes last sees the token's full count
+                cand = max(cand, (unsigned long long)((uint64_t(votes) << 32) | uint32_t(0x7fffffff - t[u])));
+              }
+              const unsigned ball = __ballot_sync(0xffffffffu, alive[u]);
+              uint32_t at = 0;
+              if (ball && lane == 0) at = atomicAdd(&s_count, uint32_t(__popc(ball)));
+              at = __shfl_sync(0xffffffffu, at, 0) + __popc(ball & ((1u << lane) - 1));
+              if (alive[u] && at < kBigList) s_list[at] = v[u] & ~kRunEnd;
+            }
+            if (end != 0xffffffffu || base + kBigThreads * kBigUnroll > cut) break;
+            __syncthreads();   // (every thread has read s_end)
+          }
+          for (int o = 16; o; o >>= 1) cand = max(cand, __shfl_xor_sync(0xffffffffu, cand, o));
+          if (lane == 0 && cand) atomicMax(&s_best, cand);
+          const uint32_t verified = __syncthreads_count(n_ok > 0);
+          if (len == 0) total = verified;
+          if (s_best == 0) break;                 // nothing continues
+          for (int x = tid; x < vocab_bound; x += kBigThreads) s_hist[x] = 0;
+          if (tid == 0) s_cur[j - 1] = 0x7fffffff - int32_t(uint32_t(s_best));
+          len = j;
+          listed = s_count <= kBigList;
+          __syncthreads();
+          if (listed || len == a.K) break;
+        }
+        // the list holds the positions alive before the last vote: keep the winner's, then go on with the list alone
+        while (listed && len < a.K) {
+          const int32_t pick = s_cur[len - 1];
+          const uint32_t count = s_count;
+          uint32_t mine[kBigList / kBigThreads];
+          bool keep[kBigList / kBigThreads];
+#pragma unroll
+          for (int u = 0; u < kBigList / kBigThreads; ++u) {
+            const uint32_t idx = u * kBigThreads + tid;
+            mine[u] = idx < count ? s_list[idx] : 0u;
+            keep[u] = idx < count && int64_t(mine[u]) + len < hi && pv.tok[int64_t(mine[u]) + len] == pick;
+          }
+          __syncthreads();
+          if (tid == 0) { s_count = 0; s_best = 0; }
+          __syncthreads();
+          const int j = len + 1;
+          unsigned long long cand = 0;
+          int32_t t[kBigList / kBigThreads];
+#pragma unroll
+          for (int u = 0; u < kBigList / kBigThreads; ++u) {
+            t[u] = keep[u] && int64_t(mine[u]) + j < hi ? pv.tok[int64_t(mine[u]) + j] : -1;
+            keep[u] = t[u] >= 0;
+            const unsigned ball = __ballot_sync(0xffffffffu, keep[u]);
+            uint32_t at = 0;
+            if (ball && lane == 0) at = atomicAdd(&s_count, uint32_t(__popc(ball)));
+            at = __shfl_sync(0xffffffffu, at, 0) + __popc(ball & ((1u << lane) - 1));
+            if (keep[u]) s_list[at] = mine[u];
+          }
+          __syncthreads();
+          if (s_count <= 64) break;
+#pragma unroll
+          for (int u = 0; u < kBigList / kBigThreads; ++u)
+            if (keep[u]) {
+              const uint32_t votes = atomicAdd(&s_hist[t[u]], 1u) + 1;
+              cand = max(cand, (unsigned long long)((uint64_t(votes) << 32) | uint32_t(0x7fffffff - t[u])));
+            }
+          for (int o = 16; o; o >>= 1) cand = max(cand, __shfl_xor_sync(0xffffffffu, cand, o));
+          if (lane == 0 && cand) atomicMax(&s_best, cand);
+          __syncthreads();
+#pragma unroll
+          for (int u = 0; u < kBigList / kBigThreads; ++u)
+            if (keep[u]) s_hist[t[u]] = 0;
+          if (tid == 0) s_cur[j - 1] = 0x7fffffff - int32_t(uint32_t(s_best));
+          len = j;
+          __syncthreads();
+        }
+        if (listed && len < a.K && s_count > 0) {   // up to 64 survivors, all of which have a token at depth len + 1
+          if (warp == 0) {
+            const uint32_t c = s_count;
+            const int l = walk_occurrences(pv.tok, hi, nullptr, 0, lane < c ? s_list[lane] : 0u, lane + 32 < c ? s_list[lane + 32] : 0u,
+                                           lane < c, lane + 32 < c, len, a.K, lane, s_cur);
+            if (lane == 0) s_found = l;
+          }
+          __syncthreads();
+          len = s_found;
+        }
       }
       if (len > best_len) {
         for (int j = tid; j < len; j += kBigThreads) out[j] = s_cur[j];
@@ -687,8 +786,9 @@ draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound) {
     }
     for (int j = best_len + tid; j < a.K; j += kBigThreads) out[j] = -1;
     if (tid == 0) { a.draft_len[q] = best_len; a.match_n[q] = best_len ? best_n : 0; }
-    __syncthreads();
   }
+  // the last CTA leaves the work list empty for the next call
+  if (tid == 0 && atomicAdd(&a.work[2], 1) == int(gridDim.x) - 1) { a.work[0] = 0; a.work[1] = 0; a.work[2] = 0; }
 }
 
 __global__ void make_rows_kernel(const int32_t* __restrict__ last, const int32_t* __restrict__ draft,
@@ -703,21 +803,17 @@ __global__ void make_rows_kernel(const int32_t* __restrict__ last, const int32_t
   if (j == 0) n_rows[b] = lt < 0 ? 0 : 1 + m;
 }
 
-template <typename T>
-laser_status dev_alloc(T** p, size_t count, int64_t* bytes) {
-  LASER_CUDA(cudaMalloc(reinterpret_cast<void**>(p), std::max<size_t>(count, 1) * sizeof(T)));
-  *bytes += int64_t(count * sizeof(T));
-  return LASER_OK;
-}
-
 }  // namespace
 }  // namespace laser
 
 LASER_API laser_status laser_pool_free(laser_pool* pool) {
   if (!pool) return LASER_OK;
-  cudaFree(pool->tokens);
-  cudaFree(pool->group_offsets);
-  for (auto& lv : pool->level) { cudaFree(lv.table); cudaFree(lv.positions); }
+  int dev = 0;
+  const bool other = cudaGetDevice(&dev) == cudaSuccess && dev != pool->device;
+  if (other) cudaSetDevice(pool->device);
+  cudaDeviceSynchronize();                 // lookups on any stream may still read it
+  laser::pooled_free(pool->memory, nullptr);
+  if (other) cudaSetDevice(dev);
   delete pool;
   return LASER_OK;
 }
@@ -739,75 +835,68 @@ LASER_API laser_status laser_pool_build(const int32_t* tokens, int64_t n_tokens,
   P->n_tokens = n_tokens; P->n_groups = n_groups; P->n_min = n_min; P->n_max = n_max;
   struct Guard { laser_pool* p; ~Guard() { if (p) laser_pool_free(p); } } guard{P};
 
-  LASER_TRY(dev_alloc(&P->tokens, size_t(n_tokens), &P->device_bytes));
-  LASER_TRY(dev_alloc(&P->group_offsets, size_t(n_groups) + 1, &P->device_bytes));
-  LASER_CUDA(cudaMemcpyAsync(P->tokens, tokens, size_t(n_tokens) * 4, cudaMemcpyDefault, stream));
-  LASER_CUDA(cudaMemcpyAsync(P->group_offsets, group_offsets, (size_t(n_groups) + 1) * 8,
-                             cudaMemcpyHostToDevice, stream));
+  LASER_CUDA(cudaGetDevice(&P->device));
 
-  // transient build buffers
-  uint64_t *keys = nullptr, *keys_alt = nullptr;
-  uint32_t *pos = nullptr, *pos_alt = nullptr;
-  void* cub_tmp = nullptr;
-  unsigned long long* counters = nullptr;  // [0] valid keys, [1] heads
-  int* max_tok = nullptr;
-  struct Tmp { void** p; ~Tmp() { cudaFree(*p); } };
-  Tmp t1{(void**)&keys}, t2{(void**)&keys_alt}, t3{(void**)&pos}, t4{(void**)&pos_alt},
-      t5{&cub_tmp}, t6{(void**)&counters}, t7{(void**)&max_tok};
+  // One allocation for the index, sized before any key is counted (at most one key per token and level, tables at most 5/8
+  // full), so that the levels run back to back without the host; one for the build's own buffers.
   const size_t N = size_t(n_tokens);
-  LASER_CUDA(cudaMalloc(&keys, N * 8));
-  LASER_CUDA(cudaMalloc(&keys_alt, N * 8));
-  LASER_CUDA(cudaMalloc(&pos, N * 4));
-  LASER_CUDA(cudaMalloc(&pos_alt, N * 4));
-  LASER_CUDA(cudaMalloc(&counters, 16));
-  LASER_CUDA(cudaMalloc(&max_tok, 4));
-  LASER_CUDA(cudaMemsetAsync(max_tok, 0xff, 4, stream));
-  size_t cub_bytes = 0;
-  {
-    cub::DoubleBuffer<uint64_t> kb(keys, keys_alt);
-    cub::DoubleBuffer<uint32_t> vb(pos, pos_alt);
-    LASER_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, cub_bytes, kb, vb, int64_t(N), 0, 64, stream));
-  }
-  LASER_CUDA(cudaMalloc(&cub_tmp, std::max<size_t>(cub_bytes, 16)));
-
-  const int threads = 256;
-  const unsigned blocks = unsigned(ceil_div<size_t>(N, threads));
+  const uint32_t slots = uint32_t(N + N * 3 / 5 + 64);
+  auto padded = [](size_t bytes) { return (bytes + 255) & ~size_t(255); };
+  const size_t b_tok = padded(N * 4), b_goff = padded((size_t(n_groups) + 1) * 8), b_tab = padded(size_t(slots) * 8), b_pos = padded((N + 32) * 4);
+  P->device_bytes = int64_t(b_tok + b_goff + (n_max - n_min + 1) * (b_tab + b_pos));
+  LASER_TRY(pooled_alloc(&P->memory, size_t(P->device_bytes), stream));
+  uint8_t* at = static_cast<uint8_t*>(P->memory);
+  auto take = [&](auto** p, size_t bytes) { *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(at); at += bytes; };
+  take(&P->tokens, b_tok);
+  take(&P->group_offsets, b_goff);
   for (int n = n_min; n <= n_max; ++n) {
     auto& lv = P->level[n];
-    LASER_CUDA(cudaMemsetAsync(counters, 0, 16, stream));
-    make_keys_kernel<<<blocks, threads, 0, stream>>>(P->tokens, n_tokens, P->group_offsets, n_groups, n,
-                                                     keys, pos, counters, max_tok);
+    lv.slots = slots;
+    take(&lv.table, b_tab);
+    take(&lv.positions, b_pos);
+  }
+  LASER_CUDA(cudaMemcpyAsync(P->tokens, tokens, N * 4, cudaMemcpyDefault, stream));
+  LASER_CUDA(cudaMemcpyAsync(P->group_offsets, group_offsets, (size_t(n_groups) + 1) * 8, cudaMemcpyHostToDevice, stream));
+
+  size_t cub_bytes = 0;
+  {
+    cub::DoubleBuffer<uint64_t> kb(nullptr, nullptr);
+    cub::DoubleBuffer<uint32_t> vb(nullptr, nullptr);
+    LASER_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, cub_bytes, kb, vb, int64_t(N), 0, 64, stream));
+  }
+  constexpr size_t kCounters = (kMaxN + 2) * 8;   // distinct keys per level, then the largest token
+  struct Tmp { void* p = nullptr; cudaStream_t s; ~Tmp() { pooled_free(p, s); } } tmp{nullptr, stream};
+  LASER_TRY(pooled_alloc(&tmp.p, 2 * padded(N * 8) + 2 * padded(N * 4) + kCounters + 256 + cub_bytes, stream));
+  at = static_cast<uint8_t*>(tmp.p);
+  uint64_t *keys, *keys_alt;
+  uint32_t *pos, *pos_alt;
+  unsigned long long* counters;
+  uint8_t* cub_tmp;
+  take(&keys, padded(N * 8)); take(&keys_alt, padded(N * 8)); take(&pos, padded(N * 4)); take(&pos_alt, padded(N * 4));
+  take(&counters, padded(kCounters)); take(&cub_tmp, cub_bytes);
+  int* max_tok = reinterpret_cast<int*>(counters + kMaxN + 1);
+  LASER_CUDA(cudaMemsetAsync(counters, 0, kCounters, stream));
+  LASER_CUDA(cudaMemsetAsync(max_tok, 0xff, 4, stream));
+  const unsigned blocks = unsigned(ceil_div<size_t>(N, kKeyThreads));
+  for (int n = n_min; n <= n_max; ++n) {
+    auto& lv = P->level[n];
+    make_keys_kernel<<<blocks, kKeyThreads, 0, stream>>>(P->tokens, n_tokens, P->group_offsets, n_groups, n, keys, pos,
+                                                         n == n_min ? max_tok : nullptr);
     cub::DoubleBuffer<uint64_t> kb(keys, keys_alt);
     cub::DoubleBuffer<uint32_t> vb(pos, pos_alt);
     LASER_CUDA(cub::DeviceRadixSort::SortPairs(cub_tmp, cub_bytes, kb, vb, int64_t(N), 0, 64, stream));
-    unsigned long long h_cnt[2] = {0, 0};
-    LASER_CUDA(cudaMemcpyAsync(h_cnt, counters, 8, cudaMemcpyDeviceToHost, stream));
-    LASER_CUDA(cudaStreamSynchronize(stream));
-    const int64_t n_valid = int64_t(h_cnt[0]);  // invalid keys (all ones) sort to the end
-    count_heads_kernel<<<unsigned(ceil_div<int64_t>(std::max<int64_t>(n_valid, 1), threads)), threads, 0, stream>>>(
-        kb.Current(), n_valid, counters + 1);
-    LASER_CUDA(cudaMemcpyAsync(h_cnt + 1, counters + 1, 8, cudaMemcpyDeviceToHost, stream));
-    LASER_CUDA(cudaStreamSynchronize(stream));
-    lv.n_keys = int64_t(h_cnt[1]);
-    lv.n_positions = n_valid;
-    uint64_t slots = 64;
-    while (slots < 2 * uint64_t(lv.n_keys)) slots <<= 1;
-    lv.mask = slots - 1;
-    LASER_TRY(dev_alloc(&lv.table, size_t(slots), &P->device_bytes));
-    LASER_CUDA(cudaMemsetAsync(lv.table, 0xff, size_t(slots) * sizeof(uint4), stream));
-    LASER_TRY(dev_alloc(&lv.positions, size_t(n_valid), &P->device_bytes));
-    if (n_valid > 0) {
-      LASER_CUDA(cudaMemcpyAsync(lv.positions, vb.Current(), size_t(n_valid) * 4, cudaMemcpyDeviceToDevice, stream));
-      insert_heads_kernel<<<unsigned(ceil_div<int64_t>(n_valid, threads)), threads, 0, stream>>>(
-          kb.Current(), n_valid, lv.table, lv.mask);
-    }
+    LASER_CUDA(cudaMemsetAsync(lv.table, 0xff, size_t(slots) * 8, stream));
+    LASER_CUDA(cudaMemsetAsync(lv.positions + N, 0xff, 32 * 4, stream));
+    index_runs_kernel<<<blocks, kKeyThreads, 0, stream>>>(kb.Current(), vb.Current(), n_tokens, lv.positions,
+                                                          reinterpret_cast<unsigned long long*>(lv.table), slots, counters + n);
+    count_launch(2);
     LASER_CUDA(cudaGetLastError());
-    LASER_CUDA(cudaStreamSynchronize(stream));
   }
-  int h_max = -1;
-  LASER_CUDA(cudaMemcpyAsync(&h_max, max_tok, 4, cudaMemcpyDeviceToHost, stream));
+  unsigned long long h_cnt[kMaxN + 2] = {};
+  LASER_CUDA(cudaMemcpyAsync(h_cnt, counters, kCounters, cudaMemcpyDeviceToHost, stream));
   LASER_CUDA(cudaStreamSynchronize(stream));
-  P->vocab_bound = h_max + 1;
+  for (int n = n_min; n <= n_max; ++n) P->level[n].n_keys = int64_t(h_cnt[n]);
+  P->vocab_bound = int32_t(uint32_t(h_cnt[kMaxN + 1])) + 1;
   guard.p = nullptr;
   *out = P;
   return LASER_OK;
@@ -835,28 +924,23 @@ LASER_API laser_status laser_draft(const laser_pool* pool, const int32_t* tails,
   LASER_REQUIRE(p->max_occ >= 0 && p->min_draft >= 0, "max_occ / min_draft negative");
   if (B == 0) return LASER_OK;
   cudaStream_t stream = as_stream(stream_);
-  PoolView pv{};
-  pv.tok = pool->tokens; pv.goff = pool->group_offsets; pv.G = pool->n_groups;
-  for (int n = pool->n_min; n <= pool->n_max; ++n) {
-    pv.table[n] = pool->level[n].table; pv.mask[n] = pool->level[n].mask;
-    pv.positions[n] = pool->level[n].positions;
-  }
+  const PoolView pv = view_of(pool);
   const bool big = (p->max_occ == 0 || p->max_occ > 64);
-  const size_t smem = size_t(pool->vocab_bound) * sizeof(uint32_t);
-  if (big && smem > 200 * 1024) {
+  const size_t hist = size_t(pool->vocab_bound) * sizeof(uint32_t);
+  if (big && hist > 200 * 1024) {
     set_error("vocabulary bound %d too large for the unlimited-occurrence path", pool->vocab_bound);
     return LASER_ERR_UNSUPPORTED;
   }
   void* scratch = nullptr;
-  LASER_TRY(scratch_get(SCRATCH_DRAFT, sizeof(int32_t) * (size_t(B) + 1), &scratch));
+  if (big) LASER_TRY(scratch_get(SCRATCH_DRAFT, sizeof(int32_t) * (size_t(kWorkHead) + 2 * size_t(B)), &scratch));
   DraftArgs a{tails, tail_len, group_id, B, p->K, p->n_min, p->n_max, p->min_draft, p->max_occ,
-              draft, draft_len, match_n, static_cast<int32_t*>(scratch)};
-  LASER_CUDA(cudaMemsetAsync(scratch, 0, sizeof(int32_t), stream));
+              draft, draft_len, match_n, static_cast<int32_t*>(scratch), pool->n_tokens};
   draft_warp_kernel<<<ceil_div(B, kDraftWarps), kDraftWarps * 32, 0, stream>>>(pv, a);
   count_launch();
   if (big) {
+    const size_t smem = hist + kBigList * sizeof(uint32_t);
     LASER_CUDA(cudaFuncSetAttribute(draft_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-    draft_cta_kernel<<<std::min(B, 296), kBigThreads, smem, stream>>>(pv, a, pool->vocab_bound);
+    draft_cta_kernel<<<std::min(B, 148), kBigThreads, smem, stream>>>(pv, a, pool->vocab_bound);
     count_launch();
   }
   LASER_CUDA(cudaGetLastError());
@@ -877,14 +961,9 @@ LASER_API laser_status laser_draft_temp(const laser_pool* pool, const int32_t* t
                 "max_occ = %d: the temporary-branch draft keeps 1..64 occurrences", p->max_occ);
   if (B == 0) return LASER_OK;
   cudaStream_t stream = as_stream(stream_);
-  PoolView pv{};
-  pv.tok = pool->tokens; pv.goff = pool->group_offsets; pv.G = pool->n_groups;
-  for (int n = pool->n_min; n <= pool->n_max; ++n) {
-    pv.table[n] = pool->level[n].table; pv.mask[n] = pool->level[n].mask;
-    pv.positions[n] = pool->level[n].positions;
-  }
+  const PoolView pv = view_of(pool);
   DraftArgs a{tails, tail_len, group_id, B, p->K, p->n_min, p->n_max, p->min_draft, p->max_occ,
-              draft, draft_len, match_n, nullptr};
+              draft, draft_len, match_n, nullptr, pool->n_tokens};
   TempArgs t{hist, hist_len, hist_stride};
   draft_temp_kernel<<<ceil_div(B, kDraftWarps), kDraftWarps * 32, 0, stream>>>(pv, a, t);
   count_launch();
@@ -906,14 +985,9 @@ LASER_API laser_status laser_draft_tree(const laser_pool* pool, const int32_t* t
   LASER_REQUIRE(p->max_occ >= 1 && p->max_occ <= 64 && p->min_draft >= 0,
                 "max_occ = %d: tree drafting keeps 1..64 occurrences", p->max_occ);
   if (B == 0) return LASER_OK;
-  PoolView pv{};
-  pv.tok = pool->tokens; pv.goff = pool->group_offsets; pv.G = pool->n_groups;
-  for (int n = pool->n_min; n <= pool->n_max; ++n) {
-    pv.table[n] = pool->level[n].table; pv.mask[n] = pool->level[n].mask;
-    pv.positions[n] = pool->level[n].positions;
-  }
+  const PoolView pv = view_of(pool);
   DraftArgs a{tails, tail_len, group_id, B, p->K, p->n_min, p->n_max, p->min_draft, p->max_occ,
-              draft, draft_len, match_n, nullptr};
+              draft, draft_len, match_n, nullptr, pool->n_tokens};
   TempArgs t{hist, hist_len, hist_stride};
   draft_tree_kernel<<<B, 32, 0, as_stream(stream_)>>>(pv, a, t, draft_parents);
   count_launch();

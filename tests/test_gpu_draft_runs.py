@@ -1,0 +1,58 @@
+"""Long runs of the retrieval index (csrc/pool.cu): lookups whose occurrences fill one warp, overflow to the kernel with the
+vocabulary histogram, overflow that kernel's list for one or several depths, or are cut by max_occ anywhere on the way."""
+import numpy as np
+import pytest
+
+from helpers import dev_i32, ensure_built
+from oracle import retrieval as R
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    ensure_built()
+    from paper_2408_05676_b200 import binding
+    return binding
+
+
+def _compare(L, toks, offs, tails, gids, n_max, **prm):
+    pool = L.pool_build(toks, offs, 1, n_max)
+    p = L.make_params(n_min=1, n_max=n_max, **prm)
+    B = len(tails)
+    tails, lens, gids = np.asarray(tails, np.int32), np.full(B, n_max, np.int32), np.asarray(gids, np.int32)
+    want = R.draft_batch(toks, offs, tails, lens, gids, p.K, 1, n_max, p.min_draft, p.max_occ)
+    for _ in range(2):                         # the work list is left empty by the first call
+        got = L.draft(pool, dev_i32(tails), dev_i32(lens), dev_i32(gids), p)
+        for g, w in zip(got, want):
+            assert (g.cpu().numpy() == w).all()
+
+
+# vocabulary sizes that leave about `run` occurrences of a token in 20 thousand; 2 keeps thousands alive for several depths
+@pytest.mark.parametrize("vocab,n_max,K,max_occ,min_draft", [
+    (2, 2, 20, 0, 1), (2, 3, 64, 5000, 1), (4, 1, 9, 4097, 1), (5, 2, 16, 0, 16), (40, 2, 8, 65, 1), (310, 1, 16, 0, 1), (310, 3, 33, 64, 4),
+])
+def test_runs_of_every_length(L, vocab, n_max, K, max_occ, min_draft):
+    rng = np.random.default_rng(vocab * 100 + K)
+    toks = rng.integers(0, vocab, 20000, dtype=np.int64).astype(np.int32)
+    toks[rng.integers(0, 20000, 12)] = -1                     # documents
+    offs = np.array([0, 15000, 15000, 20000], dtype=np.int64)  # one group is empty
+    B = 6
+    at = rng.integers(10, 14000, B)
+    tails = np.stack([np.maximum(toks[a:a + n_max], 0) for a in at]).astype(np.int32)
+    gids = np.array([0, 0, 2, 0, 1, 2])
+    _compare(L, toks, offs, tails, gids, n_max, K=K, max_occ=max_occ, min_draft=min_draft)
+
+
+@pytest.mark.parametrize("copies", [31, 32, 33, 63, 64, 65, 66])
+def test_a_run_around_one_warp(L, copies):
+    # `copies` documents "7 7 a ..": the winner is decided by counts that span both of a lane's occurrences
+    rng = np.random.default_rng(copies)
+    toks = []
+    for c in range(copies):
+        toks += [7, 8, 20 + c % 3, 30 + c % 2] + rng.integers(40, 60, int(rng.integers(0, 12))).tolist() + [-1]
+    toks = np.array(toks + list(range(100, 140)), dtype=np.int32)
+    offs = np.array([0, len(toks)], dtype=np.int64)
+    for max_occ in (0, 33, 64):
+        _compare(L, toks, offs, np.array([[7, 8], [8, 20], [3, 7]], dtype=np.int32), np.zeros(3, dtype=np.int64), 2, K=12, max_occ=max_occ,
+                 min_draft=1)
