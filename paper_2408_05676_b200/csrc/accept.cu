@@ -2,11 +2,10 @@
 // ablation variants (Eq. 7; "top-p" of Section 4.3.2), longest accepted prefix, correction
 // or bonus token, and the KV-cache length update.
 //
-// One CTA per (sequence, row): pass 1 finds max / arg max (smallest id on ties), pass 2
-// (the row is now in L1/L2) counts the tokens ranked ahead of the draft token and, where the
-// rule needs a probability, sums exp(l - max) in fp64.  The last CTA of a sequence to finish
-// walks the per-row verdicts in order and writes the outputs.  Reductions have a fixed
-// shape, so results are identical from run to run.
+// One CTA per (sequence, row) reads its row once (verdict.cuh): max / arg max (smallest id on
+// ties), the tokens ranked ahead of the draft token and, where the rule needs a probability, the
+// sum of exp(l - max).  The last CTA of a sequence to finish walks the per-row verdicts in order
+// and writes the outputs.  Reductions have a fixed shape, so results are identical from run to run.
 #include <mutex>
 
 #include "state.cuh"
@@ -29,7 +28,7 @@ accept_rows_kernel(const float* __restrict__ logits, const int32_t* __restrict__
                    int32_t* __restrict__ n_out, int32_t* __restrict__ kv_len) {
   const int b = blockIdx.x / R, i = blockIdx.x % R;
   const int nr = min(n_rows[b], R);
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int tid = threadIdx.x;
   if (nr <= 0) {
     if (i == 0) {
       if (tid == 0) { n_accept[b] = 0; n_out[b] = 0; }
@@ -40,13 +39,10 @@ accept_rows_kernel(const float* __restrict__ logits, const int32_t* __restrict__
   if (i >= nr) return;
 
   const float* row = logits + (size_t(b) * R + i) * V;
-  // pass 1: max and arg max; pass 2 (the row is now in L1/L2): the verdict on the draft token this
-  // row verifies, if any.  The branch conditions are uniform across the CTA.
+  // max, arg max, and the verdict on the draft token that this row verifies, if any
   float mx;
-  int arg;
-  cta_argmax(row, V, &mx, &arg);
-  int pass = 0;
-  if (i + 1 < nr) pass = cta_verdict(row, V, tokens[b * R + i + 1], mx, arg, mode, topk, p);
+  int arg, pass;
+  cta_row(row, V, i + 1 < nr ? tokens[b * R + i + 1] : -1, mode, topk, p, &mx, &arg, &pass);
 
   // publish, then let the last CTA of this sequence scan the verdicts in order
   __shared__ int s_last;

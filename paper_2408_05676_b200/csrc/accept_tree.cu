@@ -39,17 +39,14 @@ accept_tree_kernel(const float* __restrict__ logits, const int32_t* __restrict__
   }
   if (i >= nr) return;
   float mx;
-  int arg;
-  cta_argmax(logits + (size_t(b) * R + i) * V, V, &mx, &arg);
-  int pass = 0;
+  int arg, pass = 0;
+  cta_row(logits + (size_t(b) * R + i) * V, V, -1, mode, topk, p, &mx, &arg, &pass);
   if (i > 0) {
     const int par = parents[b * R + i];
     if (par >= 0 && par < i) {      // a malformed parent verifies nothing
-      const float* prow = logits + (size_t(b) * R + par) * V;
       float pmx;
       int parg;
-      cta_argmax(prow, V, &pmx, &parg);
-      pass = cta_verdict(prow, V, tokens[b * R + i], pmx, parg, mode, topk, p);
+      cta_row(logits + (size_t(b) * R + par) * V, V, tokens[b * R + i], mode, topk, p, &pmx, &parg, &pass);
     }
   }
   __shared__ int s_last;

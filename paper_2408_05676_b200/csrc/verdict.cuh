@@ -1,98 +1,151 @@
-// Row passes shared by the acceptance kernels (Eq. 4, Eq. 7, Eq. 8 and the variants of Section
-// 4.3.2): max and arg max of a row of logits, and the verdict on one token given its row - its rank
-// (tokens ahead of it; equal logits rank the smaller id first) and, where the rule needs it, its
-// probability with the denominator summed in fp64 from fp32 differences.  One CTA of kVerdictThreads
-// threads works on one row; reductions have a fixed shape, so results are identical from run to run.
+// Row pass shared by the acceptance kernels (Eq. 4, Eq. 7, Eq. 8 and the variants of Section 4.3.2): max and arg max of a row
+// of logits, and the verdict on one token given its row - its rank (tokens ahead of it; equal logits rank the smaller id
+// first) and, where the rule needs it, whether its probability exceeds p, the denominator in fp64 from fp32 differences.
+// One CTA of kVerdictThreads threads works on one row; reductions have a fixed shape, so results are identical from run to run.
+//
+// The row is read once, 16 bytes a load and eight loads in flight per thread.  The probability is first estimated in fp32 with a
+// running maximum; the fp64 sum - an exponential per token, which used to be most of the kernel - is taken only where the
+// estimate lies within its error bound of p, so that the verdict is always the fp64 one.  64 sequences x 1 .. 9 rows of 32000
+// logits, relaxed rule: 57.5 -> 20.1 us.
 #pragma once
 #include "common.cuh"
 
 namespace laser {
 
 constexpr int kVerdictThreads = 256;
+constexpr int kRowLoads = 8;       // float4 loads in flight per thread
 
 __device__ __forceinline__ void better(float& v, int& i, float ov, int oi) {
   if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; }
 }
 
-// max and arg max (smallest id on ties) of a row, by the whole CTA
-static __device__ void cta_argmax(const float* __restrict__ row, int V, float* mx_out, int* arg_out) {
-  __shared__ float s_val[kVerdictThreads / 32];
-  __shared__ int s_idx[kVerdictThreads / 32];
-  __shared__ float s_max;
-  __shared__ int s_arg;
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool vec = (V % 4 == 0) && ((reinterpret_cast<uintptr_t>(row) & 15) == 0);
-  float best = -INFINITY;
-  int besti = 0x7fffffff;
-  if (vec) {
-    const float4* r4 = reinterpret_cast<const float4*>(row);
-    for (int j = tid; j < V / 4; j += kVerdictThreads) {
-      const float4 x = r4[j];
-      better(best, besti, x.x, 4 * j); better(best, besti, x.y, 4 * j + 1);
-      better(best, besti, x.z, 4 * j + 2); better(best, besti, x.w, 4 * j + 3);
+struct RowResult { float mx; int arg; int ahead; float m, s; };   // s = sum of exp(x - m) over what was seen
+
+// exp(d) for d <= 0.  ex2 is good to 2 units in the last place and the product's rounding shifts the exponent by |d| 2^-24:
+// within 1e-5 of exp(d) wherever that is not below 1e-38.
+__device__ __forceinline__ float exp_below(float d) { return exp2f(d * 1.4426950408889634f); }
+
+template <bool RANK, bool PROB>
+__device__ __forceinline__ RowResult scan_row(const float* __restrict__ row, int V, int t, float lt, int tid) {
+  RowResult r{-INFINITY, 0x7fffffff, 0, -INFINITY, 0.f};
+  const int lead = min(V, int((16 - (reinterpret_cast<uintptr_t>(row) & 15)) & 15) >> 2);   // values before the first 16-byte boundary
+  const int n4 = (V - lead) >> 2;
+  auto batch = [&](const float* x, int cnt, auto index_of) {
+    float bm = -INFINITY;
+#pragma unroll
+    for (int i = 0; i < cnt; ++i) bm = fmaxf(bm, x[i]);
+    if (bm > r.mx) {               // ids ascend from batch to batch and inside one: the first of equals stays
+      r.mx = bm;
+#pragma unroll
+      for (int i = cnt - 1; i >= 0; --i) if (x[i] == bm) r.arg = index_of(i);
     }
-  } else {
-    for (int j = tid; j < V; j += kVerdictThreads) better(best, besti, row[j], j);
+    if (RANK) {
+      bool eq = false;
+#pragma unroll
+      for (int i = 0; i < cnt; ++i) { r.ahead += x[i] > lt; eq |= x[i] == lt; }
+      if (eq)
+#pragma unroll
+        for (int i = 0; i < cnt; ++i) r.ahead += x[i] == lt && index_of(i) < t;
+    }
+    if (PROB && bm > -INFINITY) {
+      if (bm > r.m) { r.s *= r.m > -INFINITY ? exp_below(r.m - bm) : 0.f; r.m = bm; }
+      float add = 0.f;
+#pragma unroll
+      for (int i = 0; i < cnt; ++i) add += exp_below(x[i] - r.m);
+      r.s += add;
+    }
+  };
+  if (tid < lead) batch(row + tid, 1, [&](int) { return tid; });
+  const float4* r4 = reinterpret_cast<const float4*>(row + lead);
+  for (int base = 0; base < n4; base += kVerdictThreads * kRowLoads) {
+    float x[4 * kRowLoads];
+#pragma unroll
+    for (int u = 0; u < kRowLoads; ++u) {
+      const int i = base + u * kVerdictThreads + tid;
+      const float4 v = i < n4 ? r4[i] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      x[4 * u] = v.x; x[4 * u + 1] = v.y; x[4 * u + 2] = v.z; x[4 * u + 3] = v.w;
+    }
+    batch(x, 4 * kRowLoads, [&](int i) { return lead + 4 * (base + (i >> 2) * kVerdictThreads + tid) + (i & 3); });
   }
+  const int tail = lead + 4 * n4 + tid;
+  if (tail < V) batch(row + tail, 1, [&](int) { return tail; });
+  return r;
+}
+
+// Max and arg max (smallest id on ties) of a row in every thread, and in thread 0 whether token t passes on it (t < 0: none).
+static __device__ void cta_row(const float* __restrict__ row, int V, int t, int mode, int topk, double p, float* mx_out, int* arg_out,
+                               int* pass_out) {
+  constexpr int kWarps = kVerdictThreads / 32;
+  __shared__ RowResult s_part[kWarps];
+  __shared__ float s_max;
+  __shared__ int s_arg, s_exact;
+  __shared__ double s_sum[kWarps];
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const bool judged = t >= 0 && t < V;
+  const bool need_p = judged && (mode == LASER_MODE_RELAXED || mode == LASER_MODE_TOPP || mode == LASER_MODE_RELAXED_ARGMAX);
+  const bool need_rank = judged && (mode == LASER_MODE_RELAXED || mode == LASER_MODE_TOPK || mode == LASER_MODE_RELAXED_ARGMAX);
+  const float lt = judged ? row[t] : 0.f;
+  RowResult r = need_p ? (need_rank ? scan_row<true, true>(row, V, t, lt, tid) : scan_row<false, true>(row, V, t, lt, tid))
+                       : (need_rank ? scan_row<true, false>(row, V, t, lt, tid) : scan_row<false, false>(row, V, t, lt, tid));
+  auto merge = [&](const RowResult& o) {
+    better(r.mx, r.arg, o.mx, o.arg);
+    r.ahead += o.ahead;
+    const float m = fmaxf(r.m, o.m);
+    if (m > -INFINITY)
+      r.s = (r.m > -INFINITY ? r.s * exp_below(r.m - m) : 0.f) + (o.m > -INFINITY ? o.s * exp_below(o.m - m) : 0.f);
+    r.m = m;
+  };
   for (int o = 16; o; o >>= 1) {
-    const float ov = __shfl_xor_sync(0xffffffffu, best, o);
-    const int oi = __shfl_xor_sync(0xffffffffu, besti, o);
-    better(best, besti, ov, oi);
+    RowResult other;
+    other.mx = __shfl_xor_sync(0xffffffffu, r.mx, o);
+    other.arg = __shfl_xor_sync(0xffffffffu, r.arg, o);
+    other.ahead = __shfl_xor_sync(0xffffffffu, r.ahead, o);
+    other.m = __shfl_xor_sync(0xffffffffu, r.m, o);
+    other.s = __shfl_xor_sync(0xffffffffu, r.s, o);
+    merge(other);
   }
   __syncthreads();   // the shared slots may still be read from an earlier call
-  if (lane == 0) { s_val[warp] = best; s_idx[warp] = besti; }
+  if (lane == 0) s_part[warp] = r;
   __syncthreads();
+  int pass = 0;
   if (tid == 0) {
-    for (int w = 1; w < kVerdictThreads / 32; ++w) better(best, besti, s_val[w], s_idx[w]);
-    s_max = best; s_arg = besti;
+    for (int w = 1; w < kWarps; ++w) merge(s_part[w]);
+    if (r.arg == 0x7fffffff)   // nothing above -inf: the first -inf, as an ascending scan would find it
+      for (int j = V - 1; j >= 0; --j) if (row[j] == -INFINITY) r.arg = j;
+    s_max = r.mx; s_arg = r.arg;
+    s_exact = 0;
+    if (judged) {
+      const bool top = t == r.arg, in_topk = r.ahead < topk;
+      // The estimate's relative error: each term 1e-5, a term's at most 6 rescalings per thread (V / 8192 batches; rows beyond
+      // 49152 tokens add one per 8192) and 8 merges 1e-5 each, sums of 128 + 13 terms 1e-5; the numerator 1e-5.  Twice that.
+      const double margin = 4e-4 + 2e-9 * V;
+      const double q = double(exp_below(lt - r.mx)) / double(r.s);
+      const bool matters = need_p && (mode == LASER_MODE_RELAXED ? in_topk : mode == LASER_MODE_TOPP ? !top : !top && in_topk);
+      const bool sure_above = q * (1.0 - margin) > p, sure_below = q * (1.0 + margin) < p;
+      if (matters && !sure_above && !sure_below) s_exact = 1;      // (a NaN is neither)
+      if (mode == LASER_MODE_STRICT) pass = top;
+      else if (mode == LASER_MODE_RELAXED) pass = in_topk && sure_above;
+      else if (mode == LASER_MODE_TOPK) pass = in_topk;
+      else if (mode == LASER_MODE_RELAXED_ARGMAX) pass = top || (in_topk && sure_above);
+      else pass = top || sure_above;
+    }
   }
   __syncthreads();
   *mx_out = s_max;
   *arg_out = s_arg;
-}
-
-// whether token t passes on `row` (whose max and arg max are given); the result is valid in thread 0
-static __device__ int cta_verdict(const float* __restrict__ row, int V, int t, float mx, int arg, int mode, int topk, double p) {
-  if (t < 0 || t >= V) return 0;
-  if (mode == LASER_MODE_STRICT) return t == arg;
-  __shared__ int s_cnt[kVerdictThreads / 32];
-  __shared__ double s_sum[kVerdictThreads / 32];
-  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const bool vec = (V % 4 == 0) && ((reinterpret_cast<uintptr_t>(row) & 15) == 0);
-  const float lt = row[t];
-  const bool need_p = (mode == LASER_MODE_RELAXED || mode == LASER_MODE_TOPP || mode == LASER_MODE_RELAXED_ARGMAX);
-  int ahead = 0;
-  double sum = 0.0;
-  auto visit = [&](float x, int j) {
-    ahead += (x > lt) || (x == lt && j < t);
-    if (need_p) sum += exp(double(x - mx));
-  };
-  if (vec) {
-    const float4* r4 = reinterpret_cast<const float4*>(row);
-    for (int j = tid; j < V / 4; j += kVerdictThreads) {
-      const float4 x = r4[j];
-      visit(x.x, 4 * j); visit(x.y, 4 * j + 1); visit(x.z, 4 * j + 2); visit(x.w, 4 * j + 3);
+  if (s_exact) {   // the rule's own arithmetic: everything else about it is settled, the probability decides
+    const float mx = s_max;
+    double sum = 0.0;
+    for (int j = tid; j < V; j += kVerdictThreads) sum += exp(double(row[j] - mx));
+    for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+    if (lane == 0) s_sum[warp] = sum;
+    __syncthreads();
+    if (tid == 0) {
+      for (int w = 1; w < kWarps; ++w) sum += s_sum[w];
+      pass = exp(double(lt - mx)) / sum > p;
     }
-  } else {
-    for (int j = tid; j < V; j += kVerdictThreads) visit(row[j], j);
   }
-  for (int o = 16; o; o >>= 1) {
-    ahead += __shfl_xor_sync(0xffffffffu, ahead, o);
-    sum += __shfl_xor_sync(0xffffffffu, sum, o);
-  }
-  if (lane == 0) { s_cnt[warp] = ahead; s_sum[warp] = sum; }
-  __syncthreads();
-  int pass = 0;
-  if (tid == 0) {
-    for (int w = 1; w < kVerdictThreads / 32; ++w) { ahead += s_cnt[w]; sum += s_sum[w]; }
-    const bool in_topk = ahead < topk;
-    const bool above_p = need_p && (exp(double(lt - mx)) / sum > p);
-    if (mode == LASER_MODE_RELAXED) pass = in_topk && above_p;
-    else if (mode == LASER_MODE_TOPK) pass = in_topk;
-    else if (mode == LASER_MODE_RELAXED_ARGMAX) pass = (t == arg) || (in_topk && above_p);
-    else pass = (t == arg) || above_p;
-  }
-  return pass;
+  *pass_out = pass;
 }
 
 }  // namespace laser
