@@ -9,6 +9,13 @@
 // 16 rows per sequence (TPC = 1) the four warps take pages round-robin; with more rows (K + 1 > 16
 // or a large token tree, TPC = 2) two warps serve each of two row tiles and both tiles use the same
 // staged page, so a page is still read from HBM once per 32 rows.  Every mbarrier wait is bounded.
+//
+// With few (sequence, head) pairs the walk over one sequence's pages is a latency chain that leaves most SMs idle: up to eight
+// CTAs then take a run of the pages each, and the one that finishes last sums the partial results (through L2, in the order of
+// the runs).  A cluster and distributed shared memory would merge faster, but its CTAs must find their slots together, beside
+// those of the neighbouring kernels: a step of one short sequence lost 4 us a layer to that.
+#include <type_traits>
+
 #include "model.cuh"
 #include "tma.cuh"
 
@@ -19,6 +26,9 @@ using bf16 = __nv_bfloat16;
 constexpr int kConsumers = 4;
 constexpr int kAttnThreads = (kConsumers + 1) * 32;
 constexpr int kStages = 4;   // a multiple of kConsumers: stage s always serves warp s % 4
+constexpr int kMaxPageSplits = 8;  // CTAs that share a sequence's pages
+constexpr int kSplitFrom = 16;      // pages from which a split pays for the merge (about 3 us, ten pages of one CTA's walk),
+constexpr int kSplitPages = 4;      // and pages a run has at least
 constexpr int kCtasPerSm = 4;  // registers and shared memory are sized for four resident CTAs
 
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
@@ -40,16 +50,19 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// PR (precise mode): the queries come in fp32 (qf) and enter the score MMA as hi + lo bf16 pairs, the probabilities
-// enter the value MMA as pairs as well, and the output is written as pairs ([hi | lo] rows of 2 H DH).
-template <int DH, int TPC, bool PR>
+// SP: the pages are split over `splits` CTAs (grid x = sequences x splits).  PR (precise mode): the queries come in fp32 (qf) and
+// enter the score MMA as hi + lo bf16 pairs, the probabilities enter the value MMA as pairs as well, and the output is written
+// as pairs ([hi | lo] rows of 2 H DH).
+template <int DH, int TPC, bool PR, bool SP>
 __global__ void __launch_bounds__(kAttnThreads, PR ? 3 : kCtasPerSm)
 attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restrict__ q, const float* __restrict__ qf,
                   const int32_t* __restrict__ seq_ids, const int32_t* __restrict__ row_ctx,
                   const int32_t* __restrict__ row_n, int Rs, int H, int Hkv,
                   const int32_t* __restrict__ page_table, int pages_per_seq, int layer_row0,
                   bf16* __restrict__ out, int32_t* __restrict__ status,
-                  const unsigned long long* __restrict__ row_mask, int fresh) {
+                  const unsigned long long* __restrict__ row_mask, int fresh, int splits,
+                  float* __restrict__ part, int32_t* __restrict__ arrived) {
+  constexpr int kPartFloats = 16 * TPC * (DH + 2);   // SP: a partial result: O [rows][DH], max [rows], sum [rows]
   constexpr int HALVES = DH / 64;                 // 64-element (128-byte) column blocks per row
   constexpr int SUB = 16 * 128;                   // bytes of one 16-token x 64-element sub-tile
   constexpr int STAGE = 2 * HALVES * SUB;         // K then V
@@ -58,13 +71,14 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
   __shared__ uint64_t full_bar[kStages], empty_bar[kStages];
   __shared__ float s_m[kConsumers][16], s_l[kConsumers][16], s_wgt[kConsumers][16];
   __shared__ int abort_flag;
+  __shared__ int s_last;
 
   // Programmatic dependent launch: let the next kernel start its prologue.  The kernel before this
   // one produces Q and the K/V of the step's own rows; pages that lie wholly below the committed
   // length were written by earlier steps, so the producer requests those before it waits for that
   // kernel, and the wait and the Q tile overlap their flight.
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int b = blockIdx.x, h = blockIdx.y, mt = blockIdx.z;
+  const int b = SP ? blockIdx.x / splits : blockIdx.x, krank = SP ? blockIdx.x % splits : 0, h = blockIdx.y, mt = blockIdx.z;
   const int hk = h / (H / Hkv);
   const int nr = row_n[b], ctx = row_ctx[b];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
@@ -91,7 +105,14 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
   const uint32_t q_smem = tiles + kStages * STAGE;
   bf16* q_ptr = reinterpret_cast<bf16*>(tiles_ptr + kStages * STAGE);
   const int n_keys = ctx + (row_mask ? nr : min(nr, cta_row0 + 16 * TPC));   // chain: no row here sees a later one
-  const int n_pg = (n_keys + 15) >> 4;
+  const int all_pg = (n_keys + 15) >> 4;
+  const int parts = SP ? (all_pg < kSplitFrom ? 1 : min(splits, all_pg / kSplitPages)) : 1;
+  if (SP && krank >= parts) return;
+  const int per = (all_pg + parts - 1) / parts, pg0 = krank * per;
+  const int n_pg = SP ? max(0, min(per, all_pg - pg0)) : all_pg;   // this CTA's pages are pg0 .. pg0 + n_pg - 1
+  const bool whole = !SP || parts == 1;
+  const int unit = (b * H + h) * gridDim.z + mt;
+  float* const my_part = SP ? part + size_t(unit * splits + krank) * kPartFloats : nullptr;
 
   if (tid == 0) {
     abort_flag = 0;
@@ -105,7 +126,7 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
     if (lane == 0) {
       const int32_t* pt = page_table + size_t(seq_ids[b]) * pages_per_seq;
       // whole pages of older tokens that fit the ring (none where the kernel before may have written them)
-      const int n_early = fresh ? 0 : min(min(ctx >> 4, n_pg), kStages);
+      const int n_early = fresh ? 0 : min(min(max(0, (ctx >> 4) - pg0), n_pg), kStages);
       bool ok = true;
       int issued = 0;
       const uint64_t kv_policy = make_policy_evict_first();   // a page is read once per step
@@ -117,7 +138,7 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
         const uint32_t bar = smem_u32(&full_bar[s]);
         const uint32_t dst = tiles + uint32_t(s) * STAGE;
         mbar_expect_tx(bar, STAGE);
-        const int phys = pt[p];
+        const int phys = pt[pg0 + p];
         const int rowk = layer_row0 + ((phys * 2) * Hkv + hk) * 16;
         const int rowv = layer_row0 + ((phys * 2 + 1) * Hkv + hk) * 16;
 #pragma unroll
@@ -202,7 +223,7 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
       }
     }
     // causal mask, online softmax (rows g and g+8 of the tile)
-    const int key0 = p * 16 + 2 * qd;
+    const int key0 = (pg0 + p) * 16 + 2 * qd;
     float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
     for (int t = 0; t < 2; ++t)
@@ -283,6 +304,14 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
     *reinterpret_cast<float2*>(s_o + (warp * 16 + g + 8) * DH + t * 8 + 2 * qd) = make_float2(o[t][2], o[t][3]);
   }
   asm volatile("bar.sync 1, 128;" ::: "memory");
+  auto store_out = [&](int rr, int d, float4 acc) {
+    const __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x, acc.y), hi = __floats2bfloat162_rn(acc.z, acc.w);
+    *reinterpret_cast<uint2*>(obase + size_t(rr) * H * DH * OW + d) =
+        make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
+    if (PR)   // the part of the result that the first bf16 value leaves
+      *reinterpret_cast<uint2*>(obase + size_t(rr) * H * DH * OW + size_t(H) * DH + d) =
+          make_uint2(pack_bf16(acc.x - __low2float(lo), acc.y - __high2float(lo)), pack_bf16(acc.z - __low2float(hi), acc.w - __high2float(hi)));
+  };
   // weight of each warp's partial result per row, normalisation included: e_w / sum_w e_w l_w
   if (tid < 16 * kConsumers) {
     const int r = tid % 16, wsel = tid / 16, tsel = TPC == 1 ? 0 : (wsel & (TPC - 1));
@@ -298,8 +327,13 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
       den += e * s_l[w][r];
       if (w == wsel) mine = e;
     }
-    const bool live = cta_row0 + tsel * 16 + r < nr && den > 0.f && !abort_flag;
-    s_wgt[wsel][r] = live ? mine / den : 0.f;
+    if (!whole) {      // weights against this CTA's max; the runs are weighed against each other below
+      s_wgt[wsel][r] = mine;
+      if (wsel == tsel) { __stcg(my_part + 16 * TPC * DH + tsel * 16 + r, mt_); __stcg(my_part + 16 * TPC * (DH + 1) + tsel * 16 + r, den); }
+    } else {
+      const bool live = cta_row0 + tsel * 16 + r < nr && den > 0.f && !abort_flag;
+      s_wgt[wsel][r] = live ? mine / den : 0.f;
+    }
   }
   asm volatile("bar.sync 1, 128;" ::: "memory");
   for (int idx = tid; idx < 16 * TPC * (DH / 4); idx += kConsumers * 32) {   // four features per thread
@@ -314,12 +348,45 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
       const float4 x = *reinterpret_cast<const float4*>(s_o + (w * 16 + r) * DH + d);
       acc.x += e * x.x; acc.y += e * x.y; acc.z += e * x.z; acc.w += e * x.w;
     }
-    const __nv_bfloat162 lo = __floats2bfloat162_rn(acc.x, acc.y), hi = __floats2bfloat162_rn(acc.z, acc.w);
-    *reinterpret_cast<uint2*>(obase + size_t(rr) * H * DH * OW + d) =
-        make_uint2(*reinterpret_cast<const uint32_t*>(&lo), *reinterpret_cast<const uint32_t*>(&hi));
-    if (PR)   // the part of the result that the first bf16 value leaves
-      *reinterpret_cast<uint2*>(obase + size_t(rr) * H * DH * OW + size_t(H) * DH + d) =
-          make_uint2(pack_bf16(acc.x - __low2float(lo), acc.y - __high2float(lo)), pack_bf16(acc.z - __low2float(hi), acc.w - __high2float(hi)));
+    if (whole) store_out(rr, d, acc);
+    else __stcg(reinterpret_cast<float4*>(my_part + rr * DH + d), acc);
+  }
+  if (!whole) {
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    if (tid == 0) {
+      __threadfence();
+      s_last = atomicAdd(arrived + unit, 1) == parts - 1;
+      __threadfence();
+      if (s_last) arrived[unit] = 0;      // for the next layer
+    }
+    asm volatile("bar.sync 1, 128;" ::: "memory");
+    if (s_last) {   // a warp a row, four features a lane
+      const float* first = part + size_t(unit * splits) * kPartFloats;
+      for (int rr = warp; rr < 16 * TPC && cta_row0 + rr < Rs; rr += kConsumers) {
+        float mx[kMaxPageSplits], den[kMaxPageSplits];
+        float4 x[kMaxPageSplits];
+#pragma unroll
+        for (int q = 0; q < kMaxPageSplits; ++q) {
+          const float* pq = first + size_t(min(q, parts - 1)) * kPartFloats;
+          mx[q] = __ldcg(pq + 16 * TPC * DH + rr);
+          den[q] = __ldcg(pq + 16 * TPC * (DH + 1) + rr);
+          x[q] = 4 * lane < DH ? __ldcg(reinterpret_cast<const float4*>(pq + rr * DH + 4 * lane)) : make_float4(0.f, 0.f, 0.f, 0.f);
+        }
+        float top = -INFINITY, total = 0.f;
+#pragma unroll
+        for (int q = 0; q < kMaxPageSplits; ++q) if (q < parts) top = fmaxf(top, mx[q]);
+        float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int q = 0; q < kMaxPageSplits; ++q) {
+          const float e = q < parts && mx[q] > -INFINITY ? exp2f((mx[q] - top) * sl2) : 0.f;
+          total += e * den[q];
+          acc.x += e * x[q].x; acc.y += e * x[q].y; acc.z += e * x[q].z; acc.w += e * x[q].w;
+        }
+        const float inv = cta_row0 + rr < nr && total > 0.f && !abort_flag ? 1.f / total : 0.f;
+        acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv;
+        if (4 * lane < DH) store_out(rr, 4 * lane, acc);
+      }
+    }
   }
   if (tid == 0 && abort_flag) atomicCAS(status, 0, LASER_ERR_TIMEOUT);
 }
@@ -336,10 +403,18 @@ laser_status attention_tma_launch(laser_model* m, laser_kv* kv, int layer, const
   const int64_t rows_per_layer = int64_t(kv->n_pages) * 2 * Hkv * 16;
   const int layer_row0 = int(rows_per_layer * layer);
   const int tiles = ceil_div(Rs, 16), tpc = tiles > 1 ? 2 : 1;   // row tiles of a sequence; tiles per CTA
+  // Page splits while the grid stays at what the SMs hold at once, where the cache can hold pages enough; what a sequence has
+  // is known on the device alone, and CTAs that find no run to take leave.  7B, 6 layers, 32 / 512 / 1000 cached tokens, one
+  // sequence of 9 rows: 561 / 636 / 707 us unsplit, 560 / 609 / 626 in four, 561 / 605 / 615 in eight; 2 sequences 572 / 650 / 724,
+  // in eight 571 / 622 / 639; 4 sequences 628 / 709 / 779, in four 637 / 701 / 728; 8 sequences 646 / 736 / 822, in two 646 / 726 /
+  // 781.  (A prefill's chunks are many.)
+  const int units = B * H * ceil_div(tiles, tpc), most = kv->pages_per_seq;
+  const int splits = fresh || most < kSplitFrom ? 1 : units * 8 <= kAttnSplitCtas ? 8 : most < 2 * kSplitFrom ? 1 :
+                     units * 4 <= kAttnSplitCtas ? 4 : units * 2 <= kAttnSplitCtas ? 2 : 1;
   const bool pr = m->precise;
   const size_t smem = 1024 + size_t(kStages) * (2 * (dh / 64) * 16 * 128) + size_t(16) * tpc * (dh + 8) * 2 * (pr ? 2 : 1);
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(unsigned(B), unsigned(H), unsigned(ceil_div(tiles, tpc)));
+  cfg.gridDim = dim3(unsigned(B * splits), unsigned(H), unsigned(ceil_div(tiles, tpc)));
   cfg.blockDim = dim3(kAttnThreads, 1, 1);
   cfg.dynamicSmemBytes = smem;
   cfg.stream = stream;
@@ -352,22 +427,21 @@ laser_status attention_tma_launch(laser_model* m, laser_kv* kv, int layer, const
   const int32_t *rc = m->row_ctx, *rn = m->row_n, *pt = kv->page_table;
   const unsigned long long* mask = tree ? m->row_mask : nullptr;
   const float* qf = m->qf;
-#define LASER_ATTN_LAUNCH(DH_, TPC_, PR_)                                                                                \
-  do {                                                                                                                   \
-    LASER_CUDA(cudaFuncSetAttribute(attn_paged_kernel<DH_, TPC_, PR_>, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem))); \
-    LASER_CUDA(cudaLaunchKernelEx(&cfg, attn_paged_kernel<DH_, TPC_, PR_>, kv->pages_map, q, qf, seq_ids, rc, rn, Rs, H, Hkv, pt, \
-                                  kv->pages_per_seq, layer_row0, m->attn, m->status, mask, fresh ? 1 : 0));                              \
-  } while (0)
-  if (pr) {
-    if (dh == 128 && tpc == 1) LASER_ATTN_LAUNCH(128, 1, true);
-    else if (dh == 128) LASER_ATTN_LAUNCH(128, 2, true);
-    else if (tpc == 1) LASER_ATTN_LAUNCH(64, 1, true);
-    else LASER_ATTN_LAUNCH(64, 2, true);
-  } else if (dh == 128 && tpc == 1) LASER_ATTN_LAUNCH(128, 1, false);
-  else if (dh == 128) LASER_ATTN_LAUNCH(128, 2, false);
-  else if (tpc == 1) LASER_ATTN_LAUNCH(64, 1, false);
-  else LASER_ATTN_LAUNCH(64, 2, false);
-#undef LASER_ATTN_LAUNCH
+  auto launch = [&](auto kernel) -> laser_status {
+    LASER_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    LASER_CUDA(cudaLaunchKernelEx(&cfg, kernel, kv->pages_map, q, qf, seq_ids, rc, rn, Rs, H, Hkv, pt, kv->pages_per_seq, layer_row0,
+                                  m->attn, m->status, mask, fresh ? 1 : 0, splits, m->attn_part, m->attn_arrived));
+    return LASER_OK;
+  };
+  auto by_split = [&](auto dh_tag, auto tpc_tag, auto pr_tag) -> laser_status {
+    constexpr int D = decltype(dh_tag)::value, T = decltype(tpc_tag)::value;
+    constexpr bool P = decltype(pr_tag)::value;
+    return splits > 1 ? launch(attn_paged_kernel<D, T, P, true>) : launch(attn_paged_kernel<D, T, P, false>);
+  };
+  auto by_mode = [&](auto dh_tag, auto tpc_tag) { return pr ? by_split(dh_tag, tpc_tag, std::true_type{}) : by_split(dh_tag, tpc_tag, std::false_type{}); };
+  using std::integral_constant;
+  auto by_rows = [&](auto dh_tag) { return tpc == 1 ? by_mode(dh_tag, integral_constant<int, 1>{}) : by_mode(dh_tag, integral_constant<int, 2>{}); };
+  LASER_TRY(dh == 128 ? by_rows(integral_constant<int, 128>{}) : by_rows(integral_constant<int, 64>{}));
   count_launch();
   LASER_CUDA(cudaGetLastError());
   return LASER_OK;

@@ -359,6 +359,8 @@ LASER_API laser_status laser_model_create(const laser_model_cfg* cfg, const lase
   part(&m->top_idx, Rv * v_tiles);
   part(&m->tile_sum, Rv * v_tiles);
   part(&m->status, 1);
+  part(&m->attn_part, size_t(kAttnSplitCtas) * 32 * (cfg->head_dim + 2));
+  part(&m->attn_arrived, kAttnSplitCtas);
   part(&m->pair_scratch, gemm_pair_scratch_floats(m->R_cap));
   part(&m->pair_state, kPairStateInts);
   size_t total = 0;
@@ -489,6 +491,7 @@ LASER_API laser_status laser_check(laser_model* m, void* stream) {
   if (st != 0) {
     LASER_CUDA(cudaMemsetAsync(m->status, 0, 4, as_stream(stream)));
     // (a contraction that gave up may have left its tiles' state)
+    LASER_CUDA(cudaMemsetAsync(m->attn_arrived, 0, kAttnSplitCtas * sizeof(int32_t), as_stream(stream)));
     LASER_CUDA(cudaMemsetAsync(m->pair_state, 0, kPairStateInts * sizeof(int32_t), as_stream(stream)));
     set_error(st == LASER_ERR_CAPACITY ? "a sequence outgrew its KV pages"
               : st == LASER_ERR_TIMEOUT ? "a device-side wait ran out" : "a step was given a bad sequence id");

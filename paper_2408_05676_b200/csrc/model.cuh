@@ -37,6 +37,8 @@ struct laser_model {
   int4* top_idx = nullptr;         // [R_pad][vocab tiles] their token ids
   float* tile_sum = nullptr;       // [R_pad][vocab tiles] sum over the tile of exp(l - tile max)
   int32_t* status = nullptr;       // first device-side error of the stream, 0 = none
+  float* attn_part = nullptr;      // partial attention results where a sequence's pages are split, and arrivals per (sequence, head, tile)
+  int32_t* attn_arrived = nullptr;
   float* pair_scratch = nullptr;   // partial sums of the contractions for many rows (gemm_pair.cu), and the cut tiles' state
   int32_t* pair_state = nullptr;
   void* gemm_state = nullptr;      // tensor-map cache of the tensor-core GEMM
@@ -54,6 +56,7 @@ namespace laser {
 // (7B, 4 layers: 3.6 us a row at 144 rows, 1.6 us at 1024).  16 prompts of 256 .. 1024 tokens and 32 new tokens each, 7B: 456 -> 233
 // ms against passes of 128 rows of one prompt.
 constexpr int kPrefillRows = 1024;
+constexpr int kAttnSplitCtas = 512; // most CTAs of an attention launch that splits pages
 constexpr int kPrefillChunk = 32;   // rows that share each staged K/V page in the attention kernel
 
 // What the GEMM does with a finished 128-feature x NT-row accumulator tile.

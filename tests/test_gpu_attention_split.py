@@ -1,0 +1,50 @@
+"""Attention with a sequence's pages split over a cluster (csrc/attn.cu): page counts on both sides of every split, uneven
+runs, one and several row tiles, chain and tree masks, grouped heads, against the fp64 oracle."""
+import numpy as np
+import pytest
+
+from helpers import dev_i32, ensure_built, weights_to
+from oracle import forward as O
+from paper_2408_05676_b200 import synth
+from test_gpu_forward import TOL, _fill_both, _step
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module")
+def L():
+    ensure_built()
+    from paper_2408_05676_b200 import binding
+    return binding
+
+
+# pages are split from 16 on (256 tokens, the cache holding as many), in up to eight runs of four or more
+@pytest.mark.parametrize("over,ctx,precise", [
+    (dict(), [230], 0), (dict(), [231], 1), (dict(), [247], 1), (dict(), [248, 3], 1), (dict(), [300], 0), (dict(), [640, 77], 1), (dict(), [1000], 0),
+    (dict(max_draft=16), [700], 1), (dict(max_draft=40), [300, 9, 500], 1), (dict(n_kv_heads=2, max_draft=3), [410, 0, 170], 1),
+    (dict(d_model=512, head_dim=128, d_ffn=512), [333], 0),
+])
+def test_split_pages_match_the_oracle(L, over, ctx, precise):
+    cfg = synth.model_cfg("tiny", **dict(over, precise=precise))
+    Wc = synth.make_weights(cfg, seed=0, gain_jitter=0.1)
+    B, K = len(ctx), cfg["max_draft"]
+    pages = max(32, (max(ctx) + K + 16) // 16 + 1)
+    m = L.model_create(cfg, weights_to(Wc, "cuda"), max_batch=B)
+    kv = L.kv_create(m, B, B * pages)
+    L.kv_set_page_table(kv, np.random.default_rng(1).permutation(B * pages).astype(np.int32))
+    okv = O.KVCache(cfg, B, pages * 16)
+    _fill_both(L, cfg, kv, okv, range(B), ctx, seed=7)
+    rows = [synth.make_prompt(K + 1 - b % 2, cfg["vocab"], 30 + b) for b in range(B)]
+    err, logits = _step(L, m, kv, cfg, Wc, okv, list(range(B)), rows)
+    print("max-abs logit error %.2e" % err)
+    assert err <= (TOL / 10 if precise else TOL)
+    # a chain given as a tree uses the row masks instead of the causal limit
+    tokens, parents = np.full((B, K + 1), -1, np.int32), np.full((B, K + 1), -1, np.int32)
+    for b, r in enumerate(rows):
+        tokens[b, :len(r)] = r
+        parents[b, 1:len(r)] = np.arange(len(r) - 1)
+    n_rows = [len(r) for r in rows]
+    tree = L.verify_step_tree(m, kv, dev_i32(range(B)), dev_i32(tokens), dev_i32(parents), dev_i32(n_rows))
+    L.check(m)
+    for b in range(B):
+        assert (tree[b, :n_rows[b]] - logits[b, :n_rows[b]]).abs().max().item() <= (TOL / 100 if precise else TOL / 2)
