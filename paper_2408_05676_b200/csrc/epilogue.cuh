@@ -51,14 +51,14 @@ __device__ __forceinline__ LaneCtx make_lane_ctx(const GemmEpilogue& e, int n0, 
   c.vec_out = c.n + 3 < N && (e.ldo & 3) == 0;
   c.kind = 0; c.idx = 0; c.shift = 0; c.sg = 0.f; c.kv_off = 0; c.rope_off = 0;
   if (EPI == EPI_QKV) {
-    const int dh = e.dh, half = dh >> 1, dq = e.H * dh, dkv = e.Hkv * dh;
+    const int dh = e.dh, half = dh >> 1, dq = e.H * dh, dkv = e.Hkv * dh;   // dh is a power of two
     c.shift = dh >> 3;
     c.kind = c.n < dq ? 0 : (c.n < dq + dkv ? 1 : 2);
-    c.idx = c.n % dh;          // four consecutive features stay inside one half of one head
+    c.idx = c.n & (dh - 1);       // four consecutive features stay inside one half of one head
     c.sg = c.idx < half ? -1.f : 1.f;
-    c.rope_off = (c.idx % half) * 2;
+    c.rope_off = (c.idx & (half - 1)) * 2;
     if (c.kind) {
-      const int h = (c.n - dq - (c.kind - 1) * dkv) / dh;
+      const int h = (c.n - dq - (c.kind - 1) * dkv) >> (31 - __clz(dh));
       c.kv_off = (size_t(c.kind - 1) * e.Hkv + h) * 16 * dh + c.idx;
     }
   }

@@ -23,6 +23,10 @@
 // Variants: activations as hi + lo bf16 pairs (the model's precise mode: every weight block is multiplied with
 // both parts into the same accumulator); and, for the LM head, an epilogue that leaves what the acceptance rule
 // needs per (row, vocabulary tile) instead of the logits.  Steps of many token rows run in gemm_pair.cu.
+// The kernel is compiled per cluster size S and per number RB of rows a warp finishes at once, so that a launch fetches no code
+// it does not run: a step is 129 launches of five kernels that run for 5 .. 30 us each, and instruction fetch is in every one's
+// critical path.  With a switch over S inside the kernel a 7B step of 6 layers took 604 us for 9 rows and 727 for 72; per S
+// and RB 577 and 714; with the drain loop rolled up 570 and 709.
 // Every mbarrier wait is bounded: on expiry the CTA records LASER_ERR_TIMEOUT, drains its
 // copies, still joins the cluster barriers, frees its tensor memory and exits.
 #include <map>
@@ -58,11 +62,14 @@ __device__ __forceinline__ float4 ld_cluster_f4(uint32_t cluster_addr) {
 __device__ __forceinline__ void st_shared_f32(uint32_t addr, float v) {
   asm volatile("st.shared.f32 [%0], %1;" ::"r"(addr), "f"(v));
 }
-template <int EPI>
+// S: CTAs of the cluster = K ranges.  RB: token rows a warp finishes at once (few where the CTA has few, so that all warps have
+// some).
+template <int EPI, int S, int RB>
 __global__ void __launch_bounds__(kTcThreads, 2)
 gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ CUtensorMap tmA, const GemmEpilogue e,
-               int N, int NT, int total_kb, int kb_per_split, int splits, int stages, int tmem_cols,
+               int N, int NT, int total_kb, int kb_per_split, int stages, int tmem_cols,
                int32_t* __restrict__ status) {
+  constexpr int splits = S;
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], acc_bar;
   __shared__ uint32_t tmem_slot;
@@ -127,6 +134,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   // requested now, long before the epilogue uses it
   uint2 gain4 = make_uint2(0u, 0u);
   if (EPI == EPI_RESID && n0 + 4 * lane < N) gain4 = *reinterpret_cast<const uint2*>(e.gain_next + n0 + 4 * lane);
+  const LaneCtx lc = make_lane_ctx<EPI>(e, n0, lane, N);
   bool acc_ok = true;
   // the accumulator from tensor memory to shared memory, token-major [NT][128] (epilogue warps; a warp may
   // only touch its own 32 TMEM lanes)
@@ -134,24 +142,23 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     const int quarter = warp & 3;
     const uint32_t src = tmem_acc + (uint32_t(quarter * 32) << 16);
     const uint32_t dst0 = tiles + uint32_t((quarter * 32 + lane) * 4);
-    for (int c = 0; c < NT; c += 48) {   // three loads in flight, one wait; reads past NT stay inside the allocation
-      uint32_t v0[16], v1[16], v2[16];
+#pragma unroll 1
+    for (int c = 0; c < NT; c += 32) {   // (NT is a multiple of 16; what is read past it stays inside the allocation)
+      uint32_t v0[16], v1[16];
       if (acc_ok && nkb > 0) {
         tmem_ld16(src + uint32_t(c), v0);
-        if (c + 16 < NT) tmem_ld16(src + uint32_t(c + 16), v1);
-        if (c + 32 < NT) tmem_ld16(src + uint32_t(c + 32), v2);
+        tmem_ld16(src + uint32_t(c + 16), v1);
         tmem_ld_wait();
       } else {
 #pragma unroll
-        for (int x = 0; x < 16; ++x) v0[x] = v1[x] = v2[x] = 0u;
+        for (int x = 0; x < 16; ++x) v0[x] = v1[x] = 0u;
       }
       const uint32_t dst = dst0 + uint32_t(c) * (kRow * 4);
 #pragma unroll
-      for (int x = 0; x < 16; ++x) {
-        if (c + x < NT) st_shared_f32(dst + x * (kRow * 4), __uint_as_float(v0[x]));
-        if (c + 16 + x < NT) st_shared_f32(dst + (16 + x) * (kRow * 4), __uint_as_float(v1[x]));
-        if (c + 32 + x < NT) st_shared_f32(dst + (32 + x) * (kRow * 4), __uint_as_float(v2[x]));
-      }
+      for (int x = 0; x < 16; ++x) st_shared_f32(dst + x * (kRow * 4), __uint_as_float(v0[x]));
+      if (c + 16 < NT)
+#pragma unroll
+        for (int x = 0; x < 16; ++x) st_shared_f32(dst + (16 + x) * (kRow * 4), __uint_as_float(v1[x]));
     }
   };
 
@@ -244,7 +251,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   __syncthreads();
   if (splits > 1) cluster_sync_all();  // every partial tile of the cluster is staged
   const int nfeat = n0 + 4 * lane;
-  const LaneCtx lc = make_lane_ctx<EPI>(e, n0, lane, N);
   auto fetch_operands = [&](int jj, float4& g0, float4& g1) {
     g0 = make_float4(0.f, 0.f, 0.f, 0.f); g1 = g0;
     const int r = r0 + krank * slice + jj;
@@ -275,7 +281,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
   } else if ((EPI == EPI_SWIGLU || EPI == EPI_PLAIN) && splits == 1) {
     // part 3 without partial tiles to sum or operands to prefetch: all six warps finish rows,
     // in wide groups whose loads are issued first.
-    constexpr int kWide = 12;
+    constexpr int kWide = RB;
     for (int jb = warp * kWide; jb < NT; jb += (kTcThreads / 32) * kWide) {
       float4 acc[kWide];
 #pragma unroll
@@ -299,8 +305,7 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
     // flight per lane: every partial column of the group and its epilogue operands are requested
     // first (independent loads, one round trip through distributed shared memory), then summed in
     // rank order and finished.
-    auto reduce_rows = [&](auto s_tag, auto rb_tag) {
-      constexpr int S = decltype(s_tag)::value, RB = decltype(rb_tag)::value;
+    {
       uint32_t rank_base[S];
 #pragma unroll
       for (int q = 0; q < S; ++q) rank_base[q] = S > 1 ? map_to_rank(tiles, uint32_t(q)) : tiles;
@@ -331,17 +336,6 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
           else epi_qkv(e, lc, r, live, acc, rstd, s_pos[j], s_page[j], g0[b], g1[b]);
         }
       }
-    };
-    using std::integral_constant;
-    switch (splits) {
-      case 1: reduce_rows(integral_constant<int, 1>{}, integral_constant<int, 6>{}); break;
-      case 2: reduce_rows(integral_constant<int, 2>{}, integral_constant<int, 6>{}); break;
-      case 3: reduce_rows(integral_constant<int, 3>{}, integral_constant<int, 4>{}); break;
-      case 4: reduce_rows(integral_constant<int, 4>{}, integral_constant<int, 3>{}); break;
-      case 5: reduce_rows(integral_constant<int, 5>{}, integral_constant<int, 2>{}); break;
-      case 6: reduce_rows(integral_constant<int, 6>{}, integral_constant<int, 2>{}); break;
-      case 7: reduce_rows(integral_constant<int, 7>{}, integral_constant<int, 2>{}); break;
-      default: reduce_rows(integral_constant<int, 8>{}, integral_constant<int, 1>{}); break;
     }
   }
   __syncwarp();
@@ -354,9 +348,13 @@ gemm_tc_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant__ 
 }
 
 // ---- host side --------------------------------------------------------------------------
+// Which kernels of a model have been given their dynamic shared memory
+struct SizedTable { bool done[5][8][16] = {}; };
+
 struct GemmState {
   // (pointer, rows, cols, box rows) -> tensor map
   std::map<std::tuple<const void*, int, int, int>, CUtensorMap> maps;
+  SizedTable sized;
   bool ready = false, pair_fits = false;
 };
 
@@ -391,9 +389,15 @@ TcShape tc_shape(int R_pad) {
   return s;
 }
 
-template <int EPI>
-laser_status launch_epi(const CUtensorMap& tw, const CUtensorMap& ta, const GemmEpilogue& e, int N, const TcShape& sh,
-                        int n_wtiles, int total_kb, int kbps, int splits, int32_t* status, cudaStream_t stream) {
+template <int EPI, int S, int RB>
+laser_status launch_tc(const CUtensorMap& tw, const CUtensorMap& ta, const GemmEpilogue& e, int N, const TcShape& sh,
+                        int n_wtiles, int total_kb, int kbps, SizedTable& sized_tab, int32_t* status, cudaStream_t stream) {
+  constexpr int splits = S;
+  bool& sized = sized_tab.done[EPI][S - 1][RB];
+  if (!sized) {
+    LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI, S, RB>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget + 2048));
+    sized = true;
+  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(sh.n_ttiles * splits), unsigned(n_wtiles), 1);
   cfg.blockDim = dim3(kTcThreads, 1, 1);
@@ -410,19 +414,42 @@ laser_status launch_epi(const CUtensorMap& tw, const CUtensorMap& ta, const Gemm
   attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 2;
-  LASER_CUDA(cudaLaunchKernelEx(&cfg, gemm_tc_kernel<EPI>, tw, ta, e, N, sh.NT, total_kb, kbps, splits, sh.stages,
+  LASER_CUDA(cudaLaunchKernelEx(&cfg, gemm_tc_kernel<EPI, S, RB>, tw, ta, e, N, sh.NT, total_kb, kbps, sh.stages,
                                 sh.tmem_cols, status));
   return LASER_OK;
 }
 
+template <int EPI, int S>
+laser_status launch_split(const CUtensorMap& tw, const CUtensorMap& ta, const GemmEpilogue& e, int N, const TcShape& sh,
+                          int n_wtiles, int total_kb, int kbps, SizedTable& sized_tab, int32_t* status, cudaStream_t stream) {
+  const int own = ceil_div(sh.NT, S);
+  constexpr bool direct = S == 1 && (EPI == EPI_SWIGLU || EPI == EPI_PLAIN);
+  constexpr int kMany = direct ? 12 : S <= 2 ? 6 : S == 3 ? 4 : S == 4 ? 3 : S == 8 ? 1 : 2;
+  if (direct ? own <= 24 : own <= 12) {
+    if (own <= 6) return launch_tc<EPI, S, 1>(tw, ta, e, N, sh, n_wtiles, total_kb, kbps, sized_tab, status, stream);
+    constexpr int kFew = direct ? 4 : S == 8 ? 1 : 2;
+    return launch_tc<EPI, S, kFew>(tw, ta, e, N, sh, n_wtiles, total_kb, kbps, sized_tab, status, stream);
+  }
+  return launch_tc<EPI, S, kMany>(tw, ta, e, N, sh, n_wtiles, total_kb, kbps, sized_tab, status, stream);
+}
+
+template <int EPI>
+laser_status launch_epi(const CUtensorMap& tw, const CUtensorMap& ta, const GemmEpilogue& e, int N, const TcShape& sh,
+                        int n_wtiles, int total_kb, int kbps, int splits, SizedTable& sized_tab, int32_t* status, cudaStream_t stream) {
+  switch (splits) {
+    case 1: return launch_split<EPI, 1>(tw, ta, e, N, sh, n_wtiles, total_kb, kbps, sized_tab, status, stream);
+    case 2: return launch_split<EPI, 2>(tw, ta, e, N, sh, n_wtiles, total_kb, kbps, sized_tab, status, stream);
+    case 3: return launch_split<EPI, 3>(tw, ta, e, N, sh, n_wtiles, total_kb, kbps, sized_tab, status, stream);
+    case 4: return launch_split<EPI, 4>(tw, ta, e, N, sh, n_wtiles, total_kb, kbps, sized_tab, status, stream);
+    case 5: return launch_split<EPI, 5>(tw, ta, e, N, sh, n_wtiles, total_kb, kbps, sized_tab, status, stream);
+    case 6: return launch_split<EPI, 6>(tw, ta, e, N, sh, n_wtiles, total_kb, kbps, sized_tab, status, stream);
+    case 7: return launch_split<EPI, 7>(tw, ta, e, N, sh, n_wtiles, total_kb, kbps, sized_tab, status, stream);
+    default: return launch_split<EPI, 8>(tw, ta, e, N, sh, n_wtiles, total_kb, kbps, sized_tab, status, stream);
+  }
+}
+
 laser_status prepare(GemmState* st) {
   if (st->ready) return LASER_OK;
-  const int bytes = kSmemBudget + 2048;
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_PLAIN>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_RESID>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_SWIGLU>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_QKV>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-  LASER_CUDA(cudaFuncSetAttribute(gemm_tc_kernel<EPI_VERDICT>, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
   st->pair_fits = gemm_pair_fits();
   st->ready = true;
   return LASER_OK;
@@ -465,7 +492,7 @@ laser_status gemm_fused(laser_model* m, const __nv_bfloat16* A, const __nv_bfloa
   const TcShape sh = tc_shape(R_pad);
   LASER_TRY(tensor_map(st, A, m->R_cap, e.a_lo_off ? 2 * K : K, sh.NT, &ta));
   const int total_kb = ceil_div(K, kBK) * (e.a_lo_off ? 2 : 1), kbps = ceil_div(total_kb, splits);
-  auto launch = [&](auto tag) { return launch_epi<decltype(tag)::value>(*tw, *ta, e, N, sh, n_wtiles, total_kb, kbps, splits, m->status, stream); };
+  auto launch = [&](auto tag) { return launch_epi<decltype(tag)::value>(*tw, *ta, e, N, sh, n_wtiles, total_kb, kbps, splits, st->sized, m->status, stream); };
   using std::integral_constant;
   switch (epi) {
     case EPI_PLAIN: LASER_TRY(launch(integral_constant<int, EPI_PLAIN>{})); break;
