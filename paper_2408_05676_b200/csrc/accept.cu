@@ -20,13 +20,15 @@ constexpr int kMaxAcceptSeqs = 1 << 16;  // counters live at the start of the sc
 struct RowVerdict { int32_t argmax; int32_t pass; };
 
 __global__ void __launch_bounds__(kAcceptThreads)
-accept_rows_kernel(const float* __restrict__ logits, const int32_t* __restrict__ tokens,
-                   const int32_t* __restrict__ n_rows, const int32_t* __restrict__ seq_ids,
+accept_rows_kernel(const float* logits, const int32_t* tokens, const int32_t* n_rows, const int32_t* seq_ids,
                    int32_t R, int32_t V, int32_t mode, int32_t topk, double p,
                    int32_t* __restrict__ counters, RowVerdict* __restrict__ verdicts,
                    int32_t* __restrict__ n_accept, int32_t* __restrict__ out_tokens,
-                   int32_t* __restrict__ n_out, int32_t* __restrict__ kv_len) {
+                   int32_t* __restrict__ n_out, int32_t* __restrict__ kv_len, unsigned long long* stamp) {
   const int b = blockIdx.x / R, i = blockIdx.x % R;
+  next_may_launch();
+  wait_for_earlier();
+  if (stamp && blockIdx.x == 0 && threadIdx.x == 0) *stamp = device_ns();
   const int nr = min(n_rows[b], R);
   const int tid = threadIdx.x;
   if (nr <= 0) {
@@ -126,20 +128,18 @@ LASER_API laser_status laser_accept_commit_noalloc(laser_kv* kv, const int32_t* 
   // the array keeps whatever the previous call left: the arrival counters must start at zero
   LASER_CUDA(cudaMemsetAsync(counters, 0, sizeof(int32_t) * size_t(B), as_stream(stream)));
   const int R = p->K + 1;
-  accept_rows_kernel<<<B * R, kAcceptThreads, 0, as_stream(stream)>>>(
+  LASER_CUDA(launch_overlapped(accept_rows_kernel, dim3(unsigned(B * R)), kAcceptThreads, 0, as_stream(stream),
       logits, tokens, n_rows, seq_ids, R, V, p->mode, p->topk, double(p->p), counters, verdicts,
-      n_accept, out_tokens, n_out, kv ? kv->seq_len : nullptr);
+      n_accept, out_tokens, n_out, kv ? kv->seq_len : nullptr, static_cast<unsigned long long*>(nullptr)));
   count_launch();
   LASER_CUDA(cudaGetLastError());
   return LASER_OK;
 }
 
-LASER_API laser_status laser_accept_commit(laser_kv* kv, const int32_t* seq_ids,
-                                           const float* logits, const int32_t* tokens,
-                                           const int32_t* n_rows, int32_t B, int32_t V,
-                                           const laser_params* p, int32_t* n_accept,
-                                           int32_t* out_tokens, int32_t* n_out, void* stream) {
-  using namespace laser;
+namespace laser {
+laser_status accept_commit(laser_kv* kv, const int32_t* seq_ids, const float* logits, const int32_t* tokens, const int32_t* n_rows,
+                           int32_t B, int32_t V, const laser_params* p, int32_t* n_accept, int32_t* out_tokens, int32_t* n_out,
+                           unsigned long long* stamp, cudaStream_t stream) {
   LASER_REQUIRE(p && logits && tokens && n_rows && n_accept && out_tokens && n_out, "null argument");
   LASER_REQUIRE(B >= 0 && B <= kMaxAcceptSeqs, "B = %d outside [0, %d]", B, kMaxAcceptSeqs);
   LASER_REQUIRE(V >= 1, "V = %d", V);
@@ -155,10 +155,19 @@ LASER_API laser_status laser_accept_commit(laser_kv* kv, const int32_t* seq_ids,
   LASER_TRY(scratch_get(SCRATCH_ACCEPT, counters_bytes + sizeof(RowVerdict) * size_t(B) * R, &scratch));
   int32_t* counters = static_cast<int32_t*>(scratch);
   RowVerdict* verdicts = reinterpret_cast<RowVerdict*>(static_cast<char*>(scratch) + counters_bytes);
-  accept_rows_kernel<<<B * R, kAcceptThreads, 0, as_stream(stream)>>>(
+  LASER_CUDA(launch_overlapped(accept_rows_kernel, dim3(unsigned(B * R)), kAcceptThreads, 0, stream,
       logits, tokens, n_rows, seq_ids, R, V, p->mode, p->topk, double(p->p), counters, verdicts,
-      n_accept, out_tokens, n_out, kv ? kv->seq_len : nullptr);
+      n_accept, out_tokens, n_out, kv ? kv->seq_len : nullptr, stamp));
   count_launch();
   LASER_CUDA(cudaGetLastError());
   return LASER_OK;
+}
+}  // namespace laser
+
+LASER_API laser_status laser_accept_commit(laser_kv* kv, const int32_t* seq_ids,
+                                           const float* logits, const int32_t* tokens,
+                                           const int32_t* n_rows, int32_t B, int32_t V,
+                                           const laser_params* p, int32_t* n_accept,
+                                           int32_t* out_tokens, int32_t* n_out, void* stream) {
+  return laser::accept_commit(kv, seq_ids, logits, tokens, n_rows, B, V, p, n_accept, out_tokens, n_out, nullptr, laser::as_stream(stream));
 }

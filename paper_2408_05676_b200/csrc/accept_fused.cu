@@ -21,15 +21,16 @@ namespace {
 constexpr int kFusedThreads = 256;
 
 __global__ void __launch_bounds__(kFusedThreads)
-accept_fused_kernel(const float4* __restrict__ top_val, const int4* __restrict__ top_idx, const float* __restrict__ tile_sum,
-                    const float* __restrict__ draft_logit, const int32_t* __restrict__ tokens, const int32_t* __restrict__ n_rows,
-                    const int32_t* __restrict__ seq_ids, int32_t R, int32_t V, int32_t n_vtiles, int32_t top_n, int32_t mode,
+accept_fused_kernel(const float4* top_val, const int4* top_idx, const float* tile_sum, const float* draft_logit, const int32_t* tokens,
+                    const int32_t* n_rows, const int32_t* seq_ids, int32_t R, int32_t V, int32_t n_vtiles, int32_t top_n, int32_t mode,
                     int32_t topk, double p, int32_t* __restrict__ n_accept, int32_t* __restrict__ out_tokens,
                     int32_t* __restrict__ n_out, int32_t* __restrict__ kv_len) {
   extern __shared__ int32_t s_row[];   // [R] arg max, [R] verdict
   int32_t* s_arg = s_row;
   int32_t* s_pass = s_row + R;
   const int b = blockIdx.x, tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  next_may_launch();
+  wait_for_earlier();
   const int nr = min(n_rows[b], R);
   if (nr <= 0) {
     if (tid == 0) { n_accept[b] = 0; n_out[b] = 0; }
@@ -121,10 +122,10 @@ LASER_API laser_status laser_verify_accept(laser_model* m, laser_kv* kv, const i
   const int top_n = need_rank ? p->topk : 1;
   LASER_TRY(verify_fused(m, kv, seq_ids, tokens, n_rows, B, logits, top_n, need_p, stream));
   const int R = m->rows_per_seq;
-  accept_fused_kernel<<<B, kFusedThreads, size_t(2) * R * sizeof(int32_t), stream>>>(
+  LASER_CUDA(launch_overlapped(accept_fused_kernel, dim3(unsigned(B)), kFusedThreads, size_t(2) * R * sizeof(int32_t), stream,
       m->top_val, m->top_idx, m->tile_sum, m->draft_logit, tokens, n_rows, seq_ids, R, m->cfg.vocab,
       ceil_div(m->cfg.vocab, 128), top_n, p->mode, p->topk, double(p->p), n_accept, out_tokens, n_out,
-      commit ? kv->seq_len : nullptr);
+      commit ? kv->seq_len : nullptr));
   count_launch();
   LASER_CUDA(cudaGetLastError());
   return LASER_OK;

@@ -22,12 +22,15 @@ constexpr int kMaxTreeRows = 64;
 struct NodeVerdict { int32_t argmax; int32_t pass; };
 
 __global__ void __launch_bounds__(kThreads)
-accept_tree_kernel(const float* __restrict__ logits, const int32_t* __restrict__ tokens,
-                   const int32_t* __restrict__ parents, const int32_t* __restrict__ n_rows, int32_t R, int32_t V,
+accept_tree_kernel(const float* logits, const int32_t* tokens, const int32_t* parents, const int32_t* n_rows, int32_t R, int32_t V,
                    int32_t mode, int32_t topk, double p, int32_t* __restrict__ counters,
                    NodeVerdict* __restrict__ verdicts, int32_t* __restrict__ n_accept,
-                   int32_t* __restrict__ out_tokens, int32_t* __restrict__ n_out, int32_t* __restrict__ path_rows) {
+                   int32_t* __restrict__ out_tokens, int32_t* __restrict__ n_out, int32_t* __restrict__ path_rows,
+                   unsigned long long* stamp) {
+  next_may_launch();
   const int b = blockIdx.x / R, i = blockIdx.x % R;
+  wait_for_earlier();
+  if (stamp && blockIdx.x == 0 && threadIdx.x == 0) *stamp = device_ns();
   const int nr = min(n_rows[b], R);
   const int tid = threadIdx.x;
   if (nr <= 0) {
@@ -95,9 +98,10 @@ accept_tree_kernel(const float* __restrict__ logits, const int32_t* __restrict__
 // rows ascend).  One block per (sequence, layer); a thread owns fixed 16-byte chunks of a token.
 __global__ void compact_path_kernel(__nv_bfloat16* __restrict__ pages, size_t layer_elems, size_t page_elems,
                                     const int32_t* __restrict__ page_table, int pages_per_seq, int Hkv, int dh,
-                                    const int32_t* __restrict__ seq_ids, const int32_t* __restrict__ seq_len,
-                                    const int32_t* __restrict__ path_rows, const int32_t* __restrict__ n_accept,
-                                    int row_stride, int max_seqs, int capacity) {
+                                    const int32_t* seq_ids, const int32_t* seq_len, const int32_t* path_rows,
+                                    const int32_t* n_accept, int row_stride, int max_seqs, int capacity) {
+  next_may_launch();
+  wait_for_earlier();
   const int b = blockIdx.x, layer = blockIdx.y;
   const int seq = seq_ids[b];
   if (seq < 0 || seq >= max_seqs) return;
@@ -118,8 +122,9 @@ __global__ void compact_path_kernel(__nv_bfloat16* __restrict__ pages, size_t la
   }
 }
 
-__global__ void advance_len_kernel(const int32_t* __restrict__ seq_ids, const int32_t* __restrict__ n_out, int B,
-                                   int max_seqs, int32_t* __restrict__ seq_len) {
+__global__ void advance_len_kernel(const int32_t* seq_ids, const int32_t* n_out, int B, int max_seqs, int32_t* seq_len) {
+  next_may_launch();
+  wait_for_earlier();
   const int b = blockIdx.x * blockDim.x + threadIdx.x;
   if (b < B && seq_ids[b] >= 0 && seq_ids[b] < max_seqs) seq_len[seq_ids[b]] += n_out[b];
 }
@@ -135,19 +140,18 @@ LASER_API laser_status laser_kv_compact_path(laser_kv* kv, const int32_t* seq_id
   LASER_REQUIRE(kv->head_dim % 8 == 0, "head_dim = %d is not a multiple of 8", kv->head_dim);
   if (B == 0) return LASER_OK;
   const int capacity = int(std::min<int64_t>(kv->capacity_tokens(), INT32_MAX));
-  compact_path_kernel<<<dim3(unsigned(B), unsigned(kv->n_layers)), 128, 0, as_stream(stream)>>>(
+  LASER_CUDA(launch_overlapped(compact_path_kernel, dim3(unsigned(B), unsigned(kv->n_layers)), 128, 0, as_stream(stream),
       kv->pages, kv->layer_elems(), kv->page_elems(), kv->page_table, kv->pages_per_seq, kv->n_kv_heads, kv->head_dim,
-      seq_ids, kv->seq_len, path_rows, n_accept, row_stride, kv->max_seqs, capacity);
+      seq_ids, kv->seq_len, path_rows, n_accept, row_stride, kv->max_seqs, capacity));
   count_launch();
   LASER_CUDA(cudaGetLastError());
   return LASER_OK;
 }
 
-LASER_API laser_status laser_accept_tree(laser_kv* kv, const int32_t* seq_ids, const float* logits,
-                                         const int32_t* tokens, const int32_t* parents, const int32_t* n_rows,
-                                         int32_t B, int32_t V, const laser_params* p, int32_t* n_accept,
-                                         int32_t* out_tokens, int32_t* n_out, int32_t* path_rows, void* stream) {
-  using namespace laser;
+namespace laser {
+laser_status accept_tree(laser_kv* kv, const int32_t* seq_ids, const float* logits, const int32_t* tokens, const int32_t* parents,
+                         const int32_t* n_rows, int32_t B, int32_t V, const laser_params* p, int32_t* n_accept, int32_t* out_tokens,
+                         int32_t* n_out, int32_t* path_rows, unsigned long long* stamp, cudaStream_t stream) {
   LASER_REQUIRE(p && logits && tokens && parents && n_rows && n_accept && out_tokens && n_out && path_rows, "null argument");
   LASER_REQUIRE(B >= 0 && B <= kMaxSeqs, "B = %d outside [0, %d]", B, kMaxSeqs);
   LASER_REQUIRE(V >= 1, "V = %d", V);
@@ -162,16 +166,25 @@ LASER_API laser_status laser_accept_tree(laser_kv* kv, const int32_t* seq_ids, c
   LASER_TRY(scratch_get(SCRATCH_ACCEPT_TREE, counters_bytes + sizeof(NodeVerdict) * size_t(B) * R, &scratch));
   int32_t* counters = static_cast<int32_t*>(scratch);
   NodeVerdict* verdicts = reinterpret_cast<NodeVerdict*>(static_cast<char*>(scratch) + counters_bytes);
-  accept_tree_kernel<<<B * R, kThreads, 0, as_stream(stream)>>>(logits, tokens, parents, n_rows, R, V, p->mode, p->topk,
-                                                              double(p->p), counters, verdicts, n_accept, out_tokens,
-                                                              n_out, path_rows);
+  LASER_CUDA(launch_overlapped(accept_tree_kernel, dim3(unsigned(B * R)), kThreads, 0, stream, logits, tokens, parents, n_rows,
+                               R, V, p->mode, p->topk, double(p->p), counters, verdicts, n_accept, out_tokens, n_out, path_rows, stamp));
   count_launch();
   LASER_CUDA(cudaGetLastError());
   if (kv) {   // commit: compact the accepted path, then advance the lengths by the emitted tokens
     LASER_TRY(laser_kv_compact_path(kv, seq_ids, path_rows, n_accept, B, R, stream));
-    advance_len_kernel<<<ceil_div(B, 128), 128, 0, as_stream(stream)>>>(seq_ids, n_out, B, kv->max_seqs, kv->seq_len);
+    LASER_CUDA(launch_overlapped(advance_len_kernel, dim3(unsigned(ceil_div(B, 128))), 128, 0, stream, seq_ids, n_out, B,
+                                 kv->max_seqs, kv->seq_len));
     count_launch();
     LASER_CUDA(cudaGetLastError());
   }
   return LASER_OK;
+}
+}  // namespace laser
+
+LASER_API laser_status laser_accept_tree(laser_kv* kv, const int32_t* seq_ids, const float* logits,
+                                         const int32_t* tokens, const int32_t* parents, const int32_t* n_rows,
+                                         int32_t B, int32_t V, const laser_params* p, int32_t* n_accept,
+                                         int32_t* out_tokens, int32_t* n_out, int32_t* path_rows, void* stream) {
+  return laser::accept_tree(kv, seq_ids, logits, tokens, parents, n_rows, B, V, p, n_accept, out_tokens, n_out, path_rows, nullptr,
+                            laser::as_stream(stream));
 }

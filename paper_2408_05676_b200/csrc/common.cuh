@@ -61,4 +61,37 @@ inline cudaStream_t as_stream(void* s) { return reinterpret_cast<cudaStream_t>(s
 template <typename T>
 inline T ceil_div(T a, T b) { return (a + b - 1) / b; }
 
+#ifdef __CUDACC__
+// The small kernels of a step overlap their launches: each is launched while the one before still runs (launch_overlapped),
+// lets the next one be launched from its first instruction on (next_may_launch), and waits for everything before it in the
+// stream before it reads or writes global memory (wait_for_earlier; all of a grid's blocks that do work call it, so that a
+// kernel's end implies the end of every kernel before it).  What a kernel reads after the wait must not be `const
+// __restrict__`: such loads count as invariant and may be moved ahead of it.
+__device__ __forceinline__ void next_may_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void wait_for_earlier() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
+// Device clock in ns, the same on all SMs: the generation loop's stage times are taken by its kernels, since an event between two
+// kernels stops them from overlapping.
+__device__ __forceinline__ unsigned long long device_ns() {
+  unsigned long long t;
+  asm volatile("mov.u64 %0, %globaltimer;" : "=l"(t)::"memory");
+  return t;
+}
+
+template <typename... P, typename... A>
+inline cudaError_t launch_overlapped(void (*kernel)(P...), dim3 grid, unsigned threads, size_t smem, cudaStream_t stream, A&&... args) {
+  cudaLaunchAttribute attr[1];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = dim3(threads, 1, 1);
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = stream;
+  cfg.attrs = attr;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, kernel, static_cast<P>(args)...);
+}
+#endif
+
 }  // namespace laser

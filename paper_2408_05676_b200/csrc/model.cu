@@ -17,66 +17,6 @@ namespace {
 using bf16 = __nv_bfloat16;
 
 
-// ---- row bookkeeping -------------------------------------------------------------------
-// One block per row: position, cache slot, capacity check, rotary angles (fp64 -> fp32).
-// With `parents` (token tree, Section 3.3) a row's position is ctx + its depth, its cache slot
-// stays ctx + row index, and row_mask gets the rows it attends to (its ancestors and itself).
-// With `start` (prompt chunks) row group b begins there instead of at its slot's committed length.
-__global__ void prep_rows_kernel(const int32_t* __restrict__ seq_ids, const int32_t* __restrict__ n_rows,
-                                 const int32_t* __restrict__ parents, const int32_t* __restrict__ start,
-                                 unsigned long long* __restrict__ row_mask, int B, int Rs, const int32_t* __restrict__ seq_len,
-                                 int max_seqs, int capacity, int half, double theta, int head_dim,
-                                 int32_t* __restrict__ row_pos, int32_t* __restrict__ row_seq,
-                                 int32_t* __restrict__ row_ctx, int32_t* __restrict__ row_n,
-                                 float* __restrict__ rope, int32_t* __restrict__ status) {
-  const int r = blockIdx.x;
-  const int b = r / Rs, i = r % Rs;
-  int pos = -1, seq = 0;
-  __shared__ int s_rpos;
-  int rpos = 0;                      // position the rotary embedding uses
-  unsigned long long mask = 0ull;
-  if (r < B * Rs) {
-    seq = seq_ids[b];
-    int nr = min(max(n_rows[b], 0), Rs);
-    int ctx = 0;
-    if (seq < 0 || seq >= max_seqs) {
-      nr = 0; seq = 0;
-      if (threadIdx.x == 0) atomicCAS(status, 0, LASER_ERR_INVALID_ARG);
-    } else {
-      ctx = start ? start[b] : seq_len[seq];
-      if (ctx + nr > capacity) {
-        nr = 0;
-        if (threadIdx.x == 0) atomicCAS(status, 0, LASER_ERR_CAPACITY);
-      }
-    }
-    if (i < nr) pos = ctx + i;
-    rpos = max(pos, 0);
-    if (parents && i < nr && threadIdx.x == 0) {
-      int depth = 0, j = i;
-      mask = 1ull << i;
-      while (j > 0) {                // parents are earlier rows: at most i steps
-        const int pj = parents[b * Rs + j];
-        if (pj < 0 || pj >= j) { atomicCAS(status, 0, LASER_ERR_INVALID_ARG); break; }
-        j = pj;
-        mask |= 1ull << j;
-        ++depth;
-      }
-      rpos = ctx + depth;
-    }
-    if (i == 0 && threadIdx.x == 0) { row_ctx[b] = ctx; row_n[b] = nr; }
-  }
-  if (threadIdx.x == 0) { row_pos[r] = pos; row_seq[r] = seq; s_rpos = rpos; if (row_mask) row_mask[r] = mask; }
-  __syncthreads();
-  rpos = s_rpos;
-  for (int j = threadIdx.x; j < half; j += blockDim.x) {
-    const double inv_freq = pow(theta, -2.0 * double(j) / double(head_dim));
-    double s, c;
-    sincos(double(rpos) * inv_freq, &s, &c);
-    rope[(size_t(r) * half + j) * 2] = float(c);
-    rope[(size_t(r) * half + j) * 2 + 1] = float(s);
-  }
-}
-
 __device__ __forceinline__ float block_sum(float v, float* red) {
   for (int o = 16; o; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -88,35 +28,127 @@ __device__ __forceinline__ float block_sum(float v, float* red) {
   return t;
 }
 
-// Embedding gather: resid = emb[token]; xb = bf16(resid * gain of the first norm); the sum of
-// squares of the row goes to tile plane 0 (the consumer GEMM turns it into the RMSNorm scale).
-__global__ void __launch_bounds__(256)
-embed_kernel(const int32_t* __restrict__ tokens, int R, int d, int vocab, const bf16* __restrict__ emb,
-             const bf16* __restrict__ gain, float* __restrict__ resid, bf16* __restrict__ xb,
-             float* __restrict__ sumsq, const int32_t* __restrict__ n_rows, int Rs, int32_t* __restrict__ row_draft,
-             int split) {
-  __shared__ float red[8];
-  const int r = blockIdx.x;
+// ---- the rows of a step: bookkeeping and embedding --------------------------------------
+// One block per row: position, cache slot, capacity check, rotary angles (fp64 -> fp32); and
+// the embedding gather: resid = emb[token], xb = bf16(resid * gain of the first norm), the sum of
+// squares of the row in tile plane 0 (the consumer GEMM turns it into the RMSNorm scale).
+// With `parents` (token tree, Section 3.3) a row's position is ctx + its depth, its cache slot
+// stays ctx + row index, and row_mask gets the rows it attends to (its ancestors and itself).
+// With `start` (prompt chunks) row group b begins there instead of at its slot's committed length.
+// Bound by its latency: a few dependent loads.  The angles' frequencies need no input and are computed while the kernel
+// before still runs; the gather moves four values a thread at a time.  It does not let the next kernel start early: the attention
+// kernels read row_ctx, row_n and the pages of earlier steps ahead of their own wait, which is safe because nothing of the
+// forward starts before this kernel, and so everything before it, has ended.  `vec`: d is a multiple of four, the tables are aligned.
+constexpr int kRowThreads = 256;
+struct RowTables {
+  int32_t *row_pos, *row_seq, *row_ctx, *row_n;
+  unsigned long long* row_mask;
+  float* rope;
+  int32_t *row_draft, *status;
+};
+
+__global__ void __launch_bounds__(kRowThreads)
+rows_kernel(const int32_t* seq_ids, const int32_t* n_rows, const int32_t* parents, const int32_t* start, int B, int Rs,
+            const int32_t* seq_len, int max_seqs, int capacity, int half, double theta, int head_dim, const RowTables out,
+            const int32_t* tokens, int d, int vocab, const bf16* __restrict__ emb, const bf16* __restrict__ gain,
+            float* __restrict__ resid, bf16* __restrict__ xb, float* __restrict__ sumsq, int split, int vec) {
+  __shared__ float red[kRowThreads / 32];
+  __shared__ int s_depth;
+  const int r = blockIdx.x, R = B * Rs;
+  const int b = r / Rs, i = r % Rs;
+  double inv_freq = 0.0;
+  if (int(threadIdx.x) < half) inv_freq = pow(theta, -2.0 * double(threadIdx.x) / double(head_dim));
+  wait_for_earlier();
   const int tok = r < R ? tokens[r] : -1;
-  if (row_draft && threadIdx.x == 0) {   // fused acceptance: the draft token that this row's distribution verifies
-    int dt = -1;
-    if (r < R && (r % Rs) + 1 < min(n_rows[r / Rs], Rs)) dt = tokens[r + 1];
-    row_draft[r] = dt;
+  int pos = -1, seq = 0, rpos = 0, n_raw = 0;   // rpos: position the rotary embedding uses
+  if (r < R) {
+    seq = seq_ids[b];
+    n_raw = n_rows[b];
+    int nr = min(max(n_raw, 0), Rs);
+    int ctx = 0;
+    if (seq < 0 || seq >= max_seqs) {
+      nr = 0; seq = 0;
+      if (threadIdx.x == 0) atomicCAS(out.status, 0, LASER_ERR_INVALID_ARG);
+    } else {
+      ctx = start ? start[b] : seq_len[seq];
+      if (ctx + nr > capacity) {
+        nr = 0;
+        if (threadIdx.x == 0) atomicCAS(out.status, 0, LASER_ERR_CAPACITY);
+      }
+    }
+    if (i < nr) pos = ctx + i;
+    rpos = max(pos, 0);
+    if (parents && i < nr) {
+      if (threadIdx.x == 0) {
+        int depth = 0, j = i;
+        unsigned long long mask = 1ull << i;
+        while (j > 0) {              // parents are earlier rows: at most i steps
+          const int pj = parents[b * Rs + j];
+          if (pj < 0 || pj >= j) { atomicCAS(out.status, 0, LASER_ERR_INVALID_ARG); break; }
+          j = pj;
+          mask |= 1ull << j;
+          ++depth;
+        }
+        out.row_mask[r] = mask;
+        s_depth = depth;
+      }
+      __syncthreads();               // (pos is the same in all of the block's threads)
+      rpos = ctx + s_depth;
+    } else if (parents && threadIdx.x == 0) {
+      out.row_mask[r] = 0ull;
+    }
+    if (i == 0 && threadIdx.x == 0) { out.row_ctx[b] = ctx; out.row_n[b] = nr; }
+  } else if (parents && threadIdx.x == 0) {
+    out.row_mask[r] = 0ull;
   }
+  if (threadIdx.x == 0) {
+    out.row_pos[r] = pos; out.row_seq[r] = seq;
+    // fused acceptance: the draft token that this row's distribution verifies
+    if (out.row_draft) out.row_draft[r] = r < R && i + 1 < min(n_raw, Rs) ? tokens[r + 1] : -1;
+  }
+
   const bool ok = tok >= 0 && tok < vocab;
   float ss = 0.f;
-  for (int j = threadIdx.x; j < d; j += blockDim.x) {
-    const float x = ok ? __bfloat162float(emb[size_t(tok) * d + j]) : 0.f;
-    resid[size_t(r) * d + j] = x;
-    const float y = x * __bfloat162float(gain[j]);
-    const bf16 hi = __float2bfloat16(y);
-    if (split) {   // operand as a hi + lo pair: [hi | lo] in a row of 2 d
-      xb[size_t(r) * (2 * d) + j] = hi;
-      xb[size_t(r) * (2 * d) + d + j] = __float2bfloat16(y - __bfloat162float(hi));
-    } else {
-      xb[size_t(r) * d + j] = hi;
+  if (vec) {
+    for (int j = threadIdx.x * 4; j < d; j += kRowThreads * 4) {
+      uint2 raw = make_uint2(0u, 0u);
+      if (ok) raw = *reinterpret_cast<const uint2*>(emb + size_t(tok) * d + j);
+      const uint2 g = *reinterpret_cast<const uint2*>(gain + j);
+      const bf16 *x4 = reinterpret_cast<const bf16*>(&raw), *g4 = reinterpret_cast<const bf16*>(&g);
+      float x[4];
+      uint2 hi, lo;
+      bf16 *h4 = reinterpret_cast<bf16*>(&hi), *l4 = reinterpret_cast<bf16*>(&lo);
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        x[u] = __bfloat162float(x4[u]);
+        const float y = x[u] * __bfloat162float(g4[u]);
+        h4[u] = __float2bfloat16(y);
+        l4[u] = __float2bfloat16(y - __bfloat162float(h4[u]));
+        ss += x[u] * x[u];
+      }
+      *reinterpret_cast<float4*>(resid + size_t(r) * d + j) = make_float4(x[0], x[1], x[2], x[3]);
+      bf16* row = xb + size_t(r) * (split ? 2 * d : d);
+      *reinterpret_cast<uint2*>(row + j) = hi;
+      if (split) *reinterpret_cast<uint2*>(row + d + j) = lo;   // operand as a hi + lo pair: [hi | lo] in a row of 2 d
     }
-    ss += x * x;
+  } else {
+    for (int j = threadIdx.x; j < d; j += kRowThreads) {
+      const float x = ok ? __bfloat162float(emb[size_t(tok) * d + j]) : 0.f;
+      resid[size_t(r) * d + j] = x;
+      const float y = x * __bfloat162float(gain[j]);
+      const bf16 hi = __float2bfloat16(y);
+      bf16* row = xb + size_t(r) * (split ? 2 * d : d);
+      row[j] = hi;
+      if (split) row[d + j] = __float2bfloat16(y - __bfloat162float(hi));
+      ss += x * x;
+    }
+  }
+  for (int j = threadIdx.x; j < half; j += kRowThreads) {
+    if (j >= kRowThreads) inv_freq = pow(theta, -2.0 * double(j) / double(head_dim));
+    double s, c;
+    sincos(double(rpos) * inv_freq, &s, &c);
+    out.rope[(size_t(r) * half + j) * 2] = float(c);
+    out.rope[(size_t(r) * half + j) * 2 + 1] = float(s);
   }
   ss = block_sum(ss, red);
   if (threadIdx.x == 0) sumsq[r] = ss;
@@ -278,6 +310,7 @@ LASER_API laser_status laser_profile_read(laser_model* m, int32_t cls, double* m
 LASER_API laser_status laser_model_free(laser_model* m) {
   if (!m) return LASER_OK;
   gemm_state_free(m);
+  gen_host_free(m);
   for (auto& v : m->prof_events) for (cudaEvent_t e : v) cudaEventDestroy(e);
   for (void* p : m->owned) cudaFree(p);
   delete m;
@@ -557,13 +590,13 @@ static laser_status verify_impl(laser_model* m, laser_kv* kv, const int32_t* seq
 
   // (rows are independent columns of every product: what a token tile finds beyond these is multiplied and dropped)
   const bool tree = parents != nullptr;
-  prep_rows_kernel<<<Rp, 64, 0, stream>>>(seq_ids, n_rows, parents, start, tree ? m->row_mask : nullptr, B, Rs, kv->seq_len, kv->max_seqs, capacity, dh / 2,
-                                          double(c.rope_theta), dh, m->row_pos, m->row_seq, m->row_ctx, m->row_n,
-                                          m->rope, m->status);
   const __nv_bfloat16* first_gain = c.n_layers > 0 ? m->attn_norm[0] : m->final_norm;
-  embed_kernel<<<Rp, 256, 0, stream>>>(tokens, R, d, c.vocab, m->tok_emb, first_gain, m->resid, m->xn, m->sumsq, n_rows, Rs,
-                                             fused ? m->row_draft : nullptr, m->precise ? 1 : 0);
-  count_launch(2);
+  const RowTables rt{m->row_pos, m->row_seq, m->row_ctx, m->row_n, m->row_mask, m->rope, fused ? m->row_draft : nullptr, m->status};
+  const bool vec = d % 4 == 0 && ((reinterpret_cast<uintptr_t>(m->tok_emb) | reinterpret_cast<uintptr_t>(first_gain)) & 7) == 0;
+  LASER_CUDA(launch_overlapped(rows_kernel, dim3(unsigned(Rp)), kRowThreads, 0, stream, seq_ids, n_rows, parents, start, B, Rs, kv->seq_len,
+                               kv->max_seqs, capacity, dh / 2, double(c.rope_theta), dh, rt, tokens, d, c.vocab, m->tok_emb, first_gain,
+                               m->resid, m->xn, m->sumsq, m->precise ? 1 : 0, vec ? 1 : 0));
+  count_launch();
   const bool use_tma_attn = attention_tma_supported(m, kv);
   const size_t attn_smem = (size_t(dh) + size_t(capacity) + 8) * sizeof(float);
   if (!use_tma_attn && attn_smem > 48 * 1024) {

@@ -4,6 +4,8 @@
 
 #include "state.cuh"
 
+namespace laser { struct GenHost; }
+
 struct laser_model {
   laser_model_cfg cfg{};
   int rows_per_seq = 0;  // max_draft + 1
@@ -44,6 +46,7 @@ struct laser_model {
   void* gemm_state = nullptr;      // tensor-map cache of the tensor-core GEMM
   void* gen_buf = nullptr;         // work buffers of laser_generate, kept between calls (in `owned`)
   size_t gen_bytes = 0;
+  laser::GenHost* gen_host = nullptr;  // pinned memory and events of laser_generate, kept between calls
   // optional per-class kernel timing (class 0 = GEMM, 1 = attention)
   bool profile = false;
   std::vector<cudaEvent_t> prof_events[2];  // begin/end pairs
@@ -58,6 +61,21 @@ namespace laser {
 constexpr int kPrefillRows = 1024;
 constexpr int kAttnSplitCtas = 512; // most CTAs of an attention launch that splits pages
 constexpr int kPrefillChunk = 32;   // rows that share each staged K/V page in the attention kernel
+
+void gen_host_free(laser_model* m);
+
+// The entry points of the same names; `stamp` (optional): the device clock at the end of the rows' making, at the start of the verdict.
+laser_status make_rows(const int32_t* last_token, const int32_t* draft, const int32_t* draft_len, int32_t B, int32_t K, int32_t* tokens,
+                       int32_t* n_rows, unsigned long long* stamp, cudaStream_t stream);
+laser_status make_rows_tree(const int32_t* last_token, const int32_t* draft, const int32_t* draft_parents, const int32_t* draft_len,
+                            int32_t B, int32_t K, int32_t* tokens, int32_t* parents, int32_t* n_rows, unsigned long long* stamp,
+                            cudaStream_t stream);
+laser_status accept_commit(laser_kv* kv, const int32_t* seq_ids, const float* logits, const int32_t* tokens, const int32_t* n_rows,
+                           int32_t B, int32_t V, const laser_params* p, int32_t* n_accept, int32_t* out_tokens, int32_t* n_out,
+                           unsigned long long* stamp, cudaStream_t stream);
+laser_status accept_tree(laser_kv* kv, const int32_t* seq_ids, const float* logits, const int32_t* tokens, const int32_t* parents,
+                         const int32_t* n_rows, int32_t B, int32_t V, const laser_params* p, int32_t* n_accept, int32_t* out_tokens,
+                         int32_t* n_out, int32_t* path_rows, unsigned long long* stamp, cudaStream_t stream);
 
 // What the GEMM does with a finished 128-feature x NT-row accumulator tile.
 enum { EPI_PLAIN = 0, EPI_RESID = 1, EPI_SWIGLU = 2, EPI_QKV = 3, EPI_VERDICT = 4 };

@@ -294,7 +294,9 @@ draft_warp_kernel(PoolView pv, DraftArgs a) {
   __shared__ int32_t s_cur[kDraftWarps][kMaxK];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = blockIdx.x * kDraftWarps + warp;
+  next_may_launch();
   if (q >= a.B) return;
+  wait_for_earlier();
   int32_t* out = a.draft + size_t(q) * a.K;
   const int g = a.group_id[q];
   int best_len = 0, best_n = 0;
@@ -354,7 +356,9 @@ draft_temp_kernel(PoolView pv, DraftArgs a, TempArgs t) {
   __shared__ int32_t s_cur[kDraftWarps][kMaxK];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = blockIdx.x * kDraftWarps + warp;
+  next_may_launch();
   if (q >= a.B) return;
+  wait_for_earlier();
   int32_t* out = a.draft + size_t(q) * a.K;
   const int g = a.group_id[q];
   const bool has_group = g >= 0 && g < pv.G;
@@ -422,7 +426,9 @@ draft_tree_kernel(PoolView pv, DraftArgs a, TempArgs t, int32_t* __restrict__ dr
   __shared__ uint8_t s_freq[64][kTreeK];           // frequency of node (o, d) at [o][d-1]
   __shared__ int s_sel_o[kTreeK], s_sel_d[kTreeK], s_rank[kTreeK];
   const int lane = threadIdx.x, q = blockIdx.x;
+  next_may_launch();
   if (q >= a.B) return;
+  wait_for_earlier();
   int32_t* out = a.draft + size_t(q) * a.K;
   int32_t* outp = draft_parents + size_t(q) * a.K;
   const int K = a.K;
@@ -570,18 +576,19 @@ draft_tree_kernel(PoolView pv, DraftArgs a, TempArgs t, int32_t* __restrict__ dr
   if (lane == 0) { a.draft_len[q] = best_len; a.match_n[q] = best_len ? best_n : 0; }
 }
 
-__global__ void make_tree_rows_kernel(const int32_t* __restrict__ last, const int32_t* __restrict__ draft,
-                                      const int32_t* __restrict__ dpar, const int32_t* __restrict__ dlen, int B, int K,
-                                      int32_t* __restrict__ tokens, int32_t* __restrict__ parents,
-                                      int32_t* __restrict__ n_rows) {
+__global__ void make_tree_rows_kernel(const int32_t* last, const int32_t* draft, const int32_t* dpar, const int32_t* dlen, int B, int K,
+                                      int32_t* tokens, int32_t* parents, int32_t* n_rows, unsigned long long* stamp) {
+  next_may_launch();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= B * (K + 1)) return;
   const int b = i / (K + 1), j = i % (K + 1);
+  wait_for_earlier();
   const int32_t lt = last[b];
   const int m = lt < 0 ? 0 : min(max(dlen[b], 0), K);
   tokens[i] = lt < 0 ? -1 : (j == 0 ? lt : (j <= m ? draft[b * K + j - 1] : -1));
   parents[i] = (lt >= 0 && j >= 1 && j <= m) ? dpar[b * K + j - 1] : -1;
   if (j == 0) n_rows[b] = lt < 0 ? 0 : 1 + m;
+  if (stamp && i == 0) *stamp = device_ns();
 }
 
 // Large-run path: one CTA per query, votes through a shared-memory histogram over the vocabulary.  The run is read once: its
@@ -604,7 +611,9 @@ draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound) {
   __shared__ int s_found, s_item, s_warp_n[kBigThreads / 32];
   __shared__ unsigned long long s_best;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  next_may_launch();
   for (int v = tid; v < vocab_bound; v += kBigThreads) s_hist[v] = 0;
+  wait_for_earlier();
   const int n_work = a.work[0];
   for (;;) {
     __syncthreads();
@@ -791,16 +800,18 @@ draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound) {
   if (tid == 0 && atomicAdd(&a.work[2], 1) == int(gridDim.x) - 1) { a.work[0] = 0; a.work[1] = 0; a.work[2] = 0; }
 }
 
-__global__ void make_rows_kernel(const int32_t* __restrict__ last, const int32_t* __restrict__ draft,
-                                 const int32_t* __restrict__ dlen, int B, int K,
-                                 int32_t* __restrict__ tokens, int32_t* __restrict__ n_rows) {
+__global__ void make_rows_kernel(const int32_t* last, const int32_t* draft, const int32_t* dlen, int B, int K,
+                                 int32_t* tokens, int32_t* n_rows, unsigned long long* stamp) {
+  next_may_launch();
   const int i = blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= B * (K + 1)) return;
   const int b = i / (K + 1), j = i % (K + 1);
+  wait_for_earlier();
   const int32_t lt = last[b];
   const int m = lt < 0 ? 0 : min(max(dlen[b], 0), K);
   tokens[i] = lt < 0 ? -1 : (j == 0 ? lt : (j <= m ? draft[b * K + j - 1] : -1));
   if (j == 0) n_rows[b] = lt < 0 ? 0 : 1 + m;
+  if (stamp && i == 0) *stamp = device_ns();
 }
 
 }  // namespace
@@ -935,12 +946,12 @@ LASER_API laser_status laser_draft(const laser_pool* pool, const int32_t* tails,
   if (big) LASER_TRY(scratch_get(SCRATCH_DRAFT, sizeof(int32_t) * (size_t(kWorkHead) + 2 * size_t(B)), &scratch));
   DraftArgs a{tails, tail_len, group_id, B, p->K, p->n_min, p->n_max, p->min_draft, p->max_occ,
               draft, draft_len, match_n, static_cast<int32_t*>(scratch), pool->n_tokens};
-  draft_warp_kernel<<<ceil_div(B, kDraftWarps), kDraftWarps * 32, 0, stream>>>(pv, a);
+  LASER_CUDA(launch_overlapped(draft_warp_kernel, dim3(unsigned(ceil_div(B, kDraftWarps))), kDraftWarps * 32, 0, stream, pv, a));
   count_launch();
   if (big) {
     const size_t smem = hist + kBigList * sizeof(uint32_t);
     LASER_CUDA(cudaFuncSetAttribute(draft_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-    draft_cta_kernel<<<std::min(B, 148), kBigThreads, smem, stream>>>(pv, a, pool->vocab_bound);
+    LASER_CUDA(launch_overlapped(draft_cta_kernel, dim3(unsigned(std::min(B, 148))), kBigThreads, smem, stream, pv, a, pool->vocab_bound));
     count_launch();
   }
   LASER_CUDA(cudaGetLastError());
@@ -965,7 +976,7 @@ LASER_API laser_status laser_draft_temp(const laser_pool* pool, const int32_t* t
   DraftArgs a{tails, tail_len, group_id, B, p->K, p->n_min, p->n_max, p->min_draft, p->max_occ,
               draft, draft_len, match_n, nullptr, pool->n_tokens};
   TempArgs t{hist, hist_len, hist_stride};
-  draft_temp_kernel<<<ceil_div(B, kDraftWarps), kDraftWarps * 32, 0, stream>>>(pv, a, t);
+  LASER_CUDA(launch_overlapped(draft_temp_kernel, dim3(unsigned(ceil_div(B, kDraftWarps))), kDraftWarps * 32, 0, stream, pv, a, t));
   count_launch();
   LASER_CUDA(cudaGetLastError());
   return LASER_OK;
@@ -989,35 +1000,45 @@ LASER_API laser_status laser_draft_tree(const laser_pool* pool, const int32_t* t
   DraftArgs a{tails, tail_len, group_id, B, p->K, p->n_min, p->n_max, p->min_draft, p->max_occ,
               draft, draft_len, match_n, nullptr, pool->n_tokens};
   TempArgs t{hist, hist_len, hist_stride};
-  draft_tree_kernel<<<B, 32, 0, as_stream(stream_)>>>(pv, a, t, draft_parents);
+  LASER_CUDA(launch_overlapped(draft_tree_kernel, dim3(unsigned(B)), 32, 0, as_stream(stream_), pv, a, t, draft_parents));
   count_launch();
   LASER_CUDA(cudaGetLastError());
   return LASER_OK;
 }
 
-LASER_API laser_status laser_make_rows_tree(const int32_t* last_token, const int32_t* draft, const int32_t* draft_parents,
-                                            const int32_t* draft_len, int32_t B, int32_t K, int32_t* tokens,
-                                            int32_t* parents, int32_t* n_rows, void* stream) {
-  using namespace laser;
+namespace laser {
+laser_status make_rows(const int32_t* last_token, const int32_t* draft, const int32_t* draft_len, int32_t B, int32_t K, int32_t* tokens,
+                       int32_t* n_rows, unsigned long long* stamp, cudaStream_t stream) {
+  LASER_REQUIRE(last_token && draft && draft_len && tokens && n_rows, "null argument");
+  LASER_REQUIRE(B >= 0 && K >= 0, "B = %d, K = %d", B, K);
+  if (B == 0) return LASER_OK;
+  LASER_CUDA(launch_overlapped(make_rows_kernel, dim3(unsigned(ceil_div(B * (K + 1), 256))), 256, 0, stream, last_token, draft, draft_len,
+                               B, K, tokens, n_rows, stamp));
+  count_launch();
+  return LASER_OK;
+}
+
+laser_status make_rows_tree(const int32_t* last_token, const int32_t* draft, const int32_t* draft_parents, const int32_t* draft_len,
+                            int32_t B, int32_t K, int32_t* tokens, int32_t* parents, int32_t* n_rows, unsigned long long* stamp,
+                            cudaStream_t stream) {
   LASER_REQUIRE(last_token && draft && draft_parents && draft_len && tokens && parents && n_rows, "null argument");
   LASER_REQUIRE(B >= 0 && K >= 0, "B = %d, K = %d", B, K);
   if (B == 0) return LASER_OK;
-  make_tree_rows_kernel<<<ceil_div(B * (K + 1), 256), 256, 0, as_stream(stream)>>>(last_token, draft, draft_parents, draft_len,
-                                                                                  B, K, tokens, parents, n_rows);
+  LASER_CUDA(launch_overlapped(make_tree_rows_kernel, dim3(unsigned(ceil_div(B * (K + 1), 256))), 256, 0, stream, last_token, draft,
+                               draft_parents, draft_len, B, K, tokens, parents, n_rows, stamp));
   count_launch();
-  LASER_CUDA(cudaGetLastError());
   return LASER_OK;
+}
+}  // namespace laser
+
+LASER_API laser_status laser_make_rows_tree(const int32_t* last_token, const int32_t* draft, const int32_t* draft_parents,
+                                            const int32_t* draft_len, int32_t B, int32_t K, int32_t* tokens,
+                                            int32_t* parents, int32_t* n_rows, void* stream) {
+  return laser::make_rows_tree(last_token, draft, draft_parents, draft_len, B, K, tokens, parents, n_rows, nullptr, laser::as_stream(stream));
 }
 
 LASER_API laser_status laser_make_rows(const int32_t* last_token, const int32_t* draft,
                                        const int32_t* draft_len, int32_t B, int32_t K,
                                        int32_t* tokens, int32_t* n_rows, void* stream) {
-  using namespace laser;
-  LASER_REQUIRE(last_token && draft && draft_len && tokens && n_rows, "null argument");
-  LASER_REQUIRE(B >= 0 && K >= 0, "B = %d, K = %d", B, K);
-  if (B == 0) return LASER_OK;
-  make_rows_kernel<<<ceil_div(B * (K + 1), 256), 256, 0, as_stream(stream)>>>(last_token, draft, draft_len, B, K, tokens, n_rows);
-  count_launch();
-  LASER_CUDA(cudaGetLastError());
-  return LASER_OK;
+  return laser::make_rows(last_token, draft, draft_len, B, K, tokens, n_rows, nullptr, laser::as_stream(stream));
 }
