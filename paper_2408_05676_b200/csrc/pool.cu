@@ -1,28 +1,31 @@
 // Customized Retrieval Pool (Section 3.2) and draft retrieval, Retrieve(D, tail, K) of Eq. 5
 // (Section 3.3).
 //
-// Index: for every n in [n_min, n_max] one open-addressing hash table keyed by a 64-bit
-// hash of (group, n-gram) whose 8-byte entries {low half of the key, start} point at a run of a
-// position array sorted by (hash, position); the last position of a run carries a mark.  A run
-// lists, ascending, every position where that n-gram ends inside that group - exactly the nodes a
-// per-group trie reaches with the n-gram as prefix, with multiplicity.  A key's home slot is its
-// high half scaled to the table, so the sorted keys fill the table from end to end and an insert
-// touches the lines of its neighbours' inserts.  Equal halves of different keys only cost a look at
-// the wrong run, a collision of whole keys only merges runs: every position read at lookup time is
-// checked against the actual pool tokens and the group bounds, so results never depend on the hash.
+// Index: for every n in [n_min, n_max] an open-addressing hash table keyed by a 64-bit hash of
+// (group, n-gram) whose 8-byte entries {low half of the key, start} point at a run of a position
+// array; the last position of a run carries a mark.  A run lists, ascending, every position where
+// that n-gram ends inside that group - exactly the nodes a per-group trie reaches with the n-gram as
+// prefix, with multiplicity.  Every group has a region of the table for itself (region_of), so that
+// a group is indexed on its own, and a key's home slot is its high half scaled to the region.
+// Equal halves of different keys only cost a look at the wrong run, a collision of whole keys only
+// merges runs: every position read at lookup time is checked against the actual pool tokens and the
+// group bounds, so results never depend on the hash.
+//
+// Build: a group whose working set fits shared memory is indexed there by one CTA per n
+// (index_group_kernel); the n-grams of larger groups are inserted into the table itself, and their
+// positions sorted by slot, all groups together, with the radix sort of CUB, the header library
+// shipped with the CUDA toolkit (nothing on the per-step path uses it).
 //
 // Lookup: one warp per query.  All 32 lanes probe 32 consecutive slots (256 B, coalesced);
 // the run is read 32 positions at a time, verified, and compacted; the greedy
 // highest-frequency walk votes over at most 64 occurrences held two per lane.  Queries that
 // need more than 64 occurrences (max_occ = 0 or > 64) go to a work list served by one CTA
 // per query with a shared-memory histogram over the vocabulary.
-//
-// The (key, position) sort of the one-off build uses the radix sort of CUB, the header
-// library shipped with the CUDA toolkit; nothing on the per-step path does.
 #include <cub/device/device_radix_sort.cuh>
 
 #include <algorithm>
 #include <type_traits>
+#include <vector>
 
 #include "common.cuh"
 
@@ -36,7 +39,6 @@ struct laser_pool {
   int64_t* group_offsets = nullptr;  // dev [n_groups + 1]
   struct Level {
     uint2* table = nullptr;          // {key's low half, start of its run}, all ones = empty
-    uint32_t slots = 0;
     uint32_t* positions = nullptr;   // [n_tokens + 32], runs end with a marked position
     int64_t n_keys = 0;
   } level[9];                        // indexed by n
@@ -57,14 +59,19 @@ __host__ __device__ __forceinline__ uint64_t mix64(uint64_t x) {
   x ^= x >> 31;
   return x;
 }
-__host__ __device__ __forceinline__ uint64_t key_begin(int g, int n) {
-  return mix64((uint64_t(uint32_t(g)) << 8) | uint64_t(n));
-}
-__host__ __device__ __forceinline__ uint64_t key_push(uint64_t h, int32_t tok) {
-  return mix64(h ^ (uint64_t(uint32_t(tok)) * 0x9E3779B97F4A7C15ULL));
-}
-__host__ __device__ __forceinline__ uint64_t key_end(uint64_t h) { return h == kEmpty ? 0 : h; }
+// A polynomial in the tokens, mixed once: a mix per token made hashing a third of the build in shared memory.
+__host__ __device__ __forceinline__ uint64_t key_begin(int g, int n) { return (uint64_t(uint32_t(g)) << 8) | uint64_t(n); }
+__host__ __device__ __forceinline__ uint64_t key_push(uint64_t h, int32_t tok) { return h * 0x9E3779B97F4A7C15ULL + uint32_t(tok); }
+__host__ __device__ __forceinline__ uint64_t key_end(uint64_t h) { return mix64(h * 0x9E3779B97F4A7C15ULL); }
 __device__ __forceinline__ uint32_t home_slot(uint64_t key, uint32_t slots) { return uint32_t(__umul64hi(key, slots)); }
+
+// A group's region of a table: 13 slots per 8 tokens, and always one more than there are tokens.
+struct Region { int64_t base; uint32_t slots; };
+__host__ __device__ __forceinline__ int64_t region_base(int64_t group_start, int64_t g) { return group_start + (group_start >> 1) + (group_start >> 3) + 2 * g; }
+__host__ __device__ __forceinline__ Region region_of(int64_t lo, int64_t hi, int g) {
+  const int64_t base = region_base(lo, g);
+  return Region{base, uint32_t(region_base(hi, int64_t(g) + 1) - base)};
+}
 
 constexpr int kKeyThreads = 256;
 
@@ -77,31 +84,75 @@ __device__ __forceinline__ int group_of(const int64_t* __restrict__ goff, int lo
   return lo;
 }
 
-// Bound by its 16 bytes a position in and out (10 M positions: 396 -> 40 us; before, every warp added to two counters and every
-// thread searched all groups).  A block's positions are consecutive: two searches bound those of its threads.
+struct IndexLevels { uint2* table[kMaxN + 1]; uint32_t* positions[kMaxN + 1]; };
+
+// The groups that the sort takes: their ids, and where the positions of each begin when they are laid end to end.
+struct LargeGroups { const int32_t* id; const int64_t* at; int n; };
+
+// Inserts the n-grams of the listed groups, for the n from n0 on, into their regions (cleared before) and leaves every (n,
+// position) with the number of its n-gram's slot among all those tables' (kNoSlot where none ends).  An entry is {key's low
+// half, a position of the n-gram} here; equal low halves are told apart by the tokens.  A block's positions are consecutive: two
+// searches bound the groups of its threads, and as they are a chain of loads a block takes kInsertItems positions a thread (2.8 M
+// positions, four n: 374 us with one, 256 with four).  Bound by the latency of the probes, in L2 for the most part.
+constexpr uint32_t kNoSlot = 0xffffffffu;
+constexpr int kInsertItems = 4, kInsertBlock = kInsertItems * kKeyThreads;
 __global__ void __launch_bounds__(kKeyThreads)
-make_keys_kernel(const int32_t* __restrict__ tok, int64_t N, const int64_t* __restrict__ goff, int G, int n,
-                 uint64_t* __restrict__ keys, uint32_t* __restrict__ pos, int* __restrict__ max_tok) {
+insert_large_kernel(const int32_t* __restrict__ tok, const int64_t* __restrict__ goff, LargeGroups lg, int64_t M, int n0,
+                    const IndexLevels lv, uint32_t table_slots, uint32_t* __restrict__ slot_of, uint32_t* __restrict__ pos,
+                    unsigned long long* __restrict__ n_valid, int* __restrict__ max_tok) {
   __shared__ int s_g[2], s_max[kKeyThreads / 32];
-  const int64_t p0 = int64_t(blockIdx.x) * kKeyThreads, p = p0 + threadIdx.x;
-  if (threadIdx.x < 2) s_g[threadIdx.x] = group_of(goff, 0, G, min(N - 1, p0 + threadIdx.x * (kKeyThreads - 1)));
+  __shared__ unsigned s_ends;
+  const int64_t i0 = int64_t(blockIdx.x) * kInsertBlock;
+  const int n = n0 + blockIdx.y;
+  unsigned long long* const table = reinterpret_cast<unsigned long long*>(lv.table[n]);
+  if (threadIdx.x < 2) s_g[threadIdx.x] = group_of(lg.at, 0, lg.n, min(M - 1, i0 + threadIdx.x * (kInsertBlock - 1)));
+  if (threadIdx.x == 0) s_ends = 0;
   __syncthreads();
-  int mt = -1;
-  if (p < N) {
-    const int g = s_g[0] == s_g[1] ? s_g[0] : group_of(goff, s_g[0], s_g[1] + 1, p);
-    bool valid = p - n + 1 >= goff[g];
-    uint64_t h = key_begin(g, n);
+  int mt = -1, ends = 0;
+  for (int64_t i = i0 + threadIdx.x; i < min(M, i0 + kInsertBlock); i += kKeyThreads) {
+    const int l = s_g[0] == s_g[1] ? s_g[0] : group_of(lg.at, s_g[0], s_g[1] + 1, i), g = lg.id[l];
+    const int64_t lo = goff[g], p = lo + (i - lg.at[l]);
+    bool valid = i - lg.at[l] >= n - 1;
+    uint64_t key = key_begin(g, n);
     if (valid)
       for (int j = 0; j < n; ++j) {
         const int32_t t = tok[p - n + 1 + j];
         if (t < 0) { valid = false; break; }
-        h = key_push(h, t);
+        key = key_push(key, t);
       }
-    keys[p] = valid ? key_end(h) : kEmpty;
-    pos[p] = uint32_t(p);
-    mt = max_tok ? tok[p] : -1;
+    uint32_t at = kNoSlot;
+    if (valid) {
+      key = key_end(key);
+      const Region rg = region_of(lo, goff[g + 1], g);
+      const unsigned long long entry = (uint64_t(uint32_t(p)) << 32) | uint32_t(key);
+      uint32_t s = home_slot(key, rg.slots);
+      for (uint32_t tries = 0; tries < rg.slots; ++tries) {   // there are more slots than positions
+        unsigned long long* e = table + rg.base + s;
+        unsigned long long old = __ldcg(e);
+        if (old == kEmpty) {
+          old = atomicCAS(e, (unsigned long long)kEmpty, entry);
+          if (old == kEmpty) break;
+        }
+        if (uint32_t(old) == uint32_t(key)) {
+          const int64_t q = int64_t(old >> 32);
+          bool same = true;
+          for (int j = 0; same && j < n; ++j) same = tok[p - j] == tok[q - j];
+          if (same) break;
+        }
+        if (++s == rg.slots) s = 0;
+      }
+      at = blockIdx.y * table_slots + uint32_t(rg.base) + s;
+      ++ends;
+    }
+    slot_of[blockIdx.y * M + i] = at;
+    pos[blockIdx.y * M + i] = uint32_t(p);
+    mt = max(mt, tok[p]);
   }
-  if (max_tok) {
+  ends = __reduce_add_sync(0xffffffffu, ends);
+  if ((threadIdx.x & 31) == 0) atomicAdd(&s_ends, unsigned(ends));
+  __syncthreads();
+  if (threadIdx.x == 0 && s_ends) atomicAdd(n_valid + n, (unsigned long long)s_ends);
+  if (blockIdx.y == 0) {
     for (int o = 16; o; o >>= 1) mt = max(mt, __shfl_xor_sync(0xffffffffu, mt, o));
     if ((threadIdx.x & 31) == 0) s_max[threadIdx.x >> 5] = mt;
     __syncthreads();
@@ -112,30 +163,206 @@ make_keys_kernel(const int32_t* __restrict__ tok, int64_t N, const int64_t* __re
   }
 }
 
-// Sorted (key, position) pairs to the position array with its run marks, and the first of every run to the table.  Bound by
-// its streams: 16 bytes a position and 8 a distinct key, whose slots ascend with the keys (10 M positions, mean of four levels:
-// count and insert 611 -> 150 us against random 16-byte slots, a search for every run's end and a counter update per warp).
+// (slot, position) pairs sorted by slot to the position arrays (from `first` on) with their run marks, and the start of every
+// run to its slot.
 __global__ void __launch_bounds__(kKeyThreads)
-index_runs_kernel(const uint64_t* __restrict__ keys, const uint32_t* __restrict__ pos, int64_t N, uint32_t* __restrict__ positions,
-                  unsigned long long* __restrict__ table, uint32_t slots, unsigned long long* __restrict__ n_heads) {
+index_runs_kernel(const uint32_t* __restrict__ slot, const uint32_t* __restrict__ pos, int64_t count, int64_t first, int n0,
+                  const IndexLevels lv, uint32_t table_slots, const unsigned long long* __restrict__ n_valid,
+                  unsigned long long* __restrict__ n_heads) {
+  __shared__ unsigned s_heads[kMaxN + 1];
+  if (threadIdx.x <= kMaxN) s_heads[threadIdx.x] = 0;
+  __syncthreads();
   const int64_t i = int64_t(blockIdx.x) * kKeyThreads + threadIdx.x;
-  bool head = false;
-  if (i < N) {
-    const uint64_t k = keys[i];
-    const bool end = i + 1 == N || keys[i + 1] != k;
-    positions[i] = pos[i] | (end ? kRunEnd : 0u);
-    head = k != kEmpty && (i == 0 || keys[i - 1] != k);
-    if (head) {
-      const unsigned long long entry = (uint64_t(uint32_t(i)) << 32) | uint32_t(k);
-      uint32_t s = home_slot(k, slots);
-      for (uint32_t tries = 0; tries < slots; ++tries) {   // there are more slots than keys
-        if (atomicCAS(&table[s], (unsigned long long)kEmpty, entry) == kEmpty) break;
-        if (++s == slots) s = 0;
-      }
+  const uint32_t s = i < count ? slot[i] : kNoSlot;
+  if (s != kNoSlot) {
+    const uint32_t l = s / table_slots;
+    int64_t rank = i;                      // among the positions of its n
+    for (uint32_t x = 0; x < l; ++x) rank -= int64_t(n_valid[n0 + x]);
+    const bool end = i + 1 == count || slot[i + 1] != s;
+    lv.positions[n0 + l][first + rank] = pos[i] | (end ? kRunEnd : 0u);
+    if (i == 0 || slot[i - 1] != s) {
+      lv.table[n0 + l][s - l * table_slots].y = uint32_t(first + rank);
+      atomicAdd(&s_heads[n0 + l], 1u);
     }
   }
-  const int heads = __syncthreads_count(head);
-  if (threadIdx.x == 0 && heads) atomicAdd(n_heads, (unsigned long long)heads);
+  __syncthreads();
+  if (threadIdx.x <= kMaxN && s_heads[threadIdx.x]) atomicAdd(n_heads + threadIdx.x, (unsigned long long)s_heads[threadIdx.x]);
+}
+
+__global__ void __launch_bounds__(kKeyThreads)
+clear_regions_kernel(const IndexLevels lv, int n_min, const int64_t* __restrict__ goff, LargeGroups lg) {
+  const int g = lg.id[blockIdx.y];
+  const Region rg = region_of(goff[g], goff[g + 1], g);
+  uint2* table = lv.table[n_min + blockIdx.z] + rg.base;
+  for (uint32_t s = blockIdx.x * kKeyThreads + threadIdx.x; s < rg.slots; s += gridDim.x * kKeyThreads) table[s] = make_uint2(0xffffffffu, 0xffffffffu);
+}
+
+// ---- a group in shared memory ------------------------------------------------------------
+// One CTA per (group, n): the region's slots as words {count | representative position}, into which the group's n-grams are
+// inserted (compared by their tokens); the counts become run starts by a prefix sum; a block of positions after the other goes
+// into the runs, and a position finds its place among those of its block by counting.  Memory sees the tokens, the runs and
+// the regions; what bounds the kernel is the latency of its steps in shared memory.  In the insert loop a lane takes its next
+// position as soon as it has placed one: a warp whose lanes wait for the longest of 32 probe walks took four times as long.
+// Groups come in three classes by size, for one, two and three CTAs an SM.  10 M tokens in 2000 groups, four levels: 820 us for
+// the 72 % of them in groups that fit and 740 us for the rest, against 4.7 ms for a sort of all positions by 64-bit key and n;
+// the whole build 4.99 -> 1.61 ms, and 4.66 -> 2.48 ms where groups are so large that few fit.
+constexpr uint32_t kFreeWord = 0x0000ffffu;
+constexpr int kScan = 128;                       // slots that a warp scans at a time
+constexpr size_t group_smem(int64_t tokens) {    // words, tokens, slot and run member of every position
+  return size_t((tokens + tokens / 2 + tokens / 8 + 4 + kScan - 1) / kScan * kScan) * 4 + size_t(tokens) * 8 + 16;
+}
+constexpr int kClasses = 3;
+constexpr int kGroupMax = 15400;                 // tokens of the largest group
+constexpr int64_t kClassMax[kClasses] = {kGroupMax, 7600, 4900};
+static_assert(group_smem(kGroupMax) <= 226 * 1024 && 2 * group_smem(kClassMax[1]) <= 224 * 1024 && 3 * group_smem(kClassMax[2]) <= 222 * 1024 &&
+              kGroupMax + kGroupMax / 2 + kGroupMax / 8 + 4 < 65535, "");
+
+template <int THREADS, int CTAS>
+__global__ void __launch_bounds__(THREADS, CTAS)
+index_group_kernel(const int32_t* __restrict__ tok, const int64_t* __restrict__ goff, const int32_t* __restrict__ group_id,
+                   const int64_t* __restrict__ group_at, int leads, int n_min, const IndexLevels lv, unsigned long long* __restrict__ n_heads,
+                   int* __restrict__ max_tok) {
+  constexpr int kWarps = THREADS / 32, kBlock = 256;
+  extern __shared__ __align__(16) uint32_t s_word[];
+  __shared__ uint32_t s_sum[kWarps];
+  __shared__ int s_heads;
+  if (leads) wait_for_earlier();  // the first class waits for its inputs, and so do those that it lets start
+  next_may_launch();
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const int g = group_id[blockIdx.x], n = n_min + blockIdx.y;
+  const int64_t lo = goff[g], hi = goff[g + 1], first = group_at[blockIdx.x];   // first: of the group's runs
+  const int T = int(hi - lo);
+  const Region rg = region_of(lo, hi, g);
+  const int slots = int(rg.slots), words = (slots + kScan - 1) / kScan * kScan;
+  int32_t* s_tok = reinterpret_cast<int32_t*>(s_word + words);
+  uint16_t* s_slot = reinterpret_cast<uint16_t*>(s_tok + T);
+  uint16_t* s_member = s_slot + T;
+  uint2* const table = lv.table[n] + rg.base;
+
+  if (tid == 0) s_heads = 0;
+  for (int s = tid; s < words; s += THREADS) s_word[s] = kFreeWord;
+  for (int s = tid; s < slots; s += THREADS) table[s] = make_uint2(0xffffffffu, 0xffffffffu);
+  int mt = -1;
+  for (int i = tid; i < T; i += THREADS) {
+    const int32_t t = tok[lo + i];
+    s_tok[i] = t;
+    mt = max(mt, t);
+  }
+  if (blockIdx.y == 0) {
+    for (int o = 16; o; o >>= 1) mt = max(mt, __shfl_xor_sync(0xffffffffu, mt, o));
+    if (lane == 0 && mt > *max_tok) atomicMax(max_tok, mt);
+  }
+  __syncthreads();
+  auto key_of = [&](int i) {      // of the n-gram that ends at i
+    uint64_t h = key_begin(g, n);
+    for (int j = i - n + 1; j <= i; ++j) h = key_push(h, s_tok[j]);
+    return key_end(h);
+  };
+
+  // home slots
+  for (int i = tid; i < T; i += THREADS) {
+    uint64_t h = key_begin(g, n);
+    int32_t least = i >= n - 1 ? 0 : -1;
+    for (int j = max(i - n + 1, 0); j <= i; ++j) {
+      const int32_t t = s_tok[j];
+      least = min(least, t);
+      h = key_push(h, t);
+    }
+    s_slot[i] = least >= 0 ? uint16_t(home_slot(key_end(h), rg.slots)) : uint16_t(0xffff);
+  }
+  // insert and count (a thread's positions are its own from here to the next barrier)
+  for (int i = tid, s = i < T ? s_slot[i] : 0, t = i < T ? s_tok[i] : 0; i < T;) {
+    bool placed = s == 0xffff;    // (none ends here)
+    if (!placed) {                // (there are more slots than positions)
+      uint32_t w = *const_cast<volatile uint32_t*>(s_word + s);
+      if (w == kFreeWord) {
+        w = atomicCAS(s_word + s, kFreeWord, 0x10000u | uint32_t(i));
+        placed = w == kFreeWord;
+      }
+      if (!placed) {
+        const int rep = int(w & 0xffffu);
+        if (s_tok[rep] == t) {
+          placed = true;
+          for (int j = 1; j < n; ++j) placed = placed && s_tok[i - j] == s_tok[rep - j];
+          if (placed) atomicAdd(s_word + s, 0x10000u);
+        }
+      }
+    }
+    if (placed) {
+      s_slot[i] = uint16_t(s);
+      i += THREADS;
+      if (i < T) { s = s_slot[i]; t = s_tok[i]; }
+    } else if (++s == slots) {
+      s = 0;
+    }
+  }
+  __syncthreads();
+
+  // counts -> {0 | start}: a warp's share of the slots is consecutive, four a lane at a time
+  const int per = (words / kScan + kWarps - 1) / kWarps * kScan, s0 = min(words, warp * per), s1 = min(words, s0 + per);
+  uint32_t sum = 0, heads = 0;
+  for (int s = s0 + lane; s < s1; s += 32) {
+    const uint32_t c = s_word[s] >> 16;
+    sum += c;
+    heads += c != 0;
+  }
+  sum = __reduce_add_sync(0xffffffffu, sum);
+  heads = __reduce_add_sync(0xffffffffu, heads);
+  if (lane == 0) { s_sum[warp] = sum; if (heads) atomicAdd(&s_heads, int(heads)); }
+  __syncthreads();
+  uint32_t start = 0, total = 0;
+  for (int w = 0; w < kWarps; ++w) { if (w < warp) start += s_sum[w]; total += s_sum[w]; }
+  for (int s = s0; s < s1; s += kScan) {
+    uint4* at = reinterpret_cast<uint4*>(s_word + s) + lane;
+    const uint4 w = *at;
+    const uint32_t c0 = w.x >> 16, c1 = c0 + (w.y >> 16), c2 = c1 + (w.z >> 16), c3 = c2 + (w.w >> 16);
+    uint32_t upto = c3;
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(0xffffffffu, upto, o);
+      if (lane >= o) upto += v;
+    }
+    const uint32_t at0 = start + upto - c3;
+    *at = make_uint4(at0, at0 + c0, at0 + c1, at0 + c2);
+    start += __shfl_sync(0xffffffffu, upto, 31);
+  }
+  __syncthreads();
+
+  // every position into its run: blocks of kBlock positions in order, within a block in the order of arrival; the words
+  // become {count | start}.  (A large block is placed quickly, a small one ranked: groups of 4,900 to 7,600 tokens, n = 1,
+  // blocks of 512 take 4 and 62 thousand cycles, of 256 7 and 41; n = 4, 4 and 13, 6 and 13.)
+  if (tid < kBlock)
+    for (int i0 = 0; i0 < T; i0 += kBlock) {
+      const int i = i0 + tid, s = i < T ? s_slot[i] : 0xffff;
+      if (s != 0xffff) {
+        const uint32_t w = atomicAdd(s_word + s, 0x10000u);
+        s_member[(w & 0xffffu) + (w >> 16)] = uint16_t(i);
+      }
+      asm volatile("bar.sync 1, %0;" ::"n"(kBlock) : "memory");
+    }
+  __syncthreads();
+
+  // to its place in the run, behind those of earlier blocks; the first of a run makes its entry
+  uint32_t* positions = lv.positions[n] + first;
+  for (uint32_t k = tid; k < total; k += THREADS) {
+    const uint32_t i = s_member[k], block = i / kBlock, s = s_slot[i], w = s_word[s], begin = w & 0xffffu, end = begin + (w >> 16);
+    uint32_t left = k, smaller = 0;
+    while (left > begin) {
+      const uint32_t m = s_member[left - 1];
+      if (m / kBlock != block) break;
+      smaller += m < i;
+      --left;
+    }
+    for (uint32_t r = k + 1; r < end; ++r) {
+      const uint32_t m = s_member[r];
+      if (m / kBlock != block) break;
+      smaller += m < i;
+    }
+    const uint32_t at = left + smaller;
+    positions[at] = (uint32_t(lo) + i) | (at + 1 == end ? kRunEnd : 0u);
+    if (k == begin) table[s] = make_uint2(uint32_t(key_of(int(i))), uint32_t(first) + begin);
+  }
+  if (tid == 0 && s_heads) atomicAdd(n_heads + n, (unsigned long long)s_heads);
+  wait_for_earlier();             // (the classes are independent; what follows in the stream waits for all)
 }
 
 // ---------------------------------------------------------------------------------------
@@ -144,7 +371,6 @@ struct PoolView {
   const int64_t* goff;
   int G;
   const uint2* table[kMaxN + 1];
-  uint32_t slots[kMaxN + 1];
   const uint32_t* positions[kMaxN + 1];
 };
 
@@ -152,7 +378,7 @@ PoolView view_of(const laser_pool* pool) {
   PoolView pv{};
   pv.tok = pool->tokens; pv.goff = pool->group_offsets; pv.G = pool->n_groups;
   for (int n = pool->n_min; n <= pool->n_max; ++n) {
-    pv.table[n] = pool->level[n].table; pv.slots[n] = pool->level[n].slots;
+    pv.table[n] = pool->level[n].table;
     pv.positions[n] = pool->level[n].positions;
   }
   return pv;
@@ -172,9 +398,8 @@ __device__ __forceinline__ bool probe(const uint2* __restrict__ table, uint32_t 
                                       uint32_t& start) {
   const uint32_t home = home_slot(key, slots);
   for (; off < slots; off += 32) {
-    uint64_t s = uint64_t(home) + off + lane;
-    if (s >= slots) s -= slots;
-    if (s >= slots) s -= slots;            // (a table has at least 64 slots)
+    uint64_t s = uint64_t(home) + off + lane;   // (a small region is seen more than once: up to its first empty slot, it counts)
+    if (s >= slots) s %= slots;
     const uint2 e = __ldg(&table[s]);
     const unsigned empty = __ballot_sync(0xffffffffu, e.x == 0xffffffffu && e.y == 0xffffffffu);
     unsigned hit = __ballot_sync(0xffffffffu, e.x == uint32_t(key) && e.y != 0xffffffffu);
@@ -201,10 +426,11 @@ __device__ __forceinline__ bool is_occurrence(const int32_t* __restrict__ tok, i
 // The group's occurrences of the n tail tokens, ascending, behind the n_occ that s_occ[64] already holds, until there are
 // `cap` (more may be counted, 64 are kept).  All lanes of a warp.
 __device__ __forceinline__ int gather_occurrences(const PoolView& pv, int64_t lo, int64_t hi, const int32_t* tail, int n, uint64_t key,
-                                                  int lane, uint32_t* s_occ, int n_occ, int cap) {
+                                                  int g, int lane, uint32_t* s_occ, int n_occ, int cap) {
   const int before = n_occ;
+  const Region rg = region_of(lo, hi, g);
   uint32_t start;
-  for (uint32_t off = 0; n_occ < cap && n_occ == before && probe(pv.table[n], pv.slots[n], key, lane, off, start); ++off) {
+  for (uint32_t off = 0; n_occ < cap && n_occ == before && probe(pv.table[n] + rg.base, rg.slots, key, lane, off, start); ++off) {
     for (uint32_t base = start; n_occ < cap; base += 32) {   // (the array is padded: lanes past its end read marked padding)
       const uint32_t v = pv.positions[n][base + lane];
       const unsigned ends = __ballot_sync(0xffffffffu, (v & kRunEnd) != 0);
@@ -315,7 +541,7 @@ draft_warp_kernel(PoolView pv, DraftArgs a) {
       }
       if (bad) continue;
       const int want = (a.max_occ > 0 && a.max_occ <= 64) ? a.max_occ : 65;
-      int n_occ = gather_occurrences(pv, lo, hi, tn, n, key_end(h), lane, s_occ[warp], 0, want);
+      int n_occ = gather_occurrences(pv, lo, hi, tn, n, key_end(h), g, lane, s_occ[warp], 0, want);
       if (want == 65 && n_occ > 64) { overflow = n; break; }
       n_occ = min(n_occ, min(want, 64));
       if (n_occ == 0) continue;
@@ -390,7 +616,7 @@ draft_temp_kernel(PoolView pv, DraftArgs a, TempArgs t) {
     }
     n_occ = min(n_occ, cap);
     if (has_group && n_occ < cap)   // the group, ascending
-      n_occ = min(cap, gather_occurrences(pv, lo, hi, tn, n, key_end(key), lane, s_occ[warp], n_occ, cap));
+      n_occ = min(cap, gather_occurrences(pv, lo, hi, tn, n, key_end(key), g, lane, s_occ[warp], n_occ, cap));
     if (n_occ == 0) continue;
     __syncwarp();
     const int len = walk_occurrences(pv.tok, hi, h, hl, lane < n_occ ? s_occ[warp][lane] : 0u, lane + 32 < n_occ ? s_occ[warp][lane + 32] : 0u,
@@ -462,7 +688,7 @@ draft_tree_kernel(PoolView pv, DraftArgs a, TempArgs t, int32_t* __restrict__ dr
       n_occ += __popc(ball);
     }
     n_occ = min(n_occ, cap);
-    if (has_group && n_occ < cap) n_occ = min(cap, gather_occurrences(pv, lo, hi, tn, n, key_end(key), lane, s_occ, n_occ, cap));
+    if (has_group && n_occ < cap) n_occ = min(cap, gather_occurrences(pv, lo, hi, tn, n, key_end(key), g, lane, s_occ, n_occ, cap));
     if (n_occ == 0) continue;
     __syncwarp();
     // ---- continuations ----
@@ -640,7 +866,8 @@ draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound) {
       for (uint32_t off = 0; total == 0; ++off) {  // (a run of another key with the same low half has none)
         if (warp == 0) {
           uint32_t st = 0;
-          const bool f = probe(pv.table[n], pv.slots[n], key_end(h), lane, off, st);
+          const Region rg = region_of(lo, hi, g);
+          const bool f = probe(pv.table[n] + rg.base, rg.slots, key_end(h), lane, off, st);
           if (lane == 0) { s_found = f; s_start = st; s_off = off; s_end = s_cut = 0xffffffffu; }
         }
         __syncthreads();
@@ -848,63 +1075,114 @@ LASER_API laser_status laser_pool_build(const int32_t* tokens, int64_t n_tokens,
 
   LASER_CUDA(cudaGetDevice(&P->device));
 
-  // One allocation for the index, sized before any key is counted (at most one key per token and level, tables at most 5/8
-  // full), so that the levels run back to back without the host; one for the build's own buffers.
+  // Groups by size: what fits shared memory, in three classes of its use (one, two and four CTAs an SM), the larger first, and
+  // the rest.  The positions of the first come first in the position arrays, those of the large groups (sorted together) behind.
   const size_t N = size_t(n_tokens);
-  const uint32_t slots = uint32_t(N + N * 3 / 5 + 64);
+  std::vector<int32_t> id[kClasses + 1];
+  for (int g = 0; g < n_groups; ++g) {
+    const int64_t size = group_offsets[g + 1] - group_offsets[g];
+    int c = 0;
+    while (c < kClasses && size <= kClassMax[c]) ++c;
+    id[c].push_back(g);            // 0: large
+  }
+  // [n_groups] ids, [n_groups + 1] starts: of the small groups their runs' place, of the large ones their place among those
+  std::vector<int64_t> lists(size_t(n_groups) * 2 + 2);
+  int64_t* const h_at = lists.data();
+  int32_t* const h_id = reinterpret_cast<int32_t*>(h_at + n_groups + 1);
+  int64_t n_small = 0, n_large = 0;
+  size_t fill = 0;
+  for (int c = 1; c <= kClasses; ++c)
+    for (int32_t g : id[c]) { h_id[fill] = g; h_at[fill++] = n_small; n_small += group_offsets[g + 1] - group_offsets[g]; }
+  for (int32_t g : id[0]) { h_id[fill] = g; h_at[fill++] = n_large; n_large += group_offsets[g + 1] - group_offsets[g]; }
+  h_at[fill] = n_large;
+  const size_t M = size_t(n_large);
+
+  // One allocation for the index, sized before any key is counted; one for the build's own buffers.
+  const size_t slots = size_t(region_base(n_tokens, n_groups));
+  LASER_REQUIRE(slots < kNoSlot, "%lld tokens in %d groups are too many for one index", (long long)n_tokens, n_groups);
   auto padded = [](size_t bytes) { return (bytes + 255) & ~size_t(255); };
-  const size_t b_tok = padded(N * 4), b_goff = padded((size_t(n_groups) + 1) * 8), b_tab = padded(size_t(slots) * 8), b_pos = padded((N + 32) * 4);
+  const size_t b_tok = padded(N * 4), b_goff = padded((size_t(n_groups) + 1) * 8), b_tab = padded(slots * 8), b_pos = padded((N + 32) * 4);
   P->device_bytes = int64_t(b_tok + b_goff + (n_max - n_min + 1) * (b_tab + b_pos));
   LASER_TRY(pooled_alloc(&P->memory, size_t(P->device_bytes), stream));
   uint8_t* at = static_cast<uint8_t*>(P->memory);
   auto take = [&](auto** p, size_t bytes) { *p = reinterpret_cast<std::remove_reference_t<decltype(*p)>>(at); at += bytes; };
   take(&P->tokens, b_tok);
   take(&P->group_offsets, b_goff);
+  IndexLevels lvs{};
   for (int n = n_min; n <= n_max; ++n) {
     auto& lv = P->level[n];
-    lv.slots = slots;
     take(&lv.table, b_tab);
     take(&lv.positions, b_pos);
+    lvs.table[n] = lv.table; lvs.positions[n] = lv.positions;
   }
   LASER_CUDA(cudaMemcpyAsync(P->tokens, tokens, N * 4, cudaMemcpyDefault, stream));
   LASER_CUDA(cudaMemcpyAsync(P->group_offsets, group_offsets, (size_t(n_groups) + 1) * 8, cudaMemcpyHostToDevice, stream));
 
+  // The large groups' n-grams go through one sort for as many n as 32-bit slot numbers and 64 M pairs hold.
+  const int levels = n_max - n_min + 1;
+  const int batch = int(std::max<size_t>(1, std::min({size_t(levels), size_t(kNoSlot) / slots, (size_t(64) << 20) / std::max<size_t>(M, 1)})));
+  int slot_bits = 1;             // all that kNoSlot needs to sort behind every slot
+  while (slot_bits < 32 && (slots * batch) >> slot_bits) ++slot_bits;
+  const size_t pairs = M * batch;
   size_t cub_bytes = 0;
-  {
-    cub::DoubleBuffer<uint64_t> kb(nullptr, nullptr);
-    cub::DoubleBuffer<uint32_t> vb(nullptr, nullptr);
-    LASER_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, cub_bytes, kb, vb, int64_t(N), 0, 64, stream));
+  if (M) {
+    cub::DoubleBuffer<uint32_t> kb(nullptr, nullptr), vb(nullptr, nullptr);
+    LASER_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, cub_bytes, kb, vb, int64_t(pairs), 0, slot_bits, stream));
   }
-  constexpr size_t kCounters = (kMaxN + 2) * 8;   // distinct keys per level, then the largest token
+  constexpr size_t kCounters = (2 * kMaxN + 3) * 8;   // distinct keys per n, the largest token, n-grams of the large groups per n
+  const size_t b_lists = lists.size() * 8;
   struct Tmp { void* p = nullptr; cudaStream_t s; ~Tmp() { pooled_free(p, s); } } tmp{nullptr, stream};
-  LASER_TRY(pooled_alloc(&tmp.p, 2 * padded(N * 8) + 2 * padded(N * 4) + kCounters + 256 + cub_bytes, stream));
+  LASER_TRY(pooled_alloc(&tmp.p, 4 * padded(pairs * 4) + padded(kCounters) + padded(b_lists) + cub_bytes + 256, stream));
   at = static_cast<uint8_t*>(tmp.p);
-  uint64_t *keys, *keys_alt;
-  uint32_t *pos, *pos_alt;
+  uint32_t *slot_of, *slot_alt, *pos, *pos_alt;
   unsigned long long* counters;
+  int64_t* d_at;
   uint8_t* cub_tmp;
-  take(&keys, padded(N * 8)); take(&keys_alt, padded(N * 8)); take(&pos, padded(N * 4)); take(&pos_alt, padded(N * 4));
-  take(&counters, padded(kCounters)); take(&cub_tmp, cub_bytes);
+  take(&slot_of, padded(pairs * 4)); take(&slot_alt, padded(pairs * 4)); take(&pos, padded(pairs * 4)); take(&pos_alt, padded(pairs * 4));
+  take(&counters, padded(kCounters)); take(&d_at, padded(b_lists)); take(&cub_tmp, cub_bytes);
+  const int32_t* d_id = reinterpret_cast<const int32_t*>(d_at + n_groups + 1);
   int* max_tok = reinterpret_cast<int*>(counters + kMaxN + 1);
+  unsigned long long* n_valid = counters + kMaxN + 2;
+  LASER_CUDA(cudaMemcpyAsync(d_at, lists.data(), b_lists, cudaMemcpyHostToDevice, stream));
   LASER_CUDA(cudaMemsetAsync(counters, 0, kCounters, stream));
   LASER_CUDA(cudaMemsetAsync(max_tok, 0xff, 4, stream));
-  const unsigned blocks = unsigned(ceil_div<size_t>(N, kKeyThreads));
-  for (int n = n_min; n <= n_max; ++n) {
-    auto& lv = P->level[n];
-    make_keys_kernel<<<blocks, kKeyThreads, 0, stream>>>(P->tokens, n_tokens, P->group_offsets, n_groups, n, keys, pos,
-                                                         n == n_min ? max_tok : nullptr);
-    cub::DoubleBuffer<uint64_t> kb(keys, keys_alt);
-    cub::DoubleBuffer<uint32_t> vb(pos, pos_alt);
-    LASER_CUDA(cub::DeviceRadixSort::SortPairs(cub_tmp, cub_bytes, kb, vb, int64_t(N), 0, 64, stream));
-    LASER_CUDA(cudaMemsetAsync(lv.table, 0xff, size_t(slots) * 8, stream));
-    LASER_CUDA(cudaMemsetAsync(lv.positions + N, 0xff, 32 * 4, stream));
-    index_runs_kernel<<<blocks, kKeyThreads, 0, stream>>>(kb.Current(), vb.Current(), n_tokens, lv.positions,
-                                                          reinterpret_cast<unsigned long long*>(lv.table), slots, counters + n);
-    count_launch(2);
-    LASER_CUDA(cudaGetLastError());
+  for (int n = n_min; n <= n_max; ++n) LASER_CUDA(cudaMemsetAsync(P->level[n].positions + N, 0xff, 32 * 4, stream));
+  size_t done = 0;
+  for (int c = 1; c <= kClasses; ++c) {
+    if (id[c].empty()) continue;
+    auto index = [&](auto kernel, unsigned threads) -> laser_status {
+      const size_t smem = group_smem(kClassMax[c - 1]);
+      LASER_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+      LASER_CUDA(launch_overlapped(kernel, dim3(unsigned(id[c].size()), unsigned(n_max - n_min + 1)), threads, smem, stream, P->tokens,
+                                   P->group_offsets, d_id + done, d_at + done, done == 0 ? 1 : 0, n_min, lvs, counters, max_tok));
+      return LASER_OK;
+    };
+    LASER_TRY(c == 1 ? index(index_group_kernel<1024, 1>, 1024) : c == 2 ? index(index_group_kernel<512, 2>, 512) : index(index_group_kernel<512, 3>, 512));
+    count_launch();
+    done += id[c].size();
+  }
+  if (M) {
+    const LargeGroups lg{d_id + done, d_at + done, int(id[0].size())};
+    const unsigned blocks = unsigned(ceil_div<size_t>(M, kInsertBlock));
+    for (int l0 = 0; l0 < lg.n; l0 += 65535)
+      clear_regions_kernel<<<dim3(16, unsigned(std::min(lg.n - l0, 65535)), unsigned(levels)), kKeyThreads, 0, stream>>>(
+          lvs, n_min, P->group_offsets, LargeGroups{lg.id + l0, lg.at + l0, lg.n - l0});
+    count_launch();
+    for (int n0 = n_min; n0 <= n_max; n0 += batch) {
+      const int nb = std::min(batch, n_max - n0 + 1);
+      const int64_t count = int64_t(M) * nb;
+      insert_large_kernel<<<dim3(blocks, unsigned(nb)), kKeyThreads, 0, stream>>>(P->tokens, P->group_offsets, lg, n_large, n0, lvs,
+                                                                                  uint32_t(slots), slot_of, pos, n_valid, max_tok);
+      cub::DoubleBuffer<uint32_t> kb(slot_of, slot_alt), vb(pos, pos_alt);
+      LASER_CUDA(cub::DeviceRadixSort::SortPairs(cub_tmp, cub_bytes, kb, vb, count, 0, slot_bits, stream));
+      index_runs_kernel<<<unsigned(ceil_div<int64_t>(count, kKeyThreads)), kKeyThreads, 0, stream>>>(
+          kb.Current(), vb.Current(), count, n_small, n0, lvs, uint32_t(slots), n_valid, counters);
+      count_launch(2);
+      LASER_CUDA(cudaGetLastError());
+    }
   }
   unsigned long long h_cnt[kMaxN + 2] = {};
-  LASER_CUDA(cudaMemcpyAsync(h_cnt, counters, kCounters, cudaMemcpyDeviceToHost, stream));
+  LASER_CUDA(cudaMemcpyAsync(h_cnt, counters, sizeof(h_cnt), cudaMemcpyDeviceToHost, stream));
   LASER_CUDA(cudaStreamSynchronize(stream));
   for (int n = n_min; n <= n_max; ++n) P->level[n].n_keys = int64_t(h_cnt[n]);
   P->vocab_bound = int32_t(uint32_t(h_cnt[kMaxN + 1])) + 1;
