@@ -2,10 +2,12 @@
 // ablation variants (Eq. 7; "top-p" of Section 4.3.2), longest accepted prefix, correction
 // or bonus token, and the KV-cache length update.
 //
-// One CTA per (sequence, row) reads its row once (verdict.cuh): max / arg max (smallest id on
+// A row is read once (verdict.cuh), by one CTA or in parts by several: max / arg max (smallest id on
 // ties), the tokens ranked ahead of the draft token and, where the rule needs a probability, the
-// sum of exp(l - max).  The last CTA of a sequence to finish walks the per-row verdicts in order
-// and writes the outputs.  Reductions have a fixed shape, so results are identical from run to run.
+// sum of exp(l - max).  The last CTA of a sequence to finish puts the parts together, walks the rows'
+// verdicts in order and writes the outputs.  Reductions have a fixed shape, so results are identical
+// from run to run.
+#include <algorithm>
 #include <mutex>
 
 #include "state.cuh"
@@ -17,22 +19,27 @@ namespace {
 constexpr int kAcceptThreads = kVerdictThreads;
 constexpr int kMaxAcceptSeqs = 1 << 16;  // counters live at the start of the scratch
 
-struct RowVerdict { int32_t argmax; int32_t pass; };
+constexpr int kMaxParts = 8;
+
+// Parts of a row: a CTA goes through its part in batches of 8192 values, a memory round trip each, so few rows are cut until the
+// SMs are full (two CTAs for every one that can be resident: of a step's rows many are inactive) or a part is half a batch.
+int parts_of(int64_t rows, int32_t V) {
+  return int(std::max<int64_t>(1, std::min<int64_t>({kMaxParts, 8 * 148 / rows, V / 4096})));
+}
 
 __global__ void __launch_bounds__(kAcceptThreads)
 accept_rows_kernel(const float* logits, const int32_t* tokens, const int32_t* n_rows, const int32_t* seq_ids,
-                   int32_t R, int32_t V, int32_t mode, int32_t topk, double p,
-                   int32_t* __restrict__ counters, RowVerdict* __restrict__ verdicts,
+                   int32_t R, int32_t V, const Rule rule, int32_t* __restrict__ counters, RowResult* results,
                    int32_t* __restrict__ n_accept, int32_t* __restrict__ out_tokens,
                    int32_t* __restrict__ n_out, int32_t* __restrict__ kv_len, unsigned long long* stamp) {
-  const int b = blockIdx.x / R, i = blockIdx.x % R;
+  const int b = blockIdx.x / R, i = blockIdx.x % R, part = blockIdx.y, parts = gridDim.y;
   next_may_launch();
   wait_for_earlier();
-  if (stamp && blockIdx.x == 0 && threadIdx.x == 0) *stamp = device_ns();
+  if (stamp && blockIdx.x == 0 && part == 0 && threadIdx.x == 0) *stamp = device_ns();
   const int nr = min(n_rows[b], R);
   const int tid = threadIdx.x;
   if (nr <= 0) {
-    if (i == 0) {
+    if (i == 0 && part == 0) {
       if (tid == 0) { n_accept[b] = 0; n_out[b] = 0; }
       for (int j = tid; j < R; j += kAcceptThreads) out_tokens[b * R + j] = -1;
     }
@@ -40,45 +47,59 @@ accept_rows_kernel(const float* logits, const int32_t* tokens, const int32_t* n_
   }
   if (i >= nr) return;
 
-  const float* row = logits + (size_t(b) * R + i) * V;
-  // max, arg max, and the verdict on the draft token that this row verifies, if any
-  float mx;
-  int arg, pass;
-  cta_row(row, V, i + 1 < nr ? tokens[b * R + i + 1] : -1, mode, topk, p, &mx, &arg, &pass);
+  // row x verifies draft token x + 1, if there is one
+  auto row_of = [&](int x) { return logits + (size_t(b) * R + x) * V; };
+  auto token_of = [&](int x) { return x + 1 < nr ? tokens[b * R + x + 1] : -1; };
+  RowResult mine = cta_scan(row_of(i), V, part, parts, token_of(i), rule);
 
-  // publish, then let the last CTA of this sequence scan the verdicts in order
+  // publish, then let the last CTA of this sequence go through the rows in order
   __shared__ int s_last;
   if (tid == 0) {
-    verdicts[b * R + i] = RowVerdict{arg, pass};
+    if (parts == 1) mine.ahead = judge(row_of(i), V, token_of(i), rule, mine);   // (its verdict: 0, 1 or 2)
+    results[(size_t(b) * R + i) * parts + part] = mine;
     __threadfence();
-    const int done = atomicAdd(&counters[b], 1);
-    s_last = (done == nr - 1);
+    s_last = atomicAdd(&counters[b], 1) == nr * parts - 1;
   }
   __syncthreads();
   if (!s_last) return;
   __threadfence();
-  __shared__ int s_a;
-  const volatile RowVerdict* v = verdicts + b * R;
+  __shared__ int s_arg[kAcceptThreads], s_pass[kAcceptThreads];
+  __shared__ float s_max[kAcceptThreads];
+  int a = 0, base = 0;           // (the same in every thread)
+  for (bool go = true;; base += kAcceptThreads) {   // a row a thread: rows base .. base + kAcceptThreads - 1
+    const int x = base + tid;
+    if (x < nr) {
+      const volatile RowResult* v = results + (size_t(b) * R + x) * parts;
+      RowResult r{v->mx, v->arg, v->ahead, v->m, v->s, v->lt};
+      for (int q = 1; q < parts; ++q) merge_rows(r, RowResult{v[q].mx, v[q].arg, v[q].ahead, v[q].m, v[q].s, 0.f});
+      s_pass[tid] = parts == 1 ? r.ahead : judge(row_of(x), V, token_of(x), rule, r);
+      s_arg[tid] = r.arg;
+      s_max[tid] = r.mx;
+    }
+    __syncthreads();
+    for (const int end = min(nr - 1, base + kAcceptThreads); go && a < end; a += go) {
+      const int pass = s_pass[a - base];
+      go = (pass == 2 ? exact_pass(row_of(a), V, token_of(a), s_max[a - base], rule.p) : pass) != 0;
+    }
+    if (!go || a < base + kAcceptThreads) break;
+    __syncthreads();
+  }
   if (tid == 0) {
-    int a = 0;
-    while (a < nr - 1 && v[a].pass) ++a;
-    s_a = a;
     n_accept[b] = a;
     n_out[b] = a + 1;
     if (kv_len) kv_len[seq_ids[b]] += a + 1;
     counters[b] = 0;  // ready for the next call
   }
-  __syncthreads();
-  const int a = s_a;
   for (int j = tid; j < R; j += kAcceptThreads)
-    out_tokens[b * R + j] = j < a ? tokens[b * R + j + 1] : (j == a ? v[a].argmax : -1);
+    out_tokens[b * R + j] = j < a ? tokens[b * R + j + 1] : (j == a ? s_arg[a - base] : -1);
 }
 
-// Fixed scratch of the allocation-free entry point: per-sequence counters, then row verdicts.
+// Fixed scratch of the allocation-free entry point: per-sequence counters, then the rows' results (rows in parts are few).
 constexpr int kNoAllocMaxSeqs = 1024;
 constexpr int kNoAllocMaxRows = 16384;
 constexpr size_t kNoAllocCounterBytes = sizeof(int32_t) * kNoAllocMaxSeqs;
-constexpr size_t kNoAllocBytes = kNoAllocCounterBytes + sizeof(RowVerdict) * kNoAllocMaxRows;
+constexpr size_t kNoAllocBytes = kNoAllocCounterBytes + sizeof(RowResult) * kNoAllocMaxRows;
+static_assert(8 * 148 <= kNoAllocMaxRows, "");
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
 // Device address of g_noalloc_scratch on the current device, resolved once per device.  Host threads
@@ -124,12 +145,12 @@ LASER_API laser_status laser_accept_commit_noalloc(laser_kv* kv, const int32_t* 
   void* scratch = nullptr;
   LASER_TRY(noalloc_scratch(&scratch));
   int32_t* counters = static_cast<int32_t*>(scratch);
-  RowVerdict* verdicts = reinterpret_cast<RowVerdict*>(static_cast<char*>(scratch) + kNoAllocCounterBytes);
+  RowResult* results = reinterpret_cast<RowResult*>(static_cast<char*>(scratch) + kNoAllocCounterBytes);
   // the array keeps whatever the previous call left: the arrival counters must start at zero
   LASER_CUDA(cudaMemsetAsync(counters, 0, sizeof(int32_t) * size_t(B), as_stream(stream)));
-  const int R = p->K + 1;
-  LASER_CUDA(launch_overlapped(accept_rows_kernel, dim3(unsigned(B * R)), kAcceptThreads, 0, as_stream(stream),
-      logits, tokens, n_rows, seq_ids, R, V, p->mode, p->topk, double(p->p), counters, verdicts,
+  const int R = p->K + 1, parts = parts_of(rows, V);
+  LASER_CUDA(launch_overlapped(accept_rows_kernel, dim3(unsigned(B * R), unsigned(parts)), kAcceptThreads, 0, as_stream(stream),
+      logits, tokens, n_rows, seq_ids, R, V, Rule{p->mode, p->topk, double(p->p)}, counters, results,
       n_accept, out_tokens, n_out, kv ? kv->seq_len : nullptr, static_cast<unsigned long long*>(nullptr)));
   count_launch();
   LASER_CUDA(cudaGetLastError());
@@ -149,14 +170,14 @@ laser_status accept_commit(laser_kv* kv, const int32_t* seq_ids, const float* lo
                 "topk = %d", p->topk);
   LASER_REQUIRE(kv == nullptr || seq_ids != nullptr, "seq_ids is required when committing");
   if (B == 0) return LASER_OK;
-  const int R = p->K + 1;
+  const int R = p->K + 1, parts = parts_of(int64_t(B) * R, V);
   void* scratch = nullptr;
   const size_t counters_bytes = sizeof(int32_t) * kMaxAcceptSeqs;
-  LASER_TRY(scratch_get(SCRATCH_ACCEPT, counters_bytes + sizeof(RowVerdict) * size_t(B) * R, &scratch));
+  LASER_TRY(scratch_get(SCRATCH_ACCEPT, counters_bytes + sizeof(RowResult) * size_t(B) * R * parts, &scratch));
   int32_t* counters = static_cast<int32_t*>(scratch);
-  RowVerdict* verdicts = reinterpret_cast<RowVerdict*>(static_cast<char*>(scratch) + counters_bytes);
-  LASER_CUDA(launch_overlapped(accept_rows_kernel, dim3(unsigned(B * R)), kAcceptThreads, 0, stream,
-      logits, tokens, n_rows, seq_ids, R, V, p->mode, p->topk, double(p->p), counters, verdicts,
+  RowResult* results = reinterpret_cast<RowResult*>(static_cast<char*>(scratch) + counters_bytes);
+  LASER_CUDA(launch_overlapped(accept_rows_kernel, dim3(unsigned(B * R), unsigned(parts)), kAcceptThreads, 0, stream,
+      logits, tokens, n_rows, seq_ids, R, V, Rule{p->mode, p->topk, double(p->p)}, counters, results,
       n_accept, out_tokens, n_out, kv ? kv->seq_len : nullptr, stamp));
   count_launch();
   LASER_CUDA(cudaGetLastError());

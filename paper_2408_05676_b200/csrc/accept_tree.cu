@@ -41,15 +41,14 @@ accept_tree_kernel(const float* logits, const int32_t* tokens, const int32_t* pa
     return;
   }
   if (i >= nr) return;
-  float mx;
+  const Rule rule{mode, topk, p};
   int arg, pass = 0;
-  cta_row(logits + (size_t(b) * R + i) * V, V, -1, mode, topk, p, &mx, &arg, &pass);
+  cta_row(logits + (size_t(b) * R + i) * V, V, -1, rule, &arg, &pass);
   if (i > 0) {
     const int par = parents[b * R + i];
     if (par >= 0 && par < i) {      // a malformed parent verifies nothing
-      float pmx;
       int parg;
-      cta_row(logits + (size_t(b) * R + par) * V, V, tokens[b * R + i], mode, topk, p, &pmx, &parg, &pass);
+      cta_row(logits + (size_t(b) * R + par) * V, V, tokens[b * R + i], rule, &parg, &pass);
     }
   }
   __shared__ int s_last;

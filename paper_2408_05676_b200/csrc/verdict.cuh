@@ -1,12 +1,13 @@
 // Row pass shared by the acceptance kernels (Eq. 4, Eq. 7, Eq. 8 and the variants of Section 4.3.2): max and arg max of a row
 // of logits, and the verdict on one token given its row - its rank (tokens ahead of it; equal logits rank the smaller id
 // first) and, where the rule needs it, whether its probability exceeds p, the denominator in fp64 from fp32 differences.
-// One CTA of kVerdictThreads threads works on one row; reductions have a fixed shape, so results are identical from run to run.
+// One CTA of kVerdictThreads threads works on one row or a part of it; reductions have a fixed shape, so results are identical from
+// run to run.
 //
 // The row is read once, 16 bytes a load and eight loads in flight per thread.  The probability is first estimated in fp32 with a
 // running maximum; the fp64 sum - an exponential per token, which used to be most of the kernel - is taken only where the
 // estimate lies within its error bound of p, so that the verdict is always the fp64 one.  64 sequences x 1 .. 9 rows of 32000
-// logits, relaxed rule: 57.5 -> 20.1 us.
+// logits, relaxed rule: 57.5 -> 20.1 us; 18.4 with launches overlapped, 16.2 with the rows in two parts each.
 #pragma once
 #include "common.cuh"
 
@@ -19,15 +20,15 @@ __device__ __forceinline__ void better(float& v, int& i, float ov, int oi) {
   if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; }
 }
 
-struct RowResult { float mx; int arg; int ahead; float m, s; };   // s = sum of exp(x - m) over what was seen
+struct RowResult { float mx; int arg; int ahead; float m, s, lt; };   // s = sum of exp(x - m) over what was seen; lt = the token's
 
 // exp(d) for d <= 0.  ex2 is good to 2 units in the last place and the product's rounding shifts the exponent by |d| 2^-24:
 // within 1e-5 of exp(d) wherever that is not below 1e-38.
 __device__ __forceinline__ float exp_below(float d) { return exp2f(d * 1.4426950408889634f); }
 
 template <bool RANK, bool PROB>
-__device__ __forceinline__ RowResult scan_row(const float* __restrict__ row, int V, int t, float lt, int tid) {
-  RowResult r{-INFINITY, 0x7fffffff, 0, -INFINITY, 0.f};
+__device__ __forceinline__ RowResult scan_row(const float* __restrict__ row, int V, int part, int parts, int t, float lt, int tid) {
+  RowResult r{-INFINITY, 0x7fffffff, 0, -INFINITY, 0.f, lt};
   const int lead = min(V, int((16 - (reinterpret_cast<uintptr_t>(row) & 15)) & 15) >> 2);   // values before the first 16-byte boundary
   const int n4 = (V - lead) >> 2;
   auto batch = [&](const float* x, int cnt, auto index_of) {
@@ -55,46 +56,50 @@ __device__ __forceinline__ RowResult scan_row(const float* __restrict__ row, int
       r.s += add;
     }
   };
-  if (tid < lead) batch(row + tid, 1, [&](int) { return tid; });
+  const int per = (n4 + parts - 1) / parts, end = min(n4, (part + 1) * per);   // (float4s of this part: part * per .. end - 1)
+  if (part == 0 && tid < lead) batch(row + tid, 1, [&](int) { return tid; });
   const float4* r4 = reinterpret_cast<const float4*>(row + lead);
-  for (int base = 0; base < n4; base += kVerdictThreads * kRowLoads) {
+  for (int base = part * per; base < end; base += kVerdictThreads * kRowLoads) {
     float x[4 * kRowLoads];
 #pragma unroll
     for (int u = 0; u < kRowLoads; ++u) {
       const int i = base + u * kVerdictThreads + tid;
-      const float4 v = i < n4 ? r4[i] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+      const float4 v = i < end ? r4[i] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
       x[4 * u] = v.x; x[4 * u + 1] = v.y; x[4 * u + 2] = v.z; x[4 * u + 3] = v.w;
     }
     batch(x, 4 * kRowLoads, [&](int i) { return lead + 4 * (base + (i >> 2) * kVerdictThreads + tid) + (i & 3); });
   }
   const int tail = lead + 4 * n4 + tid;
-  if (tail < V) batch(row + tail, 1, [&](int) { return tail; });
+  if (part == parts - 1 && tail < V) batch(row + tail, 1, [&](int) { return tail; });
   return r;
 }
 
-// Max and arg max (smallest id on ties) of a row in every thread, and in thread 0 whether token t passes on it (t < 0: none).
-static __device__ void cta_row(const float* __restrict__ row, int V, int t, int mode, int topk, double p, float* mx_out, int* arg_out,
-                               int* pass_out) {
+__device__ __forceinline__ void merge_rows(RowResult& r, const RowResult& o) {
+  better(r.mx, r.arg, o.mx, o.arg);
+  r.ahead += o.ahead;
+  const float m = fmaxf(r.m, o.m);
+  if (m > -INFINITY)
+    r.s = (r.m > -INFINITY ? r.s * exp_below(r.m - m) : 0.f) + (o.m > -INFINITY ? o.s * exp_below(o.m - m) : 0.f);
+  r.m = m;
+}
+
+struct Rule {
+  int mode, topk;
+  double p;
+  __device__ bool needs_p() const { return mode == LASER_MODE_RELAXED || mode == LASER_MODE_TOPP || mode == LASER_MODE_RELAXED_ARGMAX; }
+  __device__ bool needs_rank() const { return mode == LASER_MODE_RELAXED || mode == LASER_MODE_TOPK || mode == LASER_MODE_RELAXED_ARGMAX; }
+};
+
+// What a CTA finds in its part of a row, in thread 0.  t: the token whose verdict the row gives (t < 0: none).
+static __device__ RowResult cta_scan(const float* row, int V, int part, int parts, int t, const Rule& rule) {
   constexpr int kWarps = kVerdictThreads / 32;
   __shared__ RowResult s_part[kWarps];
-  __shared__ float s_max;
-  __shared__ int s_arg, s_exact;
-  __shared__ double s_sum[kWarps];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   const bool judged = t >= 0 && t < V;
-  const bool need_p = judged && (mode == LASER_MODE_RELAXED || mode == LASER_MODE_TOPP || mode == LASER_MODE_RELAXED_ARGMAX);
-  const bool need_rank = judged && (mode == LASER_MODE_RELAXED || mode == LASER_MODE_TOPK || mode == LASER_MODE_RELAXED_ARGMAX);
+  const bool need_p = judged && rule.needs_p(), need_rank = judged && rule.needs_rank();
   const float lt = judged ? row[t] : 0.f;
-  RowResult r = need_p ? (need_rank ? scan_row<true, true>(row, V, t, lt, tid) : scan_row<false, true>(row, V, t, lt, tid))
-                       : (need_rank ? scan_row<true, false>(row, V, t, lt, tid) : scan_row<false, false>(row, V, t, lt, tid));
-  auto merge = [&](const RowResult& o) {
-    better(r.mx, r.arg, o.mx, o.arg);
-    r.ahead += o.ahead;
-    const float m = fmaxf(r.m, o.m);
-    if (m > -INFINITY)
-      r.s = (r.m > -INFINITY ? r.s * exp_below(r.m - m) : 0.f) + (o.m > -INFINITY ? o.s * exp_below(o.m - m) : 0.f);
-    r.m = m;
-  };
+  RowResult r = need_p ? (need_rank ? scan_row<true, true>(row, V, part, parts, t, lt, tid) : scan_row<false, true>(row, V, part, parts, t, lt, tid))
+                       : (need_rank ? scan_row<true, false>(row, V, part, parts, t, lt, tid) : scan_row<false, false>(row, V, part, parts, t, lt, tid));
   for (int o = 16; o; o >>= 1) {
     RowResult other;
     other.mx = __shfl_xor_sync(0xffffffffu, r.mx, o);
@@ -102,50 +107,72 @@ static __device__ void cta_row(const float* __restrict__ row, int V, int t, int 
     other.ahead = __shfl_xor_sync(0xffffffffu, r.ahead, o);
     other.m = __shfl_xor_sync(0xffffffffu, r.m, o);
     other.s = __shfl_xor_sync(0xffffffffu, r.s, o);
-    merge(other);
+    merge_rows(r, other);
   }
   __syncthreads();   // the shared slots may still be read from an earlier call
   if (lane == 0) s_part[warp] = r;
   __syncthreads();
-  int pass = 0;
+  if (tid == 0)
+    for (int w = 1; w < kWarps; ++w) merge_rows(r, s_part[w]);
+  return r;
+}
+
+// One thread, from a whole row's result: the arg max (smallest id on ties), and whether t passes: 0, 1, or 2 where only the rule's
+// own arithmetic (exact_pass) can tell.
+static __device__ int judge(const float* row, int V, int t, const Rule& rule, RowResult& r) {
+  if (r.arg == 0x7fffffff)   // nothing above -inf: the first -inf, as an ascending scan would find it
+    for (int j = V - 1; j >= 0; --j) if (row[j] == -INFINITY) r.arg = j;
+  if (t < 0 || t >= V) return 0;
+  const bool top = t == r.arg, in_topk = r.ahead < rule.topk;
+  // The estimate's relative error: each term 1e-5, a term's at most 6 rescalings per thread (V / 8192 batches; rows beyond
+  // 49152 tokens add one per 8192) and 8 + 7 merges (lanes and warps, parts) 1e-5 each, sums of 128 + 20 terms 1e-5; the numerator
+  // 1e-5.  Twice that.
+  const double margin = 5.2e-4 + 2e-9 * V;
+  const double q = double(exp_below(r.lt - r.mx)) / double(r.s);
+  const bool matters = rule.needs_p() && (rule.mode == LASER_MODE_RELAXED ? in_topk : rule.mode == LASER_MODE_TOPP ? !top : !top && in_topk);
+  const bool sure_above = q * (1.0 - margin) > rule.p, sure_below = q * (1.0 + margin) < rule.p;
+  if (matters && !sure_above && !sure_below) return 2;      // (a NaN is neither)
+  if (rule.mode == LASER_MODE_STRICT) return top;
+  if (rule.mode == LASER_MODE_RELAXED) return in_topk && sure_above;
+  if (rule.mode == LASER_MODE_TOPK) return in_topk;
+  if (rule.mode == LASER_MODE_RELAXED_ARGMAX) return top || (in_topk && sure_above);
+  return top || sure_above;
+}
+
+// The rule's own arithmetic, by the whole CTA: everything else about the row is settled, the probability decides.  Every thread
+// gets the answer.
+static __device__ int exact_pass(const float* row, int V, int t, float mx, double p) {
+  constexpr int kWarps = kVerdictThreads / 32;
+  __shared__ double s_sum[kWarps];
+  __shared__ int s_pass;
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  double sum = 0.0;
+  for (int j = tid; j < V; j += kVerdictThreads) sum += exp(double(row[j] - mx));
+  for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  __syncthreads();   // (the slots of an earlier call)
+  if (lane == 0) s_sum[warp] = sum;
+  __syncthreads();
   if (tid == 0) {
-    for (int w = 1; w < kWarps; ++w) merge(s_part[w]);
-    if (r.arg == 0x7fffffff)   // nothing above -inf: the first -inf, as an ascending scan would find it
-      for (int j = V - 1; j >= 0; --j) if (row[j] == -INFINITY) r.arg = j;
-    s_max = r.mx; s_arg = r.arg;
-    s_exact = 0;
-    if (judged) {
-      const bool top = t == r.arg, in_topk = r.ahead < topk;
-      // The estimate's relative error: each term 1e-5, a term's at most 6 rescalings per thread (V / 8192 batches; rows beyond
-      // 49152 tokens add one per 8192) and 8 merges 1e-5 each, sums of 128 + 13 terms 1e-5; the numerator 1e-5.  Twice that.
-      const double margin = 4e-4 + 2e-9 * V;
-      const double q = double(exp_below(lt - r.mx)) / double(r.s);
-      const bool matters = need_p && (mode == LASER_MODE_RELAXED ? in_topk : mode == LASER_MODE_TOPP ? !top : !top && in_topk);
-      const bool sure_above = q * (1.0 - margin) > p, sure_below = q * (1.0 + margin) < p;
-      if (matters && !sure_above && !sure_below) s_exact = 1;      // (a NaN is neither)
-      if (mode == LASER_MODE_STRICT) pass = top;
-      else if (mode == LASER_MODE_RELAXED) pass = in_topk && sure_above;
-      else if (mode == LASER_MODE_TOPK) pass = in_topk;
-      else if (mode == LASER_MODE_RELAXED_ARGMAX) pass = top || (in_topk && sure_above);
-      else pass = top || sure_above;
-    }
+    for (int w = 1; w < kWarps; ++w) sum += s_sum[w];
+    s_pass = exp(double(row[t] - mx)) / sum > p;
   }
   __syncthreads();
-  *mx_out = s_max;
-  *arg_out = s_arg;
-  if (s_exact) {   // the rule's own arithmetic: everything else about it is settled, the probability decides
-    const float mx = s_max;
-    double sum = 0.0;
-    for (int j = tid; j < V; j += kVerdictThreads) sum += exp(double(row[j] - mx));
-    for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == 0) s_sum[warp] = sum;
-    __syncthreads();
-    if (tid == 0) {
-      for (int w = 1; w < kWarps; ++w) sum += s_sum[w];
-      pass = exp(double(lt - mx)) / sum > p;
-    }
+  return s_pass;
+}
+
+// Max and arg max (smallest id on ties) of a row, and whether token t passes on it (t < 0: none), in every thread.
+static __device__ void cta_row(const float* row, int V, int t, const Rule& rule, int* arg_out, int* pass_out) {
+  __shared__ float s_max;
+  __shared__ int s_arg, s_verdict;
+  RowResult r = cta_scan(row, V, 0, 1, t, rule);
+  if (threadIdx.x == 0) {
+    s_verdict = judge(row, V, t, rule, r);
+    s_max = r.mx; s_arg = r.arg;
   }
-  *pass_out = pass;
+  __syncthreads();
+  *arg_out = s_arg;
+  const int verdict = s_verdict;
+  *pass_out = verdict == 2 ? exact_pass(row, V, t, s_max, rule.p) : verdict;
 }
 
 }  // namespace laser
