@@ -1,4 +1,4 @@
-"""Acceptance with a row's CTAs (csrc/accept.cu): few rows are cut into up to eight parts, many rows are read whole, and more
+"""Acceptance with a row's CTAs (csrc/accept.cu): few rows are cut into two or four parts, many rows are read whole, and more
 rows of a sequence than the last CTA has threads are judged in turn; against the oracle's rule, the fp64 decision included."""
 import numpy as np
 import pytest
@@ -17,7 +17,7 @@ def L():
     return binding
 
 
-# rows x parts: 8 * 148 // rows parts of at least 4096 values, eight at most
+# parts of at least 4096 values while there are at most 1184 launched and 640 active ones
 @pytest.mark.parametrize("B,R,V", [
     (1, 2, 8195), (1, 3, 12287), (2, 5, 32003), (13, 9, 33001), (66, 9, 32002), (65, 9, 8200), (1, 256, 40), (1, 257, 31), (2, 300, 17), (1, 513, 9),
 ])
