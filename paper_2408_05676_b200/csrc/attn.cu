@@ -28,7 +28,7 @@ constexpr int kAttnThreads = (kConsumers + 1) * 32;
 constexpr int kStages = 4;   // a multiple of kConsumers: stage s always serves warp s % 4
 constexpr int kMaxPageSplits = 8;  // CTAs that share a sequence's pages
 constexpr int kSplitFrom = 16;      // pages from which a split pays for the merge (about 3 us, ten pages of one CTA's walk),
-constexpr int kSplitPages = 4;      // and pages a run has at least
+constexpr int kSplitPages = 8;      // and pages a run has at least
 constexpr int kCtasPerSm = 4;  // registers and shared memory are sized for four resident CTAs
 
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
@@ -72,6 +72,7 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
   __shared__ float s_m[kConsumers][16], s_l[kConsumers][16], s_wgt[kConsumers][16];
   __shared__ int abort_flag;
   __shared__ int s_last;
+  __shared__ float s_inv[SP ? 16 * TPC : 1];
 
   // Programmatic dependent launch: let the next kernel start its prologue.  The kernel before this
   // one produces Q and the K/V of the step's own rows; pages that lie wholly below the committed
@@ -106,9 +107,10 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
   bf16* q_ptr = reinterpret_cast<bf16*>(tiles_ptr + kStages * STAGE);
   const int n_keys = ctx + (row_mask ? nr : min(nr, cta_row0 + 16 * TPC));   // chain: no row here sees a later one
   const int all_pg = (n_keys + 15) >> 4;
-  const int parts = SP ? (all_pg < kSplitFrom ? 1 : min(splits, all_pg / kSplitPages)) : 1;
+  // (the runs do not depend on how many rows the step has, so that a row's result is the same among drafts and alone)
+  const int per = SP ? max(kSplitPages, (pages_per_seq + splits - 1) / splits) : all_pg, parts = SP ? (all_pg + per - 1) / per : 1;
   if (SP && krank >= parts) return;
-  const int per = (all_pg + parts - 1) / parts, pg0 = krank * per;
+  const int pg0 = krank * per;
   const int n_pg = SP ? max(0, min(per, all_pg - pg0)) : all_pg;   // this CTA's pages are pg0 .. pg0 + n_pg - 1
   const bool whole = !SP || parts == 1;
   const int unit = (b * H + h) * gridDim.z + mt;
@@ -332,7 +334,8 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
       if (wsel == tsel) { __stcg(my_part + 16 * TPC * DH + tsel * 16 + r, mt_); __stcg(my_part + 16 * TPC * (DH + 1) + tsel * 16 + r, den); }
     } else {
       const bool live = cta_row0 + tsel * 16 + r < nr && den > 0.f && !abort_flag;
-      s_wgt[wsel][r] = live ? mine / den : 0.f;
+      s_wgt[wsel][r] = !live ? 0.f : SP ? mine : mine / den;
+      if (SP && wsel == tsel) s_inv[tsel * 16 + r] = live ? 1.f / den : 0.f;   // (the same arithmetic as the merge of runs)
     }
   }
   asm volatile("bar.sync 1, 128;" ::: "memory");
@@ -348,6 +351,7 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
       const float4 x = *reinterpret_cast<const float4*>(s_o + (w * 16 + r) * DH + d);
       acc.x += e * x.x; acc.y += e * x.y; acc.z += e * x.z; acc.w += e * x.w;
     }
+    if (SP && whole) { const float inv = s_inv[rr]; acc.x *= inv; acc.y *= inv; acc.z *= inv; acc.w *= inv; }
     if (whole) store_out(rr, d, acc);
     else __stcg(reinterpret_cast<float4*>(my_part + rr * DH + d), acc);
   }
