@@ -20,11 +20,11 @@ constexpr int kAcceptThreads = kVerdictThreads;
 constexpr int kMaxAcceptSeqs = 1 << 16;  // counters live at the start of the scratch
 
 // Parts of a row: a CTA goes through its part in batches of 8192 values, a memory round trip each, so rows are cut into two or
-// four while all CTAs with work can be resident at once (four an SM).  How many rows are active is known on the device alone: the
+// four while about all CTAs with work can be resident at once (four an SM).  How many rows are active is known on the device alone: the
 // host launches up to twice the CTAs that fit, and the kernel takes so many parts that those with work do.  32000 logits, relaxed
 // rule, all rows active, in one / two / four / eight parts: 9 rows 9.8 / 8.0 / 7.3 / 8.4 us, 144 rows 12.7 / 11.0 / 10.3 / 16.6, 288
 // rows 15.3 / 12.5 / 15.8 / 26.7, 576 rows 18.2 / 20.4 / 26.1 / 45.4.
-constexpr int kFewCtas = 640;
+constexpr int kFewCtas = 800;   // (592 can be resident; a third more still ends sooner than whole rows)
 int parts_of(int64_t rows, int32_t V) {
   int parts = 4;
   while (parts > 1 && (rows * parts > 8 * 148 || V < 4096 * parts)) parts /= 2;
