@@ -7,8 +7,10 @@
 // 128 B instead of 16 KB + NT x 128 B.  The kernel is persistent: pair p walks the tiles p, p + P, .., and two
 // accumulators in tensor memory let the epilogue of one tile run under the main loop of the next.  The tiles left
 // over after the last full wave are cut along K over all pairs where that pays; the pairs that share a tile exchange
-// fp32 partial sums through a scratch in L2 and each finishes a slice of its token rows, in a fixed order of summation
-// (results are the same from run to run).
+// fp32 partial sums through a scratch in L2 and each finishes a slice of its token rows, in a fixed order of summation.
+// How a tile is cut follows from its weight tile alone: all token tiles of a weight tile are whole, or all are cut at the
+// same K blocks.  A row's result then does not depend on its place in the step, so that a token among drafts gets the
+// logits that it gets alone (and results are the same from run to run).
 //   warps 0, 10  TMA producers of the CTA's own halves (weights, activations); completion bytes count on the pair's
 //              first CTA
 //   warp 1     MMA issuer (first CTA only); commits free the stages of both CTAs
@@ -46,31 +48,26 @@ constexpr int kPairSmem = 220 * 1024;   // + up to 6.2 KB of static shared memor
 struct PairPlan {
   int N, NT, n_tt, KB, stages;
   int P;                        // pairs in the grid
-  int full_tiles, rem_tiles;    // whole tiles; tiles cut along K
-  int KBp, u;                   // cut tiles: units per tile (>= KB), units per pair
-  float* scratch;               // [pair][segment][rank][NT][128 features]
+  int full_tiles, rem_tiles;    // whole tiles; tiles cut along K: every token tile of the last weight tiles
+  int S, k;                     // cut tiles: K ranges of a tile, K blocks of a range
+  float* scratch;               // [pair][rank][NT][128 features]
   int32_t* state;               // [cut tile][rank][kPairState]
 };
 
-struct Item { int tile, kb0, kb1, C, c, seg; };   // C contributors, this pair is number c, its segment seg
+struct Item { int tile, kb0, kb1, C, c; };   // C contributors, this pair is number c
 
+// A pair's whole tiles, then at most one range of a cut tile.
 __device__ __forceinline__ bool get_item(const PairPlan& pl, int p, int idx, Item& it) {
   const int n_whole = pl.full_tiles > p ? (pl.full_tiles - 1 - p) / pl.P + 1 : 0;
   if (idx < n_whole) {
-    it.tile = p + idx * pl.P; it.kb0 = 0; it.kb1 = pl.KB; it.C = 1; it.c = 0; it.seg = 0;
+    it.tile = p + idx * pl.P; it.kb0 = 0; it.kb1 = pl.KB; it.C = 1; it.c = 0;
     return true;
   }
-  const int s = idx - n_whole;
-  if (s > 1 || pl.rem_tiles == 0) return false;
-  const int ua = p * pl.u, ub = min(ua + pl.u, pl.rem_tiles * pl.KBp);
-  if (ua >= ub) return false;
-  const int i0 = ua / pl.KBp, i = i0 + s;
-  if (i * pl.KBp >= ub) return false;
-  it.kb0 = s == 0 ? ua - i0 * pl.KBp : 0;
-  it.kb1 = min(pl.KB, ub - i * pl.KBp);
-  it.tile = pl.full_tiles + i;
-  const int first = i * pl.KBp / pl.u, last = (i * pl.KBp + pl.KB - 1) / pl.u;
-  it.C = last - first + 1; it.c = p - first; it.seg = s;
+  if (idx > n_whole || p >= pl.rem_tiles * pl.S) return false;
+  const int i = p / pl.S;
+  it.tile = pl.full_tiles + i; it.C = pl.S; it.c = p - i * pl.S;
+  it.kb0 = it.c * pl.k;
+  it.kb1 = min(pl.KB, it.kb0 + pl.k);
   return true;
 }
 
@@ -119,7 +116,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
   extern __shared__ uint8_t smem_raw[];
   __shared__ uint64_t full_bar[kMaxStages], empty_bar[kMaxStages], acc_full[2], acc_empty[2];
   __shared__ uint32_t tmem_slot;
-  __shared__ int abort_flag, s_last[2], s_go;
+  __shared__ int abort_flag, s_last, s_go;
   __shared__ float s_rstd[256];
   __shared__ int s_pos[256], s_page[256];
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
@@ -316,7 +313,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
       // tensor memory -> staging buffer -> rows: finished, or (cut tile) published as partial sums
       if (finish || publish) {
         const uint32_t src = tmem + uint32_t(buf) * 256 + lanes;
-        float* part = pl.scratch + (size_t(p * 2 + it.seg) * 2 + rank) * NT * kBM + 4 * lane;
+        float* part = pl.scratch + (size_t(p) * 2 + rank) * NT * kBM + 4 * lane;
         for (int ch = group; ch * kChunk < NT; ch += 2) {
           uint32_t v0[16], v1[16];
           tmem_ld16(src + uint32_t(ch * kChunk), v0);
@@ -352,20 +349,18 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         epi_barrier();
         if (et == 0) {
           __threadfence();
-          s_last[it.seg] = atomicAdd(tile_state(it), 1) == it.C - 1;
+          s_last = atomicAdd(tile_state(it), 1) == it.C - 1;
         }
       }
     }
-    // Cut tiles: each contributor sums and finishes a slice of the token rows, after all its partial sums are published
-    // (no chain of waits).  It waits for its peers only so long: they may not be running, if other kernels hold their SMs.
+    // A cut tile (a pair's last item): each contributor sums and finishes a slice of the token rows, after its partial sums
+    // are published.  It waits for its peers only so long: they may not be running, if other kernels hold their SMs.
     // A slice given up is marked, and the contributor that arrives last takes it over; between the mark and the arrival
     // count each side writes its own before it reads the other's, and a compare-and-swap settles who goes on.
-    for (int at = max(0, idx - 2); at < idx; ++at) {
-      get_item(pl, p, at, it);
-      if (it.C == 1) continue;
+    if (idx > 0 && get_item(pl, p, idx - 1, it) && it.C > 1) {
       const int wt = (it.tile / pl.n_tt) * 2 + rank, r0 = (it.tile % pl.n_tt) * NT;
       row_context(r0);
-      const int rel = it.tile - pl.full_tiles, first = p - it.c;
+      const int first = p - it.c;
       int32_t* state = tile_state(it);             // arrived, slices finished, one mark per slice
       const int sl = (NT / 4 + it.C - 1) / it.C;   // rows of a slice, in units of four
       // RB rows x all contributors' partial sums of a warp are requested together: one L2 round trip per batch
@@ -381,8 +376,8 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
             float4 v[CB][RB];
 #pragma unroll
             for (int c = 0; c < CB; ++c) {
-              const int pair = first + min(cb + c, it.C - 1), seg = rel - pair * pl.u / pl.KBp;
-              const float* b = pl.scratch + ((size_t(pair * 2 + seg) * 2 + rank) * NT + q) * kBM + 4 * lane;
+              const int pair = first + min(cb + c, it.C - 1);
+              const float* b = pl.scratch + ((size_t(pair) * 2 + rank) * NT + q) * kBM + 4 * lane;
 #pragma unroll
               for (int x = 0; x < RB; ++x)
                 v[c][x] = cb + c < it.C ? __ldcg(reinterpret_cast<const float4*>(b + size_t(x) * kBM)) : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -418,7 +413,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         s_go = mine;
       }
       epi_barrier();
-      const bool last = s_last[it.seg], mine = s_go;
+      const bool last = s_last, mine = s_go;
       if (mine) finish_slice(it.c);
       if (last) {
         for (int j = 0; j < it.C; ++j) {
@@ -433,7 +428,6 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
           if (s_go) finish_slice(j);
         }
       }
-      epi_barrier();   // (s_go is free again)
     }
   }
   asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
@@ -483,9 +477,22 @@ int stage_count(int NT, int parts) {
   return std::min(kMaxStages, (kPairSmem - 1024 - 2 * kStgBytes) / (kBM * 128 + parts * (NT / 2) * 128));
 }
 
+// The tiles of a launch: whole ones in full waves, and the rest cut, from a weight tile's first token tile on.  Every cut
+// tile has at least two pairs, which take one range each (no cut where the rest fills more than half of the pairs).
+struct Cut { int full_tiles, rem_tiles, S, k; };
+Cut cut_of(int tiles, int n_tt, int KB, bool split) {
+  Cut c{tiles, 0, 1, KB};
+  const int full = tiles / kPairCount * kPairCount / n_tt * n_tt, rem = tiles - full;
+  if (!split || rem == 0 || 2 * rem > kPairCount) return c;
+  c.full_tiles = full; c.rem_tiles = rem;
+  c.k = ceil_div(KB, kPairCount / rem);
+  c.S = ceil_div(KB, c.k);
+  return c;
+}
+
 }  // namespace
 
-size_t gemm_pair_scratch_floats(int R_pad) { return size_t(kPairCount) * 4 * std::min(R_pad, 256) * kBM; }
+size_t gemm_pair_scratch_floats(int R_pad) { return size_t(kPairCount) * 2 * std::min(R_pad, 256) * kBM; }
 
 GemmPairShape gemm_pair_shape(int R_pad, int N, int K, int epi, bool pairs) {
   const int parts = pairs ? 2 : 1, KB = ceil_div(K, kBK);
@@ -499,23 +506,19 @@ GemmPairShape gemm_pair_shape(int R_pad, int N, int K, int epi, bool pairs) {
     const int tiles = w256 * n_tt;
     // Constants fitted on the 7B and 13B layer shapes at 16 .. 2048 rows, each launch varied alone inside the step.  A K
     // block's MMAs take 1.2 ns per token row (1.75 PFLOP/s while the clock holds); below about 100 rows its 16 KB of
-    // weights per SM take 0.16 us.  A tile cut into whole splits costs 7 us of exchange, a run that leaves a pair with two
-    // ends 16 us; a launch ends with the last tile's epilogue, NT / 40 us.
+    // weights per SM take 0.16 us.  A cut tile costs 7 us of exchange; a launch ends with the last tile's epilogue, NT / 40 us.
     const double kb_us = std::max(0.16, 0.035 + 0.0012 * NT * parts);
     auto wave_us = [&](int wave_tiles, int kbs) {   // its distinct weight tiles come from HBM
       const double fresh = std::min(double(w256), double(wave_tiles) / n_tt);
       return std::max(kbs * kb_us, fresh * KB * (256 * kBK * 2) / 6.1e6);
     };
     for (int split = 0; split < 2; ++split) {
-      const int rem = tiles % kPairCount;
-      if (split && rem == 0) continue;
-      double us = NT / 40.0 + tiles / kPairCount * wave_us(kPairCount, KB);
-      if (rem) {
-        const int S = split ? kPairCount / rem : 1;
-        if (!split) us += wave_us(rem, KB);
-        else if (S >= 2) us += wave_us(rem, ceil_div(KB, S)) + 7.0;
-        else us += wave_us(rem, ceil_div(rem * KB, kPairCount)) + 16.0;
-      }
+      const Cut cut = cut_of(tiles, n_tt, KB, split != 0);
+      if (split && cut.rem_tiles == 0) continue;
+      const int waves = split ? ceil_div(cut.full_tiles, kPairCount) : tiles / kPairCount;
+      double us = NT / 40.0 + waves * wave_us(kPairCount, KB);
+      if (split) us += wave_us(cut.rem_tiles, cut.k) + 7.0;
+      else if (tiles % kPairCount) us += wave_us(tiles % kPairCount, KB);
       if (us < best.us) best = GemmPairShape{NT, n_tt, split, us};
     }
   }
@@ -546,21 +549,9 @@ laser_status gemm_pair_launch(laser_model* m, const GemmPairShape& sh, const CUt
   pl.P = kPairCount;
   const int w256 = ceil_div(epi == EPI_SWIGLU ? ceil_div(N / 2, 64) : ceil_div(N, kBM), 2);
   const int tiles = w256 * pl.n_tt;
-  pl.full_tiles = sh.split ? tiles / pl.P * pl.P : tiles;
-  pl.rem_tiles = tiles - pl.full_tiles;
-  pl.KBp = pl.u = 1;
-  if (pl.rem_tiles) {
-    // the left-over tiles along K: whole splits of one tile where at least two pairs serve each, else one run of
-    // units over all pairs (a pair then holds the end of one tile and the start of the next)
-    int S = pl.P / pl.rem_tiles;
-    if (S >= 2) {
-      const int k = ceil_div(pl.KB, S);
-      S = ceil_div(pl.KB, k);
-      pl.KBp = S * k; pl.u = k;
-    } else {
-      pl.KBp = pl.KB; pl.u = ceil_div(pl.rem_tiles * pl.KB, pl.P);
-    }
-  }
+  const Cut cut = cut_of(tiles, pl.n_tt, pl.KB, sh.split != 0);
+  pl.full_tiles = cut.full_tiles; pl.rem_tiles = cut.rem_tiles;
+  pl.S = cut.S; pl.k = cut.k;
   pl.scratch = m->pair_scratch;
   pl.state = m->pair_state;
   switch (epi) {

@@ -20,10 +20,11 @@ constexpr int gemm_pair_rows(bool pairs) { return pairs ? 64 : 160; }
 struct GemmPairShape { int NT, n_tt, split; double us; };
 GemmPairShape gemm_pair_shape(int R_pad, int N, int K, int epi, bool pairs);
 // The scratch for partial sums (fp32 values), and per cut tile and half of it: contributors arrived, slices finished, a
-// mark per slice (a tile has at most kPairCount contributors).  The state is zero between launches.
+// mark per slice (a tile has at most kPairCount contributors, and at most kPairCount / 2 tiles are cut).  The state is zero
+// between launches.
 size_t gemm_pair_scratch_floats(int R_pad);
 constexpr int kPairState = kPairCount + 2;
-constexpr int kPairStateInts = 2 * kPairCount * kPairState;
+constexpr int kPairStateInts = kPairCount * kPairState;
 
 laser_status gemm_pair_launch(laser_model* m, const GemmPairShape& sh, const CUtensorMap& tw, const CUtensorMap& ta, int N, int K, int epi,
                               const GemmEpilogue& e, cudaStream_t stream);

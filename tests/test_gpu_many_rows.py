@@ -36,7 +36,7 @@ def test_layers_at_the_tile_edges(L, B, K, precise):
 
 
 # No layers: the LM head alone, whose [vocab, d_model] shape sets how its 256-row tiles fall on the 74 SM pairs.
-# Left-over tiles: 2 of 74 (many contributors each), 20 (three), 30 (two), 60 (two pairs' ends meet), 125 - 74 = 51, none.
+# Left-over tiles: 2 of 74 (many contributors each), 20 (three), 30 (two), 60 (more than half of the pairs: whole), 125 - 74 = 51 (whole), none.
 @pytest.mark.parametrize("tiles,d,precise", [(2, 8192, 0), (20, 8192, 0), (30, 8192, 0), (60, 8192, 1), (125, 2048, 1), (74, 512, 0)])
 def test_left_over_tiles_cut_along_k(L, tiles, d, precise):
     B, K = 20, 8                                     # 180 rows
