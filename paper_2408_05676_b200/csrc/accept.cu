@@ -24,16 +24,23 @@ constexpr int kMaxAcceptSeqs = 1 << 16;  // counters live at the start of the sc
 // host launches up to twice the CTAs that fit, and the kernel takes so many parts that those with work do.  32000 logits, relaxed
 // rule, all rows active, in one / two / four / eight parts: 9 rows 9.8 / 8.0 / 7.3 / 8.4 us, 144 rows 12.7 / 11.0 / 10.3 / 16.6, 288
 // rows 15.3 / 12.5 / 15.8 / 26.7, 576 rows 18.2 / 20.4 / 26.1 / 45.4.
+constexpr int kLaunchedCtas = 8 * 148;
 constexpr int kFewCtas = 800;   // (592 can be resident; a third more still ends sooner than whole rows)
 int parts_of(int64_t rows, int32_t V) {
   int parts = 4;
-  while (parts > 1 && (rows * parts > 8 * 148 || V < 4096 * parts)) parts /= 2;
+  while (parts > 1 && (rows * parts > kLaunchedCtas || V < 4096 * parts)) parts /= 2;
   return parts;
+}
+
+// What the CTAs leave in the scratch: the verdict of a row read whole, or the RowResult of each part.
+struct WholeRow { int arg, pass; };
+size_t results_bytes(int64_t rows, int parts) {
+  return size_t(rows) * std::max(sizeof(WholeRow), parts > 1 ? sizeof(RowResult) * parts : size_t(0));
 }
 
 __global__ void __launch_bounds__(kAcceptThreads)
 accept_rows_kernel(const float* logits, const int32_t* tokens, const int32_t* n_rows, const int32_t* seq_ids,
-                   int32_t R, int32_t V, const Rule rule, int32_t* __restrict__ counters, RowResult* results,
+                   int32_t R, int32_t V, const Rule rule, int32_t* __restrict__ counters, void* results,
                    int32_t* __restrict__ n_accept, int32_t* __restrict__ out_tokens,
                    int32_t* __restrict__ n_out, int32_t* __restrict__ kv_len, unsigned long long* stamp) {
   const int b = blockIdx.x / R, i = blockIdx.x % R, part = blockIdx.y;
@@ -72,8 +79,12 @@ accept_rows_kernel(const float* logits, const int32_t* tokens, const int32_t* n_
   // publish, then let the last CTA of this sequence go through the rows in order
   __shared__ int s_last;
   if (tid == 0) {
-    if (parts == 1) mine.ahead = judge(row_of(i), V, token_of(i), rule, mine);   // (its verdict: 0, 1 or 2)
-    results[(size_t(b) * R + i) * parts + part] = mine;
+    if (parts == 1) {
+      const int pass = judge(row_of(i), V, token_of(i), rule, mine);
+      static_cast<WholeRow*>(results)[size_t(b) * R + i] = WholeRow{mine.arg, pass};
+    } else {
+      static_cast<RowResult*>(results)[(size_t(b) * R + i) * parts + part] = mine;
+    }
     __threadfence();
     s_last = atomicAdd(&counters[b], 1) == nr * parts - 1;
   }
@@ -81,22 +92,24 @@ accept_rows_kernel(const float* logits, const int32_t* tokens, const int32_t* n_
   if (!s_last) return;
   __threadfence();
   __shared__ int s_arg[kAcceptThreads], s_pass[kAcceptThreads];
-  __shared__ float s_max[kAcceptThreads];
   int a = 0, base = 0;           // (the same in every thread)
   for (bool go = true;; base += kAcceptThreads) {   // a row a thread: rows base .. base + kAcceptThreads - 1
     const int x = base + tid;
-    if (x < nr) {
-      const volatile RowResult* v = results + (size_t(b) * R + x) * parts;
+    if (x < nr && parts == 1) {
+      const volatile WholeRow* v = static_cast<const WholeRow*>(results) + size_t(b) * R + x;
+      s_pass[tid] = v->pass;
+      s_arg[tid] = v->arg;
+    } else if (x < nr) {
+      const volatile RowResult* v = static_cast<const RowResult*>(results) + (size_t(b) * R + x) * parts;
       RowResult r{v->mx, v->arg, v->ahead, v->m, v->s, v->lt};
       for (int q = 1; q < parts; ++q) merge_rows(r, RowResult{v[q].mx, v[q].arg, v[q].ahead, v[q].m, v[q].s, 0.f});
-      s_pass[tid] = parts == 1 ? r.ahead : judge(row_of(x), V, token_of(x), rule, r);
+      s_pass[tid] = judge(row_of(x), V, token_of(x), rule, r);
       s_arg[tid] = r.arg;
-      s_max[tid] = r.mx;
     }
     __syncthreads();
     for (const int end = min(nr - 1, base + kAcceptThreads); go && a < end; a += go) {
       const int pass = s_pass[a - base];
-      go = (pass == 2 ? exact_pass(row_of(a), V, token_of(a), s_max[a - base], rule.p) : pass) != 0;
+      go = (pass == 2 ? exact_pass(row_of(a), V, token_of(a), s_arg[a - base], rule.p) : pass) != 0;
     }
     if (!go || a < base + kAcceptThreads) break;
     __syncthreads();
@@ -111,12 +124,13 @@ accept_rows_kernel(const float* logits, const int32_t* tokens, const int32_t* n_
     out_tokens[b * R + j] = j < a ? tokens[b * R + j + 1] : (j == a ? s_arg[a - base] : -1);
 }
 
-// Fixed scratch of the allocation-free entry point: per-sequence counters, then the rows' results (rows in parts are few).
+// Fixed scratch of the allocation-free entry point: per-sequence counters, then the rows' results (rows in parts are few).  Its
+// size is part of that entry point's contract (laser.h).
 constexpr int kNoAllocMaxSeqs = 1024;
 constexpr int kNoAllocMaxRows = 16384;
 constexpr size_t kNoAllocCounterBytes = sizeof(int32_t) * kNoAllocMaxSeqs;
-constexpr size_t kNoAllocBytes = kNoAllocCounterBytes + sizeof(RowResult) * kNoAllocMaxRows;
-static_assert(8 * 148 <= kNoAllocMaxRows, "");   // (rows in parts)
+constexpr size_t kNoAllocBytes = kNoAllocCounterBytes + sizeof(WholeRow) * kNoAllocMaxRows;
+static_assert(kNoAllocBytes == 132 * 1024 && kLaunchedCtas * sizeof(RowResult) <= sizeof(WholeRow) * kNoAllocMaxRows, "");
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoAllocBytes];
 
 // Device address of g_noalloc_scratch on the current device, resolved once per device.  Host threads
@@ -162,7 +176,7 @@ LASER_API laser_status laser_accept_commit_noalloc(laser_kv* kv, const int32_t* 
   void* scratch = nullptr;
   LASER_TRY(noalloc_scratch(&scratch));
   int32_t* counters = static_cast<int32_t*>(scratch);
-  RowResult* results = reinterpret_cast<RowResult*>(static_cast<char*>(scratch) + kNoAllocCounterBytes);
+  void* results = static_cast<char*>(scratch) + kNoAllocCounterBytes;
   // the array keeps whatever the previous call left: the arrival counters must start at zero
   LASER_CUDA(cudaMemsetAsync(counters, 0, sizeof(int32_t) * size_t(B), as_stream(stream)));
   const int R = p->K + 1, parts = parts_of(rows, V);
@@ -190,9 +204,9 @@ laser_status accept_commit(laser_kv* kv, const int32_t* seq_ids, const float* lo
   const int R = p->K + 1, parts = parts_of(int64_t(B) * R, V);
   void* scratch = nullptr;
   const size_t counters_bytes = sizeof(int32_t) * kMaxAcceptSeqs;
-  LASER_TRY(scratch_get(SCRATCH_ACCEPT, counters_bytes + sizeof(RowResult) * size_t(B) * R * parts, &scratch));
+  LASER_TRY(scratch_get(SCRATCH_ACCEPT, counters_bytes + results_bytes(int64_t(B) * R, parts), &scratch));
   int32_t* counters = static_cast<int32_t*>(scratch);
-  RowResult* results = reinterpret_cast<RowResult*>(static_cast<char*>(scratch) + counters_bytes);
+  void* results = static_cast<char*>(scratch) + counters_bytes;
   LASER_CUDA(launch_overlapped(accept_rows_kernel, dim3(unsigned(B * R), unsigned(parts)), kAcceptThreads, 0, stream,
       logits, tokens, n_rows, seq_ids, R, V, Rule{p->mode, p->topk, double(p->p)}, counters, results,
       n_accept, out_tokens, n_out, kv ? kv->seq_len : nullptr, stamp));

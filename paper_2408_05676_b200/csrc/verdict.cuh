@@ -139,13 +139,14 @@ static __device__ int judge(const float* row, int V, int t, const Rule& rule, Ro
   return top || sure_above;
 }
 
-// The rule's own arithmetic, by the whole CTA: everything else about the row is settled, the probability decides.  Every thread
-// gets the answer.
-static __device__ int exact_pass(const float* row, int V, int t, float mx, double p) {
+// The rule's own arithmetic, by the whole CTA: everything else about the row (whose arg max is given) is settled, the
+// probability decides.  Every thread gets the answer.
+static __device__ int exact_pass(const float* row, int V, int t, int arg, double p) {
   constexpr int kWarps = kVerdictThreads / 32;
   __shared__ double s_sum[kWarps];
   __shared__ int s_pass;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const float mx = arg < V ? row[arg] : -INFINITY;   // (no arg max: nothing but NaN)
   double sum = 0.0;
   for (int j = tid; j < V; j += kVerdictThreads) sum += exp(double(row[j] - mx));
   for (int o = 16; o; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
@@ -162,17 +163,16 @@ static __device__ int exact_pass(const float* row, int V, int t, float mx, doubl
 
 // Max and arg max (smallest id on ties) of a row, and whether token t passes on it (t < 0: none), in every thread.
 static __device__ void cta_row(const float* row, int V, int t, const Rule& rule, int* arg_out, int* pass_out) {
-  __shared__ float s_max;
   __shared__ int s_arg, s_verdict;
   RowResult r = cta_scan(row, V, 0, 1, t, rule);
   if (threadIdx.x == 0) {
     s_verdict = judge(row, V, t, rule, r);
-    s_max = r.mx; s_arg = r.arg;
+    s_arg = r.arg;
   }
   __syncthreads();
   *arg_out = s_arg;
   const int verdict = s_verdict;
-  *pass_out = verdict == 2 ? exact_pass(row, V, t, s_max, rule.p) : verdict;
+  *pass_out = verdict == 2 ? exact_pass(row, V, t, s_arg, rule.p) : verdict;
 }
 
 }  // namespace laser

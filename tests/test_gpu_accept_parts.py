@@ -40,3 +40,19 @@ def test_parts_and_many_rows(L, B, R, V):
         want = A.accept_batch(logits, tokens, n_rows, mode, k, float(np.float32(p)))
         for g, w in zip(got, want):
             assert (g.cpu().numpy() == w).all(), (mode, k, p)
+
+
+# the allocation-free call keeps whole rows and parts in one array of fixed size: parts, then whole rows, then parts again
+def test_parts_in_the_fixed_array(L):
+    for B, R, V in [(2, 5, 32003), (66, 9, 8200), (130, 9, 8200), (1, 2, 16384)]:
+        rng = np.random.default_rng(B)
+        logits = torch.as_tensor((rng.standard_normal((B, R, V)) * 3).astype(np.float32), device="cuda")
+        tokens = torch.zeros(B, R, dtype=torch.int32, device="cuda")
+        tokens[:, 1:] = logits.topk(2, 2).indices[:, :-1, int(rng.integers(0, 2))]
+        n_rows = dev_i32(rng.integers(0, R + 1, B))
+        prm = L.make_params(K=R - 1, mode=L.MODE_RELAXED, topk=2, p=0.02)
+        want = L.accept_commit(None, None, logits, tokens, n_rows, prm)
+        for _ in range(2):
+            out = [torch.full(s, -7, dtype=torch.int32, device="cuda") for s in ((B,), (B, R), (B,))]
+            got = L.accept_commit_noalloc(None, None, logits, tokens, n_rows, prm, out)
+            assert all(torch.equal(g, w) for g, w in zip(got, want)), (B, R, V)
