@@ -20,6 +20,8 @@ __device__ __forceinline__ void better(float& v, int& i, float ov, int oi) {
   if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; }
 }
 
+constexpr int kNoId = 0x7fffffff;   // no arg max (a row of NaN alone); padding
+
 struct RowResult { float mx; int arg; int ahead; float m, s, lt; };   // s = sum of exp(x - m) over what was seen; lt = the token's
 
 // exp(d) for d <= 0.  ex2 is good to 2 units in the last place and the product's rounding shifts the exponent by |d| 2^-24:
@@ -28,9 +30,10 @@ __device__ __forceinline__ float exp_below(float d) { return exp2f(d * 1.4426950
 
 template <bool RANK, bool PROB>
 __device__ __forceinline__ RowResult scan_row(const float* __restrict__ row, int V, int part, int parts, int t, float lt, int tid) {
-  RowResult r{-INFINITY, 0x7fffffff, 0, -INFINITY, 0.f, lt};
+  RowResult r{-INFINITY, kNoId, 0, -INFINITY, 0.f, lt};
   const int lead = min(V, int((16 - (reinterpret_cast<uintptr_t>(row) & 15)) & 15) >> 2);   // values before the first 16-byte boundary
   const int n4 = (V - lead) >> 2;
+  // cnt values and their ids; a value with an id of kNoId is padding (-inf)
   auto batch = [&](const float* x, int cnt, auto index_of) {
     float bm = -INFINITY;
 #pragma unroll
@@ -67,7 +70,10 @@ __device__ __forceinline__ RowResult scan_row(const float* __restrict__ row, int
       const float4 v = i < end ? r4[i] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
       x[4 * u] = v.x; x[4 * u + 1] = v.y; x[4 * u + 2] = v.z; x[4 * u + 3] = v.w;
     }
-    batch(x, 4 * kRowLoads, [&](int i) { return lead + 4 * (base + (i >> 2) * kVerdictThreads + tid) + (i & 3); });
+    batch(x, 4 * kRowLoads, [&](int i) {
+      const int at = base + (i >> 2) * kVerdictThreads + tid;
+      return at < end ? lead + 4 * at + (i & 3) : kNoId;
+    });
   }
   const int tail = lead + 4 * n4 + tid;
   if (part == parts - 1 && tail < V) batch(row + tail, 1, [&](int) { return tail; });
@@ -120,7 +126,7 @@ static __device__ RowResult cta_scan(const float* row, int V, int part, int part
 // One thread, from a whole row's result: the arg max (smallest id on ties), and whether t passes: 0, 1, or 2 where only the rule's
 // own arithmetic (exact_pass) can tell.
 static __device__ int judge(const float* row, int V, int t, const Rule& rule, RowResult& r) {
-  if (r.arg == 0x7fffffff)   // nothing above -inf: the first -inf, as an ascending scan would find it
+  if (r.arg == kNoId)   // nothing above -inf: the first -inf, as an ascending scan would find it
     for (int j = V - 1; j >= 0; --j) if (row[j] == -INFINITY) r.arg = j;
   if (t < 0 || t >= V) return 0;
   const bool top = t == r.arg, in_topk = r.ahead < rule.topk;

@@ -65,3 +65,20 @@ def test_ends_of_the_range(L):
     out = L.accept_commit(None, None, torch.as_tensor(logits[2:], device="cuda"), dev_i32(tokens[2:]), dev_i32([1]),
                           L.make_params(K=1, mode=L.MODE_STRICT))
     assert out[1].cpu().tolist() == [[0, -1]]           # nothing above -inf: the smallest id
+
+
+# A masked draft token (-inf) ranks behind every finite logit and behind the masked tokens of smaller id, and nothing else: the
+# lanes' padding past a part's end must not count.  Whole rows and rows in parts, masks of all but one token and of every second.
+@pytest.mark.parametrize("V", [5, 6, 7, 1003, 8195, 16390, 32003])
+def test_rank_of_a_masked_token(L, V):
+    logits = np.full((2, 2, V), -np.inf, dtype=np.float32)
+    logits[0, 0, V // 2] = 1.0
+    logits[1, 0, ::2] = np.arange((V + 1) // 2, dtype=np.float32) * 1e-3
+    for t in sorted({0, 1, V // 3 | 1, V - 3, V - 2, V - 1}):
+        tokens = np.array([[0, t], [0, t]], dtype=np.int32)
+        for b in range(2):
+            row = logits[b, 0]
+            rank = int((row > row[t]).sum() + (row[:t] == row[t]).sum())
+            for k in (rank, rank + 1):
+                if k >= 1:
+                    _check(L, logits[b:b + 1], tokens[b:b + 1], np.array([2], dtype=np.int32), A.TOPK, k, 0.0)
