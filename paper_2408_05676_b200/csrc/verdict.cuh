@@ -52,11 +52,14 @@ __device__ __forceinline__ RowResult scan_row(const float* __restrict__ row, int
         for (int i = 0; i < cnt; ++i) r.ahead += x[i] == lt && index_of(i) < t;
     }
     if (PROB && bm > -INFINITY) {
-      if (bm > r.m) { r.s *= r.m > -INFINITY ? exp_below(r.m - bm) : 0.f; r.m = bm; }
+      if (bm > r.m) { r.s *= r.m > -INFINITY ? exp_below(r.m - bm) : 0.f; r.m = bm; }   // (a NaN stays)
       float add = 0.f;
 #pragma unroll
       for (int i = 0; i < cnt; ++i) add += exp_below(x[i] - r.m);
       r.s += add;
+    } else if (PROB) {              // -inf adds nothing, NaN makes the sum NaN
+#pragma unroll
+      for (int i = 0; i < cnt; ++i) if (x[i] != x[i]) r.s = x[i];
     }
   };
   const int per = (n4 + parts - 1) / parts, end = min(n4, (part + 1) * per);   // (float4s of this part: part * per .. end - 1)
@@ -84,8 +87,7 @@ __device__ __forceinline__ void merge_rows(RowResult& r, const RowResult& o) {
   better(r.mx, r.arg, o.mx, o.arg);
   r.ahead += o.ahead;
   const float m = fmaxf(r.m, o.m);
-  if (m > -INFINITY)
-    r.s = (r.m > -INFINITY ? r.s * exp_below(r.m - m) : 0.f) + (o.m > -INFINITY ? o.s * exp_below(o.m - m) : 0.f);
+  r.s = (r.m > -INFINITY ? r.s * exp_below(r.m - m) : r.s) + (o.m > -INFINITY ? o.s * exp_below(o.m - m) : o.s);   // (without a maximum: 0 or NaN)
   r.m = m;
 }
 

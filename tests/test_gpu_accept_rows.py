@@ -82,3 +82,23 @@ def test_rank_of_a_masked_token(L, V):
             for k in (rank, rank + 1):
                 if k >= 1:
                     _check(L, logits[b:b + 1], tokens[b:b + 1], np.array([2], dtype=np.int32), A.TOPK, k, 0.0)
+
+
+# One NaN anywhere in a row makes every probability on it NaN, which exceeds no p: at the ends that are read singly, in a batch
+# of its own among masked tokens, and in another part than the rest.
+@pytest.mark.parametrize("V", [7, 8195, 16390, 32003])
+def test_a_nan_leaves_no_probability(L, V):
+    rng = np.random.default_rng(V)
+    for masked in (False, True):
+        for at in sorted({0, 1, 2, 3, V // 2, V - 3, V - 2, V - 1}):
+            for shift in range(4):                       # the row's distance from a 16-byte boundary
+                row = np.full(V, -np.inf, dtype=np.float32) if masked else rng.standard_normal(V).astype(np.float32)
+                top = (at + V // 3 + 1) % V
+                row[top] = 20.0
+                row[at] = np.nan
+                logits = torch.zeros(shift + 2 * V, device="cuda")[shift:].view(1, 2, V)
+                logits[0, 0] = torch.as_tensor(row)
+                for mode in (L.MODE_RELAXED, L.MODE_TOPP):
+                    tokens = dev_i32([[0, top if mode == L.MODE_RELAXED else (top + 1) % V]])
+                    n = L.accept_commit(None, None, logits, tokens, dev_i32([2]), L.make_params(K=1, mode=mode, topk=2, p=1e-6))[0]
+                    assert int(n[0]) == 0, (masked, at, shift, mode)
