@@ -137,9 +137,10 @@ static __device__ int judge(const float* row, int V, int t, const Rule& rule, Ro
   // 1e-5.  Twice that.
   const double margin = 5.2e-4 + 2e-9 * V;
   const double q = double(exp_below(r.lt - r.mx)) / double(r.s);
+  const bool estimated = rule.p <= 0.0 || rule.p >= 1e-30;   // (a probability near a smaller p has lost digits in fp32)
   const bool matters = rule.needs_p() && (rule.mode == LASER_MODE_RELAXED ? in_topk : rule.mode == LASER_MODE_TOPP ? !top : !top && in_topk);
   const bool sure_above = q * (1.0 - margin) > rule.p, sure_below = q * (1.0 + margin) < rule.p;
-  if (matters && !sure_above && !sure_below) return 2;      // (a NaN is neither)
+  if (matters && !(estimated && (sure_above || sure_below))) return 2;      // (a NaN is neither)
   if (rule.mode == LASER_MODE_STRICT) return top;
   if (rule.mode == LASER_MODE_RELAXED) return in_topk && sure_above;
   if (rule.mode == LASER_MODE_TOPK) return in_topk;

@@ -102,3 +102,14 @@ def test_a_nan_leaves_no_probability(L, V):
                     tokens = dev_i32([[0, top if mode == L.MODE_RELAXED else (top + 1) % V]])
                     n = L.accept_commit(None, None, logits, tokens, dev_i32([2]), L.make_params(K=1, mode=mode, topk=2, p=1e-6))[0]
                     assert int(n[0]) == 0, (masked, at, shift, mode)
+
+
+def test_thresholds_below_the_normal_range(L):
+    """Probabilities of a few of the smallest fp32 steps (2^-149): exponentials in fp32 have lost their digits there."""
+    logits = np.zeros((600, 2, 3), dtype=np.float32)
+    logits[:, 0, 1] = -2.0
+    logits[:, 0, 2] = np.linspace(-104.0, -101.0, 600, dtype=np.float32)
+    tokens = np.tile(np.array([[0, 2]], dtype=np.int32), (600, 1))
+    for j in (1, 2, 3, 5, 7):
+        for mode in (A.TOPP, A.RELAXED):
+            _check(L, logits, tokens, np.full(600, 2, dtype=np.int32), mode, 3, j * 2.0 ** -149)
