@@ -20,7 +20,7 @@ __device__ __forceinline__ void better(float& v, int& i, float ov, int oi) {
   if (ov > v || (ov == v && oi < i)) { v = ov; i = oi; }
 }
 
-constexpr int kNoId = 0x7fffffff;   // no arg max (a row of NaN alone); padding
+constexpr int kNoId = 0x7fffffff;   // no arg max (a row of NaN alone)
 
 struct RowResult { float mx; int arg; int ahead; float m, s, lt; };   // s = sum of exp(x - m) over what was seen; lt = the token's
 
@@ -33,8 +33,8 @@ __device__ __forceinline__ RowResult scan_row(const float* __restrict__ row, int
   RowResult r{-INFINITY, kNoId, 0, -INFINITY, 0.f, lt};
   const int lead = min(V, int((16 - (reinterpret_cast<uintptr_t>(row) & 15)) & 15) >> 2);   // values before the first 16-byte boundary
   const int n4 = (V - lead) >> 2;
-  // cnt values and their ids; a value with an id of kNoId is padding (-inf)
-  auto batch = [&](const float* x, int cnt, auto index_of) {
+  // cnt values and their ids; equal logits rank ahead of the token where their id is below `before` (padding, -inf, must not be)
+  auto batch = [&](const float* x, int cnt, auto index_of, int before) {
     float bm = -INFINITY;
 #pragma unroll
     for (int i = 0; i < cnt; ++i) bm = fmaxf(bm, x[i]);
@@ -49,21 +49,19 @@ __device__ __forceinline__ RowResult scan_row(const float* __restrict__ row, int
       for (int i = 0; i < cnt; ++i) { r.ahead += x[i] > lt; eq |= x[i] == lt; }
       if (eq)
 #pragma unroll
-        for (int i = 0; i < cnt; ++i) r.ahead += x[i] == lt && index_of(i) < t;
+        for (int i = 0; i < cnt; ++i) r.ahead += x[i] == lt && index_of(i) < before;
     }
-    if (PROB && bm > -INFINITY) {
+    if (PROB) {
       if (bm > r.m) { r.s *= r.m > -INFINITY ? exp_below(r.m - bm) : 0.f; r.m = bm; }   // (a NaN stays)
+      const float ref = r.m > -INFINITY ? r.m : 0.f;   // (nothing above -inf so far: the terms are 0, or NaN)
       float add = 0.f;
 #pragma unroll
-      for (int i = 0; i < cnt; ++i) add += exp_below(x[i] - r.m);
+      for (int i = 0; i < cnt; ++i) add += exp_below(x[i] - ref);
       r.s += add;
-    } else if (PROB) {              // -inf adds nothing, NaN makes the sum NaN
-#pragma unroll
-      for (int i = 0; i < cnt; ++i) if (x[i] != x[i]) r.s = x[i];
     }
   };
   const int per = (n4 + parts - 1) / parts, end = min(n4, (part + 1) * per);   // (float4s of this part: part * per .. end - 1)
-  if (part == 0 && tid < lead) batch(row + tid, 1, [&](int) { return tid; });
+  if (part == 0 && tid < lead) batch(row + tid, 1, [&](int) { return tid; }, t);
   const float4* r4 = reinterpret_cast<const float4*>(row + lead);
   for (int base = part * per; base < end; base += kVerdictThreads * kRowLoads) {
     float x[4 * kRowLoads];
@@ -73,21 +71,18 @@ __device__ __forceinline__ RowResult scan_row(const float* __restrict__ row, int
       const float4 v = i < end ? r4[i] : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
       x[4 * u] = v.x; x[4 * u + 1] = v.y; x[4 * u + 2] = v.z; x[4 * u + 3] = v.w;
     }
-    batch(x, 4 * kRowLoads, [&](int i) {
-      const int at = base + (i >> 2) * kVerdictThreads + tid;
-      return at < end ? lead + 4 * at + (i & 3) : kNoId;
-    });
+    batch(x, 4 * kRowLoads, [&](int i) { return lead + 4 * (base + (i >> 2) * kVerdictThreads + tid) + (i & 3); }, min(t, lead + 4 * end));
   }
   const int tail = lead + 4 * n4 + tid;
-  if (part == parts - 1 && tail < V) batch(row + tail, 1, [&](int) { return tail; });
+  if (part == parts - 1 && tail < V) batch(row + tail, 1, [&](int) { return tail; }, t);
   return r;
 }
 
 __device__ __forceinline__ void merge_rows(RowResult& r, const RowResult& o) {
   better(r.mx, r.arg, o.mx, o.arg);
   r.ahead += o.ahead;
-  const float m = fmaxf(r.m, o.m);
-  r.s = (r.m > -INFINITY ? r.s * exp_below(r.m - m) : r.s) + (o.m > -INFINITY ? o.s * exp_below(o.m - m) : o.s);   // (without a maximum: 0 or NaN)
+  const float m = fmaxf(r.m, o.m), ref = m > -INFINITY ? m : 0.f;   // (a sum without a maximum is 0 or NaN)
+  r.s = r.s * exp_below(r.m - ref) + o.s * exp_below(o.m - ref);
   r.m = m;
 }
 
