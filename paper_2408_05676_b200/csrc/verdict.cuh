@@ -38,7 +38,7 @@ __device__ __forceinline__ RowResult scan_row(const float* __restrict__ row, int
     float bm = -INFINITY;
 #pragma unroll
     for (int i = 0; i < cnt; ++i) bm = fmaxf(bm, x[i]);
-    if (bm > r.mx) {               // ids ascend from batch to batch and inside one: the first of equals stays
+    if (bm > r.mx || r.arg == kNoId) {   // ids ascend from batch to batch and inside one: the first of equals stays
       r.mx = bm;
 #pragma unroll
       for (int i = cnt - 1; i >= 0; --i) if (x[i] == bm) r.arg = index_of(i);
@@ -73,6 +73,7 @@ __device__ __forceinline__ RowResult scan_row(const float* __restrict__ row, int
     }
     batch(x, 4 * kRowLoads, [&](int i) { return lead + 4 * (base + (i >> 2) * kVerdictThreads + tid) + (i & 3); }, min(t, lead + 4 * end));
   }
+  if (r.arg >= lead + 4 * end) r.arg = kNoId;   // (padding, where nothing was above -inf)
   const int tail = lead + 4 * n4 + tid;
   if (part == parts - 1 && tail < V) batch(row + tail, 1, [&](int) { return tail; }, t);
   return r;
@@ -122,9 +123,7 @@ static __device__ RowResult cta_scan(const float* row, int V, int part, int part
 
 // One thread, from a whole row's result: the arg max (smallest id on ties), and whether t passes: 0, 1, or 2 where only the rule's
 // own arithmetic (exact_pass) can tell.
-static __device__ int judge(const float* row, int V, int t, const Rule& rule, RowResult& r) {
-  if (r.arg == kNoId)   // nothing above -inf: the first -inf, as an ascending scan would find it
-    for (int j = V - 1; j >= 0; --j) if (row[j] == -INFINITY) r.arg = j;
+static __device__ int judge(const float* row, int V, int t, const Rule& rule, const RowResult& r) {
   if (t < 0 || t >= V) return 0;
   const bool top = t == r.arg, in_topk = r.ahead < rule.topk;
   // The estimate's relative error: each term 1e-5, a term's at most 6 rescalings per thread (V / 8192 batches; rows beyond

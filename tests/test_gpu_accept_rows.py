@@ -113,3 +113,14 @@ def test_thresholds_below_the_normal_range(L):
     for j in (1, 2, 3, 5, 7):
         for mode in (A.TOPP, A.RELAXED):
             _check(L, logits, tokens, np.full(600, 2, dtype=np.int32), mode, 3, j * 2.0 ** -149)
+
+
+# Rows with nothing above -inf: the smallest id that is -inf is the arg max, also behind NaN and in any part
+@pytest.mark.parametrize("V", [3, 9, 1003, 16390, 32003])
+def test_arg_max_of_masked_rows(L, V):
+    for first in sorted({0, 1, V // 2, V - 2, V - 1}):
+        row = np.full(V, -np.inf, dtype=np.float32)
+        row[:first] = np.nan
+        logits = torch.as_tensor(np.stack([row, row])[None], device="cuda")
+        out = L.accept_commit(None, None, logits, dev_i32([[0, first]]), dev_i32([2]), L.make_params(K=1, mode=L.MODE_STRICT))
+        assert out[1].cpu().tolist() == [[first, first]], first
