@@ -11,8 +11,8 @@
 // staged page, so a page is still read from HBM once per 32 rows.  Every mbarrier wait is bounded.
 //
 // With few (sequence, head) pairs the walk over one sequence's pages is a latency chain that leaves most SMs idle: up to eight
-// CTAs then take a run of the pages each, and the one that finishes last sums the partial results (through L2, in the order of
-// the runs).  A cluster and distributed shared memory would merge faster, but its CTAs must find their slots together, beside
+// CTAs then take runs of eight pages in turn, and the one that finishes last sums the partial results (through L2, in the order
+// of the CTAs).  A cluster and distributed shared memory would merge faster, but its CTAs must find their slots together, beside
 // those of the neighbouring kernels: a step of one short sequence lost 4 us a layer to that.
 #include <type_traits>
 
@@ -28,7 +28,7 @@ constexpr int kAttnThreads = (kConsumers + 1) * 32;
 constexpr int kStages = 4;   // a multiple of kConsumers: stage s always serves warp s % 4
 constexpr int kMaxPageSplits = 8;  // CTAs that share a sequence's pages
 constexpr int kSplitFrom = 16;      // pages from which a split pays for the merge (about 3 us, ten pages of one CTA's walk),
-constexpr int kSplitPages = 8;      // and pages a run has at least
+constexpr int kRunPages = 8;        // and pages of a run (a multiple of kStages: a warp's pages stay the same ones)
 constexpr int kCtasPerSm = 4;  // registers and shared memory are sized for four resident CTAs
 
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
@@ -107,11 +107,17 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
   bf16* q_ptr = reinterpret_cast<bf16*>(tiles_ptr + kStages * STAGE);
   const int n_keys = ctx + (row_mask ? nr : min(nr, cta_row0 + 16 * TPC));   // chain: no row here sees a later one
   const int all_pg = (n_keys + 15) >> 4;
-  // (the runs do not depend on how many rows the step has, so that a row's result is the same among drafts and alone)
-  const int per = SP ? max(kSplitPages, (pages_per_seq + splits - 1) / splits) : all_pg, parts = SP ? (all_pg + per - 1) / per : 1;
+  // SP: run j of the pages belongs to CTA j % splits.  Which pages a CTA sums follows from their numbers alone, neither from the
+  // step's rows (a row's result is the same among drafts and alone) nor from the cache's capacity.
+  const int parts = SP ? min(splits, (all_pg + kRunPages - 1) / kRunPages) : 1;
   if (SP && krank >= parts) return;
-  const int pg0 = krank * per;
-  const int n_pg = SP ? max(0, min(per, all_pg - pg0)) : all_pg;   // this CTA's pages are pg0 .. pg0 + n_pg - 1
+  auto page_of = [&](int p) { return SP ? ((p / kRunPages) * splits + krank) * kRunPages + p % kRunPages : p; };   // the CTA's p-th page
+  auto pages_below = [&](int x) {   // how many of its pages come before page x
+    if (!SP) return x;
+    const int runs = x / kRunPages;
+    return (runs - krank + splits - 1) / splits * kRunPages + (runs % splits == krank ? x % kRunPages : 0);
+  };
+  const int n_pg = pages_below(all_pg);
   const bool whole = !SP || parts == 1;
   const int unit = (b * H + h) * gridDim.z + mt;
   float* const my_part = SP ? part + size_t(unit * splits + krank) * kPartFloats : nullptr;
@@ -128,7 +134,7 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
     if (lane == 0) {
       const int32_t* pt = page_table + size_t(seq_ids[b]) * pages_per_seq;
       // whole pages of older tokens that fit the ring (none where the kernel before may have written them)
-      const int n_early = fresh ? 0 : min(min(max(0, (ctx >> 4) - pg0), n_pg), kStages);
+      const int n_early = fresh ? 0 : min(pages_below(min(ctx >> 4, all_pg)), kStages);
       bool ok = true;
       int issued = 0;
       const uint64_t kv_policy = make_policy_evict_first();   // a page is read once per step
@@ -140,7 +146,7 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
         const uint32_t bar = smem_u32(&full_bar[s]);
         const uint32_t dst = tiles + uint32_t(s) * STAGE;
         mbar_expect_tx(bar, STAGE);
-        const int phys = pt[pg0 + p];
+        const int phys = pt[page_of(p)];
         const int rowk = layer_row0 + ((phys * 2) * Hkv + hk) * 16;
         const int rowv = layer_row0 + ((phys * 2 + 1) * Hkv + hk) * 16;
 #pragma unroll
@@ -225,7 +231,7 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
       }
     }
     // causal mask, online softmax (rows g and g+8 of the tile)
-    const int key0 = (pg0 + p) * 16 + 2 * qd;
+    const int key0 = page_of(p) * 16 + 2 * qd;
     float mx0 = -INFINITY, mx1 = -INFINITY;
 #pragma unroll
     for (int t = 0; t < 2; ++t)
@@ -408,10 +414,12 @@ laser_status attention_tma_launch(laser_model* m, laser_kv* kv, int layer, const
   const int layer_row0 = int(rows_per_layer * layer);
   const int tiles = ceil_div(Rs, 16), tpc = tiles > 1 ? 2 : 1;   // row tiles of a sequence; tiles per CTA
   // Page splits while the grid stays at what the SMs hold at once, where the cache can hold pages enough; what a sequence has
-  // is known on the device alone, and CTAs that find no run to take leave.  7B, 6 layers, 32 / 512 / 1000 cached tokens, one
-  // sequence of 9 rows: 561 / 636 / 707 us unsplit, 560 / 609 / 626 in four, 561 / 605 / 615 in eight; 2 sequences 572 / 650 / 724,
-  // in eight 571 / 622 / 639; 4 sequences 628 / 709 / 779, in four 637 / 701 / 728; 8 sequences 646 / 736 / 822, in two 646 / 726 /
-  // 781.  (A prefill's chunks are many.)
+  // is known on the device alone, and CTAs that find no run to take leave.  7B, 6 layers, steps of 9 rows, 128 / 256 / 512 / 1000
+  // cached tokens in a cache of 256 pages a sequence: one sequence 526 / 544 / 580 / 649 us unsplit, 543 / 546 / 552 / 563 in
+  // eight; two 551 / 569 / 606 / 679, in eight 569 / 577 / 583 / 593; four 612 / 630 / 665 / 734, in four 636 / 643 / 660 / 686; eight
+  // 650 / 670 / 705 / 787, in two 660 / 672 / 700 / 755.  The merge costs 3 us a layer, which texts of 9 to 16 pages do not win
+  // back; a cache that holds no more is not split.  Runs of 12 or 16 pages: one sequence of 512 / 1000 tokens 560 / 567, 567 / 573.
+  // (A prefill's chunks are many.)
   const int units = B * H * ceil_div(tiles, tpc), most = kv->pages_per_seq;
   const int splits = fresh || most < kSplitFrom ? 1 : units * 8 <= kAttnSplitCtas ? 8 : most < 2 * kSplitFrom ? 1 :
                      units * 4 <= kAttnSplitCtas ? 4 : units * 2 <= kAttnSplitCtas ? 2 : 1;

@@ -1,7 +1,8 @@
-"""Attention with a sequence's pages split over a cluster (csrc/attn.cu): page counts on both sides of every split, uneven
+"""Attention with a sequence's pages split over several CTAs (csrc/attn.cu): page counts on both sides of every split, uneven
 runs, one and several row tiles, chain and tree masks, grouped heads, against the fp64 oracle."""
 import numpy as np
 import pytest
+import torch
 
 from helpers import dev_i32, ensure_built, weights_to
 from oracle import forward as O
@@ -18,7 +19,7 @@ def L():
     return binding
 
 
-# pages are split from 16 on (256 tokens, the cache holding as many), in up to eight runs of four or more
+# caches of 16 pages or more are split: runs of eight pages (128 tokens), dealt to up to eight CTAs in turn
 @pytest.mark.parametrize("over,ctx,precise", [
     (dict(), [230], 0), (dict(), [231], 1), (dict(), [247], 1), (dict(), [248, 3], 1), (dict(), [300], 0), (dict(), [640, 77], 1), (dict(), [1000], 0),
     (dict(max_draft=16), [700], 1), (dict(max_draft=40), [300, 9, 500], 1), (dict(n_kv_heads=2, max_draft=3), [410, 0, 170], 1),
@@ -48,3 +49,48 @@ def test_split_pages_match_the_oracle(L, over, ctx, precise):
     L.check(m)
     for b in range(B):
         assert (tree[b, :n_rows[b]] - logits[b, :n_rows[b]]).abs().max().item() <= (TOL / 100 if precise else TOL / 2)
+
+
+# Four-way (96 pairs of sequence and head) and two-way splits (192), one run against two (128 and 129 keys) and uneven deals of
+# runs to CTAs, in a cache that is larger than the texts
+@pytest.mark.parametrize("B,K,precise", [(24, 8, 0), (24, 8, 1), (48, 2, 1)])
+def test_four_and_two_way_splits(L, B, K, precise):
+    cfg = synth.model_cfg("tiny", max_draft=K, precise=precise)
+    Wc = synth.make_weights(cfg, seed=0, gain_jitter=0.1)
+    pages = 64
+    m = L.model_create(cfg, weights_to(Wc, "cuda"), max_batch=B)
+    kv = L.kv_create(m, B, B * pages)
+    okv = O.KVCache(cfg, B, pages * 16)
+    ctx = ([128 - K - 1, 128 - K, 127, 128, 255 - K, 256 - K, 500, 640, 650, 0, 1000] * 5)[:B]
+    _fill_both(L, cfg, kv, okv, range(B), ctx, seed=7)
+    rows = [synth.make_prompt(K + 1, cfg["vocab"], 30 + b) for b in range(B)]
+    err, _ = _step(L, m, kv, cfg, Wc, okv, list(range(B)), rows)
+    print("max-abs logit error %.2e" % err)
+    assert err <= (TOL / 10 if precise else TOL)
+
+
+# What is summed in which order follows from the page numbers alone: the same bits in a cache of any capacity, and for a row
+# among drafts and alone, also where the drafts reach into another page or run
+@pytest.mark.parametrize("B,K,ctx", [(1, 8, 125), (2, 8, 505), (1, 20, 250), (24, 8, 380), (48, 4, 254)])
+def test_same_bits_in_any_capacity_and_alone(L, B, K, ctx):
+    cfg = synth.model_cfg("tiny", max_draft=K)
+    m = L.model_create(cfg, weights_to(synth.make_weights(cfg, seed=0, gain_jitter=0.1), "cuda"), max_batch=B)
+    text, ids = synth.make_prompt(K + 1, cfg["vocab"], 30), dev_i32(range(B))
+    first = None
+    for pages in (34, 100, 256):
+        kv = L.kv_create(m, B, B * pages)
+        for l in range(cfg["n_layers"]):
+            k, v = synth.make_kv_layer(ctx, cfg["n_kv_heads"] * cfg["head_dim"], 7, l, device="cuda")
+            for b in range(B):
+                L.kv_import(kv, b, l, 0, k, v)
+        L.kv_set_len(kv, list(range(B)), [ctx] * B)
+        full = L.verify_step(m, kv, ids, dev_i32(np.tile(text, (B, 1))), dev_i32([K + 1] * B))
+        first = full if first is None else first
+        assert torch.equal(first, full), "%d pages" % pages
+        rows = np.full((B, K + 1), -1, np.int32)
+        for i in range(K + 1):
+            rows[:, 0] = text[i]
+            L.kv_set_len(kv, list(range(B)), [ctx + i] * B)
+            alone = L.verify_step(m, kv, ids, dev_i32(rows), dev_i32([1] * B))
+            assert torch.equal(alone[:, 0], full[:, i]), "row %d, %d pages" % (i, pages)
+    L.check(m)
