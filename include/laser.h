@@ -140,6 +140,12 @@ laser_status laser_pool_build(const int32_t* tokens, int64_t n_tokens,
                               const int64_t* group_offsets, int32_t n_groups,
                               int32_t n_min, int32_t n_max, void* stream, laser_pool** out);
 laser_status laser_pool_free(laser_pool* pool);
+/* Pools come from a reserve of the library's own.  Of the memory that laser_pool_free and the
+ * build's work buffers return, up to 2 GB per device stay there for the next build; what is above
+ * goes back to the device at the next synchronisation, and all of it when one of the library's own
+ * allocations finds no memory.  A process whose other allocators need the rest calls laser_trim:
+ * it synchronises the current device and gives back whatever no pool holds.  Errors: CUDA. */
+laser_status laser_trim(void);
 /* Host-side facts: tokens, distinct (group, n-gram) keys over all n, device bytes held. */
 laser_status laser_pool_info(const laser_pool* pool, int64_t* n_tokens, int64_t* n_keys,
                              int64_t* device_bytes);

@@ -58,7 +58,7 @@ class Stats(C.Structure):
 
 
 EXPORTS = ["laser_version", "laser_last_error", "laser_launch_count", "laser_pool_build", "laser_pool_free",
-           "laser_pool_info", "laser_draft", "laser_draft_temp", "laser_draft_tree", "laser_make_rows", "laser_make_rows_tree", "laser_model_create", "laser_model_free",
+           "laser_pool_info", "laser_trim", "laser_draft", "laser_draft_temp", "laser_draft_tree", "laser_make_rows", "laser_make_rows_tree", "laser_model_create", "laser_model_free",
            "laser_kv_create", "laser_kv_free", "laser_kv_set_page_table", "laser_kv_set_len",
            "laser_kv_get_len", "laser_kv_reset", "laser_kv_set_len_dev", "laser_kv_import", "laser_kv_export",
            "laser_verify_step", "laser_verify_step_tree", "laser_check", "laser_profile_enable", "laser_profile_read", "laser_accept_commit", "laser_accept_commit_noalloc", "laser_accept_tree", "laser_kv_compact_path",
@@ -143,6 +143,11 @@ def pool_build(tokens, group_offsets: np.ndarray, n_min: int, n_max: int, stream
     _chk(lib.laser_pool_build(_ptr(tokens), C.c_int64(len(tokens)), _ptr(offs), C.c_int32(len(offs) - 1),
                               C.c_int32(n_min), C.c_int32(n_max), _stream(stream), C.byref(h)))
     return Pool(h)
+
+
+def trim() -> None:
+    """Gives the device memory that freed pools left with the library back to the current device."""
+    _chk(lib.laser_trim())
 
 
 def draft(pool: Pool, tails, tail_len, group_id, params: Params, draft_out=None, draft_len=None,

@@ -50,11 +50,13 @@ laser_status current_pool(bool make, cudaMemPool_t* out) {
 }
 
 // Gives the pool's unused memory back to the device.
-void trim_pool() {
+laser_status trim_pool() {
   cudaMemPool_t pool = nullptr;
-  if (current_pool(false, &pool) != LASER_OK || !pool) return;
-  cudaDeviceSynchronize();
-  cudaMemPoolTrimTo(pool, 0);
+  LASER_TRY(current_pool(false, &pool));
+  if (!pool) return LASER_OK;
+  LASER_CUDA(cudaDeviceSynchronize());
+  LASER_CUDA(cudaMemPoolTrimTo(pool, 0));
+  return LASER_OK;
 }
 }  // namespace
 
@@ -146,3 +148,4 @@ laser_status encode_bf16_2d(CUtensorMap* tm, const void* ptr, uint64_t rows, uin
 LASER_API const char* laser_version(void) { return "laser-b200 0.1.0 (sm_100a)"; }
 LASER_API const char* laser_last_error(void) { return laser::t_err; }
 LASER_API int64_t laser_launch_count(void) { return laser::g_launches; }
+LASER_API laser_status laser_trim(void) { return laser::trim_pool(); }

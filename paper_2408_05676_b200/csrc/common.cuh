@@ -46,7 +46,8 @@ laser_status scratch_get(int slot, size_t bytes, void** out);
 // Stream-ordered device memory from a pool of the library's own (one per device, any thread and stream).  Memory given back
 // stays with the pool up to 2 GB, so that building and dropping retrieval pools does not go through the driver each time (a
 // gigabyte takes it 4 .. 100 ms to hand out and 4 to take back); what is above goes back to the device at the next
-// synchronisation, and all of it when one of the library's allocations finds no memory (device_malloc, pooled_alloc).
+// synchronisation, and all of it at laser_trim or when one of the library's allocations finds no memory (device_malloc,
+// pooled_alloc).
 laser_status pooled_alloc(void** p, size_t bytes, cudaStream_t stream);
 void pooled_free(void* p, cudaStream_t stream);
 // cudaMalloc for the library's long-lived buffers

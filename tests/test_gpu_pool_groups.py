@@ -64,3 +64,28 @@ def test_build_by_group_size(L, sizes, vocab, n_min, n_max):
         got = L.draft(pool, dev_i32(tails), dev_i32(lens), dev_i32(gids), p)
         for g, w in zip(got, want):
             assert (g.cpu().numpy() == w).all()
+
+
+def test_freed_pools_are_given_back(L):
+    """What freed pools leave with the library is bounded, serves the next build, and goes back to the device on request."""
+    import torch
+
+    toks = np.random.default_rng(3).integers(0, 5000, 4_000_000).astype(np.int32)
+    offs = np.linspace(0, len(toks), 401).astype(np.int64)
+    L.pool_build(toks[:1000], np.array([0, 1000]), 1, 2).free()    # (whatever the first use loads)
+    L.trim()
+    free0 = torch.cuda.mem_get_info()[0]
+    keep = L.pool_build(toks[:1000], np.array([0, 1000]), 1, 2)
+    pool = L.pool_build(toks, offs, 1, 4)
+    size = pool.info()["device_bytes"]
+    pool.free()
+    assert free0 - torch.cuda.mem_get_info()[0] < (2 << 30) + (64 << 20)
+    L.trim()
+    assert free0 - torch.cuda.mem_get_info()[0] < size / 2         # (a block beside the small pool's may stay)
+    got = L.draft(keep, dev_i32([toks[10:12]]), dev_i32([2]), dev_i32([0]), L.make_params(K=4, n_min=1, n_max=2, max_occ=64))
+    want = R.draft_batch(toks[:1000], np.array([0, 1000]), toks[None, 10:12], np.array([2]), np.array([0]), 4, 1, 2, 1, 64)
+    for g, w in zip(got, want):
+        assert (g.cpu().numpy() == w).all()
+    keep.free()
+    L.trim()
+    assert torch.cuda.mem_get_info()[0] >= free0
