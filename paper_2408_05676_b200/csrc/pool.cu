@@ -12,7 +12,7 @@
 // group bounds, so results never depend on the hash.
 //
 // Build: a group whose working set fits shared memory is indexed there by one CTA per n
-// (index_group_kernel); the n-grams of larger groups are inserted into the table itself, and their
+// (index_group_kernel); the n-grams of larger groups, and of many tiny ones, are inserted into the table itself, and their
 // positions sorted by slot, all groups together, with the radix sort of CUB, the header library
 // shipped with the CUDA toolkit (nothing on the per-step path uses it).
 //
@@ -24,8 +24,9 @@
 #include <cub/device/device_radix_sort.cuh>
 
 #include <algorithm>
+#include <memory>
+#include <new>
 #include <type_traits>
-#include <vector>
 
 #include "common.cuh"
 
@@ -75,11 +76,11 @@ __host__ __device__ __forceinline__ Region region_of(int64_t lo, int64_t hi, int
 
 constexpr int kKeyThreads = 256;
 
-// Largest g in [lo, hi) with goff[g] <= p (skips empty groups)
-__device__ __forceinline__ int group_of(const int64_t* __restrict__ goff, int lo, int hi, int64_t p) {
+// Largest g in [lo, hi) with at[g] <= p (skips empty groups)
+__device__ __forceinline__ int group_of(const uint32_t* __restrict__ at, int lo, int hi, int64_t p) {
   while (hi - lo > 1) {
     int mid = (lo + hi) >> 1;
-    if (goff[mid] <= p) lo = mid; else hi = mid;
+    if (at[mid] <= p) lo = mid; else hi = mid;
   }
   return lo;
 }
@@ -87,7 +88,7 @@ __device__ __forceinline__ int group_of(const int64_t* __restrict__ goff, int lo
 struct IndexLevels { uint2* table[kMaxN + 1]; uint32_t* positions[kMaxN + 1]; };
 
 // The groups that the sort takes: their ids, and where the positions of each begin when they are laid end to end.
-struct LargeGroups { const int32_t* id; const int64_t* at; int n; };
+struct SortedGroups { const uint32_t* id; const uint32_t* at; int n; };
 
 // Inserts the n-grams of the listed groups, for the n from n0 on, into their regions (cleared before) and leaves every (n,
 // position) with the number of its n-gram's slot among all those tables' (kNoSlot where none ends).  An entry is {key's low
@@ -97,7 +98,7 @@ struct LargeGroups { const int32_t* id; const int64_t* at; int n; };
 constexpr uint32_t kNoSlot = 0xffffffffu;
 constexpr int kInsertItems = 4, kInsertBlock = kInsertItems * kKeyThreads;
 __global__ void __launch_bounds__(kKeyThreads)
-insert_large_kernel(const int32_t* __restrict__ tok, const int64_t* __restrict__ goff, LargeGroups lg, int64_t M, int n0,
+insert_sorted_kernel(const int32_t* __restrict__ tok, const int64_t* __restrict__ goff, SortedGroups lg, int64_t M, int n0,
                     const IndexLevels lv, uint32_t table_slots, uint32_t* __restrict__ slot_of, uint32_t* __restrict__ pos,
                     unsigned long long* __restrict__ n_valid, int* __restrict__ max_tok) {
   __shared__ int s_g[2], s_max[kKeyThreads / 32];
@@ -110,7 +111,7 @@ insert_large_kernel(const int32_t* __restrict__ tok, const int64_t* __restrict__
   __syncthreads();
   int mt = -1, ends = 0;
   for (int64_t i = i0 + threadIdx.x; i < min(M, i0 + kInsertBlock); i += kKeyThreads) {
-    const int l = s_g[0] == s_g[1] ? s_g[0] : group_of(lg.at, s_g[0], s_g[1] + 1, i), g = lg.id[l];
+    const int l = s_g[0] == s_g[1] ? s_g[0] : group_of(lg.at, s_g[0], s_g[1] + 1, i), g = int(lg.id[l]);
     const int64_t lo = goff[g], p = lo + (i - lg.at[l]);
     bool valid = i - lg.at[l] >= n - 1;
     uint64_t key = key_begin(g, n);
@@ -190,8 +191,8 @@ index_runs_kernel(const uint32_t* __restrict__ slot, const uint32_t* __restrict_
 }
 
 __global__ void __launch_bounds__(kKeyThreads)
-clear_regions_kernel(const IndexLevels lv, int n_min, const int64_t* __restrict__ goff, LargeGroups lg) {
-  const int g = lg.id[blockIdx.y];
+clear_regions_kernel(const IndexLevels lv, int n_min, const int64_t* __restrict__ goff, SortedGroups lg) {
+  const int g = int(lg.id[blockIdx.y]);
   const Region rg = region_of(goff[g], goff[g + 1], g);
   uint2* table = lv.table[n_min + blockIdx.z] + rg.base;
   for (uint32_t s = blockIdx.x * kKeyThreads + threadIdx.x; s < rg.slots; s += gridDim.x * kKeyThreads) table[s] = make_uint2(0xffffffffu, 0xffffffffu);
@@ -217,10 +218,16 @@ constexpr int64_t kClassMax[kClasses] = {kGroupMax, 7600, 4900};
 static_assert(group_smem(kGroupMax) <= 226 * 1024 && 2 * group_smem(kClassMax[1]) <= 224 * 1024 && 3 * group_smem(kClassMax[2]) <= 222 * 1024 &&
               kGroupMax + kGroupMax / 2 + kGroupMax / 8 + 4 < 65535, "");
 
+// A CTA per (group, n) costs about 15 ns of the device whatever the group's size, so tiny groups are sorted with the large ones
+// where they are so many that the sort's own launches (0.2 ms) do not show.  10 M tokens in groups of 5 / 20 / 100 / 200 / 250: a CTA
+// each 92 / 25.7 / 6.9 / 3.95 / 3.31 ms, sorted 15.2 / 5.6 / 3.5 / 3.24 / 3.13; 1 M tokens in groups of 20 / 100 / 200: 2.42 / 0.71 / 0.46,
+// sorted 0.70 / 0.49 / 0.46; 200 k tokens in groups of 20 / 100 (2000 of them): 0.54 / 0.21, sorted 0.25 / 0.21.
+constexpr int kTinyGroup = 256, kManyTiny = 4096;
+
 template <int THREADS, int CTAS>
 __global__ void __launch_bounds__(THREADS, CTAS)
-index_group_kernel(const int32_t* __restrict__ tok, const int64_t* __restrict__ goff, const int32_t* __restrict__ group_id,
-                   const int64_t* __restrict__ group_at, int leads, int n_min, const IndexLevels lv, unsigned long long* __restrict__ n_heads,
+index_group_kernel(const int32_t* __restrict__ tok, const int64_t* __restrict__ goff, const uint32_t* __restrict__ group_id,
+                   const uint32_t* __restrict__ group_at, int leads, int n_min, const IndexLevels lv, unsigned long long* __restrict__ n_heads,
                    int* __restrict__ max_tok) {
   constexpr int kWarps = THREADS / 32, kBlock = 256;
   extern __shared__ __align__(16) uint32_t s_word[];
@@ -229,7 +236,7 @@ index_group_kernel(const int32_t* __restrict__ tok, const int64_t* __restrict__ 
   if (leads) wait_for_earlier();  // the first class waits for its inputs, and so do those that it lets start
   next_may_launch();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  const int g = group_id[blockIdx.x], n = n_min + blockIdx.y;
+  const int g = int(group_id[blockIdx.x]), n = n_min + blockIdx.y;
   const int64_t lo = goff[g], hi = goff[g + 1], first = group_at[blockIdx.x];   // first: of the group's runs
   const int T = int(hi - lo);
   const Region rg = region_of(lo, hi, g);
@@ -1075,27 +1082,41 @@ LASER_API laser_status laser_pool_build(const int32_t* tokens, int64_t n_tokens,
 
   LASER_CUDA(cudaGetDevice(&P->device));
 
-  // Groups by size: what fits shared memory, in three classes of its use (one, two and four CTAs an SM), the larger first, and
-  // the rest.  The positions of the first come first in the position arrays, those of the large groups (sorted together) behind.
+  // Groups by size: what fits shared memory, in three classes of its use (one, two and three CTAs an SM), the larger first, and
+  // the rest, which are sorted together: larger groups, and tiny ones where they are many.  The positions of the first come first
+  // in the position arrays, those of the sorted groups behind.
   const size_t N = size_t(n_tokens);
-  std::vector<int32_t> id[kClasses + 1];
+  auto class_of = [&](int64_t size) { int c = 0; while (c < kClasses && size <= kClassMax[c]) ++c; return c; };   // 0: large
+  int count[kClasses + 1] = {}, n_tiny = 0;
+  int64_t sum[kClasses + 1] = {}, tiny_sum = 0;
   for (int g = 0; g < n_groups; ++g) {
     const int64_t size = group_offsets[g + 1] - group_offsets[g];
-    int c = 0;
-    while (c < kClasses && size <= kClassMax[c]) ++c;
-    id[c].push_back(g);            // 0: large
+    const int c = class_of(size);
+    ++count[c]; sum[c] += size;
+    if (size < kTinyGroup) { ++n_tiny; tiny_sum += size; }
   }
-  // [n_groups] ids, [n_groups + 1] starts: of the small groups their runs' place, of the large ones their place among those
-  std::vector<int64_t> lists(size_t(n_groups) * 2 + 2);
-  int64_t* const h_at = lists.data();
-  int32_t* const h_id = reinterpret_cast<int32_t*>(h_at + n_groups + 1);
-  int64_t n_small = 0, n_large = 0;
-  size_t fill = 0;
-  for (int c = 1; c <= kClasses; ++c)
-    for (int32_t g : id[c]) { h_id[fill] = g; h_at[fill++] = n_small; n_small += group_offsets[g + 1] - group_offsets[g]; }
-  for (int32_t g : id[0]) { h_id[fill] = g; h_at[fill++] = n_large; n_large += group_offsets[g + 1] - group_offsets[g]; }
-  h_at[fill] = n_large;
-  const size_t M = size_t(n_large);
+  const int64_t least = n_tiny >= kManyTiny ? kTinyGroup : 0;    // of a group in shared memory
+  if (least) { count[kClasses] -= n_tiny; sum[kClasses] -= tiny_sum; count[0] += n_tiny; sum[0] += tiny_sum; }
+  // [n_groups] ids, [n_groups + 1] starts: of the groups in shared memory their runs' place, of the others their place among those
+  std::unique_ptr<uint32_t[]> lists(new (std::nothrow) uint32_t[size_t(n_groups) * 2 + 1]);
+  if (!lists) { set_error("no host memory for %d groups", n_groups); return LASER_ERR_OOM; }
+  uint32_t *const h_id = lists.get(), *const h_at = h_id + n_groups;
+  int fill[kClasses + 1];
+  int64_t place[kClasses + 1];
+  const int n_small_groups = n_groups - count[0];
+  int64_t n_small = 0;
+  for (int c = 1, f = 0; c <= kClasses; ++c) { fill[c] = f; place[c] = n_small; f += count[c]; n_small += sum[c]; }
+  fill[0] = n_small_groups; place[0] = 0;
+  for (int g = 0; g < n_groups; ++g) {
+    const int64_t size = group_offsets[g + 1] - group_offsets[g];
+    const int c = size < least ? 0 : class_of(size);
+    h_id[fill[c]] = uint32_t(g);
+    h_at[fill[c]++] = uint32_t(place[c]);
+    place[c] += size;
+  }
+  h_at[n_groups] = uint32_t(sum[0]);
+  const int64_t n_sorted = sum[0];
+  const size_t M = size_t(n_sorted);
 
   // One allocation for the index, sized before any key is counted; one for the build's own buffers.
   const size_t slots = size_t(region_base(n_tokens, n_groups));
@@ -1118,7 +1139,7 @@ LASER_API laser_status laser_pool_build(const int32_t* tokens, int64_t n_tokens,
   LASER_CUDA(cudaMemcpyAsync(P->tokens, tokens, N * 4, cudaMemcpyDefault, stream));
   LASER_CUDA(cudaMemcpyAsync(P->group_offsets, group_offsets, (size_t(n_groups) + 1) * 8, cudaMemcpyHostToDevice, stream));
 
-  // The large groups' n-grams go through one sort for as many n as 32-bit slot numbers and 64 M pairs hold.
+  // The sorted groups' n-grams go through one sort for as many n as 32-bit slot numbers and 64 M pairs hold.
   const int levels = n_max - n_min + 1;
   const int batch = int(std::max<size_t>(1, std::min({size_t(levels), size_t(kNoSlot) / slots, (size_t(64) << 20) / std::max<size_t>(M, 1)})));
   int slot_bits = 1;             // all that kNoSlot needs to sort behind every slot
@@ -1129,49 +1150,51 @@ LASER_API laser_status laser_pool_build(const int32_t* tokens, int64_t n_tokens,
     cub::DoubleBuffer<uint32_t> kb(nullptr, nullptr), vb(nullptr, nullptr);
     LASER_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, cub_bytes, kb, vb, int64_t(pairs), 0, slot_bits, stream));
   }
-  constexpr size_t kCounters = (2 * kMaxN + 3) * 8;   // distinct keys per n, the largest token, n-grams of the large groups per n
-  const size_t b_lists = lists.size() * 8;
+  constexpr size_t kCounters = (2 * kMaxN + 3) * 8;   // distinct keys per n, the largest token, n-grams of the sorted groups per n
+  const size_t b_lists = (size_t(n_groups) * 2 + 1) * 4;
   struct Tmp { void* p = nullptr; cudaStream_t s; ~Tmp() { pooled_free(p, s); } } tmp{nullptr, stream};
   LASER_TRY(pooled_alloc(&tmp.p, 4 * padded(pairs * 4) + padded(kCounters) + padded(b_lists) + cub_bytes + 256, stream));
   at = static_cast<uint8_t*>(tmp.p);
   uint32_t *slot_of, *slot_alt, *pos, *pos_alt;
   unsigned long long* counters;
-  int64_t* d_at;
+  uint32_t* d_id;
   uint8_t* cub_tmp;
   take(&slot_of, padded(pairs * 4)); take(&slot_alt, padded(pairs * 4)); take(&pos, padded(pairs * 4)); take(&pos_alt, padded(pairs * 4));
-  take(&counters, padded(kCounters)); take(&d_at, padded(b_lists)); take(&cub_tmp, cub_bytes);
-  const int32_t* d_id = reinterpret_cast<const int32_t*>(d_at + n_groups + 1);
+  take(&counters, padded(kCounters)); take(&d_id, padded(b_lists)); take(&cub_tmp, cub_bytes);
+  const uint32_t* d_at = d_id + n_groups;
   int* max_tok = reinterpret_cast<int*>(counters + kMaxN + 1);
   unsigned long long* n_valid = counters + kMaxN + 2;
-  LASER_CUDA(cudaMemcpyAsync(d_at, lists.data(), b_lists, cudaMemcpyHostToDevice, stream));
+  LASER_CUDA(cudaMemcpyAsync(d_id, lists.get(), b_lists, cudaMemcpyHostToDevice, stream));
   LASER_CUDA(cudaMemsetAsync(counters, 0, kCounters, stream));
   LASER_CUDA(cudaMemsetAsync(max_tok, 0xff, 4, stream));
   for (int n = n_min; n <= n_max; ++n) LASER_CUDA(cudaMemsetAsync(P->level[n].positions + N, 0xff, 32 * 4, stream));
+  if (least)                     // (so many regions are cleared as whole tables)
+    for (int n = n_min; n <= n_max; ++n) LASER_CUDA(cudaMemsetAsync(P->level[n].table, 0xff, slots * 8, stream));
   size_t done = 0;
   for (int c = 1; c <= kClasses; ++c) {
-    if (id[c].empty()) continue;
+    if (!count[c]) continue;
     auto index = [&](auto kernel, unsigned threads) -> laser_status {
       const size_t smem = group_smem(kClassMax[c - 1]);
       LASER_CUDA(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-      LASER_CUDA(launch_overlapped(kernel, dim3(unsigned(id[c].size()), unsigned(n_max - n_min + 1)), threads, smem, stream, P->tokens,
+      LASER_CUDA(launch_overlapped(kernel, dim3(unsigned(count[c]), unsigned(n_max - n_min + 1)), threads, smem, stream, P->tokens,
                                    P->group_offsets, d_id + done, d_at + done, done == 0 ? 1 : 0, n_min, lvs, counters, max_tok));
       return LASER_OK;
     };
     LASER_TRY(c == 1 ? index(index_group_kernel<1024, 1>, 1024) : c == 2 ? index(index_group_kernel<512, 2>, 512) : index(index_group_kernel<512, 3>, 512));
     count_launch();
-    done += id[c].size();
+    done += size_t(count[c]);
   }
   if (M) {
-    const LargeGroups lg{d_id + done, d_at + done, int(id[0].size())};
+    const SortedGroups lg{d_id + done, d_at + done, count[0]};
     const unsigned blocks = unsigned(ceil_div<size_t>(M, kInsertBlock));
-    for (int l0 = 0; l0 < lg.n; l0 += 65535)
+    for (int l0 = 0; l0 < lg.n && !least; l0 += 65535)
       clear_regions_kernel<<<dim3(16, unsigned(std::min(lg.n - l0, 65535)), unsigned(levels)), kKeyThreads, 0, stream>>>(
-          lvs, n_min, P->group_offsets, LargeGroups{lg.id + l0, lg.at + l0, lg.n - l0});
+          lvs, n_min, P->group_offsets, SortedGroups{lg.id + l0, lg.at + l0, lg.n - l0});
     count_launch();
     for (int n0 = n_min; n0 <= n_max; n0 += batch) {
       const int nb = std::min(batch, n_max - n0 + 1);
       const int64_t count = int64_t(M) * nb;
-      insert_large_kernel<<<dim3(blocks, unsigned(nb)), kKeyThreads, 0, stream>>>(P->tokens, P->group_offsets, lg, n_large, n0, lvs,
+      insert_sorted_kernel<<<dim3(blocks, unsigned(nb)), kKeyThreads, 0, stream>>>(P->tokens, P->group_offsets, lg, n_sorted, n0, lvs,
                                                                                   uint32_t(slots), slot_of, pos, n_valid, max_tok);
       cub::DoubleBuffer<uint32_t> kb(slot_of, slot_alt), vb(pos, pos_alt);
       LASER_CUDA(cub::DeviceRadixSort::SortPairs(cub_tmp, cub_bytes, kb, vb, count, 0, slot_bits, stream));

@@ -89,3 +89,29 @@ def test_freed_pools_are_given_back(L):
     keep.free()
     L.trim()
     assert torch.cuda.mem_get_info()[0] >= free0
+
+
+def test_many_tiny_groups(L):
+    """Tiny groups that are many are sorted together with the large ones, beside groups of shared memory, on both sides of either
+    limit; more groups than a grid's second dimension holds."""
+    rng = np.random.default_rng(12)
+    sizes = np.concatenate([rng.integers(0, 12, 66000), [15401, 3000, 255, 256, 257, 0, 5000]])
+    rng.shuffle(sizes)
+    N, n_max, vocab = int(sizes.sum()), 3, 30
+    toks = rng.integers(0, vocab, N).astype(np.int32)
+    toks[rng.integers(0, N, N // 50)] = -1
+    offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    pool = L.pool_build(toks, offs, 1, n_max)
+    assert pool.info()["n_keys"] == _n_keys(toks, offs, 1, n_max)
+    gids = np.concatenate([np.flatnonzero(sizes >= 200), rng.integers(0, len(sizes), 300)]).astype(np.int32)
+    tails = np.zeros((len(gids), n_max), np.int32)
+    for b, g in enumerate(gids):
+        at = offs[g] + int(rng.integers(0, max(1, sizes[g] - n_max)))
+        t = np.maximum(toks[at:min(at + n_max, N)], 0)
+        tails[b, n_max - len(t):] = t
+    lens = np.full(len(gids), n_max, np.int32)
+    for max_occ in (64, 0):
+        want = R.draft_batch(toks, offs, tails, lens, gids, 6, 1, n_max, 2, max_occ)
+        got = L.draft(pool, dev_i32(tails), dev_i32(lens), dev_i32(gids), L.make_params(K=6, n_min=1, n_max=n_max, min_draft=2, max_occ=max_occ))
+        for g, w in zip(got, want):
+            assert (g.cpu().numpy() == w).all()
