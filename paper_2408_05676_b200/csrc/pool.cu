@@ -226,9 +226,8 @@ constexpr int kTinyGroup = 256, kManyTiny = 4096;
 
 template <int THREADS, int CTAS>
 __global__ void __launch_bounds__(THREADS, CTAS)
-index_group_kernel(const int32_t* __restrict__ tok, const int64_t* __restrict__ goff, const uint32_t* __restrict__ group_id,
-                   const uint32_t* __restrict__ group_at, int leads, int n_min, const IndexLevels lv, unsigned long long* __restrict__ n_heads,
-                   int* __restrict__ max_tok) {
+index_group_kernel(const int32_t* tok, const int64_t* goff, const uint32_t* group_id, const uint32_t* group_at, int leads, int n_min,
+                   const IndexLevels lv, unsigned long long* n_heads, int* max_tok) {
   constexpr int kWarps = THREADS / 32, kBlock = 256;
   extern __shared__ __align__(16) uint32_t s_word[];
   __shared__ uint32_t s_sum[kWarps];
