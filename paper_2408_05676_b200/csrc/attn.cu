@@ -55,12 +55,12 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
 // as pairs ([hi | lo] rows of 2 H DH).
 template <int DH, int TPC, bool PR, bool SP>
 __global__ void __launch_bounds__(kAttnThreads, PR ? 3 : kCtasPerSm)
-attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restrict__ q, const float* __restrict__ qf,
+attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* q, const float* qf,
                   const int32_t* __restrict__ seq_ids, const int32_t* __restrict__ row_ctx,
                   const int32_t* __restrict__ row_n, int Rs, int H, int Hkv,
                   const int32_t* __restrict__ page_table, int pages_per_seq, int layer_row0,
                   bf16* __restrict__ out, int32_t* __restrict__ status,
-                  const unsigned long long* __restrict__ row_mask, int fresh, int splits,
+                  const unsigned long long* row_mask, int fresh, int splits,
                   float* __restrict__ part, int32_t* __restrict__ arrived) {
   constexpr int kPartFloats = 16 * TPC * (DH + 2);   // SP: a partial result: O [rows][DH], max [rows], sum [rows]
   constexpr int HALVES = DH / 64;                 // 64-element (128-byte) column blocks per row
@@ -77,7 +77,8 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* __restr
   // Programmatic dependent launch: let the next kernel start its prologue.  The kernel before this
   // one produces Q and the K/V of the step's own rows; pages that lie wholly below the committed
   // length were written by earlier steps, so the producer requests those before it waits for that
-  // kernel, and the wait and the Q tile overlap their flight.
+  // kernel, and the wait and the Q tile overlap their flight.  (q and qf are written while this kernel may be running already:
+  // they are not const __restrict__.)
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int b = SP ? blockIdx.x / splits : blockIdx.x, krank = SP ? blockIdx.x % splits : 0, h = blockIdx.y, mt = blockIdx.z;
   const int hk = h / (H / Hkv);
