@@ -383,6 +383,13 @@ laser_status laser_verify_accept(laser_model* m, laser_kv* kv, const int32_t* se
  *           producer role, [2] the producer saw its copy land, [3] cycles the wait took.
  * Asynchronous on `stream`.  Errors: INVALID_ARG. */
 laser_status laser_selftest_wait(laser_model* m, int64_t limit_cycles, int32_t* report, void* stream);
+/* Self-test of the hand-over between the SMs that share a tile of a contraction of many token rows:
+ * each waits `wait_cycles` clock cycles for the others' partial sums (200000 unless this call changes
+ * it for the model, 0 .. 2e6), then leaves its share to the one that arrives last.  Results are the
+ * same whoever does the work.  Synchronises the device.
+ *   state_left  host int32 out: words of the hand-over's state that earlier steps did not leave zero
+ * Errors: INVALID_ARG, CUDA. */
+laser_status laser_selftest_peers(laser_model* m, int32_t wait_cycles, int32_t* state_left);
 
 /* ---- Grouping (Section 3.2, Collaborative-based Grouping) ------------------------------
  * K-means over embeddings (Lloyd's iteration): the clustering by which the paper assigns users

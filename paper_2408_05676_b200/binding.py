@@ -63,7 +63,7 @@ EXPORTS = ["laser_version", "laser_last_error", "laser_launch_count", "laser_poo
            "laser_kv_get_len", "laser_kv_reset", "laser_kv_set_len_dev", "laser_kv_import", "laser_kv_export",
            "laser_verify_step", "laser_verify_step_tree", "laser_check", "laser_profile_enable", "laser_profile_read", "laser_accept_commit", "laser_accept_commit_noalloc", "laser_accept_tree", "laser_kv_compact_path",
            "laser_verify_accept",
-           "laser_selftest_wait", "laser_group_kmeans", "laser_generate"]
+           "laser_selftest_wait", "laser_selftest_peers", "laser_group_kmeans", "laser_generate"]
 
 lib.laser_version.restype = C.c_char_p
 lib.laser_last_error.restype = C.c_char_p
@@ -370,6 +370,13 @@ def selftest_wait(model: Model, limit_cycles: int, stream=None) -> torch.Tensor:
     report = torch.zeros(4, dtype=torch.int32, device="cuda")
     _chk(lib.laser_selftest_wait(model.handle, C.c_int64(int(limit_cycles)), _ptr(report), _stream(stream)))
     return report
+
+
+def selftest_peers(model: Model, wait_cycles: int = 200000) -> int:
+    """Sets the wait for each other of the SMs that share a tile; returns the state words that are not zero."""
+    left = C.c_int32()
+    _chk(lib.laser_selftest_peers(model.handle, C.c_int32(wait_cycles), C.byref(left)))
+    return left.value
 
 
 def accept_commit_noalloc(kv: Optional[KV], seq_ids, logits, tokens, n_rows, params: Params, out, stream=None):

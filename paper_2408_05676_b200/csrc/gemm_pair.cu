@@ -42,7 +42,6 @@ constexpr int kMaxStages = 8;
 constexpr int kChunk = 32;                       // token rows in a group's staging buffer
 constexpr int kStgRow = 132;                     // floats per staged row
 constexpr int kStgBytes = kChunk * kStgRow * 4;  // 16.5 KB per group
-constexpr long long kPeerCycles = 200000;        // about 0.1 ms: many times the skew between pairs that are running
 constexpr int kPairSmem = 220 * 1024;   // + up to 6.2 KB of static shared memory
 
 struct PairPlan {
@@ -50,6 +49,7 @@ struct PairPlan {
   int P;                        // pairs in the grid
   int full_tiles, rem_tiles;    // whole tiles; tiles cut along K: every token tile of the last weight tiles
   int S, k;                     // cut tiles: K ranges of a tile, K blocks of a range
+  int peer_cycles;              // how long a contributor waits for the others of its tile
   float* scratch;               // [pair][rank][NT][128 features]
   int32_t* state;               // [cut tile][rank][kPairState]
 };
@@ -402,7 +402,7 @@ gemm_pair_kernel(const __grid_constant__ CUtensorMap tmW, const __grid_constant_
         const long long t0 = clock64();
         int have = 0;
         do asm volatile("ld.acquire.gpu.global.s32 %0, [%1];" : "=r"(have) : "l"(state) : "memory");
-        while (have < it.C && clock64() - t0 < kPeerCycles);
+        while (have < it.C && clock64() - t0 < pl.peer_cycles);
         bool mine = have >= it.C;
         if (!mine) {
           atomicExch(state + 2 + it.c, 1);
@@ -552,6 +552,7 @@ laser_status gemm_pair_launch(laser_model* m, const GemmPairShape& sh, const CUt
   const Cut cut = cut_of(tiles, pl.n_tt, pl.KB, sh.split != 0);
   pl.full_tiles = cut.full_tiles; pl.rem_tiles = cut.rem_tiles;
   pl.S = cut.S; pl.k = cut.k;
+  pl.peer_cycles = m->peer_cycles;
   pl.scratch = m->pair_scratch;
   pl.state = m->pair_state;
   switch (epi) {

@@ -43,6 +43,7 @@ struct laser_model {
   int32_t* attn_arrived = nullptr;
   float* pair_scratch = nullptr;   // partial sums of the contractions for many rows (gemm_pair.cu), and the cut tiles' state
   int32_t* pair_state = nullptr;
+  int peer_cycles = 200000;        // how long they wait for each other: about 0.1 ms, many times the skew between pairs that are running
   void* gemm_state = nullptr;      // tensor-map cache of the tensor-core GEMM
   void* gen_buf = nullptr;         // work buffers of laser_generate, kept between calls (in `owned`)
   size_t gen_bytes = 0;

@@ -3,6 +3,10 @@
 // copies it still has in flight, and surface LASER_ERR_TIMEOUT through the model's status word -
 // leaving the context usable.  Nothing faults or hangs: the wait is on a barrier nobody arrives
 // on, with a limit the caller passes (the production limit kWaitCycles is not touched).
+#include <algorithm>
+#include <vector>
+
+#include "gemm_pair.cuh"
 #include "model.cuh"
 #include "tma.cuh"
 
@@ -48,6 +52,20 @@ selftest_wait_kernel(const float* __restrict__ src, long long limit_cycles, int3
 
 }  // namespace
 }  // namespace laser
+
+// The hand-over of slices in the contractions for many token rows (gemm_pair.cu) is reached only where the SMs of a tile's
+// contributors are held by other kernels; with a wait of zero cycles every contributor that is not the last gives its slice up.
+LASER_API laser_status laser_selftest_peers(laser_model* m, int32_t wait_cycles, int32_t* state_left) {
+  using namespace laser;
+  LASER_REQUIRE(m && state_left, "null argument");
+  LASER_REQUIRE(wait_cycles >= 0 && wait_cycles <= 2000000, "wait_cycles = %d outside [0, 2e6]", wait_cycles);
+  std::vector<int32_t> state(kPairStateInts);
+  LASER_CUDA(cudaDeviceSynchronize());
+  LASER_CUDA(cudaMemcpy(state.data(), m->pair_state, sizeof(int32_t) * kPairStateInts, cudaMemcpyDeviceToHost));
+  *state_left = int32_t(std::count_if(state.begin(), state.end(), [](int32_t v) { return v != 0; }));
+  m->peer_cycles = wait_cycles;
+  return LASER_OK;
+}
 
 LASER_API laser_status laser_selftest_wait(laser_model* m, int64_t limit_cycles, int32_t* report, void* stream) {
   using namespace laser;

@@ -36,8 +36,10 @@ def test_layers_at_the_tile_edges(L, B, K, precise):
 
 
 # No layers: the LM head alone, whose [vocab, d_model] shape sets how its 256-row tiles fall on the 74 SM pairs.
-# Left-over tiles: 2 of 74 (many contributors each), 20 (three), 30 (two), 60 (more than half of the pairs: whole), 125 - 74 = 51 (whole), none.
-@pytest.mark.parametrize("tiles,d,precise", [(2, 8192, 0), (20, 8192, 0), (30, 8192, 0), (60, 8192, 1), (125, 2048, 1), (74, 512, 0)])
+# Cut: 2 weight tiles x 3 token tiles (twelve contributors each), 12 x 2 (three), with operands as pairs 2 x 4 (nine) and 12 x 3
+# (two).  Whole: 20 x 3, 30 x 2, 60 x 1 (more than half of the pairs), 125 x 2 (three waves and part of a fourth), 74 x 3.
+@pytest.mark.parametrize("tiles,d,precise", [(2, 8192, 0), (20, 8192, 0), (30, 8192, 0), (60, 8192, 1), (125, 2048, 1), (74, 512, 0),
+                                             (12, 8192, 0), (2, 8192, 1), (12, 8192, 1)])
 def test_left_over_tiles_cut_along_k(L, tiles, d, precise):
     B, K = 20, 8                                     # 180 rows
     V = tiles * 256 - 8                              # the last weight tile overhangs
@@ -58,4 +60,27 @@ def test_left_over_tiles_cut_along_k(L, tiles, d, precise):
     for _ in range(3):                               # the partial sums are added in a fixed order
         again = L.verify_step(m, kv, dev_i32(range(B)), dev_i32(np.stack(rows)), dev_i32([K + 1] * B))
         assert torch.equal(first, again)
+    L.check(m)
+
+
+# A contributor that finds its peers late leaves its slice of the rows to the last one: with no time to wait nearly every slice
+# is handed over.  LM heads whose tiles have twelve, three, four and (behind a full wave) two contributors; a layer whose gate/up
+# and down projections are cut.
+@pytest.mark.parametrize("over", [dict(n_layers=0, d_model=8192, vocab=2 * 256 - 8), dict(n_layers=0, d_model=8192, vocab=12 * 256),
+                                  dict(n_layers=0, d_model=8192, vocab=30 * 256, precise=1), dict(n_layers=0, d_model=8192, vocab=60 * 256, precise=1),
+                                  dict(shape="7b", n_layers=1, vocab=4096)])
+def test_slices_handed_to_the_last_contributor(L, over):
+    B, K = 30, 8                                     # 270 rows
+    over = dict(over)
+    cfg = synth.model_cfg(over.pop("shape", "tiny"), max_draft=K, **over)
+    m = L.model_create(cfg, synth.make_weights(cfg, seed=1, device="cuda", gain_jitter=0.1), max_batch=B)
+    kv = L.kv_create(m, B, B * 2)
+    ids, n_rows = dev_i32(range(B)), dev_i32([K + 1] * B)
+    tokens = dev_i32(np.stack([synth.make_prompt(K + 1, cfg["vocab"], 70 + b) for b in range(B)]))
+    want = L.verify_step(m, kv, ids, tokens, n_rows)
+    for cycles in (0, 0, 300, 1500, 200000):
+        assert L.selftest_peers(m, cycles) == 0
+        for _ in range(4):
+            assert torch.equal(want, L.verify_step(m, kv, ids, tokens, n_rows))
+    assert L.selftest_peers(m) == 0
     L.check(m)
