@@ -20,12 +20,14 @@ constexpr int kAcceptThreads = kVerdictThreads;
 constexpr int kMaxAcceptSeqs = 1 << 16;  // counters live at the start of the scratch
 
 // Parts of a row: a CTA goes through its part in batches of 8192 values, a memory round trip each, so rows are cut into two or
-// four while about all CTAs with work can be resident at once (four an SM).  How many rows are active is known on the device alone: the
-// host launches up to twice the CTAs that fit, and the kernel takes so many parts that those with work do.  32000 logits, relaxed
-// rule, all rows active, in one / two / four / eight parts: 9 rows 9.8 / 8.0 / 7.3 / 8.4 us, 144 rows 12.7 / 11.0 / 10.3 / 16.6, 288
-// rows 15.3 / 12.5 / 15.8 / 26.7, 576 rows 18.2 / 20.4 / 26.1 / 45.4.
+// four while all CTAs with work can be resident at once (four an SM).  How many rows are active is known on the device alone: the
+// host launches up to twice the CTAs that fit, and the kernel takes so many parts that those with work do.  All rows active,
+// relaxed rule, device time in one / two / four parts: 32000 logits, 9 rows 8.7 / 7.3 / 6.8 us, 144 rows 12.9 / 10.5 / 9.6, 288 rows 13.8 /
+// 12.0 / 15.0; 12000 logits, 9 rows 6.6 / 6.2 / 6.7, 288 rows 9.9 / 9.2 / 14.8.  Where a whole row takes four batches or more, two parts still
+// end sooner with a third more CTAs than fit, and not otherwise: 324 / 396 / 432 rows of 28000 logits 16.4 / 16.4 / 16.5 whole, 14.6 /
+// 16.2 / 17.1 in two; of 24000 13.8 / 13.8 / 13.9, 14.5 / 16.2 / 17.0; of 50257 logits 400 / 440 rows 26.5 / 26.7, 25.9 / 27.2.
 constexpr int kLaunchedCtas = 8 * 148;
-constexpr int kFewCtas = 800;   // (592 can be resident; a third more still ends sooner than whole rows)
+constexpr int kResidentCtas = 4 * 148, kFewCtas = 800, kLongRow = 3 * 8192;
 int parts_of(int64_t rows, int32_t V) {
   int parts = 4;
   while (parts > 1 && (rows * parts > kLaunchedCtas || V < 4096 * parts)) parts /= 2;
@@ -59,7 +61,8 @@ accept_rows_kernel(const float* logits, const int32_t* tokens, const int32_t* n_
     mine = __reduce_add_sync(0xffffffffu, mine);
     if ((tid & 31) == 0 && mine) atomicAdd(&s_rows, mine);
     __syncthreads();
-    while (parts > 1 && s_rows * parts > kFewCtas) parts /= 2;
+    const int few = V > kLongRow ? kFewCtas : kResidentCtas;
+    while (parts > 1 && s_rows * parts > few) parts /= 2;
     if (part >= parts) return;
   }
   if (nr <= 0) {

@@ -17,9 +17,9 @@ def L():
     return binding
 
 
-# parts of at least 4096 values while there are at most 1184 launched and 800 active ones
+# parts of at least 4096 values while there are at most 1184 launched and 592 active ones (800 of rows longer than 24576)
 @pytest.mark.parametrize("B,R,V", [
-    (1, 2, 8195), (1, 3, 12287), (2, 5, 32003), (13, 9, 33001), (66, 9, 32002), (65, 9, 8200), (1, 256, 40), (1, 257, 31), (2, 300, 17), (1, 513, 9),
+    (1, 2, 8195), (1, 3, 12287), (2, 5, 32003), (13, 9, 33001), (66, 9, 32002), (65, 9, 8200), (65, 9, 12001), (1, 256, 40), (1, 257, 31), (2, 300, 17), (1, 513, 9),
 ])
 def test_parts_and_many_rows(L, B, R, V):
     rng = np.random.default_rng(B * 1000 + R)
