@@ -167,29 +167,37 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* q, cons
   asm volatile("griddepcontrol.wait;" ::: "memory");
   // Q tiles: rows of this sequence, zero beyond the active ones
   constexpr int QLO = 16 * TPC * QLD;             // PR: the lo parts of the Q tile follow the hi parts
-  for (int idx = tid; idx < 16 * TPC * (DH / 8); idx += kConsumers * 32) {
-    const int r = idx / (DH / 8), c = idx % (DH / 8);
-    uint4 v = make_uint4(0, 0, 0, 0), vl = v;
-    if (cta_row0 + r < nr) {
-      const size_t at = (size_t(b) * Rs + cta_row0 + r) * H * DH + size_t(h) * DH + c * 8;
-      if (PR) {
-        const float4 f0 = *reinterpret_cast<const float4*>(qf + at), f1 = *reinterpret_cast<const float4*>(qf + at + 4);
-        const float f[8] = {f0.x, f0.y, f0.z, f0.w, f1.x, f1.y, f1.z, f1.w};
-        uint32_t hi[4], lo[4];
+  constexpr int kQLoads = 16 * TPC * (DH / 8) / (kConsumers * 32);   // (all requested before the first is used)
+  uint4 qv[kQLoads][PR ? 2 : 1];
 #pragma unroll
-        for (int x = 0; x < 4; ++x) {
-          const __nv_bfloat162 hh = __floats2bfloat162_rn(f[2 * x], f[2 * x + 1]);
-          hi[x] = *reinterpret_cast<const uint32_t*>(&hh);
-          lo[x] = pack_bf16(f[2 * x] - __low2float(hh), f[2 * x + 1] - __high2float(hh));
-        }
-        v = make_uint4(hi[0], hi[1], hi[2], hi[3]);
-        vl = make_uint4(lo[0], lo[1], lo[2], lo[3]);
-      } else {
-        v = *reinterpret_cast<const uint4*>(q + at);
+  for (int x = 0; x < kQLoads; ++x) {
+    const int idx = tid + x * kConsumers * 32, r = idx / (DH / 8), c = idx % (DH / 8);
+    const size_t at = (size_t(b) * Rs + cta_row0 + r) * H * DH + size_t(h) * DH + c * 8;
+#pragma unroll
+    for (int y = 0; y < (PR ? 2 : 1); ++y) {
+      qv[x][y] = make_uint4(0, 0, 0, 0);
+      if (cta_row0 + r < nr) qv[x][y] = PR ? *reinterpret_cast<const uint4*>(qf + at + 4 * y) : *reinterpret_cast<const uint4*>(q + at);
+    }
+  }
+#pragma unroll
+  for (int x = 0; x < kQLoads; ++x) {
+    const int idx = tid + x * kConsumers * 32, r = idx / (DH / 8), c = idx % (DH / 8);
+    uint4 v = qv[x][0];
+    if (PR) {
+      const float* f0 = reinterpret_cast<const float*>(&qv[x][0]);
+      const float* f1 = reinterpret_cast<const float*>(&qv[x][PR ? 1 : 0]);
+      const float f[8] = {f0[0], f0[1], f0[2], f0[3], f1[0], f1[1], f1[2], f1[3]};
+      uint32_t hi[4], lo[4];
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const __nv_bfloat162 hh = __floats2bfloat162_rn(f[2 * u], f[2 * u + 1]);
+        hi[u] = *reinterpret_cast<const uint32_t*>(&hh);
+        lo[u] = pack_bf16(f[2 * u] - __low2float(hh), f[2 * u + 1] - __high2float(hh));
       }
+      v = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+      *reinterpret_cast<uint4*>(q_ptr + QLO + r * QLD + c * 8) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
     }
     *reinterpret_cast<uint4*>(q_ptr + r * QLD + c * 8) = v;
-    if (PR) *reinterpret_cast<uint4*>(q_ptr + QLO + r * QLD + c * 8) = vl;
   }
   asm volatile("bar.sync 1, 128;" ::: "memory");
   const int g = lane >> 2, qd = lane & 3;
