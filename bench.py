@@ -33,7 +33,7 @@ WORKLOAD = "verify-step-7b: batch 16, ctx 512 (16-token pages), 1+8 rows/seq, dr
 B, K, CTX, N_MAX = 16, 8, 512, 4
 POOL_TOKENS, POOL_GROUPS = 5_000_000, 1000
 # read + write MB of the QKV, O, gate/up and down launches of a layer x 32 + the LM head, from the ncu capture
-GEMM_DRAM_TRAFFIC_PER_STEP = int((105.3 + 37.2 + 187.1 + 99.8) * 32e6 + 269.1e6)
+GEMM_DRAM_TRAFFIC_PER_STEP = int((105.1 + 37.1 + 181.9 + 99.8) * 32e6 + 264.2e6)
 
 
 def measured_peaks():

@@ -459,7 +459,8 @@ __device__ __forceinline__ int gather_occurrences(const PoolView& pv, int64_t lo
 // The tokens of eight depths are requested together, so the walk costs a memory round trip per eight tokens; a vote takes one
 // step per distinct token (the first of those left names it, ballots count it) and stops at a majority, and a lone
 // occurrence is copied.  Each lane comparing its token with all 64 in shared memory cost 400 instructions a depth; 4096 queries
-// on 50 M tokens, max_occ 64: 34.8 -> 17.1 us with this and the 8-byte table entries.
+// on 50 M tokens, max_occ 64, with this and the 8-byte table entries: 33 -> 15.3 us a batch that is asked again (its part of the index
+// in L2), 38 -> 19 us batches not asked before.
 __device__ __forceinline__ int walk_occurrences(const int32_t* __restrict__ tok, int64_t hi, const int32_t* __restrict__ h, int hl,
                                                 uint32_t e0, uint32_t e1, bool a0, bool a1, int len, int K, int lane, int32_t* s_cur) {
   auto next = [&](uint32_t e, int j) -> int32_t {
@@ -829,7 +830,8 @@ __global__ void make_tree_rows_kernel(const int32_t* last, const int32_t* draft,
 // small share of them, as token frequencies fall fast.  A run that overflows the list is read again at every depth, with the
 // draft so far compared, until what is left fits.  Up to 64 survivors are walked by one warp in registers.
 // Bound by the latency of the longest run's passes; 4096 queries on 50 M tokens in 10,000 groups, the warp kernel included:
-// 1350 .. 2650 us (by the box) with three passes over the run at every depth and 256 threads -> 73 us.
+// 1200 .. 1800 us with three passes over the run at every depth and 256 threads -> 51 .. 58 us a batch that is asked again, 60 .. 64
+// us batches not asked before.
 constexpr int kBigThreads = 1024;
 constexpr int kBigUnroll = 4;
 constexpr int kBigList = 4096;      // positions: four a thread

@@ -7,7 +7,8 @@
 // The row is read once, 16 bytes a load and eight loads in flight per thread.  The probability is first estimated in fp32 with a
 // running maximum; the fp64 sum - an exponential per token, which used to be most of the kernel - is taken only where the
 // estimate lies within its error bound of p, so that the verdict is always the fp64 one.  64 sequences x 1 .. 9 rows of 32000
-// logits, relaxed rule: 57.5 -> 20.1 us; 18.4 with launches overlapped, 17.7 with the rows in two parts each.
+// logits, relaxed rule: 57.5 -> 20.1 us; 18.4 with launches overlapped, 17.6 with the rows in two parts each, 16.7 with sums that take
+// the same steps whether there is a maximum yet or not.
 #pragma once
 #include "common.cuh"
 
