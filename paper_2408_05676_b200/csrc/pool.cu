@@ -76,19 +76,25 @@ __host__ __device__ __forceinline__ Region region_of(int64_t lo, int64_t hi, int
 
 constexpr int kKeyThreads = 256;
 
-// Largest g in [lo, hi) with at[g] <= p (skips empty groups)
-__device__ __forceinline__ int group_of(const uint32_t* __restrict__ at, int lo, int hi, int64_t p) {
-  while (hi - lo > 1) {
-    int mid = (lo + hi) >> 1;
-    if (at[mid] <= p) lo = mid; else hi = mid;
-  }
-  return lo;
-}
-
 struct IndexLevels { uint2* table[kMaxN + 1]; uint32_t* positions[kMaxN + 1]; };
 
 // The groups that the sort takes: their ids, and where the positions of each begin when they are laid end to end.
-struct SortedGroups { const uint32_t* id; const uint32_t* at; int n; };
+// (null lists: all groups are, in their own order)
+struct SortedGroups {
+  const uint32_t *id, *at;
+  int n;
+  __device__ __forceinline__ int group(int l) const { return id ? int(id[l]) : l; }
+  __device__ __forceinline__ int64_t start(const int64_t* __restrict__ goff, int l) const { return at ? int64_t(at[l]) : goff[l]; }
+};
+
+// Largest l in [lo, hi) with start(l) <= i (skips empty groups)
+__device__ __forceinline__ int group_of(const SortedGroups& lg, const int64_t* __restrict__ goff, int lo, int hi, int64_t i) {
+  while (hi - lo > 1) {
+    int mid = (lo + hi) >> 1;
+    if (lg.start(goff, mid) <= i) lo = mid; else hi = mid;
+  }
+  return lo;
+}
 
 // Inserts the n-grams of the listed groups, for the n from n0 on, into their regions (cleared before) and leaves every (n,
 // position) with the number of its n-gram's slot among all those tables' (kNoSlot where none ends).  An entry is {key's low
@@ -106,14 +112,14 @@ insert_sorted_kernel(const int32_t* __restrict__ tok, const int64_t* __restrict_
   const int64_t i0 = int64_t(blockIdx.x) * kInsertBlock;
   const int n = n0 + blockIdx.y;
   unsigned long long* const table = reinterpret_cast<unsigned long long*>(lv.table[n]);
-  if (threadIdx.x < 2) s_g[threadIdx.x] = group_of(lg.at, 0, lg.n, min(M - 1, i0 + threadIdx.x * (kInsertBlock - 1)));
+  if (threadIdx.x < 2) s_g[threadIdx.x] = group_of(lg, goff, 0, lg.n, min(M - 1, i0 + threadIdx.x * (kInsertBlock - 1)));
   if (threadIdx.x == 0) s_ends = 0;
   __syncthreads();
   int mt = -1, ends = 0;
   for (int64_t i = i0 + threadIdx.x; i < min(M, i0 + kInsertBlock); i += kKeyThreads) {
-    const int l = s_g[0] == s_g[1] ? s_g[0] : group_of(lg.at, s_g[0], s_g[1] + 1, i), g = int(lg.id[l]);
-    const int64_t lo = goff[g], p = lo + (i - lg.at[l]);
-    bool valid = i - lg.at[l] >= n - 1;
+    const int l = s_g[0] == s_g[1] ? s_g[0] : group_of(lg, goff, s_g[0], s_g[1] + 1, i), g = lg.group(l);
+    const int64_t lo = goff[g], inside = i - lg.start(goff, l), p = lo + inside;
+    bool valid = inside >= n - 1;
     uint64_t key = key_begin(g, n);
     if (valid)
       for (int j = 0; j < n; ++j) {
@@ -191,8 +197,8 @@ index_runs_kernel(const uint32_t* __restrict__ slot, const uint32_t* __restrict_
 }
 
 __global__ void __launch_bounds__(kKeyThreads)
-clear_regions_kernel(const IndexLevels lv, int n_min, const int64_t* __restrict__ goff, SortedGroups lg) {
-  const int g = int(lg.id[blockIdx.y]);
+clear_regions_kernel(const IndexLevels lv, int n_min, const int64_t* __restrict__ goff, SortedGroups lg, int first) {
+  const int g = lg.group(first + blockIdx.y);
   const Region rg = region_of(goff[g], goff[g + 1], g);
   uint2* table = lv.table[n_min + blockIdx.z] + rg.base;
   for (uint32_t s = blockIdx.x * kKeyThreads + threadIdx.x; s < rg.slots; s += gridDim.x * kKeyThreads) table[s] = make_uint2(0xffffffffu, 0xffffffffu);
@@ -219,9 +225,9 @@ static_assert(group_smem(kGroupMax) <= 226 * 1024 && 2 * group_smem(kClassMax[1]
               kGroupMax + kGroupMax / 2 + kGroupMax / 8 + 4 < 65535, "");
 
 // A CTA per (group, n) costs about 15 ns of the device whatever the group's size, so tiny groups are sorted with the large ones
-// where they are so many that the sort's own launches (0.2 ms) do not show.  10 M tokens in groups of 5 / 20 / 100 / 200 / 250: a CTA
-// each 92 / 25.7 / 6.9 / 3.95 / 3.31 ms, sorted 15.2 / 5.6 / 3.5 / 3.24 / 3.13; 1 M tokens in groups of 20 / 100 / 200: 2.42 / 0.71 / 0.46,
-// sorted 0.70 / 0.49 / 0.46; 200 k tokens in groups of 20 / 100 (2000 of them): 0.54 / 0.21, sorted 0.25 / 0.21.
+// where they are so many that the sort's own launches (0.2 ms) do not show.  10 M tokens in groups of 2 / 5 / 10 / 100 / 200 / 250: a
+// CTA each 255 / 92 / 48 / 6.9 / 3.95 / 3.31 ms, sorted 11 / 5.4 / 4.0 / 3.1 / 3.24 / 3.13; 1 M tokens in groups of 10 / 100 / 200: 4.4 / 0.71 /
+// 0.46, sorted 0.53 / 0.45 / 0.46; 200 k tokens in groups of 20 / 100 (2000 of them): 0.54 / 0.21, sorted 0.25 / 0.21.
 constexpr int kTinyGroup = 256, kManyTiny = 4096;
 
 template <int THREADS, int CTAS>
@@ -1099,8 +1105,10 @@ LASER_API laser_status laser_pool_build(const int32_t* tokens, int64_t n_tokens,
   const int64_t least = n_tiny >= kManyTiny ? kTinyGroup : 0;    // of a group in shared memory
   if (least) { count[kClasses] -= n_tiny; sum[kClasses] -= tiny_sum; count[0] += n_tiny; sum[0] += tiny_sum; }
   // [n_groups] ids, [n_groups + 1] starts: of the groups in shared memory their runs' place, of the others their place among those
-  std::unique_ptr<uint32_t[]> lists(new (std::nothrow) uint32_t[size_t(n_groups) * 2 + 1]);
-  if (!lists) { set_error("no host memory for %d groups", n_groups); return LASER_ERR_OOM; }
+  // (none where all are sorted)
+  const bool listed = count[0] < n_groups;
+  std::unique_ptr<uint32_t[]> lists(listed ? new (std::nothrow) uint32_t[size_t(n_groups) * 2 + 1] : nullptr);
+  if (listed && !lists) { set_error("no host memory for %d groups", n_groups); return LASER_ERR_OOM; }
   uint32_t *const h_id = lists.get(), *const h_at = h_id + n_groups;
   int fill[kClasses + 1];
   int64_t place[kClasses + 1];
@@ -1108,14 +1116,14 @@ LASER_API laser_status laser_pool_build(const int32_t* tokens, int64_t n_tokens,
   int64_t n_small = 0;
   for (int c = 1, f = 0; c <= kClasses; ++c) { fill[c] = f; place[c] = n_small; f += count[c]; n_small += sum[c]; }
   fill[0] = n_small_groups; place[0] = 0;
-  for (int g = 0; g < n_groups; ++g) {
+  for (int g = 0; listed && g < n_groups; ++g) {
     const int64_t size = group_offsets[g + 1] - group_offsets[g];
     const int c = size < least ? 0 : class_of(size);
     h_id[fill[c]] = uint32_t(g);
     h_at[fill[c]++] = uint32_t(place[c]);
     place[c] += size;
   }
-  h_at[n_groups] = uint32_t(sum[0]);
+  if (listed) h_at[n_groups] = uint32_t(sum[0]);
   const int64_t n_sorted = sum[0];
   const size_t M = size_t(n_sorted);
 
@@ -1152,7 +1160,7 @@ LASER_API laser_status laser_pool_build(const int32_t* tokens, int64_t n_tokens,
     LASER_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, cub_bytes, kb, vb, int64_t(pairs), 0, slot_bits, stream));
   }
   constexpr size_t kCounters = (2 * kMaxN + 3) * 8;   // distinct keys per n, the largest token, n-grams of the sorted groups per n
-  const size_t b_lists = (size_t(n_groups) * 2 + 1) * 4;
+  const size_t b_lists = listed ? (size_t(n_groups) * 2 + 1) * 4 : 0;
   struct Tmp { void* p = nullptr; cudaStream_t s; ~Tmp() { pooled_free(p, s); } } tmp{nullptr, stream};
   LASER_TRY(pooled_alloc(&tmp.p, 4 * padded(pairs * 4) + padded(kCounters) + padded(b_lists) + cub_bytes + 256, stream));
   at = static_cast<uint8_t*>(tmp.p);
@@ -1165,7 +1173,7 @@ LASER_API laser_status laser_pool_build(const int32_t* tokens, int64_t n_tokens,
   const uint32_t* d_at = d_id + n_groups;
   int* max_tok = reinterpret_cast<int*>(counters + kMaxN + 1);
   unsigned long long* n_valid = counters + kMaxN + 2;
-  LASER_CUDA(cudaMemcpyAsync(d_id, lists.get(), b_lists, cudaMemcpyHostToDevice, stream));
+  if (listed) LASER_CUDA(cudaMemcpyAsync(d_id, lists.get(), b_lists, cudaMemcpyHostToDevice, stream));
   LASER_CUDA(cudaMemsetAsync(counters, 0, kCounters, stream));
   LASER_CUDA(cudaMemsetAsync(max_tok, 0xff, 4, stream));
   for (int n = n_min; n <= n_max; ++n) LASER_CUDA(cudaMemsetAsync(P->level[n].positions + N, 0xff, 32 * 4, stream));
@@ -1186,11 +1194,11 @@ LASER_API laser_status laser_pool_build(const int32_t* tokens, int64_t n_tokens,
     done += size_t(count[c]);
   }
   if (M) {
-    const SortedGroups lg{d_id + done, d_at + done, count[0]};
+    const SortedGroups lg{listed ? d_id + done : nullptr, listed ? d_at + done : nullptr, count[0]};
     const unsigned blocks = unsigned(ceil_div<size_t>(M, kInsertBlock));
     for (int l0 = 0; l0 < lg.n && !least; l0 += 65535)
       clear_regions_kernel<<<dim3(16, unsigned(std::min(lg.n - l0, 65535)), unsigned(levels)), kKeyThreads, 0, stream>>>(
-          lvs, n_min, P->group_offsets, SortedGroups{lg.id + l0, lg.at + l0, lg.n - l0});
+          lvs, n_min, P->group_offsets, lg, l0);
     count_launch();
     for (int n0 = n_min; n0 <= n_max; n0 += batch) {
       const int nb = std::min(batch, n_max - n0 + 1);

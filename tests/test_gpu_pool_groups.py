@@ -115,3 +115,21 @@ def test_many_tiny_groups(L):
         got = L.draft(pool, dev_i32(tails), dev_i32(lens), dev_i32(gids), L.make_params(K=6, n_min=1, n_max=n_max, min_draft=2, max_occ=max_occ))
         for g, w in zip(got, want):
             assert (g.cpu().numpy() == w).all()
+
+
+@pytest.mark.parametrize("sizes", ["tiny", "large"])
+def test_pools_of_sorted_groups_alone(L, sizes):
+    rng = np.random.default_rng(5)
+    sizes = rng.integers(0, 4, 70000) if sizes == "tiny" else np.array([16000, 15401, 20000])
+    N, n_max = int(sizes.sum()), 2
+    toks = rng.integers(0, 6, N).astype(np.int32)
+    offs = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    pool = L.pool_build(toks, offs, 1, n_max)
+    assert pool.info()["n_keys"] == _n_keys(toks, offs, 1, n_max)
+    gids = rng.integers(0, len(sizes), 200).astype(np.int32)
+    tails = rng.integers(0, 6, (200, n_max)).astype(np.int32)
+    lens = np.full(200, n_max, np.int32)
+    want = R.draft_batch(toks, offs, tails, lens, gids, 3, 1, n_max, 1, 64)
+    got = L.draft(pool, dev_i32(tails), dev_i32(lens), dev_i32(gids), L.make_params(K=3, n_min=1, n_max=n_max, max_occ=64))
+    for g, w in zip(got, want):
+        assert (g.cpu().numpy() == w).all()
