@@ -11,9 +11,10 @@
 // staged page, so a page is still read from HBM once per 32 rows.  Every mbarrier wait is bounded.
 //
 // With few (sequence, head) pairs the walk over one sequence's pages is a latency chain that leaves most SMs idle: up to eight
-// CTAs then take runs of eight pages in turn, and the one that finishes last sums the partial results (through L2, in the order
+// CTAs then take runs of twelve pages in turn, and the one that finishes last sums the partial results (through L2, in the order
 // of the CTAs).  A cluster and distributed shared memory would merge faster, but its CTAs must find their slots together, beside
 // those of the neighbouring kernels: a step of one short sequence lost 4 us a layer to that.
+#include <algorithm>
 #include <type_traits>
 
 #include "model.cuh"
@@ -25,11 +26,13 @@ namespace {
 using bf16 = __nv_bfloat16;
 constexpr int kConsumers = 4;
 constexpr int kAttnThreads = (kConsumers + 1) * 32;
-constexpr int kStages = 4;   // a multiple of kConsumers: stage s always serves warp s % 4
+// Pages in the ring: a multiple of kConsumers, as stage s always serves warp s % 4.  A CTA's walk over its pages is paced by the bytes
+// that it has in flight, so launches whose CTAs fit three an SM take the deep ring (with four, 16 sequences lose 5 % to three).
+constexpr int stages_of(bool deep) { return deep ? 8 : 4; }
 constexpr int kMaxPageSplits = 8;  // CTAs that share a sequence's pages
 constexpr int kSplitFrom = 16;      // pages from which a split pays for the merge (about 3 us, ten pages of one CTA's walk),
-constexpr int kRunPages = 8;        // and pages of a run (a multiple of kStages: a warp's pages stay the same ones)
-constexpr int kCtasPerSm = 4;  // registers and shared memory are sized for four resident CTAs
+constexpr int kRunPages = 12;       // and pages of a run (a multiple of kConsumers: a warp's pages stay the same ones)
+constexpr int kCtasPerSm = 4;  // registers and shared memory are sized for four resident CTAs, or three with the deep ring
 
 __device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
   asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
@@ -50,11 +53,11 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// SP: the pages are split over `splits` CTAs (grid x = sequences x splits).  PR (precise mode): the queries come in fp32 (qf) and
+// SP: the pages are split over `splits` CTAs (grid x = sequences x splits).  DEEP: eight pages in the ring.  PR (precise mode): the queries come in fp32 (qf) and
 // enter the score MMA as hi + lo bf16 pairs, the probabilities enter the value MMA as pairs as well, and the output is written
 // as pairs ([hi | lo] rows of 2 H DH).
-template <int DH, int TPC, bool PR, bool SP>
-__global__ void __launch_bounds__(kAttnThreads, PR ? 3 : kCtasPerSm)
+template <int DH, int TPC, bool PR, bool SP, bool DEEP>
+__global__ void __launch_bounds__(kAttnThreads, PR && TPC == 2 && DEEP ? 2 : PR || DEEP ? 3 : kCtasPerSm)
 attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* q, const float* qf,
                   const int32_t* __restrict__ seq_ids, const int32_t* __restrict__ row_ctx,
                   const int32_t* __restrict__ row_n, int Rs, int H, int Hkv,
@@ -62,13 +65,14 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* q, cons
                   bf16* __restrict__ out, int32_t* __restrict__ status,
                   const unsigned long long* row_mask, int fresh, int splits,
                   float* __restrict__ part, int32_t* __restrict__ arrived) {
+  constexpr int ST = stages_of(DEEP);
   constexpr int kPartFloats = 16 * TPC * (DH + 2);   // SP: a partial result: O [rows][DH], max [rows], sum [rows]
   constexpr int HALVES = DH / 64;                 // 64-element (128-byte) column blocks per row
   constexpr int SUB = 16 * 128;                   // bytes of one 16-token x 64-element sub-tile
   constexpr int STAGE = 2 * HALVES * SUB;         // K then V
   constexpr int QLD = DH + 8;                     // padded row of the Q tile (elements)
   extern __shared__ uint8_t smem_raw[];
-  __shared__ uint64_t full_bar[kStages], empty_bar[kStages];
+  __shared__ uint64_t full_bar[ST], empty_bar[ST];
   __shared__ float s_m[kConsumers][16], s_l[kConsumers][16], s_wgt[kConsumers][16];
   __shared__ int abort_flag;
   __shared__ int s_last;
@@ -104,8 +108,8 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* q, cons
   const uint32_t raw = smem_u32(smem_raw);
   const uint32_t tiles = (raw + 1023u) & ~1023u;
   uint8_t* tiles_ptr = smem_raw + (tiles - raw);
-  const uint32_t q_smem = tiles + kStages * STAGE;
-  bf16* q_ptr = reinterpret_cast<bf16*>(tiles_ptr + kStages * STAGE);
+  const uint32_t q_smem = tiles + ST * STAGE;
+  bf16* q_ptr = reinterpret_cast<bf16*>(tiles_ptr + ST * STAGE);
   const int n_keys = ctx + (row_mask ? nr : min(nr, cta_row0 + 16 * TPC));   // chain: no row here sees a later one
   const int all_pg = (n_keys + 15) >> 4;
   // SP: run j of the pages belongs to CTA j % splits.  Which pages a CTA sums follows from their numbers alone, neither from the
@@ -125,7 +129,7 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* q, cons
 
   if (tid == 0) {
     abort_flag = 0;
-    for (int s = 0; s < kStages; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), TPC); }
+    for (int s = 0; s < ST; ++s) { mbar_init(smem_u32(&full_bar[s]), 1); mbar_init(smem_u32(&empty_bar[s]), TPC); }
     mbar_fence_init();
     tma_prefetch_map(&kvmap);
   }
@@ -135,14 +139,14 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* q, cons
     if (lane == 0) {
       const int32_t* pt = page_table + size_t(seq_ids[b]) * pages_per_seq;
       // whole pages of older tokens that fit the ring (none where the kernel before may have written them)
-      const int n_early = fresh ? 0 : min(pages_below(min(ctx >> 4, all_pg)), kStages);
+      const int n_early = fresh ? 0 : min(pages_below(min(ctx >> 4, all_pg)), ST);
       bool ok = true;
       int issued = 0;
       const uint64_t kv_policy = make_policy_evict_first();   // a page is read once per step
       for (int p = 0; p < n_pg && ok; ++p) {
-        const int s = p % kStages;
+        const int s = p % ST;
         if (p == n_early) asm volatile("griddepcontrol.wait;" ::: "memory");   // from here on: pages the kernel before may write
-        if (p >= kStages) ok = mbar_wait(smem_u32(&empty_bar[s]), ((p / kStages) - 1) & 1, &abort_flag);
+        if (p >= ST) ok = mbar_wait(smem_u32(&empty_bar[s]), ((p / ST) - 1) & 1, &abort_flag);
         if (!ok) break;
         const uint32_t bar = smem_u32(&full_bar[s]);
         const uint32_t dst = tiles + uint32_t(s) * STAGE;
@@ -158,7 +162,7 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* q, cons
         issued = p + 1;
       }
       if (!ok)
-        for (int p = max(0, issued - kStages); p < issued; ++p) mbar_drain(smem_u32(&full_bar[p % kStages]), (p / kStages) & 1);
+        for (int p = max(0, issued - ST); p < issued; ++p) mbar_drain(smem_u32(&full_bar[p % ST]), (p / ST) & 1);
     }
     return;
   }
@@ -216,8 +220,8 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* q, cons
   const unsigned long long vis1 = row_mask ? row_mask[size_t(b) * Rs + min(row0 + g + 8, nr - 1)] : 0ull;
 
   for (int p = pgrp; p < n_pg; p += NPG) {
-    const int s = p % kStages;
-    if (!mbar_wait(smem_u32(&full_bar[s]), (p / kStages) & 1, &abort_flag)) break;
+    const int s = p % ST;
+    if (!mbar_wait(smem_u32(&full_bar[s]), (p / ST) & 1, &abort_flag)) break;
     const uint32_t kbase = tiles + uint32_t(s) * STAGE, vbase = kbase + HALVES * SUB;
     float sc[2][4];
 #pragma unroll
@@ -422,18 +426,21 @@ laser_status attention_tma_launch(laser_model* m, laser_kv* kv, int layer, const
   const int64_t rows_per_layer = int64_t(kv->n_pages) * 2 * Hkv * 16;
   const int layer_row0 = int(rows_per_layer * layer);
   const int tiles = ceil_div(Rs, 16), tpc = tiles > 1 ? 2 : 1;   // row tiles of a sequence; tiles per CTA
-  // Page splits while the grid stays at what the SMs hold at once, where the cache can hold pages enough; what a sequence has
-  // is known on the device alone, and CTAs that find no run to take leave.  7B, 6 layers, steps of 9 rows, 128 / 256 / 512 / 1000
-  // cached tokens in a cache of 256 pages a sequence: one sequence 526 / 544 / 580 / 649 us unsplit, 543 / 546 / 552 / 563 in
-  // eight; two 551 / 569 / 606 / 679, in eight 569 / 577 / 583 / 593; four 612 / 630 / 665 / 734, in four 636 / 643 / 660 / 686; eight
-  // 650 / 670 / 705 / 787, in two 660 / 672 / 700 / 755.  The merge costs 3 us a layer, which texts of 9 to 16 pages do not win
-  // back; a cache that holds no more is not split.  Runs of 12 or 16 pages: one sequence of 512 / 1000 tokens 560 / 567, 567 / 573.
-  // (A prefill's chunks are many.)
-  const int units = B * H * ceil_div(tiles, tpc), most = kv->pages_per_seq;
-  const int splits = fresh || most < kSplitFrom ? 1 : units * 8 <= kAttnSplitCtas ? 8 : most < 2 * kSplitFrom ? 1 :
-                     units * 4 <= kAttnSplitCtas ? 4 : units * 2 <= kAttnSplitCtas ? 2 : 1;
+  // Page splits while the CTAs stay resident, where the cache can hold pages enough; what a sequence has is known on the device
+  // alone, and CTAs that find no run to take leave.  7B, 6 layers, steps of 9 rows, 128 / 256 / 512 / 1000 cached tokens in a cache of 256
+  // pages a sequence, us; unsplit with a ring of four: one sequence 526 / 544 / 580 / 649, two 551 / 569 / 606 / 679, four 612 / 630 / 665 /
+  // 734, eight 645 / 664 / 703 / 787; here, in eight 516 / 540 / 545 / 553, in six 539 / 569 / 576 / 581, in three 605 / 635 / 648 / 675, unsplit
+  // with the deep ring 640 / 656 / 680 / 736.  A ring of four and runs of eight pages: one sequence 543 / 545 / 551 / 563, four 635 / 643 /
+  // 659 / 687: the merge costs 3 us a layer, which a text of two runs does not win back.  Runs of 8 or 16 pages with the deep ring: one
+  // sequence 535 / 539 / 546 / 553, 518 / 551 / 557 / 565.  Caches that hold less than 32 pages are split for up to 74 pairs of sequence
+  // and head (256 tokens in such a cache: two sequences 584 unsplit, 575 in six; four 623 unsplit, 644 in three).  (A prefill's
+  // chunks are many.)
   const bool pr = m->precise;
-  const size_t smem = 1024 + size_t(kStages) * (2 * (dh / 64) * 16 * 128) + size_t(16) * tpc * (dh + 8) * 2 * (pr ? 2 : 1);
+  const int units = B * H * ceil_div(tiles, tpc), most = kv->pages_per_seq;
+  const int resident = pr && tpc == 2 ? kAttnSplitCtas / 3 * 2 : kAttnSplitCtas;   // (hi + lo queries of 32 rows take more shared memory)
+  const bool deep = !fresh && units <= resident;
+  const int splits = !deep || most < (units <= kAttnSplitCtas / 6 ? kSplitFrom : 2 * kSplitFrom) ? 1 : std::min(kMaxPageSplits, resident / units);
+  const size_t smem = 1024 + size_t(stages_of(deep)) * (2 * (dh / 64) * 16 * 128) + size_t(16) * tpc * (dh + 8) * 2 * (pr ? 2 : 1);
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(unsigned(B * splits), unsigned(H), unsigned(ceil_div(tiles, tpc)));
   cfg.blockDim = dim3(kAttnThreads, 1, 1);
@@ -457,7 +464,7 @@ laser_status attention_tma_launch(laser_model* m, laser_kv* kv, int layer, const
   auto by_split = [&](auto dh_tag, auto tpc_tag, auto pr_tag) -> laser_status {
     constexpr int D = decltype(dh_tag)::value, T = decltype(tpc_tag)::value;
     constexpr bool P = decltype(pr_tag)::value;
-    return splits > 1 ? launch(attn_paged_kernel<D, T, P, true>) : launch(attn_paged_kernel<D, T, P, false>);
+    return splits > 1 ? launch(attn_paged_kernel<D, T, P, true, true>) : deep ? launch(attn_paged_kernel<D, T, P, false, true>) : launch(attn_paged_kernel<D, T, P, false, false>);
   };
   auto by_mode = [&](auto dh_tag, auto tpc_tag) { return pr ? by_split(dh_tag, tpc_tag, std::true_type{}) : by_split(dh_tag, tpc_tag, std::false_type{}); };
   using std::integral_constant;

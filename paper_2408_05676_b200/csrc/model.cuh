@@ -60,7 +60,7 @@ namespace laser {
 // (7B, 4 layers: 3.6 us a row at 144 rows, 1.6 us at 1024).  16 prompts of 256 .. 1024 tokens and 32 new tokens each, 7B: 456 -> 233
 // ms against passes of 128 rows of one prompt.
 constexpr int kPrefillRows = 1024;
-constexpr int kAttnSplitCtas = 512; // most CTAs of an attention launch that splits pages
+constexpr int kAttnSplitCtas = 3 * 148; // most CTAs of an attention launch that splits pages: three an SM
 constexpr int kPrefillChunk = 32;   // rows that share each staged K/V page in the attention kernel
 
 void gen_host_free(laser_model* m);
