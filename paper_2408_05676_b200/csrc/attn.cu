@@ -53,9 +53,9 @@ __device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&v);
 }
 
-// SP: the pages are split over `splits` CTAs (grid x = sequences x splits).  DEEP: eight pages in the ring.  PR (precise mode): the queries come in fp32 (qf) and
-// enter the score MMA as hi + lo bf16 pairs, the probabilities enter the value MMA as pairs as well, and the output is written
-// as pairs ([hi | lo] rows of 2 H DH).
+// SP: the pages are split over `splits` CTAs (grid x = sequences x splits).  DEEP: eight pages in the ring.  PR (precise mode): the
+// queries come in fp32 (qf) and enter the score MMA as hi + lo bf16 pairs, the probabilities enter the value MMA as pairs as well,
+// and the output is written as pairs ([hi | lo] rows of 2 H DH).
 template <int DH, int TPC, bool PR, bool SP, bool DEEP>
 __global__ void __launch_bounds__(kAttnThreads, PR && TPC == 2 && DEEP ? 2 : PR || DEEP ? 3 : kCtasPerSm)
 attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* q, const float* qf,
