@@ -613,6 +613,8 @@ static laser_status verify_impl(laser_model* m, laser_kv* kv, const int32_t* seq
   int norm_tiles = 1;  // tile planes holding the sums of squares of the current residual
   for (int l = 0; l < c.n_layers; ++l) {
     __nv_bfloat16* pages_l = kv->pages + size_t(l) * kv->layer_elems();
+    // Of the last layer a prompt leaves its keys and values alone: their projections are all that it runs.
+    const bool kv_alone = start && l == c.n_layers - 1;
     {  // QKV projection of the normalised residual; rotary embedding; Q store; cache write
       GemmEpilogue e = base;
       e.sumsq_in = m->sumsq; e.sumsq_in_tiles = norm_tiles;
@@ -621,8 +623,10 @@ static laser_status verify_impl(laser_model* m, laser_kv* kv, const int32_t* seq
       e.H = H; e.Hkv = Hkv; e.dh = dh;
       if (m->precise) { e.a_lo_off = d; e.qf = m->qf; }
       ProfScope ps(m, 0, stream);
-      LASER_TRY(gemm_fused(m, m->xn, m->wqkv[l], Rp, m->dqkv, d, EPI_QKV, e, stream));
+      if (kv_alone) e.H = 0;   // (no feature is a query's)
+      LASER_TRY(gemm_fused(m, m->xn, m->wqkv[l] + (kv_alone ? size_t(m->dq) * d : 0), Rp, kv_alone ? 2 * m->dkv : m->dqkv, d, EPI_QKV, e, stream));
     }
+    if (kv_alone) break;
     {
       ProfScope ps(m, 1, stream);
       if (use_tma_attn) {
