@@ -17,6 +17,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "mma.cuh"
 #include "model.cuh"
 #include "tma.cuh"
 
@@ -33,25 +34,6 @@ constexpr int kMaxPageSplits = 8;  // CTAs that share a sequence's pages
 constexpr int kSplitFrom = 16;      // pages from which a split pays for the merge (about 3 us, ten pages of one CTA's walk),
 constexpr int kRunPages = 12;       // and pages of a run (a multiple of kConsumers: a warp's pages stay the same ones)
 constexpr int kCtasPerSm = 4;  // registers and shared memory are sized for four resident CTAs, or three with the deep ring
-
-__device__ __forceinline__ void ldsm_x4(uint32_t (&r)[4], uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void ldsm_x4_t(uint32_t (&r)[4], uint32_t addr) {
-  asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0,%1,%2,%3}, [%4];"
-               : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(addr));
-}
-__device__ __forceinline__ void mma16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
-  asm volatile(
-      "mma.sync.aligned.m16n8k16.row.col.f32.bf16.bf16.f32 {%0,%1,%2,%3}, {%4,%5,%6,%7}, {%8,%9}, {%0,%1,%2,%3};"
-      : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
-      : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
-}
-__device__ __forceinline__ uint32_t pack_bf16(float lo, float hi) {
-  __nv_bfloat162 v = __floats2bfloat162_rn(lo, hi);
-  return *reinterpret_cast<uint32_t*>(&v);
-}
 
 // SP: the pages are split over `splits` CTAs (grid x = sequences x splits).  DEEP: eight pages in the ring.  PR (precise mode): the
 // queries come in fp32 (qf) and enter the score MMA as hi + lo bf16 pairs, the probabilities enter the value MMA as pairs as well,

@@ -145,6 +145,32 @@ struct DevBuf {
   }
 };
 
+// A prompt's tokens start .. start + rows - 1, and the chunks of a pass in the order in which attention takes them: kPrefillShare
+// consecutive chunks of a prompt at a time, those that see most keys first (its CTAs differ by the keys that they walk, and one that
+// starts last and walks longest is what the launch would end with).  What a prompt has beyond a multiple of kPrefillShare is the
+// beginning of its part of the pass, which sees least, and goes behind all others.
+struct Chunk { int prompt, start, rows; };
+void order_pass(Chunk* pass, int n) {
+  struct Run { int first, n, keys; };
+  std::vector<Run> runs;
+  for (int c = 0; c < n;) {
+    int e = c;
+    while (e < n && pass[e].prompt == pass[c].prompt) ++e;
+    for (int x = c, take; x < e; x += take) {
+      take = (e - x) % kPrefillShare ? (e - x) % kPrefillShare : kPrefillShare;
+      runs.push_back(Run{x, take, pass[x + take - 1].start + pass[x + take - 1].rows});
+    }
+    c = e;
+  }
+  std::stable_sort(runs.begin(), runs.end(), [](const Run& a, const Run& b) {
+    return (a.n == kPrefillShare) != (b.n == kPrefillShare) ? a.n == kPrefillShare : a.keys > b.keys;
+  });
+  std::vector<Chunk> out;
+  out.reserve(size_t(n));
+  for (const Run& r : runs) out.insert(out.end(), pass + r.first, pass + r.first + r.n);
+  std::copy(out.begin(), out.end(), pass);
+}
+
 constexpr int kInFlight = 2;   // steps queued beyond the last whose report has been read
 constexpr int kSlots = 4;      // reports
 
@@ -257,22 +283,27 @@ LASER_API laser_status laser_generate(laser_model* m, laser_kv* kv, const laser_
   memset(h + at_out, 0xff, (n_result - at_out) * 4);
   memset(h + at_done, 0, size_t(B) * 4);
   int32_t *h_pre = h + at_pre, *h_slot = h_pre + size_t(n_chunks) * kPrefillChunk, *h_start = h_slot + n_chunks, *h_rows = h_start + n_chunks;
-  for (int b = 0, c = 0; b < B; ++b) {
-    const int32_t* prompt = prompts + prompt_offsets[b];
+  std::vector<Chunk> chunks;
+  chunks.reserve(size_t(n_chunks));
+  for (int b = 0; b < B; ++b) {
     const int len = int(prompt_offsets[b + 1] - prompt_offsets[b]);
     h[at_len + b] = len;
     h[at_ids + b] = b;
     h[at_gid + b] = pool ? group_id[b] : -1;
     int32_t* text = h + at_text + size_t(b) * max_total;
-    memcpy(text, prompt, size_t(len) * 4);
+    memcpy(text, prompts + prompt_offsets[b], size_t(len) * 4);
     memset(text + len, 0, size_t(max_total - len) * 4);
-    for (int p0 = 0; p0 < len - 1; p0 += kPrefillChunk, ++c) {
-      const int rows = std::min(kPrefillChunk, len - 1 - p0);
-      int32_t* chunk = h_pre + size_t(c) * kPrefillChunk;
-      memcpy(chunk, prompt + p0, size_t(rows) * 4);
-      std::fill(chunk + rows, chunk + kPrefillChunk, -1);
-      h_slot[c] = b; h_start[c] = p0; h_rows[c] = rows;
-    }
+    for (int p0 = 0; p0 < len - 1; p0 += kPrefillChunk) chunks.push_back(Chunk{b, p0, std::min(kPrefillChunk, len - 1 - p0)});
+  }
+  std::vector<int> passes;      // as many chunks each as the workspace holds
+  for (int left = n_chunks; left > 0; left -= passes.back()) passes.push_back(std::min(left, m->R_cap / kPrefillChunk));
+  for (int c0 = 0, i = 0; c0 < n_chunks; c0 += passes[size_t(i++)]) order_pass(chunks.data() + c0, passes[size_t(i)]);
+  for (int c = 0; c < n_chunks; ++c) {
+    const Chunk& x = chunks[size_t(c)];
+    int32_t* row = h_pre + size_t(c) * kPrefillChunk;
+    memcpy(row, prompts + prompt_offsets[x.prompt] + x.start, size_t(x.rows) * 4);
+    std::fill(row + x.rows, row + kPrefillChunk, -1);
+    h_slot[c] = x.prompt; h_start[c] = x.start; h_rows[c] = x.rows;
   }
 
   DevBuf buf;
@@ -308,12 +339,13 @@ LASER_API laser_status laser_generate(laser_model* m, laser_kv* kv, const laser_
   LASER_CUDA(cudaMemcpyAsync(init, h, words * 4, cudaMemcpyHostToDevice, stream));
   LASER_CUDA(cudaEventRecord(host.uploaded, stream));
   LASER_CUDA(cudaEventRecord(host.begin, stream));
-  // As many chunks a pass as the workspace holds, of whatever prompts; a prompt's chunks come in order, in one pass or several.
+  // A pass takes chunks of whatever prompts; what a prompt has in several passes comes in order.
   const int32_t *pre = init + at_pre, *slot = pre + size_t(n_chunks) * kPrefillChunk, *start = slot + n_chunks, *rows = start + n_chunks;
-  const int pass = m->R_cap / kPrefillChunk;
-  for (int c0 = 0, n_pass = 0; c0 < n_chunks; c0 += pass, ++n_pass) {
-    LASER_TRY(prefill_chunks(m, kv, slot + c0, start + c0, pre + size_t(c0) * kPrefillChunk, rows + c0, std::min(pass, n_chunks - c0), stream));
-    if ((n_pass & 15) == 15) LASER_TRY(laser_check(m, stream));   // do not keep launching after a device-side error
+  int c0 = 0, n_pass = 0;
+  for (const int pass : passes) {
+    LASER_TRY(prefill_chunks(m, kv, slot + c0, start + c0, pre + size_t(c0) * kPrefillChunk, rows + c0, pass, stream));
+    c0 += pass;
+    if ((n_pass++ & 15) == 15) LASER_TRY(laser_check(m, stream));   // do not keep launching after a device-side error
   }
   LASER_CUDA(cudaEventRecord(host.prefilled, stream));
   LASER_CUDA(launch_overlapped(step_kernel, dim3(1), kStepThreads, 0, stream, g, 1, 0, n_rows, n_accept, out_tokens, n_out, host.report, 0u));

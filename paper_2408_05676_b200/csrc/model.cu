@@ -629,7 +629,9 @@ static laser_status verify_impl(laser_model* m, laser_kv* kv, const int32_t* seq
     if (kv_alone) break;
     {
       ProfScope ps(m, 1, stream);
-      if (use_tma_attn) {
+      if (use_tma_attn && start && !m->precise) {
+        LASER_TRY(attention_prefill_launch(m, kv, l, seq_ids, B, stream));
+      } else if (use_tma_attn) {
         LASER_TRY(attention_tma_launch(m, kv, l, seq_ids, B, Rs, tree, start != nullptr, stream));
       } else {
         attention_kernel<<<dim3(B, H), 128, attn_smem, stream>>>(m->q, m->qf, m->precise ? 1 : 0, seq_ids, m->row_ctx, m->row_n, Rs, H, Hkv, dh,

@@ -61,7 +61,8 @@ namespace laser {
 // ms against passes of 128 rows of one prompt.
 constexpr int kPrefillRows = 1024;
 constexpr int kAttnSplitCtas = 3 * 148; // most CTAs of an attention launch that splits pages: three an SM
-constexpr int kPrefillChunk = 32;   // rows that share each staged K/V page in the attention kernel
+constexpr int kPrefillChunk = 32;   // rows of a chunk of a prompt
+constexpr int kPrefillShare = 4;    // consecutive chunks that share each staged K/V page in the attention kernel
 
 void gen_host_free(laser_model* m);
 
@@ -151,6 +152,8 @@ bool attention_tma_supported(const laser_model* m, const laser_kv* kv);
 // fresh: pages below a sequence's row_ctx may be written by the kernel right before (prompt chunks of one prefill pass).
 laser_status attention_tma_launch(laser_model* m, laser_kv* kv, int layer, const int32_t* seq_ids, int B, int Rs, bool tree, bool fresh,
                                   cudaStream_t stream);
+// The same for the chunks of a prefill pass (default mode; head_dim 64 or 128 as above).
+laser_status attention_prefill_launch(laser_model* m, laser_kv* kv, int layer, const int32_t* seq_ids, int n_chunks, cudaStream_t stream);
 
 // Prompt processing: the verify forward without the LM head over chunks of up to kPrefillChunk prompt tokens.  Chunk i is
 // n_rows[i] tokens of cache slot seq_ids[i] from position start[i] on; chunks of one prompt may share a call, in any order:
