@@ -295,8 +295,7 @@ LASER_API laser_status laser_generate(laser_model* m, laser_kv* kv, const laser_
     memset(text + len, 0, size_t(max_total - len) * 4);
     for (int p0 = 0; p0 < len - 1; p0 += kPrefillChunk) chunks.push_back(Chunk{b, p0, std::min(kPrefillChunk, len - 1 - p0)});
   }
-  std::vector<int> passes;      // as many chunks each as the workspace holds
-  for (int left = n_chunks; left > 0; left -= passes.back()) passes.push_back(std::min(left, m->R_cap / kPrefillChunk));
+  const std::vector<int> passes = prefill_passes(m, n_chunks);
   for (int c0 = 0, i = 0; c0 < n_chunks; c0 += passes[size_t(i++)]) order_pass(chunks.data() + c0, passes[size_t(i)]);
   for (int c = 0; c < n_chunks; ++c) {
     const Chunk& x = chunks[size_t(c)];

@@ -44,6 +44,7 @@ struct laser_model {
   float* pair_scratch = nullptr;   // partial sums of the contractions for many rows (gemm_pair.cu), and the cut tiles' state
   int32_t* pair_state = nullptr;
   int peer_cycles = 200000;        // how long they wait for each other: about 0.1 ms, many times the skew between pairs that are running
+  std::vector<double> prefill_us;  // [chunks] what a prefill pass of that many chunks is estimated to take
   void* gemm_state = nullptr;      // tensor-map cache of the tensor-core GEMM
   void* gen_buf = nullptr;         // work buffers of laser_generate, kept between calls (in `owned`)
   size_t gen_bytes = 0;
@@ -57,14 +58,17 @@ struct laser_model {
 namespace laser {
 
 // A prefill pass runs the contractions over up to this many prompt tokens: enough rows for the tensor pipe to be the bound
-// (7B, 4 layers: 3.6 us a row at 144 rows, 1.6 us at 1024).  16 prompts of 256 .. 1024 tokens and 32 new tokens each, 7B: 456 -> 233
-// ms against passes of 128 rows of one prompt.
-constexpr int kPrefillRows = 1024;
+// (7B, 4 layers: 3.6 us a row at 144 rows, 1.6 us at 1024), and to fill whole waves of tiles: 16 tiles of 256 weight rows, as the O and down
+// projections of 4096 features have, leave 14 % of the last wave idle at 1024 rows (64 of 74 pairs), 3 % at 2304 (144 of 148).
+constexpr int kPrefillRows = 2304;
 constexpr int kAttnSplitCtas = 3 * 148; // most CTAs of an attention launch that splits pages: three an SM
 constexpr int kPrefillChunk = 32;   // rows of a chunk of a prompt
 constexpr int kPrefillShare = 4;    // consecutive chunks that share each staged K/V page in the attention kernel
 
 void gen_host_free(laser_model* m);
+
+// Chunks of each pass of a prefill of n_chunks, in order: the division whose estimated time is least.
+std::vector<int> prefill_passes(const laser_model* m, int n_chunks);
 
 // The entry points of the same names; `stamp` (optional): the device clock at the end of the rows' making, at the start of the verdict.
 laser_status make_rows(const int32_t* last_token, const int32_t* draft, const int32_t* draft_len, int32_t B, int32_t K, int32_t* tokens,
