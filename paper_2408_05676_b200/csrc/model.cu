@@ -365,14 +365,6 @@ LASER_API laser_status laser_model_create(const laser_model_cfg* cfg, const lase
     m->ffn_norm.push_back(static_cast<const bf16*>(w->ffn_norm[l]));
   }
   m->R_cap = std::max(m->R_pad, kPrefillRows);
-  m->prefill_us.assign(size_t(m->R_cap / kPrefillChunk) + 1, 0.0);
-  for (int c = 1; c < int(m->prefill_us.size()); ++c) {
-    const int rows = c * kPrefillChunk;
-    const bool pairs = cfg->precise != 0;
-    constexpr double kEnds = 4 * 2.5 + 15;   // between launches, and what of the attention does not grow with the rows
-    m->prefill_us[c] = kEnds + gemm_pair_shape(rows, m->dqkv, d, EPI_QKV, pairs).us + gemm_pair_shape(rows, d, m->dq, EPI_RESID, pairs).us +
-                       gemm_pair_shape(rows, 2 * f, d, EPI_SWIGLU, pairs).us + gemm_pair_shape(rows, d, f, EPI_RESID, pairs).us;
-  }
   m->precise = cfg->precise != 0;
   const size_t Rp = size_t(m->R_cap), pair = m->precise ? 2 : 1;     // pair: hi + lo parts side by side in a row
   const size_t groups = std::max<size_t>(cfg->max_batch, Rp / kPrefillChunk);
@@ -565,8 +557,14 @@ LASER_API laser_status laser_verify_step_tree(laser_model* m, laser_kv* kv, cons
 namespace laser {
 // Passes as large as the workspace are not always the best: what a pass takes goes up in steps, by waves of tiles, and so does what
 // is left for the last.  7B, 10 k prompt tokens in passes of up to 1024 / 1536 / 2304 rows: 133 / 121 / 114 ms.
-std::vector<int> prefill_passes(const laser_model* m, int n_chunks) {
-  const int most = int(m->prefill_us.size()) - 1;
+std::vector<int> prefill_passes(laser_model* m, int n_chunks) {
+  const int most = std::min(n_chunks, m->R_cap / kPrefillChunk), d = m->cfg.d_model, f = m->cfg.d_ffn;
+  for (int c = int(m->prefill_us.size()); c <= most; ++c) {
+    const int rows = c * kPrefillChunk;
+    constexpr double kEnds = 4 * 2.5 + 15;   // between launches, and what of the attention does not grow with the rows
+    m->prefill_us.push_back(kEnds + gemm_pair_shape(rows, m->dqkv, d, EPI_QKV, m->precise).us + gemm_pair_shape(rows, d, m->dq, EPI_RESID, m->precise).us +
+                            gemm_pair_shape(rows, 2 * f, d, EPI_SWIGLU, m->precise).us + gemm_pair_shape(rows, d, f, EPI_RESID, m->precise).us);
+  }
   std::vector<double> us(size_t(n_chunks) + 1, 0.0);     // of the first i chunks
   std::vector<int> last(size_t(n_chunks) + 1, 0);        // their last pass
   for (int i = 1; i <= n_chunks; ++i) {

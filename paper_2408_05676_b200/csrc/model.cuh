@@ -44,7 +44,7 @@ struct laser_model {
   float* pair_scratch = nullptr;   // partial sums of the contractions for many rows (gemm_pair.cu), and the cut tiles' state
   int32_t* pair_state = nullptr;
   int peer_cycles = 200000;        // how long they wait for each other: about 0.1 ms, many times the skew between pairs that are running
-  std::vector<double> prefill_us;  // [chunks] what a prefill pass of that many chunks is estimated to take
+  std::vector<double> prefill_us{0.0};  // [chunks] what a layer of a prefill pass of that many chunks is estimated to take, as far as needed so far
   void* gemm_state = nullptr;      // tensor-map cache of the tensor-core GEMM
   void* gen_buf = nullptr;         // work buffers of laser_generate, kept between calls (in `owned`)
   size_t gen_bytes = 0;
@@ -68,7 +68,7 @@ constexpr int kPrefillShare = 4;    // consecutive chunks that share each staged
 void gen_host_free(laser_model* m);
 
 // Chunks of each pass of a prefill of n_chunks, in order: the division whose estimated time is least.
-std::vector<int> prefill_passes(const laser_model* m, int n_chunks);
+std::vector<int> prefill_passes(laser_model* m, int n_chunks);
 
 // The entry points of the same names; `stamp` (optional): the device clock at the end of the rows' making, at the start of the verdict.
 laser_status make_rows(const int32_t* last_token, const int32_t* draft, const int32_t* draft_len, int32_t B, int32_t K, int32_t* tokens,
