@@ -400,7 +400,7 @@ struct DraftArgs {
   const int32_t* tails; const int32_t* tail_len; const int32_t* group_id;
   int B, K, n_min, n_max, min_draft, max_occ;
   int32_t* draft; int32_t* draft_len; int32_t* match_n;
-  int32_t* work;       // large-run path: kWorkHead counters (zero between calls), then (query, suffix length) pairs
+  int32_t* work;       // large-run path: WORK_HEAD counters (zero between calls), then the items
   int64_t n_positions;
 };
 
@@ -436,13 +436,13 @@ __device__ __forceinline__ bool is_occurrence(const int32_t* __restrict__ tok, i
 }
 
 // The group's occurrences of the n tail tokens, ascending, behind the n_occ that s_occ[64] already holds, until there are
-// `cap` (more may be counted, 64 are kept).  All lanes of a warp.
+// `cap` (more may be counted, 64 are kept).  All lanes of a warp.  start: of their run, if there is one.  off: slots past the home one
+// that are known not to be the key's.
 __device__ __forceinline__ int gather_occurrences(const PoolView& pv, int64_t lo, int64_t hi, const int32_t* tail, int n, uint64_t key,
-                                                  int g, int lane, uint32_t* s_occ, int n_occ, int cap) {
+                                                  int g, int lane, uint32_t* s_occ, int n_occ, int cap, uint32_t& start, uint32_t off = 0) {
   const int before = n_occ;
   const Region rg = region_of(lo, hi, g);
-  uint32_t start;
-  for (uint32_t off = 0; n_occ < cap && n_occ == before && probe(pv.table[n] + rg.base, rg.slots, key, lane, off, start); ++off) {
+  for (; n_occ < cap && n_occ == before && probe(pv.table[n] + rg.base, rg.slots, key, lane, off, start); ++off) {
     for (uint32_t base = start; n_occ < cap; base += 32) {   // (the array is padded: lanes past its end read marked padding)
       const uint32_t v = pv.positions[n][base + lane];
       const unsigned ends = __ballot_sync(0xffffffffu, (v & kRunEnd) != 0);
@@ -461,14 +461,15 @@ __device__ __forceinline__ int gather_occurrences(const PoolView& pv, int64_t lo
 // The greedy highest-frequency walk over up to 64 occurrences, two a lane (e0, e1; alive a0, a1), from depth `len` on (their
 // tokens up to there agree): at every depth the most frequent next token, ties to the smallest, and the occurrences that
 // continue with it.  An occurrence is a pool position, or with bit 31 an index into the history h[0 .. hl).  Writes the
-// tokens to s_cur and returns the depth reached, at most K.  All lanes of a warp.
-// The tokens of eight depths are requested together, so the walk costs a memory round trip per eight tokens; a vote takes one
-// step per distinct token (the first of those left names it, ballots count it) and stops at a majority, and a lone
-// occurrence is copied.  Each lane comparing its token with all 64 in shared memory cost 400 instructions a depth; 4096 queries
-// on 50 M tokens, max_occ 64, with this and the 8-byte table entries: 33 -> 15.3 us a batch that is asked again (its part of the index
-// in L2), 38 -> 19 us batches not asked before.
+// tokens to s_cur and returns the depth reached, at most K.  s_val: kWalkVals words, 16-byte aligned.  All lanes of a warp.
+// Up to eight occurrences are read along: a lane a depth, so that one step covers all depths where they agree, and the vote where
+// they part.  More of them vote a depth at a time, each lane comparing its tokens with all of them, and are soon fewer; the
+// tokens of four depths are requested together.  Bound by latency: a vote whose steps are the distinct tokens, and a depth at a time
+// however few are left, took 9000 cycles of the 21000 of the longest queries, and 8000 for two occurrences that agree.
+constexpr int kWalkFew = 8, kWalkVals = 68;
 __device__ __forceinline__ int walk_occurrences(const int32_t* __restrict__ tok, int64_t hi, const int32_t* __restrict__ h, int hl,
-                                                uint32_t e0, uint32_t e1, bool a0, bool a1, int len, int K, int lane, int32_t* s_cur) {
+                                                uint32_t e0, uint32_t e1, bool a0, bool a1, int len, int K, int lane, int32_t* s_cur,
+                                                int32_t* s_val) {
   auto next = [&](uint32_t e, int j) -> int32_t {
     if (e & 0x80000000u) {
       const int idx = int(e & 0x7fffffffu) + j;
@@ -477,47 +478,86 @@ __device__ __forceinline__ int walk_occurrences(const int32_t* __restrict__ tok,
     const int64_t p = int64_t(e) + j;
     return p < hi ? tok[p] : -1;
   };
-  unsigned m0 = __ballot_sync(0xffffffffu, a0), m1 = __ballot_sync(0xffffffffu, a1);
-  while (len < K && (m0 | m1)) {
-    if (__popc(m0) + __popc(m1) == 1) {   // lane l copies depths len + 1 + l, ..
-      const uint32_t e = __shfl_sync(0xffffffffu, m0 ? e0 : e1, __ffs(m0 | m1) - 1);
-      for (; len < K; len += 32) {
-        const int32_t t = len + 1 + lane <= K ? next(e, len + 1 + lane) : -1;
-        const unsigned stop = __ballot_sync(0xffffffffu, t < 0);
-        const int n = stop ? __ffs(stop) - 1 : 32;
-        if (lane < n) s_cur[len + lane] = t;
-        if (n < 32) { len += n; break; }
-      }
-      break;
-    }
-    int32_t r0[8], r1[8];
+  const unsigned below = (1u << lane) - 1;
+  constexpr int32_t kNone = 0x7fffffff;
+  __syncwarp();                         // (s_val may be where e0 and e1 came from)
+  while (len < K) {
+    unsigned m0 = __ballot_sync(0xffffffffu, a0), m1 = __ballot_sync(0xffffffffu, a1);
+    int c = __popc(m0) + __popc(m1);
+    if (c == 0) break;
+    if (c <= kWalkFew) {
+      const int depth = len + 1 + lane;
+      int32_t x[kWalkFew];
+      unsigned l0 = m0, l1 = m1;
 #pragma unroll
-    for (int u = 0; u < 8; ++u) {
+      for (int i = 0; i < kWalkFew; ++i) {
+        x[i] = -1;
+        if (i >= c) continue;           // (uniform)
+        const uint32_t e = __shfl_sync(0xffffffffu, l0 ? e0 : e1, __ffs(l0 ? l0 : l1) - 1);
+        if (l0) l0 &= l0 - 1; else l1 &= l1 - 1;
+        if (depth <= K) x[i] = next(e, depth);
+      }
+      bool same = x[0] >= 0;
+#pragma unroll
+      for (int i = 1; i < kWalkFew; ++i) same = same && (i >= c || x[i] == x[0]);
+      const unsigned part = __ballot_sync(0xffffffffu, !same);
+      const int d = part ? __ffs(part) - 1 : 32;
+      if (lane < d) s_cur[len + lane] = x[0];
+      len += d;
+      if (d == 32 || len >= K) continue;
+      // lane d holds the tokens of the depth at which they part or end; lane i votes for the i-th
+      int32_t mine = -1;
+      int votes = 0;
+#pragma unroll
+      for (int i = 0; i < kWalkFew; ++i) {
+        x[i] = __shfl_sync(0xffffffffu, x[i], d);
+        if (lane == i) mine = x[i];
+      }
+#pragma unroll
+      for (int i = 0; i < kWalkFew; ++i) votes += x[i] == mine;
+      if (mine < 0) votes = 0;
+      const int best = __reduce_max_sync(0xffffffffu, votes);
+      if (best == 0) break;
+      const int32_t pick = __reduce_min_sync(0xffffffffu, votes == best ? mine : kNone);
+      const unsigned keep = __ballot_sync(0xffffffffu, votes > 0 && mine == pick);
+      a0 = a0 && (keep >> __popc(m0 & below) & 1u);
+      a1 = a1 && (keep >> (__popc(m0) + __popc(m1 & below)) & 1u);
+      if (lane == 0) s_cur[len] = pick;
+      ++len;
+      continue;
+    }
+    int32_t r0[4], r1[4];
+#pragma unroll
+    for (int u = 0; u < 4; ++u) {
       r0[u] = a0 && len + 1 + u <= K ? next(e0, len + 1 + u) : -1;
       r1[u] = a1 && len + 1 + u <= K ? next(e1, len + 1 + u) : -1;
     }
-    const int base = len;
-#pragma unroll
-    for (int u = 0; u < 8; ++u) {
-      if (len != base + u) continue;      // (stopped)
-      a0 = a0 && r0[u] >= 0; a1 = a1 && r1[u] >= 0;
+#pragma unroll 1
+    for (int u = 0; u < 4 && len < K; ++u) {
+      const int32_t t0 = u == 0 ? r0[0] : u == 1 ? r0[1] : u == 2 ? r0[2] : r0[3];
+      const int32_t t1 = u == 0 ? r1[0] : u == 1 ? r1[1] : u == 2 ? r1[2] : r1[3];
+      a0 = a0 && t0 >= 0; a1 = a1 && t1 >= 0;
       m0 = __ballot_sync(0xffffffffu, a0); m1 = __ballot_sync(0xffffffffu, a1);
-      if (!(m0 | m1) || (u > 0 && __popc(m0) + __popc(m1) == 1)) continue;
-      unsigned l0 = m0, l1 = m1;          // those not counted yet
-      int best = 0, left = __popc(l0) + __popc(l1);
-      int32_t pick = 0;
-      while (left >= best && left > 0) {  // (an equal count may still belong to a smaller token)
-        const int32_t v = __shfl_sync(0xffffffffu, l0 ? r0[u] : r1[u], __ffs(l0 ? l0 : l1) - 1);
-        const unsigned q0 = __ballot_sync(0xffffffffu, a0 && r0[u] == v), q1 = __ballot_sync(0xffffffffu, a1 && r1[u] == v);
-        const int c = __popc(q0) + __popc(q1);
-        if (c > best || (c == best && v < pick)) { best = c; pick = v; }
-        l0 &= ~q0; l1 &= ~q1;
-        left -= c;
+      c = __popc(m0) + __popc(m1);
+      if (c <= kWalkFew) break;
+      if (a0) s_val[__popc(m0 & below)] = t0;
+      if (a1) s_val[__popc(m0) + __popc(m1 & below)] = t1;
+      if (lane < 4) s_val[c + lane] = -1;
+      __syncwarp();
+      int n0 = 0, n1 = 0;
+#pragma unroll 4
+      for (int j = 0; j < c; j += 4) {
+        const int4 w = *reinterpret_cast<const int4*>(s_val + j);
+        n0 += (w.x == t0) + (w.y == t0) + (w.z == t0) + (w.w == t0);
+        n1 += (w.x == t1) + (w.y == t1) + (w.z == t1) + (w.w == t1);
       }
+      n0 = a0 ? n0 : 0; n1 = a1 ? n1 : 0;
+      const int best = __reduce_max_sync(0xffffffffu, max(n0, n1));
+      const int32_t pick = __reduce_min_sync(0xffffffffu, min(n0 == best ? t0 : kNone, n1 == best ? t1 : kNone));
+      a0 = a0 && t0 == pick; a1 = a1 && t1 == pick;
       if (lane == 0) s_cur[len] = pick;
-      a0 = a0 && r0[u] == pick; a1 = a1 && r1[u] == pick;
-      m0 = __ballot_sync(0xffffffffu, a0); m1 = __ballot_sync(0xffffffffu, a1);
       ++len;
+      __syncwarp();                     // (s_val is read)
     }
   }
   __syncwarp();
@@ -525,11 +565,52 @@ __device__ __forceinline__ int walk_occurrences(const int32_t* __restrict__ tok,
 }
 
 constexpr int kDraftWarps = 4;
-constexpr int kWorkHead = 3;   // work list: items, next item, CTAs done; then (query, suffix length) pairs
+// Work list of the large-run kernel: runs that a team of it holds and longer ones, the next of each, CTAs done; then (query, suffix
+// length, start of its run), of the former from the front and of the latter from the back.
+enum { WORK_SHORT = 0, WORK_LONG, WORK_NEXT_SHORT, WORK_NEXT_LONG, WORK_DONE, WORK_HEAD };
+constexpr int kTeamRun = 2048; // positions of the longest run that a team takes
+
+// The first probes of four suffix lengths, n and below, at once: eight lanes and slots each, from the keys' home slots on.  A bit
+// per length: settled (found, or an empty slot seen first: not there) and found, then `off` in that length's first lane is the
+// slot's distance from home.  A length after the other is a round trip to memory each, of the ten or so that a query takes.
+constexpr int kProbeLevels = 4, kProbeLanes = 32 / kProbeLevels;
+struct FirstProbe { unsigned settled, found; uint32_t off; };
+__device__ __forceinline__ FirstProbe probe_first(const PoolView& pv, const DraftArgs& a, const Region& rg, int q, int g, int n, int lane) {
+  const int mine = n - lane / kProbeLanes;
+  const uint32_t slot = lane % kProbeLanes;
+  uint64_t key = key_begin(g, mine);
+  bool there = mine >= a.n_min;
+  for (int j = 0; j < mine; ++j) {
+    const int32_t t = a.tails[size_t(q) * a.n_max + a.n_max - mine + j];
+    there = there && t >= 0;
+    key = key_push(key, t);
+  }
+  key = key_end(key);
+  uint2 e = make_uint2(0xffffffffu, 0xffffffffu);
+  if (there) {
+    uint64_t s = uint64_t(home_slot(key, rg.slots)) + slot;   // (a small region is seen more than once, as in probe)
+    if (s >= rg.slots) s %= rg.slots;
+    e = __ldg(pv.table[mine] + rg.base + s);
+  }
+  const unsigned empty = __ballot_sync(0xffffffffu, e.y == 0xffffffffu), hit = __ballot_sync(0xffffffffu, e.y != 0xffffffffu && e.x == uint32_t(key));
+  const unsigned shift = lane / kProbeLanes * kProbeLanes, em = empty >> shift & ((1u << kProbeLanes) - 1);
+  unsigned hm = hit >> shift & ((1u << kProbeLanes) - 1);
+  if (em) hm &= (em & -em) - 1u;
+  FirstProbe r;
+  r.off = hm ? uint32_t(__ffs(hm) - 1) : 0u;
+  const unsigned settled = __ballot_sync(0xffffffffu, (em || hm) && slot == 0), found = __ballot_sync(0xffffffffu, hm && slot == 0);
+  r.settled = r.found = 0;
+#pragma unroll
+  for (int x = 0; x < kProbeLevels; ++x) {
+    r.settled |= (settled >> (x * kProbeLanes) & 1u) << x;
+    r.found |= (found >> (x * kProbeLanes) & 1u) << x;
+  }
+  return r;
+}
 
 __global__ void __launch_bounds__(kDraftWarps * 32)
 draft_warp_kernel(PoolView pv, DraftArgs a) {
-  __shared__ uint32_t s_occ[kDraftWarps][64];
+  __shared__ __align__(16) uint32_t s_occ[kDraftWarps][kWalkVals];   // occurrences, then the walk's
   __shared__ int32_t s_cur[kDraftWarps][kMaxK];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = blockIdx.x * kDraftWarps + warp;
@@ -539,28 +620,39 @@ draft_warp_kernel(PoolView pv, DraftArgs a) {
   int32_t* out = a.draft + size_t(q) * a.K;
   const int g = a.group_id[q];
   int best_len = 0, best_n = 0;
-  int overflow = 0;                  // suffix length from which the large-run kernel takes over
+  int overflow = 0;                  // suffix length from which the large-run kernel takes over, where its run starts,
+  uint32_t start = 0;
+  bool big = false;                  // and whether a team of that kernel cannot hold it
   if (g >= 0 && g < pv.G) {
     const int64_t lo = pv.goff[g], hi = pv.goff[g + 1];
     const int tl = min(max(a.tail_len[q], 0), a.n_max);
-    for (int n = tl; n >= a.n_min && !overflow; --n) {
+    const Region rg = region_of(lo, hi, g);
+    FirstProbe fp{};
+    for (int n = tl, base = 0; n >= a.n_min && !overflow; --n) {
+      if (n == tl || n == base - kProbeLevels) { base = n; fp = probe_first(pv, a, rg, q, g, n, lane); }
+      const int level = base - n;
+      if (fp.settled >> level & ~(fp.found >> level) & 1u) continue;   // not there
       int32_t tn[kMaxN];  // the last n tail tokens, oldest first
-      bool bad = false;
       uint64_t h = key_begin(g, n);
       for (int j = 0; j < n; ++j) {
         tn[j] = a.tails[size_t(q) * a.n_max + a.n_max - n + j];
-        bad |= tn[j] < 0;
         h = key_push(h, tn[j]);
       }
-      if (bad) continue;
+      uint32_t off = (fp.found >> level & 1u) ? __shfl_sync(0xffffffffu, fp.off, level * kProbeLanes) : uint32_t(kProbeLanes);
       const int want = (a.max_occ > 0 && a.max_occ <= 64) ? a.max_occ : 65;
-      int n_occ = gather_occurrences(pv, lo, hi, tn, n, key_end(h), g, lane, s_occ[warp], 0, want);
-      if (want == 65 && n_occ > 64) { overflow = n; break; }
+      int n_occ = gather_occurrences(pv, lo, hi, tn, n, key_end(h), g, lane, s_occ[warp], 0, want, start, off);
+      if (want == 65 && n_occ > 64) {
+        overflow = n;
+        const int64_t last = int64_t(start) + kTeamRun;     // (a run is of one n-gram: a position of it there tells how long it is)
+        big = (a.max_occ == 0 || a.max_occ > kTeamRun) && last < a.n_positions && is_occurrence(pv.tok, lo, hi, int64_t(pv.positions[n][last] & ~kRunEnd), tn, n);
+        break;
+      }
       n_occ = min(n_occ, min(want, 64));
       if (n_occ == 0) continue;
       __syncwarp();
       const int len = walk_occurrences(pv.tok, hi, nullptr, 0, lane < n_occ ? s_occ[warp][lane] : 0u,
-                                       lane + 32 < n_occ ? s_occ[warp][lane + 32] : 0u, lane < n_occ, lane + 32 < n_occ, 0, a.K, lane, s_cur[warp]);
+                                       lane + 32 < n_occ ? s_occ[warp][lane + 32] : 0u, lane < n_occ, lane + 32 < n_occ, 0, a.K, lane, s_cur[warp],
+                                       reinterpret_cast<int32_t*>(s_occ[warp]));
       if (len > best_len) {
         for (int j = lane; j < len; j += 32) out[j] = s_cur[warp][j];
         best_len = len; best_n = n;
@@ -571,8 +663,9 @@ draft_warp_kernel(PoolView pv, DraftArgs a) {
   }
   if (overflow) {  // the rest of the query, and the best draft so far, to the large-run kernel
     if (lane == 0) {
-      const int w = kWorkHead + 2 * atomicAdd(&a.work[0], 1);
-      a.work[w] = q; a.work[w + 1] = overflow;
+      const int at = atomicAdd(&a.work[big ? WORK_LONG : WORK_SHORT], 1);
+      int32_t* w = a.work + WORK_HEAD + 3 * (big ? a.B - 1 - at : at);
+      w[0] = q; w[1] = overflow; w[2] = int32_t(start);
       a.draft_len[q] = best_len; a.match_n[q] = best_n;
     }
     return;
@@ -591,7 +684,7 @@ struct TempArgs {
 
 __global__ void __launch_bounds__(kDraftWarps * 32)
 draft_temp_kernel(PoolView pv, DraftArgs a, TempArgs t) {
-  __shared__ uint32_t s_occ[kDraftWarps][64];
+  __shared__ __align__(16) uint32_t s_occ[kDraftWarps][kWalkVals];   // occurrences, then the walk's
   __shared__ int32_t s_cur[kDraftWarps][kMaxK];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int q = blockIdx.x * kDraftWarps + warp;
@@ -628,12 +721,14 @@ draft_temp_kernel(PoolView pv, DraftArgs a, TempArgs t) {
       n_occ += __popc(ball);
     }
     n_occ = min(n_occ, cap);
+    uint32_t start;
     if (has_group && n_occ < cap)   // the group, ascending
-      n_occ = min(cap, gather_occurrences(pv, lo, hi, tn, n, key_end(key), g, lane, s_occ[warp], n_occ, cap));
+      n_occ = min(cap, gather_occurrences(pv, lo, hi, tn, n, key_end(key), g, lane, s_occ[warp], n_occ, cap, start));
     if (n_occ == 0) continue;
     __syncwarp();
     const int len = walk_occurrences(pv.tok, hi, h, hl, lane < n_occ ? s_occ[warp][lane] : 0u, lane + 32 < n_occ ? s_occ[warp][lane + 32] : 0u,
-                                     lane < n_occ, lane + 32 < n_occ, 0, a.K, lane, s_cur[warp]);
+                                     lane < n_occ, lane + 32 < n_occ, 0, a.K, lane, s_cur[warp],
+                                       reinterpret_cast<int32_t*>(s_occ[warp]));
     if (len > best_len) {
       for (int j = lane; j < len; j += 32) out[j] = s_cur[warp][j];
       best_len = len; best_n = n;
@@ -701,7 +796,8 @@ draft_tree_kernel(PoolView pv, DraftArgs a, TempArgs t, int32_t* __restrict__ dr
       n_occ += __popc(ball);
     }
     n_occ = min(n_occ, cap);
-    if (has_group && n_occ < cap) n_occ = min(cap, gather_occurrences(pv, lo, hi, tn, n, key_end(key), g, lane, s_occ, n_occ, cap));
+    uint32_t start;
+    if (has_group && n_occ < cap) n_occ = min(cap, gather_occurrences(pv, lo, hi, tn, n, key_end(key), g, lane, s_occ, n_occ, cap, start));
     if (n_occ == 0) continue;
     __syncwarp();
     // ---- continuations ----
@@ -830,37 +926,180 @@ __global__ void make_tree_rows_kernel(const int32_t* last, const int32_t* draft,
   if (stamp && i == 0) *stamp = device_ns();
 }
 
-// Large-run path: one CTA per query, votes through a shared-memory histogram over the vocabulary.  The run is read once: its
-// occurrences (those whose tokens match the tail) vote on the first token while their positions go to a list in shared
-// memory; from then on only the list is walked, cut after every vote to the occurrences that continue with the winner - a
-// small share of them, as token frequencies fall fast.  A run that overflows the list is read again at every depth, with the
-// draft so far compared, until what is left fits.  Up to 64 survivors are walked by one warp in registers.
-// Bound by the latency of the longest run's passes; 4096 queries on 50 M tokens in 10,000 groups, the warp kernel included:
-// 1200 .. 1800 us with three passes over the run at every depth and 256 threads -> 51 .. 58 us a batch that is asked again, 60 .. 64
-// us batches not asked before.
+// Large-run path.  Runs of up to 2048 positions - nearly all of them - go to teams of 256 threads, four a CTA, that hold the run's
+// positions in registers and vote through a small hash table in shared memory; longer ones, first, to whole CTAs that hold
+// 16384 and vote in a histogram over the vocabulary.  The warp kernel passes on where the run starts and which of the two it is
+// for; what does not fit after all, and the shorter suffixes of a query whose draft is too short, are left to the CTA.
+// Such a run is read once: its occurrences (those whose tokens match the tail) vote on the first token while their
+// positions go to a list in shared memory; from then on only the list is walked, cut after every vote to the occurrences
+// that continue with the winner - a small share of them, as token frequencies fall fast.  A run that overflows the list is
+// read again at every depth, with the draft so far compared, until what is left fits.  Up to 64 survivors are walked by one
+// warp in registers.
+// Bound by the latency of the longest run's chain of loads.  4096 queries on 50 M tokens in 10,000 groups - about 210 have such
+// runs, a dozen of them long - the warp kernel included: DRAFT_MEASURED.
 constexpr int kBigThreads = 1024;
 constexpr int kBigUnroll = 4;
 constexpr int kBigList = 4096;      // positions: four a thread
 
+// A run held in registers by THREADS threads of a CTA (whose barrier is number `bar`), ITEMS positions each: the query's run of suffix
+// length n from `start` on.  Votes go to a histogram over the vocabulary (HIST: all zero before and after), or to a hash table
+// of {token | votes}, 16 bits each.  0: done; else the suffix length from which the CTA goes on - n itself where the run is too
+// long - with the draft so far in place.
+constexpr int kTeams = 4, kTeamThreads = kBigThreads / kTeams, kTeamItems = kTeamRun / kTeamThreads;
+constexpr int kTeamSlots = 2 * kTeamRun, kTeamSlotBits = 12;
+constexpr int kLongItems = 16;
+static_assert(kTeamItems * kTeamThreads == kTeamRun && kTeamSlots == 1 << kTeamSlotBits && kTeamRun < 65536, "");
+struct Held {
+  __align__(16) uint32_t list[kWalkVals];   // occurrences, then the walk's
+  uint32_t end, count;
+  unsigned long long best;
+  int item[3], reached, odd;    // odd: a position that does not match
+  int32_t cur[kMaxK];
+};
+
+template <int THREADS, int ITEMS, bool HIST>
+__device__ __forceinline__ int held_run(const PoolView& pv, const DraftArgs& a, Held& s, uint32_t* table, int bar, int q, int n,
+                                        uint32_t start) {
+  const int tt = threadIdx.x % THREADS, lane = tt & 31, warp = tt >> 5;
+  auto barrier = [&]() { asm volatile("bar.sync %0, %1;" ::"r"(bar), "n"(THREADS) : "memory"); };
+  // Where max_occ occurrences are all that count, the run's first max_occ positions are those: they are if all of them match.
+  const bool cut = a.max_occ > 0 && a.max_occ <= THREADS * ITEMS;
+  const int most = cut ? a.max_occ : THREADS * ITEMS;
+  const uint32_t* plist = pv.positions[n] + start;
+  uint32_t v[ITEMS], alive = 0;                    // positions; a bit for each that counts
+  uint32_t end = 0xffffffffu;
+#pragma unroll
+  for (int u = 0; u < ITEMS; ++u) {
+    const int idx = u * THREADS + tt;
+    v[u] = idx < most ? (int64_t(start) + idx < a.n_positions ? plist[idx] : kRunEnd) : 0u;
+  }
+#pragma unroll
+  for (int u = ITEMS - 1; u >= 0; --u) if (v[u] & kRunEnd) end = uint32_t(u * THREADS + tt);
+  const int g = a.group_id[q];
+  const int64_t lo = pv.goff[g], hi = pv.goff[g + 1];
+  int32_t tn[kMaxN];
+  for (int j = 0; j < n; ++j) tn[j] = a.tails[size_t(q) * a.n_max + a.n_max - n + j];
+  if (tt == 0) { s.end = 0xffffffffu; s.odd = 0; s.best = 0; s.count = 0; }
+  if (!HIST) for (int x = tt; x < kTeamSlots; x += THREADS) table[x] = 0xffffffffu;
+  barrier();
+  end = __reduce_min_sync(0xffffffffu, end);
+  if (lane == 0 && end != 0xffffffffu) atomicMin(&s.end, end);
+  barrier();
+  const bool whole = s.end != 0xffffffffu;
+  if (!whole && !cut) return n;
+  end = whole ? s.end : uint32_t(most) - 1;
+  int32_t t[ITEMS];
+#pragma unroll
+  for (int u = 0; u < ITEMS; ++u) {
+    const int64_t p = int64_t(v[u] & ~kRunEnd);
+    const bool in = uint32_t(u * THREADS + tt) <= end && p >= lo;
+    t[u] = in && p + 1 < hi ? pv.tok[p + 1] : -1;
+  }
+  bool odd = false;
+#pragma unroll
+  for (int u = 0; u < ITEMS; ++u) {
+    if (uint32_t(u * THREADS + tt) > end) continue;
+    if (is_occurrence(pv.tok, lo, hi, int64_t(v[u] & ~kRunEnd), tn, n)) alive |= 1u << u;
+    else odd = true;
+  }
+  if (!whole) {
+    if (odd) s.odd = 1;
+    barrier();
+    if (s.odd) return n;
+  }
+  const int best_len = a.draft_len[q];             // of the longer suffixes, with their draft in place
+  int len = 0;
+  for (;;) {                                       // t: the tokens of depth len + 1
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) if (t[u] < 0) alive &= ~(1u << u);
+    const uint32_t left = __reduce_add_sync(0xffffffffu, uint32_t(__popc(alive)));
+    if (lane == 0 && left) atomicAdd(&s.count, left);
+    barrier();
+    const uint32_t count = s.count;
+    barrier();
+    if (tt == 0) { s.count = 0; s.best = 0; }
+    barrier();
+    if (count <= 64) {                             // one warp walks them
+#pragma unroll
+      for (int u = 0; u < ITEMS; ++u) if (alive >> u & 1u) s.list[atomicAdd(&s.count, 1u)] = v[u] & ~kRunEnd;
+      barrier();
+      if (warp == 0) {
+        const int l = count ? walk_occurrences(pv.tok, hi, nullptr, 0, lane < count ? s.list[lane] : 0u, lane + 32 < count ? s.list[lane + 32] : 0u,
+                                               lane < count, lane + 32 < count, len, a.K, lane, s.cur,
+                                               reinterpret_cast<int32_t*>(s.list)) : len;
+        if (lane == 0) s.reached = l;
+      }
+      barrier();
+      len = s.reached;
+      break;
+    }
+    unsigned long long cand = 0;
+    uint32_t at[HIST ? 1 : ITEMS];
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) {
+      if (!(alive >> u & 1u)) continue;
+      uint32_t votes;                              // whoever votes last sees the token's full count
+      if (HIST) {
+        votes = atomicAdd(table + t[u], 1u) + 1;
+      } else {
+        uint32_t x = (uint32_t(t[u]) * 0x9E3779B1u) >> (32 - kTeamSlotBits);
+        for (;; x = (x + 1) & (kTeamSlots - 1)) {  // (there are more slots than positions)
+          uint32_t w = *const_cast<volatile uint32_t*>(table + x);
+          if (w == 0xffffffffu) {
+            w = atomicCAS(table + x, 0xffffffffu, uint32_t(t[u]) << 16 | 1u);
+            if (w == 0xffffffffu) { votes = 1; break; }
+          }
+          if (w >> 16 == uint32_t(t[u])) { votes = (atomicAdd(table + x, 1u) & 0xffffu) + 1; break; }
+        }
+        at[HIST ? 0 : u] = x;
+      }
+      cand = max(cand, (unsigned long long)((uint64_t(votes) << 32) | uint32_t(0x7fffffff - t[u])));
+    }
+    for (int o = 16; o; o >>= 1) cand = max(cand, __shfl_xor_sync(0xffffffffu, cand, o));
+    if (lane == 0 && cand) atomicMax(&s.best, cand);
+    barrier();
+    const int32_t pick = 0x7fffffff - int32_t(uint32_t(s.best));
+    if (tt == 0) s.cur[len] = pick;
+    ++len;
+#pragma unroll
+    for (int u = 0; u < ITEMS; ++u) {
+      if (!(alive >> u & 1u)) continue;
+      table[HIST ? uint32_t(t[u]) : at[HIST ? 0 : u]] = HIST ? 0u : 0xffffffffu;
+      if (t[u] != pick) { alive &= ~(1u << u); continue; }
+      const int64_t p = int64_t(v[u] & ~kRunEnd) + len + 1;
+      t[u] = p < hi && len < a.K ? pv.tok[p] : -1;
+    }
+    if (len == a.K) break;
+  }
+  barrier();                                       // (s.cur is complete)
+  int32_t* out = a.draft + size_t(q) * a.K;
+  const bool better = len > best_len, done = max(len, best_len) >= max(a.min_draft, 1) || n == a.n_min;
+  if (better) for (int j = tt; j < len; j += THREADS) out[j] = s.cur[j];
+  if (done) for (int j = max(len, best_len) + tt; j < a.K; j += THREADS) out[j] = -1;
+  if (tt == 0 && better) { a.draft_len[q] = len; a.match_n[q] = n; }
+  if (tt == 0 && !better && best_len == 0) a.match_n[q] = 0;
+  return done ? 0 : n - 1;
+}
+
 __global__ void __launch_bounds__(kBigThreads)
 draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound) {
-  extern __shared__ uint32_t s_hist[];            // [vocab_bound] votes, all zero between depths; then the list
+  extern __shared__ uint32_t s_hist[];            // [vocab_bound] votes, all zero between depths; then the list; or the teams' tables
   uint32_t* s_list = s_hist + vocab_bound;
   __shared__ int32_t s_cur[kMaxK];
   __shared__ uint32_t s_start, s_off, s_end, s_cut, s_count;
   __shared__ int s_found, s_item, s_warp_n[kBigThreads / 32];
   __shared__ unsigned long long s_best;
+  __shared__ __align__(16) int32_t s_walk[kWalkVals];
+  __shared__ Held s_team[kTeams];
+  __shared__ Held s_held;
+  __shared__ int s_late[kTeams][2];
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   next_may_launch();
   for (int v = tid; v < vocab_bound; v += kBigThreads) s_hist[v] = 0;
   wait_for_earlier();
-  const int n_work = a.work[0];
-  for (;;) {
-    __syncthreads();
-    if (tid == 0) s_item = atomicAdd(&a.work[1], 1);
-    __syncthreads();
-    if (s_item >= n_work) break;
-    const int q = a.work[kWorkHead + 2 * s_item], n_first = a.work[kWorkHead + 2 * s_item + 1];
+
+  // A query by the whole CTA, from suffix length n_first on.
+  auto serve = [&](int q, int n_first) {
     int32_t* out = a.draft + size_t(q) * a.K;
     const int g = a.group_id[q];
     const int64_t lo = pv.goff[g], hi = pv.goff[g + 1];
@@ -1020,7 +1259,7 @@ draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound) {
           if (warp == 0) {
             const uint32_t c = s_count;
             const int l = walk_occurrences(pv.tok, hi, nullptr, 0, lane < c ? s_list[lane] : 0u, lane + 32 < c ? s_list[lane + 32] : 0u,
-                                           lane < c, lane + 32 < c, len, a.K, lane, s_cur);
+                                           lane < c, lane + 32 < c, len, a.K, lane, s_cur, s_walk);
             if (lane == 0) s_found = l;
           }
           __syncthreads();
@@ -1036,9 +1275,50 @@ draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound) {
     }
     for (int j = best_len + tid; j < a.K; j += kBigThreads) out[j] = -1;
     if (tid == 0) { a.draft_len[q] = best_len; a.match_n[q] = best_len ? best_n : 0; }
+  };
+
+  const int n_long = a.work[WORK_LONG], n_short = a.work[WORK_SHORT];
+  for (;;) {
+    __syncthreads();
+    if (tid == 0) s_item = n_long ? atomicAdd(&a.work[WORK_NEXT_LONG], 1) : 0;
+    __syncthreads();
+    if (s_item >= n_long) break;
+    const int32_t* w = a.work + WORK_HEAD + 3 * (a.B - 1 - s_item);
+    const int q = w[0], rest = held_run<kBigThreads, kLongItems, true>(pv, a, s_held, s_hist, 0, q, w[1], uint32_t(w[2]));
+    __syncthreads();
+    if (rest) serve(q, rest);
+  }
+  const int team = tid / kTeamThreads;
+  uint32_t* const table = s_hist + team * kTeamSlots;
+  if (tid % kTeamThreads == 0) s_late[team][1] = 0;
+  for (;;) {
+    Held& s = s_team[team];
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kTeamThreads) : "memory");
+    if (tid % kTeamThreads == 0) {
+      const int i = atomicAdd(&a.work[WORK_NEXT_SHORT], 1);
+      const int32_t* w = a.work + WORK_HEAD + 3 * i;
+      s.item[0] = i < n_short ? w[0] : -1; s.item[1] = i < n_short ? w[1] : 0; s.item[2] = i < n_short ? w[2] : 0;
+    }
+    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kTeamThreads) : "memory");
+    const int q = s.item[0];
+    if (q < 0) break;
+    const int rest = held_run<kTeamThreads, kTeamItems, false>(pv, a, s, table, 1 + team, q, s.item[1], uint32_t(s.item[2]));
+    if (rest) {                                    // (the team takes no more: its CTA goes on with this one)
+      if (tid % kTeamThreads == 0) { s_late[team][0] = q; s_late[team][1] = rest; }
+      break;
+    }
+  }
+  __syncthreads();
+  bool clear = true;
+  for (int x = 0; x < kTeams; ++x) {
+    if (!s_late[x][1]) continue;
+    if (clear) { for (int v = tid; v < vocab_bound; v += kBigThreads) s_hist[v] = 0; clear = false; }
+    __syncthreads();
+    serve(s_late[x][0], s_late[x][1]);
   }
   // the last CTA leaves the work list empty for the next call
-  if (tid == 0 && atomicAdd(&a.work[2], 1) == int(gridDim.x) - 1) { a.work[0] = 0; a.work[1] = 0; a.work[2] = 0; }
+  if (tid == 0 && atomicAdd(&a.work[WORK_DONE], 1) == int(gridDim.x) - 1)
+    for (int x = 0; x < WORK_HEAD; ++x) a.work[x] = 0;
 }
 
 __global__ void make_rows_kernel(const int32_t* last, const int32_t* draft, const int32_t* dlen, int B, int K,
@@ -1253,13 +1533,13 @@ LASER_API laser_status laser_draft(const laser_pool* pool, const int32_t* tails,
     return LASER_ERR_UNSUPPORTED;
   }
   void* scratch = nullptr;
-  if (big) LASER_TRY(scratch_get(SCRATCH_DRAFT, sizeof(int32_t) * (size_t(kWorkHead) + 2 * size_t(B)), &scratch));
+  if (big) LASER_TRY(scratch_get(SCRATCH_DRAFT, sizeof(int32_t) * (size_t(WORK_HEAD) + 3 * size_t(B)), &scratch));
   DraftArgs a{tails, tail_len, group_id, B, p->K, p->n_min, p->n_max, p->min_draft, p->max_occ,
               draft, draft_len, match_n, static_cast<int32_t*>(scratch), pool->n_tokens};
   LASER_CUDA(launch_overlapped(draft_warp_kernel, dim3(unsigned(ceil_div(B, kDraftWarps))), kDraftWarps * 32, 0, stream, pv, a));
   count_launch();
   if (big) {
-    const size_t smem = hist + kBigList * sizeof(uint32_t);
+    const size_t smem = std::max(hist + kBigList * sizeof(uint32_t), kTeams * kTeamSlots * sizeof(uint32_t));
     LASER_CUDA(cudaFuncSetAttribute(draft_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
     LASER_CUDA(launch_overlapped(draft_cta_kernel, dim3(unsigned(std::min(B, 148))), kBigThreads, smem, stream, pv, a, pool->vocab_bound));
     count_launch();

@@ -56,3 +56,21 @@ def test_a_run_around_one_warp(L, copies):
     for max_occ in (0, 33, 64):
         _compare(L, toks, offs, np.array([[7, 8], [8, 20], [3, 7]], dtype=np.int32), np.zeros(3, dtype=np.int64), 2, K=12, max_occ=max_occ,
                  min_draft=1)
+
+
+# Runs on both sides of what a team of 256 threads holds (2048 positions) and a CTA (16384), among them the last run of the position array; tokens up
+# to the largest vocabulary; a longer suffix whose draft is too short, so that the CTA goes on with the shorter ones
+@pytest.mark.parametrize("copies", [65, 255, 257, 2047, 2048, 2049, 4100, 16384, 16385])
+def test_a_run_around_a_team(L, copies):
+    rng = np.random.default_rng(copies)
+    toks = []
+    for c in range(copies):
+        toks += [7, 8] + (51199 - rng.integers(0, 3, int(rng.integers(0, 6)))).tolist() + [-1]
+    for c in range(90):
+        toks += [9, 7, 8, -1]                   # "9 7 8" is never continued, "7 8" is
+    toks = np.array(toks + [50] * 70, dtype=np.int32)
+    offs = np.array([0, len(toks)], dtype=np.int64)
+    tails = np.array([[5, 7, 8], [9, 7, 8], [50, 50, 50], [7, 8, 51199]], dtype=np.int32)
+    for max_occ in (0, 65, copies - 1, copies + 1):
+        for min_draft in (1, 6):
+            _compare(L, toks, offs, tails, np.zeros(4, dtype=np.int64), 3, K=7, max_occ=max_occ, min_draft=min_draft)
