@@ -465,7 +465,8 @@ __device__ __forceinline__ int gather_occurrences(const PoolView& pv, int64_t lo
 // Up to eight occurrences are read along: a lane a depth, so that one step covers all depths where they agree, and the vote where
 // they part.  More of them vote a depth at a time, each lane comparing its tokens with all of them, and are soon fewer; the
 // tokens of four depths are requested together.  Bound by latency: a vote whose steps are the distinct tokens, and a depth at a time
-// however few are left, took 9000 cycles of the 21000 of the longest queries, and 8000 for two occurrences that agree.
+// however few are left, took 9000 cycles of the 21000 of the longest queries, and 8000 for two occurrences that agree.  4096 queries on
+// 50 M tokens, max_occ 64, a batch asked again: 14.5 -> 11.4 us with this and the first probes at once.
 constexpr int kWalkFew = 8, kWalkVals = 68;
 __device__ __forceinline__ int walk_occurrences(const int32_t* __restrict__ tok, int64_t hi, const int32_t* __restrict__ h, int hl,
                                                 uint32_t e0, uint32_t e1, bool a0, bool a1, int len, int K, int lane, int32_t* s_cur,
@@ -936,7 +937,9 @@ __global__ void make_tree_rows_kernel(const int32_t* last, const int32_t* draft,
 // read again at every depth, with the draft so far compared, until what is left fits.  Up to 64 survivors are walked by one
 // warp in registers.
 // Bound by the latency of the longest run's chain of loads.  4096 queries on 50 M tokens in 10,000 groups - about 210 have such
-// runs, a dozen of them long - the warp kernel included: DRAFT_MEASURED.
+// runs, a dozen of them long - the warp kernel included: 62 us a batch with all of them served by whole CTAs that read the
+// run and then a list, 51 with these, 34 with the walk by lanes of depths.  Where max_occ cuts the runs (500, groups of 25 k tokens, 300
+// queries) 31 and 26.
 constexpr int kBigThreads = 1024;
 constexpr int kBigUnroll = 4;
 constexpr int kBigList = 4096;      // positions: four a thread
