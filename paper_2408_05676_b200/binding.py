@@ -100,6 +100,36 @@ def _stream(stream) -> C.c_void_p:
     return C.c_void_p(stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream))
 
 
+# The calls of a decoding step take plain addresses: with declared argument types ctypes converts an int by itself, and a call that
+# may run for ten microseconds does not wait for twelve wrapper objects and a stream object to be made.
+def _declare(name: str, n_before: int, *rest) -> None:
+    getattr(lib, name).argtypes = [C.c_void_p] * n_before + list(rest)
+
+
+_P, _I = C.c_void_p, C.c_int32
+_declare("laser_draft", 4, _I, _P, _P, _P, _P, _P)
+_declare("laser_draft_tree", 6, C.c_int64, _I, _P, _P, _P, _P, _P, _P)
+_declare("laser_make_rows", 3, _I, _I, _P, _P, _P)
+_declare("laser_make_rows_tree", 4, _I, _I, _P, _P, _P, _P)
+_declare("laser_accept_commit", 5, _I, _I, _P, _P, _P, _P, _P)
+_declare("laser_accept_commit_noalloc", 5, _I, _I, _P, _P, _P, _P, _P)
+
+
+def _at(t, dtype=None):
+    """The address of a contiguous tensor; with a dtype, of one on the GPU that holds it."""
+    if not isinstance(t, torch.Tensor):
+        return _ptr(t)
+    assert t.is_contiguous(), "tensor must be contiguous"
+    assert dtype is None or (t.is_cuda and t.dtype == dtype), (t.device, t.dtype, dtype)
+    return t.data_ptr()
+
+
+def _stream_at(stream) -> int:
+    if stream is None:
+        return torch._C._cuda_getCurrentRawStream(torch.cuda.current_device())
+    return stream.cuda_stream if hasattr(stream, "cuda_stream") else int(stream)
+
+
 def make_params(K=8, n_min=1, n_max=4, min_draft=1, max_occ=64, mode=MODE_STRICT, topk=2, p=0.1,
                 max_new=0, eos_id=-1, temp_branches=0, tree=0, fused_accept=0) -> Params:
     return Params(K, n_min, n_max, min_draft, max_occ, mode, topk, p, max_new, eos_id, temp_branches, tree, fused_accept)
@@ -158,9 +188,9 @@ def draft(pool: Pool, tails, tail_len, group_id, params: Params, draft_out=None,
         draft_out = torch.empty(B, params.K, dtype=torch.int32, device=dev)
         draft_len = torch.empty(B, dtype=torch.int32, device=dev)
         match_n = torch.empty(B, dtype=torch.int32, device=dev)
-    _chk(lib.laser_draft(pool.handle, _ptr(_dev(tails, torch.int32)), _ptr(_dev(tail_len, torch.int32)),
-                         _ptr(_dev(group_id, torch.int32)), C.c_int32(B), C.byref(params),
-                         _ptr(draft_out), _ptr(draft_len), _ptr(match_n), _stream(stream)))
+    _chk(lib.laser_draft(pool.handle, _at(tails, torch.int32), _at(tail_len, torch.int32),
+                         _at(group_id, torch.int32), B, C.byref(params),
+                         _at(draft_out), _at(draft_len), _at(match_n), _stream_at(stream)))
     return draft_out, draft_len, match_n
 
 
@@ -193,10 +223,10 @@ def draft_tree(pool: Pool, tails, tail_len, group_id, params: Params, hist=None,
     if hist is not None:
         hist, hist_len = _dev(hist, torch.int32), _dev(hist_len, torch.int32)
         stride = hist.shape[1]
-    _chk(lib.laser_draft_tree(pool.handle, _ptr(_dev(tails, torch.int32)), _ptr(_dev(tail_len, torch.int32)),
-                              _ptr(_dev(group_id, torch.int32)), _ptr(hist), _ptr(hist_len), C.c_int64(stride),
-                              C.c_int32(B), C.byref(params), _ptr(draft_out), _ptr(par_out), _ptr(draft_len),
-                              _ptr(match_n), _stream(stream)))
+    _chk(lib.laser_draft_tree(pool.handle, _at(tails, torch.int32), _at(tail_len, torch.int32),
+                              _at(group_id, torch.int32), _at(hist), _at(hist_len), stride,
+                              B, C.byref(params), _at(draft_out), _at(par_out), _at(draft_len),
+                              _at(match_n), _stream_at(stream)))
     return draft_out, par_out, draft_len, match_n
 
 
@@ -206,9 +236,9 @@ def make_rows_tree(last_token, draft_t, draft_parents, draft_len, K: int, stream
     tokens = torch.empty(B, K + 1, dtype=torch.int32, device=dev)
     parents = torch.empty(B, K + 1, dtype=torch.int32, device=dev)
     n_rows = torch.empty(B, dtype=torch.int32, device=dev)
-    _chk(lib.laser_make_rows_tree(_ptr(_dev(last_token, torch.int32)), _ptr(_dev(draft_t, torch.int32)),
-                                  _ptr(_dev(draft_parents, torch.int32)), _ptr(_dev(draft_len, torch.int32)),
-                                  C.c_int32(B), C.c_int32(K), _ptr(tokens), _ptr(parents), _ptr(n_rows), _stream(stream)))
+    _chk(lib.laser_make_rows_tree(_at(last_token, torch.int32), _at(draft_t, torch.int32),
+                                  _at(draft_parents, torch.int32), _at(draft_len, torch.int32),
+                                  B, K, _at(tokens), _at(parents), _at(n_rows), _stream_at(stream)))
     return tokens, parents, n_rows
 
 
@@ -217,9 +247,9 @@ def make_rows(last_token, draft_t, draft_len, K: int, tokens=None, n_rows=None, 
     if tokens is None:
         tokens = torch.empty(B, K + 1, dtype=torch.int32, device=last_token.device)
         n_rows = torch.empty(B, dtype=torch.int32, device=last_token.device)
-    _chk(lib.laser_make_rows(_ptr(_dev(last_token, torch.int32)), _ptr(_dev(draft_t, torch.int32)),
-                             _ptr(_dev(draft_len, torch.int32)), C.c_int32(B), C.c_int32(K),
-                             _ptr(tokens), _ptr(n_rows), _stream(stream)))
+    _chk(lib.laser_make_rows(_at(last_token, torch.int32), _at(draft_t, torch.int32),
+                             _at(draft_len, torch.int32), B, K,
+                             _at(tokens), _at(n_rows), _stream_at(stream)))
     return tokens, n_rows
 
 
@@ -384,12 +414,12 @@ def accept_commit_noalloc(kv: Optional[KV], seq_ids, logits, tokens, n_rows, par
     library.  The caller supplies every output tensor: out = (n_accept, out_tokens, n_out)."""
     B, R, V = logits.shape
     n_accept, out_tokens, n_out = out
-    _chk(lib.laser_accept_commit_noalloc(kv.handle if kv is not None else C.c_void_p(0),
-                                         _ptr(seq_ids) if seq_ids is not None else C.c_void_p(0),
-                                         _ptr(_dev(logits, torch.float32)), _ptr(_dev(tokens, torch.int32)),
-                                         _ptr(_dev(n_rows, torch.int32)), C.c_int32(B), C.c_int32(V),
-                                         C.byref(params), _ptr(n_accept), _ptr(out_tokens), _ptr(n_out),
-                                         _stream(stream)))
+    _chk(lib.laser_accept_commit_noalloc(kv.handle if kv is not None else None,
+                                         _at(seq_ids),
+                                         _at(logits, torch.float32), _at(tokens, torch.int32),
+                                         _at(n_rows, torch.int32), B, V,
+                                         C.byref(params), _at(n_accept), _at(out_tokens), _at(n_out),
+                                         _stream_at(stream)))
     return out
 
 
@@ -401,11 +431,11 @@ def accept_commit(kv: Optional[KV], seq_ids, logits, tokens, n_rows, params: Par
         out = (torch.empty(B, dtype=torch.int32, device=dev), torch.empty(B, R, dtype=torch.int32, device=dev),
                torch.empty(B, dtype=torch.int32, device=dev))
     n_accept, out_tokens, n_out = out
-    _chk(lib.laser_accept_commit(kv.handle if kv is not None else C.c_void_p(0),
-                                 _ptr(seq_ids) if seq_ids is not None else C.c_void_p(0),
-                                 _ptr(_dev(logits, torch.float32)), _ptr(_dev(tokens, torch.int32)),
-                                 _ptr(_dev(n_rows, torch.int32)), C.c_int32(B), C.c_int32(V), C.byref(params),
-                                 _ptr(n_accept), _ptr(out_tokens), _ptr(n_out), _stream(stream)))
+    _chk(lib.laser_accept_commit(kv.handle if kv is not None else None,
+                                 _at(seq_ids),
+                                 _at(logits, torch.float32), _at(tokens, torch.int32),
+                                 _at(n_rows, torch.int32), B, V, C.byref(params),
+                                 _at(n_accept), _at(out_tokens), _at(n_out), _stream_at(stream)))
     return n_accept, out_tokens, n_out
 
 
