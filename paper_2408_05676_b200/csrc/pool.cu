@@ -54,17 +54,21 @@ constexpr int kMaxK = 64;
 constexpr uint64_t kEmpty = ~0ULL;
 constexpr uint32_t kRunEnd = 0x80000000u;   // mark of a run's last position (positions are below 2^31)
 
-__host__ __device__ __forceinline__ uint64_t mix64(uint64_t x) {
-  x ^= x >> 30; x *= 0xbf58476d1ce4e5b9ULL;
-  x ^= x >> 27; x *= 0x94d049bb133111ebULL;
-  x ^= x >> 31;
-  return x;
+// Two 32-bit hashes side by side, each a polynomial in the tokens that is mixed once (the finalizer of MurmurHash3): a 64-bit one took
+// two and a half times the multiplications, and hashing was an eighth of the build in shared memory.  The upper gives a key's
+// home slot, the lower is what its entry shows of it.
+__host__ __device__ __forceinline__ uint32_t mix32(uint32_t x) {
+  x ^= x >> 16; x *= 0x85ebca6bu;
+  x ^= x >> 13; x *= 0xc2b2ae35u;
+  return x ^ (x >> 16);
 }
-// A polynomial in the tokens, mixed once: a mix per token made hashing a third of the build in shared memory.
-__host__ __device__ __forceinline__ uint64_t key_begin(int g, int n) { return (uint64_t(uint32_t(g)) << 8) | uint64_t(n); }
-__host__ __device__ __forceinline__ uint64_t key_push(uint64_t h, int32_t tok) { return h * 0x9E3779B97F4A7C15ULL + uint32_t(tok); }
-__host__ __device__ __forceinline__ uint64_t key_end(uint64_t h) { return mix64(h * 0x9E3779B97F4A7C15ULL); }
-__device__ __forceinline__ uint32_t home_slot(uint64_t key, uint32_t slots) { return uint32_t(__umul64hi(key, slots)); }
+__host__ __device__ __forceinline__ uint64_t key_of(uint32_t hi, uint32_t lo) { return uint64_t(hi) << 32 | lo; }
+__host__ __device__ __forceinline__ uint64_t key_begin(int g, int n) { return key_of(uint32_t(g) * 8u + uint32_t(n), uint32_t(g)); }
+__host__ __device__ __forceinline__ uint64_t key_push(uint64_t h, int32_t tok) {
+  return key_of(uint32_t(h >> 32) * 0x9E3779B1u + uint32_t(tok), uint32_t(h) * 0x85EBCA77u + uint32_t(tok));
+}
+__host__ __device__ __forceinline__ uint64_t key_end(uint64_t h) { return key_of(mix32(uint32_t(h >> 32)), mix32(uint32_t(h))); }
+__device__ __forceinline__ uint32_t home_slot(uint64_t key, uint32_t slots) { return __umulhi(uint32_t(key >> 32), slots); }
 
 // A group's region of a table: 13 slots per 8 tokens, and always one more than there are tokens.
 struct Region { int64_t base; uint32_t slots; };
@@ -205,15 +209,16 @@ clear_regions_kernel(const IndexLevels lv, int n_min, const int64_t* __restrict_
 }
 
 // ---- a group in shared memory ------------------------------------------------------------
-// One CTA per (group, n): the region's slots as words {count | representative position}, into which the group's n-grams are
-// inserted (compared by their tokens); the counts become run starts by a prefix sum; a block of positions after the other goes
-// into the runs, and a position finds its place among those of its block by counting.  Memory sees the tokens, the runs and
-// the regions; what bounds the kernel is the latency of its steps in shared memory.  In the insert loop a lane takes its next
-// position as soon as it has placed one: a warp whose lanes wait for the longest of 32 probe walks took four times as long.
-// Groups come in three classes by size, for one, two and three CTAs an SM.  10 M tokens in 2000 groups, four levels: 820 us for
-// the 72 % of them in groups that fit and 740 us for the rest, against 4.7 ms for a sort of all positions by 64-bit key and n;
-// the whole build 4.99 -> 1.61 ms, and 4.66 -> 2.48 ms where groups are so large that few fit.
-constexpr uint32_t kFreeWord = 0x0000ffffu;
+// One CTA per (group, n): the region's slots as words, into which the group's n-grams are inserted (told apart by 16 bits of their
+// key, then by their tokens); the counts of the slots become run starts by a prefix sum; a block of positions after the other
+// goes into the runs, and a position finds its place among those of its block by counting.  Memory sees the tokens, the runs and
+// the regions; what bounds the kernel is the latency of its steps in shared memory.  In the insert loop a lane takes the warp's
+// next position as soon as it has placed one: with positions of its own for every lane the CTA waits for the unluckiest of 512
+// probe walks, and with a warp in step for the longest of 32, four times as long again.
+// Groups come in three classes by size, for one, two and three CTAs an SM.  10 M tokens in 2000 groups, four levels: 690 us for
+// the 72 % of them in groups that fit (805 with positions per lane, representatives' tokens compared at every probe and a 64-bit
+// hash) and 735 us for the rest, against 4.7 ms for a sort of all positions by 64-bit key and n; the whole build 4.99 -> 1.49 ms.
+constexpr uint32_t kFreeWord = 0xffffffffu;
 constexpr int kScan = 128;                       // slots that a warp scans at a time
 constexpr size_t group_smem(int64_t tokens) {    // words, tokens, slot and run member of every position
   return size_t((tokens + tokens / 2 + tokens / 8 + 4 + kScan - 1) / kScan * kScan) * 4 + size_t(tokens) * 8 + 16;
@@ -234,7 +239,7 @@ template <int THREADS, int CTAS>
 __global__ void __launch_bounds__(THREADS, CTAS)
 index_group_kernel(const int32_t* tok, const int64_t* goff, const uint32_t* group_id, const uint32_t* group_at, int leads, int n_min,
                    const IndexLevels lv, unsigned long long* n_heads, int* max_tok) {
-  constexpr int kWarps = THREADS / 32, kBlock = 256;
+  constexpr int kWarps = THREADS / 32;
   extern __shared__ __align__(16) uint32_t s_word[];
   __shared__ uint32_t s_sum[kWarps];
   __shared__ int s_heads;
@@ -265,13 +270,13 @@ index_group_kernel(const int32_t* tok, const int64_t* goff, const uint32_t* grou
     if (lane == 0 && mt > *max_tok) atomicMax(max_tok, mt);
   }
   __syncthreads();
-  auto key_of = [&](int i) {      // of the n-gram that ends at i
+  auto ngram_key = [&](int i) {      // of the n-gram that ends at i
     uint64_t h = key_begin(g, n);
     for (int j = i - n + 1; j <= i; ++j) h = key_push(h, s_tok[j]);
     return key_end(h);
   };
 
-  // home slots
+  // home slots, and 16 bits of the keys where the runs' members will be
   for (int i = tid; i < T; i += THREADS) {
     uint64_t h = key_begin(g, n);
     int32_t least = i >= n - 1 ? 0 : -1;
@@ -280,34 +285,49 @@ index_group_kernel(const int32_t* tok, const int64_t* goff, const uint32_t* grou
       least = min(least, t);
       h = key_push(h, t);
     }
-    s_slot[i] = least >= 0 ? uint16_t(home_slot(key_end(h), rg.slots)) : uint16_t(0xffff);
+    h = key_end(h);
+    s_slot[i] = least >= 0 ? uint16_t(home_slot(h, rg.slots)) : uint16_t(0xffff);
+    s_member[i] = uint16_t(h);
   }
-  // insert and count (a thread's positions are its own from here to the next barrier)
-  for (int i = tid, s = i < T ? s_slot[i] : 0, t = i < T ? s_tok[i] : 0; i < T;) {
-    bool placed = s == 0xffff;    // (none ends here)
-    if (!placed) {                // (there are more slots than positions)
-      uint32_t w = *const_cast<volatile uint32_t*>(s_word + s);
-      if (w == kFreeWord) {
-        w = atomicCAS(s_word + s, kFreeWord, 0x10000u | uint32_t(i));
-        placed = w == kFreeWord;
-      }
-      if (!placed) {
-        const int rep = int(w & 0xffffu);
-        if (s_tok[rep] == t) {
+  // insert: words of {16 bits of the key | position}, so that another n-gram's slot is passed without a look at its tokens.  A
+  // warp's positions are those that its threads hashed; its lanes take them as they become free, for some walks are long
+  // (with twelve positions to each lane the CTA waited for the unluckiest of its 512).
+  __syncwarp();
+  {
+    auto position = [&](int j) { return (j >> 5) * THREADS + warp * 32 + (j & 31); };
+    int i = position(lane), given = 32;
+    int s = i < T ? s_slot[i] : 0;
+    while (__any_sync(0xffffffffu, i < T)) {
+      bool placed = i < T && s == 0xffff;       // (none ends here)
+      if (i < T && !placed) {                   // (there are more slots than positions)
+        const uint32_t word = uint32_t(s_member[i]) << 16 | uint32_t(i);
+        uint32_t w = *const_cast<volatile uint32_t*>(s_word + s);
+        if (w == kFreeWord) {
+          w = atomicCAS(s_word + s, kFreeWord, word);
+          placed = w == kFreeWord;
+        }
+        if (!placed && (w ^ word) < 0x10000u) {
+          const int rep = int(w & 0xffffu);
           placed = true;
-          for (int j = 1; j < n; ++j) placed = placed && s_tok[i - j] == s_tok[rep - j];
-          if (placed) atomicAdd(s_word + s, 0x10000u);
+          for (int j = 0; j < n; ++j) placed = placed && s_tok[i - j] == s_tok[rep - j];
         }
       }
-    }
-    if (placed) {
-      s_slot[i] = uint16_t(s);
-      i += THREADS;
-      if (i < T) { s = s_slot[i]; t = s_tok[i]; }
-    } else if (++s == slots) {
-      s = 0;
+      const unsigned done = __ballot_sync(0xffffffffu, placed);
+      if (placed) {
+        s_slot[i] = uint16_t(s);
+        i = position(given + __popc(done & ((1u << lane) - 1)));
+        if (i < T) s = s_slot[i];
+      } else if (++s == slots) {
+        s = 0;
+      }
+      given += __popc(done);
     }
   }
+  __syncthreads();
+  for (int s = 4 * tid; s < words; s += 4 * THREADS) *reinterpret_cast<uint4*>(s_word + s) = make_uint4(0u, 0u, 0u, 0u);
+  __syncthreads();
+  for (int i = tid; i < T; i += THREADS)
+    if (s_slot[i] != 0xffff) atomicAdd(s_word + s_slot[i], 0x10000u);
   __syncthreads();
 
   // counts -> {0 | start}: a warp's share of the slots is consecutive, four a lane at a time
@@ -339,39 +359,41 @@ index_group_kernel(const int32_t* tok, const int64_t* goff, const uint32_t* grou
   }
   __syncthreads();
 
-  // every position into its run: blocks of kBlock positions in order, within a block in the order of arrival; the words
+  // every position into its run: blocks of 128 or 256 positions in order, within a block in the order of arrival; the words
   // become {count | start}.  (A large block is placed quickly, a small one ranked: groups of 4,900 to 7,600 tokens, n = 1,
-  // blocks of 512 take 4 and 62 thousand cycles, of 256 7 and 41; n = 4, 4 and 13, 6 and 13.)
-  if (tid < kBlock)
-    for (int i0 = 0; i0 < T; i0 += kBlock) {
+  // blocks of 512 take 4 and 62 thousand cycles, of 256 7 and 41, of 128 12 and 28, of 32 by a warp alone 38 and 17; n = 4, 4 and 13, 6
+  // and 13, 11 and 13, 39 and 13.)
+  const uint32_t block_bits = n == 1 ? 7 : 8, in_block = 1u << block_bits;
+  if (uint32_t(tid) < in_block)
+    for (int i0 = 0; i0 < T; i0 += int(in_block)) {
       const int i = i0 + tid, s = i < T ? s_slot[i] : 0xffff;
       if (s != 0xffff) {
         const uint32_t w = atomicAdd(s_word + s, 0x10000u);
         s_member[(w & 0xffffu) + (w >> 16)] = uint16_t(i);
       }
-      asm volatile("bar.sync 1, %0;" ::"n"(kBlock) : "memory");
+      asm volatile("bar.sync 1, %0;" ::"r"(in_block) : "memory");
     }
   __syncthreads();
 
   // to its place in the run, behind those of earlier blocks; the first of a run makes its entry
   uint32_t* positions = lv.positions[n] + first;
   for (uint32_t k = tid; k < total; k += THREADS) {
-    const uint32_t i = s_member[k], block = i / kBlock, s = s_slot[i], w = s_word[s], begin = w & 0xffffu, end = begin + (w >> 16);
+    const uint32_t i = s_member[k], block = i >> block_bits, s = s_slot[i], w = s_word[s], begin = w & 0xffffu, end = begin + (w >> 16);
     uint32_t left = k, smaller = 0;
     while (left > begin) {
       const uint32_t m = s_member[left - 1];
-      if (m / kBlock != block) break;
+      if (m >> block_bits != block) break;
       smaller += m < i;
       --left;
     }
     for (uint32_t r = k + 1; r < end; ++r) {
       const uint32_t m = s_member[r];
-      if (m / kBlock != block) break;
+      if (m >> block_bits != block) break;
       smaller += m < i;
     }
     const uint32_t at = left + smaller;
     positions[at] = (uint32_t(lo) + i) | (at + 1 == end ? kRunEnd : 0u);
-    if (k == begin) table[s] = make_uint2(uint32_t(key_of(int(i))), uint32_t(first) + begin);
+    if (k == begin) table[s] = make_uint2(uint32_t(ngram_key(int(i))), uint32_t(first) + begin);
   }
   if (tid == 0 && s_heads) atomicAdd(n_heads + n, (unsigned long long)s_heads);
   wait_for_earlier();             // (the classes are independent; what follows in the stream waits for all)
