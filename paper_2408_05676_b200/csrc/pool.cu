@@ -101,9 +101,7 @@ __device__ __forceinline__ int group_of(const SortedGroups& lg, const int64_t* _
 }
 
 // Inserts the n-grams of the listed groups, for the n from n0 on, into their regions (cleared before) and leaves every (n,
-// position) with the number of its n-gram (kNoSlot where none ends): the place, among all of them, of the (n, position) that
-// inserted it, whose slot it also leaves.  (Slot numbers would do as well, but there are 13 slots to 8 positions in all groups, and
-// a bit or two more to sort by: 2.8 M positions of 10 M, four n, 24 bits and three passes instead of 26 and four.)  An entry is {key's low
+// position) with the number of its n-gram's slot among all those tables' (kNoSlot where none ends).  An entry is {key's low
 // half, a position of the n-gram} here; equal low halves are told apart by the tokens.  A block's positions are consecutive: two
 // searches bound the groups of its threads, and as they are a chain of loads a block takes kInsertItems positions a thread (2.8 M
 // positions, four n: 374 us with one, 256 with four).  Bound by the latency of the probes, in L2 for the most part.
@@ -111,7 +109,7 @@ constexpr uint32_t kNoSlot = 0xffffffffu;
 constexpr int kInsertItems = 4, kInsertBlock = kInsertItems * kKeyThreads;
 __global__ void __launch_bounds__(kKeyThreads)
 insert_sorted_kernel(const int32_t* __restrict__ tok, const int64_t* __restrict__ goff, SortedGroups lg, int64_t M, int n0,
-                    const IndexLevels lv, uint32_t* __restrict__ ngram, uint32_t* __restrict__ slot_of, uint32_t* __restrict__ pos,
+                    const IndexLevels lv, uint32_t table_slots, uint32_t* __restrict__ slot_of, uint32_t* __restrict__ pos,
                     unsigned long long* __restrict__ n_valid, int* __restrict__ max_tok) {
   __shared__ int s_g[2], s_max[kKeyThreads / 32];
   __shared__ unsigned s_ends;
@@ -139,26 +137,25 @@ insert_sorted_kernel(const int32_t* __restrict__ tok, const int64_t* __restrict_
       const Region rg = region_of(lo, goff[g + 1], g);
       const unsigned long long entry = (uint64_t(uint32_t(p)) << 32) | uint32_t(key);
       uint32_t s = home_slot(key, rg.slots);
-      int64_t first = i;
       for (uint32_t tries = 0; tries < rg.slots; ++tries) {   // there are more slots than positions
         unsigned long long* e = table + rg.base + s;
         unsigned long long old = __ldcg(e);
         if (old == kEmpty) {
           old = atomicCAS(e, (unsigned long long)kEmpty, entry);
-          if (old == kEmpty) { slot_of[blockIdx.y * M + i] = uint32_t(rg.base) + s; break; }
+          if (old == kEmpty) break;
         }
         if (uint32_t(old) == uint32_t(key)) {
           const int64_t q = int64_t(old >> 32);
           bool same = true;
           for (int j = 0; same && j < n; ++j) same = tok[p - j] == tok[q - j];
-          if (same) { first = i - (p - q); break; }
+          if (same) break;
         }
         if (++s == rg.slots) s = 0;
       }
-      at = uint32_t(blockIdx.y * M + first);
+      at = blockIdx.y * table_slots + uint32_t(rg.base) + s;
       ++ends;
     }
-    ngram[blockIdx.y * M + i] = at;
+    slot_of[blockIdx.y * M + i] = at;
     pos[blockIdx.y * M + i] = uint32_t(p);
     mt = max(mt, tok[p]);
   }
@@ -177,25 +174,25 @@ insert_sorted_kernel(const int32_t* __restrict__ tok, const int64_t* __restrict_
   }
 }
 
-// (n-gram, position) pairs sorted by n-gram to the position arrays (from `first` on) with their run marks, and the start of every
-// run to its slot.  M: positions per n.
+// (slot, position) pairs sorted by slot to the position arrays (from `first` on) with their run marks, and the start of every
+// run to its slot.
 __global__ void __launch_bounds__(kKeyThreads)
-index_runs_kernel(const uint32_t* __restrict__ ngram, const uint32_t* __restrict__ pos, int64_t count, int64_t first, int n0,
-                  const IndexLevels lv, uint32_t M, const uint32_t* __restrict__ slot_of, const unsigned long long* __restrict__ n_valid,
+index_runs_kernel(const uint32_t* __restrict__ slot, const uint32_t* __restrict__ pos, int64_t count, int64_t first, int n0,
+                  const IndexLevels lv, uint32_t table_slots, const unsigned long long* __restrict__ n_valid,
                   unsigned long long* __restrict__ n_heads) {
   __shared__ unsigned s_heads[kMaxN + 1];
   if (threadIdx.x <= kMaxN) s_heads[threadIdx.x] = 0;
   __syncthreads();
   const int64_t i = int64_t(blockIdx.x) * kKeyThreads + threadIdx.x;
-  const uint32_t k = i < count ? ngram[i] : kNoSlot;
-  if (k != kNoSlot) {
-    const uint32_t l = k / M;
+  const uint32_t s = i < count ? slot[i] : kNoSlot;
+  if (s != kNoSlot) {
+    const uint32_t l = s / table_slots;
     int64_t rank = i;                      // among the positions of its n
     for (uint32_t x = 0; x < l; ++x) rank -= int64_t(n_valid[n0 + x]);
-    const bool end = i + 1 == count || ngram[i + 1] != k;
+    const bool end = i + 1 == count || slot[i + 1] != s;
     lv.positions[n0 + l][first + rank] = pos[i] | (end ? kRunEnd : 0u);
-    if (i == 0 || ngram[i - 1] != k) {
-      lv.table[n0 + l][slot_of[k]].y = uint32_t(first + rank);
+    if (i == 0 || slot[i - 1] != s) {
+      lv.table[n0 + l][s - l * table_slots].y = uint32_t(first + rank);
       atomicAdd(&s_heads[n0 + l], 1u);
     }
   }
@@ -1456,27 +1453,27 @@ LASER_API laser_status laser_pool_build(const int32_t* tokens, int64_t n_tokens,
   LASER_CUDA(cudaMemcpyAsync(P->tokens, tokens, N * 4, cudaMemcpyDefault, stream));
   LASER_CUDA(cudaMemcpyAsync(P->group_offsets, group_offsets, (size_t(n_groups) + 1) * 8, cudaMemcpyHostToDevice, stream));
 
-  // The sorted groups' n-grams go through one sort for as many n as 64 M pairs hold.
+  // The sorted groups' n-grams go through one sort for as many n as 32-bit slot numbers and 64 M pairs hold.
   const int levels = n_max - n_min + 1;
-  const int batch = int(std::max<size_t>(1, std::min(size_t(levels), (size_t(64) << 20) / std::max<size_t>(M, 1))));
-  const size_t pairs = M * batch;   // (M where one n alone is more than 64 M: below 2^31)
-  int bits = 1;                     // all that kNoSlot needs to sort behind every n-gram
-  while (bits < 32 && pairs >> bits) ++bits;
+  const int batch = int(std::max<size_t>(1, std::min({size_t(levels), size_t(kNoSlot) / slots, (size_t(64) << 20) / std::max<size_t>(M, 1)})));
+  int slot_bits = 1;             // all that kNoSlot needs to sort behind every slot
+  while (slot_bits < 32 && (slots * batch) >> slot_bits) ++slot_bits;
+  const size_t pairs = M * batch;
   size_t cub_bytes = 0;
   if (M) {
     cub::DoubleBuffer<uint32_t> kb(nullptr, nullptr), vb(nullptr, nullptr);
-    LASER_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, cub_bytes, kb, vb, int64_t(pairs), 0, bits, stream));
+    LASER_CUDA(cub::DeviceRadixSort::SortPairs(nullptr, cub_bytes, kb, vb, int64_t(pairs), 0, slot_bits, stream));
   }
   constexpr size_t kCounters = (2 * kMaxN + 3) * 8;   // distinct keys per n, the largest token, n-grams of the sorted groups per n
   const size_t b_lists = listed ? (size_t(n_groups) * 2 + 1) * 4 : 0;
   struct Tmp { void* p = nullptr; cudaStream_t s; ~Tmp() { pooled_free(p, s); } } tmp{nullptr, stream};
-  LASER_TRY(pooled_alloc(&tmp.p, 5 * padded(pairs * 4) + padded(kCounters) + padded(b_lists) + cub_bytes + 256, stream));
+  LASER_TRY(pooled_alloc(&tmp.p, 4 * padded(pairs * 4) + padded(kCounters) + padded(b_lists) + cub_bytes + 256, stream));
   at = static_cast<uint8_t*>(tmp.p);
-  uint32_t *ngram, *ngram_alt, *pos, *pos_alt, *slot_of;
+  uint32_t *slot_of, *slot_alt, *pos, *pos_alt;
   unsigned long long* counters;
   uint32_t* d_id;
   uint8_t* cub_tmp;
-  take(&ngram, padded(pairs * 4)); take(&ngram_alt, padded(pairs * 4)); take(&pos, padded(pairs * 4)); take(&pos_alt, padded(pairs * 4)); take(&slot_of, padded(pairs * 4));
+  take(&slot_of, padded(pairs * 4)); take(&slot_alt, padded(pairs * 4)); take(&pos, padded(pairs * 4)); take(&pos_alt, padded(pairs * 4));
   take(&counters, padded(kCounters)); take(&d_id, padded(b_lists)); take(&cub_tmp, cub_bytes);
   const uint32_t* d_at = d_id + n_groups;
   int* max_tok = reinterpret_cast<int*>(counters + kMaxN + 1);
@@ -1512,11 +1509,11 @@ LASER_API laser_status laser_pool_build(const int32_t* tokens, int64_t n_tokens,
       const int nb = std::min(batch, n_max - n0 + 1);
       const int64_t count = int64_t(M) * nb;
       insert_sorted_kernel<<<dim3(blocks, unsigned(nb)), kKeyThreads, 0, stream>>>(P->tokens, P->group_offsets, lg, n_sorted, n0, lvs,
-                                                                                  ngram, slot_of, pos, n_valid, max_tok);
-      cub::DoubleBuffer<uint32_t> kb(ngram, ngram_alt), vb(pos, pos_alt);
-      LASER_CUDA(cub::DeviceRadixSort::SortPairs(cub_tmp, cub_bytes, kb, vb, count, 0, bits, stream));
+                                                                                  uint32_t(slots), slot_of, pos, n_valid, max_tok);
+      cub::DoubleBuffer<uint32_t> kb(slot_of, slot_alt), vb(pos, pos_alt);
+      LASER_CUDA(cub::DeviceRadixSort::SortPairs(cub_tmp, cub_bytes, kb, vb, count, 0, slot_bits, stream));
       index_runs_kernel<<<unsigned(ceil_div<int64_t>(count, kKeyThreads)), kKeyThreads, 0, stream>>>(
-          kb.Current(), vb.Current(), count, n_small, n0, lvs, uint32_t(M), slot_of, n_valid, counters);
+          kb.Current(), vb.Current(), count, n_small, n0, lvs, uint32_t(slots), n_valid, counters);
       count_launch(2);
       LASER_CUDA(cudaGetLastError());
     }
