@@ -364,7 +364,7 @@ LASER_API laser_status laser_model_create(const laser_model_cfg* cfg, const lase
     m->attn_norm.push_back(static_cast<const bf16*>(w->attn_norm[l]));
     m->ffn_norm.push_back(static_cast<const bf16*>(w->ffn_norm[l]));
   }
-  m->R_cap = std::max(m->R_pad, kPrefillRows);
+  m->R_cap = std::max(m->R_pad, prefill_rows(int64_t(d) * (m->dqkv + m->dq + 3 * f)));
   m->precise = cfg->precise != 0;
   const size_t Rp = size_t(m->R_cap), pair = m->precise ? 2 : 1;     // pair: hi + lo parts side by side in a row
   const size_t groups = std::max<size_t>(cfg->max_batch, Rp / kPrefillChunk);

@@ -11,7 +11,7 @@ struct laser_model {
   int rows_per_seq = 0;  // max_draft + 1
   int R = 0;             // max_batch * rows_per_seq
   int R_pad = 0;         // R rounded up to a multiple of 16
-  int R_cap = 0;         // rows of the workspace: R_pad, or kPrefillRows where that is more
+  int R_cap = 0;         // rows of the workspace: R_pad, or those of a prefill pass where that is more
   int dq = 0, dkv = 0, dqkv = 0;
   const __nv_bfloat16 *tok_emb = nullptr, *lm_head = nullptr, *final_norm = nullptr;
   std::vector<const __nv_bfloat16*> wqkv, wo, wgu, wdown, attn_norm, ffn_norm;
@@ -59,8 +59,9 @@ namespace laser {
 
 // A prefill pass runs the contractions over up to this many prompt tokens: enough rows for the tensor pipe to be the bound
 // (7B, 4 layers: 3.6 us a row at 144 rows, 1.6 us at 1024), and to fill whole waves of tiles: 16 tiles of 256 weight rows, as the O and down
-// projections of 4096 features have, leave 14 % of the last wave idle at 1024 rows (64 of 74 pairs), 3 % at 2304 (144 of 148).
-constexpr int kPrefillRows = 2304;
+// projections of 4096 features have, leave 14 % of the last wave idle at 1024 rows (64 of 74 pairs), 3 % at 2304 (144 of 148).  A
+// model of few weights a layer gains nothing by that, and would only be created more slowly.
+constexpr int prefill_rows(int64_t layer_weights) { return layer_weights >= (int64_t(16) << 20) ? 2304 : 1024; }
 constexpr int kAttnSplitCtas = 3 * 148; // most CTAs of an attention launch that splits pages: three an SM
 constexpr int kPrefillChunk = 32;   // rows of a chunk of a prompt
 constexpr int kPrefillShare = 4;    // consecutive chunks that share each staged K/V page in the attention kernel
