@@ -16,11 +16,10 @@
 // positions sorted by slot, all groups together, with the radix sort of CUB, the header library
 // shipped with the CUDA toolkit (nothing on the per-step path uses it).
 //
-// Lookup: one warp per query.  All 32 lanes probe 32 consecutive slots (256 B, coalesced);
-// the run is read 32 positions at a time, verified, and compacted; the greedy
+// Lookup: one warp per query.  Four suffix lengths are probed at once; where that does not settle one, all 32 lanes probe 32
+// consecutive slots (256 B, coalesced); the run is read 32 positions at a time, verified, and compacted; the greedy
 // highest-frequency walk votes over at most 64 occurrences held two per lane.  Queries that
-// need more than 64 occurrences (max_occ = 0 or > 64) go to a work list served by one CTA
-// per query with a shared-memory histogram over the vocabulary.
+// need more than 64 occurrences (max_occ = 0 or > 64) go to a work list served by teams of 256 threads and by whole CTAs.
 #include <cub/device/device_radix_sort.cuh>
 
 #include <algorithm>
@@ -965,6 +964,7 @@ __global__ void make_tree_rows_kernel(const int32_t* last, const int32_t* draft,
 constexpr int kBigThreads = 1024;
 constexpr int kBigUnroll = 4;
 constexpr int kBigList = 4096;      // positions: four a thread
+constexpr size_t kBigSmem = 204 * 1024;   // for the histogram and a longer list, as far as the vocabulary leaves room
 
 // A run held in registers by THREADS threads of a CTA (whose barrier is number `bar`), ITEMS positions each: the query's run of suffix
 // length n from `start` on.  Votes go to a histogram over the vocabulary (HIST: all zero before and after), or to a hash table
@@ -1107,7 +1107,7 @@ __device__ __forceinline__ int held_run(const PoolView& pv, const DraftArgs& a, 
 }
 
 __global__ void __launch_bounds__(kBigThreads)
-draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound) {
+draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound, uint32_t list_cap) {
   extern __shared__ uint32_t s_hist[];            // [vocab_bound] votes, all zero between depths; then the list; or the teams' tables
   uint32_t* s_list = s_hist + vocab_bound;
   __shared__ int32_t s_cur[kMaxK];
@@ -1217,7 +1217,7 @@ draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound) {
               uint32_t at = 0;
               if (ball && lane == 0) at = atomicAdd(&s_count, uint32_t(__popc(ball)));
               at = __shfl_sync(0xffffffffu, at, 0) + __popc(ball & ((1u << lane) - 1));
-              if (alive[u] && at < kBigList) s_list[at] = v[u] & ~kRunEnd;
+              if (alive[u] && at < list_cap) s_list[at] = v[u] & ~kRunEnd;
             }
             if (end != 0xffffffffu || base + kBigThreads * kBigUnroll > cut) break;
             __syncthreads();   // (every thread has read s_end)
@@ -1230,8 +1230,35 @@ draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound) {
           for (int x = tid; x < vocab_bound; x += kBigThreads) s_hist[x] = 0;
           if (tid == 0) s_cur[j - 1] = 0x7fffffff - int32_t(uint32_t(s_best));
           len = j;
-          listed = s_count <= kBigList;
+          const uint32_t count = s_count;
+          listed = count <= kBigList;
           __syncthreads();
+          if (!listed && count <= list_cap && len < a.K) {   // a long list, cut to the winner's occurrences where it is
+            const int32_t pick = s_cur[len - 1];
+            if (tid == 0) s_count = 0;
+            for (uint32_t base = 0; base < count; base += kBigThreads * kBigUnroll) {
+              uint32_t mine[kBigUnroll];
+              bool keep[kBigUnroll];
+#pragma unroll
+              for (int u = 0; u < kBigUnroll; ++u) {
+                const uint32_t idx = base + u * kBigThreads + tid;
+                mine[u] = idx < count ? s_list[idx] : 0u;
+                keep[u] = idx < count && int64_t(mine[u]) + len < hi && pv.tok[int64_t(mine[u]) + len] == pick;
+              }
+              __syncthreads();       // (what is written comes from here or before)
+#pragma unroll
+              for (int u = 0; u < kBigUnroll; ++u) {
+                const unsigned ball = __ballot_sync(0xffffffffu, keep[u]);
+                uint32_t at = 0;
+                if (ball && lane == 0) at = atomicAdd(&s_count, uint32_t(__popc(ball)));
+                at = __shfl_sync(0xffffffffu, at, 0) + __popc(ball & ((1u << lane) - 1));
+                if (keep[u]) s_list[at] = mine[u];
+              }
+            }
+            __syncthreads();
+            listed = s_count <= kBigList;
+            __syncthreads();
+          }
           if (listed || len == a.K) break;
         }
         // the list holds the positions alive before the last vote: keep the winner's, then go on with the list alone
@@ -1564,9 +1591,11 @@ LASER_API laser_status laser_draft(const laser_pool* pool, const int32_t* tails,
   LASER_CUDA(launch_overlapped(draft_warp_kernel, dim3(unsigned(ceil_div(B, kDraftWarps))), kDraftWarps * 32, 0, stream, pv, a));
   count_launch();
   if (big) {
-    const size_t smem = std::max(hist + kBigList * sizeof(uint32_t), kTeams * kTeamSlots * sizeof(uint32_t));
+    const size_t smem = std::max(hist + kBigList * sizeof(uint32_t), kBigSmem);
+    const uint32_t list_cap = uint32_t((smem - hist) / sizeof(uint32_t));
+    static_assert(kTeams * kTeamSlots * sizeof(uint32_t) <= kBigSmem, "");
     LASER_CUDA(cudaFuncSetAttribute(draft_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
-    LASER_CUDA(launch_overlapped(draft_cta_kernel, dim3(unsigned(std::min(B, 148))), kBigThreads, smem, stream, pv, a, pool->vocab_bound));
+    LASER_CUDA(launch_overlapped(draft_cta_kernel, dim3(unsigned(std::min(B, 148))), kBigThreads, smem, stream, pv, a, pool->vocab_bound, list_cap));
     count_launch();
   }
   LASER_CUDA(cudaGetLastError());

@@ -74,3 +74,17 @@ def test_a_run_around_a_team(L, copies):
     for max_occ in (0, 65, copies - 1, copies + 1):
         for min_draft in (1, 6):
             _compare(L, toks, offs, tails, np.zeros(4, dtype=np.int64), 3, K=7, max_occ=max_occ, min_draft=min_draft)
+
+
+# Runs beyond what a CTA holds in registers: their occurrences fit the list of a small vocabulary (more of them than its walk takes
+# at once, before and after the first vote), or do not
+@pytest.mark.parametrize("copies,spread", [(17000, 2), (17000, 40), (60000, 3)])
+def test_a_run_beyond_a_cta(L, copies, spread):
+    rng = np.random.default_rng(copies + spread)
+    doc = np.full((copies, 5), -1, np.int32)
+    doc[:, 0] = 7
+    doc[:, 1:4] = 10 + np.minimum(rng.integers(0, spread, (copies, 3)), rng.integers(0, spread, (copies, 3)))
+    toks = np.concatenate([doc.reshape(-1), np.arange(100, 140, dtype=np.int32)])
+    offs = np.array([0, len(toks)], dtype=np.int64)
+    for max_occ in (0, 16500):
+        _compare(L, toks, offs, np.array([[7], [10]], dtype=np.int32), np.zeros(2, dtype=np.int64), 1, K=6, max_occ=max_occ, min_draft=1)
