@@ -1342,31 +1342,35 @@ draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound, uint32_t list_cap) {
   }
   const int team = tid / kTeamThreads;
   uint32_t* const table = s_hist + team * kTeamSlots;
-  if (tid % kTeamThreads == 0) s_late[team][1] = 0;
-  for (;;) {
-    Held& s = s_team[team];
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kTeamThreads) : "memory");
-    if (tid % kTeamThreads == 0) {
-      const int i = atomicAdd(&a.work[WORK_NEXT_SHORT], 1);
-      const int32_t* w = a.work + WORK_HEAD + 3 * i;
-      s.item[0] = i < n_short ? w[0] : -1; s.item[1] = i < n_short ? w[1] : 0; s.item[2] = i < n_short ? w[2] : 0;
+  for (bool again = true; again;) {                // until no team has left a query and the list is empty
+    if (tid % kTeamThreads == 0) s_late[team][1] = 0;
+    for (;;) {
+      Held& s = s_team[team];
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kTeamThreads) : "memory");
+      if (tid % kTeamThreads == 0) {
+        const int i = atomicAdd(&a.work[WORK_NEXT_SHORT], 1);
+        const int32_t* w = a.work + WORK_HEAD + 3 * i;
+        s.item[0] = i < n_short ? w[0] : -1; s.item[1] = i < n_short ? w[1] : 0; s.item[2] = i < n_short ? w[2] : 0;
+      }
+      asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kTeamThreads) : "memory");
+      const int q = s.item[0];
+      if (q < 0) break;
+      const int rest = held_run<kTeamThreads, kTeamItems, false>(pv, a, s, table, 1 + team, q, s.item[1], uint32_t(s.item[2]));
+      if (rest) {                                  // (the team waits for its CTA, which goes on with this one)
+        if (tid % kTeamThreads == 0) { s_late[team][0] = q; s_late[team][1] = rest; }
+        break;
+      }
     }
-    asm volatile("bar.sync %0, %1;" ::"r"(1 + team), "n"(kTeamThreads) : "memory");
-    const int q = s.item[0];
-    if (q < 0) break;
-    const int rest = held_run<kTeamThreads, kTeamItems, false>(pv, a, s, table, 1 + team, q, s.item[1], uint32_t(s.item[2]));
-    if (rest) {                                    // (the team takes no more: its CTA goes on with this one)
-      if (tid % kTeamThreads == 0) { s_late[team][0] = q; s_late[team][1] = rest; }
-      break;
-    }
-  }
-  __syncthreads();
-  bool clear = true;
-  for (int x = 0; x < kTeams; ++x) {
-    if (!s_late[x][1]) continue;
-    if (clear) { for (int v = tid; v < vocab_bound; v += kBigThreads) s_hist[v] = 0; clear = false; }
     __syncthreads();
-    serve(s_late[x][0], s_late[x][1]);
+    again = false;
+    for (int x = 0; x < kTeams; ++x) {
+      if (!s_late[x][1]) continue;
+      if (!again) for (int v = tid; v < vocab_bound; v += kBigThreads) s_hist[v] = 0;
+      again = true;
+      __syncthreads();
+      serve(s_late[x][0], s_late[x][1]);
+    }
+    __syncthreads();                               // (s_late is read, and the histogram is the teams' tables again)
   }
   // the last CTA leaves the work list empty for the next call
   if (tid == 0 && atomicAdd(&a.work[WORK_DONE], 1) == int(gridDim.x) - 1)

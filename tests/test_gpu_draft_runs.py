@@ -88,3 +88,37 @@ def test_a_run_beyond_a_cta(L, copies, spread):
     offs = np.array([0, len(toks)], dtype=np.int64)
     for max_occ in (0, 16500):
         _compare(L, toks, offs, np.array([[7], [10]], dtype=np.int32), np.zeros(2, dtype=np.int64), 1, K=6, max_occ=max_occ, min_draft=1)
+
+
+# More queries than the large-run kernel has teams (4 on each of 148 CTAs) whose longest suffix occurs often and gives no draft, or one
+# that is too short, so that they are handed on to the shorter suffixes; among them runs beyond a team, queries that a team finishes and
+# queries that the warp kernel does.  The outputs hold other values before the call.
+@pytest.mark.parametrize("B", [592, 593, 700, 4096])
+@pytest.mark.parametrize("min_draft,max_occ", [(1, 0), (1, 500), (8, 0), (8, 500)])
+def test_more_queries_handed_on_than_teams(L, B, min_draft, max_occ):
+    rng = np.random.default_rng(B + 10 * min_draft + max_occ)
+    toks = []
+    for c in range(70):
+        toks += [9, 7, 8, -1]                                   # "9 7 8" is never continued, "7 8" is
+    for c in range(90):
+        toks += [7, 8] + rng.integers(40, 43, int(rng.integers(0, 6))).tolist() + [-1]
+    for c in range(80):
+        toks += [1, 2, 3] + rng.integers(50, 52, 12).tolist() + [-1]
+    for c in range(2100):
+        toks += [20, 21 + c % 2, -1]                            # beyond a team, and never continued
+    toks = np.array(toks + list(range(100, 140)), dtype=np.int32)
+    offs = np.array([0, len(toks)], dtype=np.int64)
+    kinds = np.array([[9, 7, 8], [1, 2, 3], [5, 5, 20], [4, 20, 21], [101, 102, 103], [6, 40, 41], [60, 60, 60]], dtype=np.int32)
+    pick = np.where(rng.random(B) < 0.8, 0, rng.integers(0, len(kinds), B))
+    pool = L.pool_build(toks, offs, 1, 3)
+    p = L.make_params(K=10, n_min=1, n_max=3, min_draft=min_draft, max_occ=max_occ)
+    n = len(kinds)
+    want = [w[pick] for w in R.draft_batch(toks, offs, kinds, np.full(n, 3, np.int32), np.zeros(n, np.int32), 10, 1, 3, min_draft, max_occ)]
+    tails, lens, gids = dev_i32(kinds[pick]), dev_i32(np.full(B, 3)), dev_i32(np.zeros(B))
+    out = [dev_i32(np.full(w.shape, -77)) for w in want]
+    for _ in range(2):                         # the work list is left empty by the first call
+        for o in out:
+            o.fill_(-77)
+        L.draft(pool, tails, lens, gids, p, *out)
+        for g, w in zip(out, want):
+            assert (g.cpu().numpy() == w).all()
