@@ -116,8 +116,11 @@ _declare("laser_accept_commit_noalloc", 5, _I, _I, _P, _P, _P, _P, _P)
 
 
 def _at(t, dtype=None):
-    """The address of a contiguous tensor; with a dtype, of one on the GPU that holds it."""
+    """The address of a contiguous tensor; with a dtype, of one on the GPU that holds it (and of nothing else: the library would read
+    a host array's address as a device one)."""
     if not isinstance(t, torch.Tensor):
+        if dtype is not None:
+            raise TypeError("expected a %s tensor on the GPU, not %s" % (dtype, type(t)))
         return _ptr(t)
     assert t.is_contiguous(), "tensor must be contiguous"
     assert dtype is None or (t.is_cuda and t.dtype == dtype), (t.device, t.dtype, dtype)
