@@ -483,12 +483,14 @@ __device__ __forceinline__ int gather_occurrences(const PoolView& pv, int64_t lo
 // tokens up to there agree): at every depth the most frequent next token, ties to the smallest, and the occurrences that
 // continue with it.  An occurrence is a pool position, or with bit 31 an index into the history h[0 .. hl).  Writes the
 // tokens to s_cur and returns the depth reached, at most K.  s_val: kWalkVals words, 16-byte aligned.  All lanes of a warp.
-// Up to eight occurrences are read along: a lane a depth, so that one step covers all depths where they agree, and the vote where
-// they part.  More of them vote a depth at a time, each lane comparing its tokens with all of them, and are soon fewer; the
-// tokens of four depths are requested together.  Bound by latency: a vote whose steps are the distinct tokens, and a depth at a time
-// however few are left, took 9000 cycles of the 21000 of the longest queries, and 8000 for two occurrences that agree.  4096 queries on
-// 50 M tokens, max_occ 64, a batch asked again: 14.5 -> 11.4 us with this and the first probes at once.
-constexpr int kWalkFew = 8, kWalkVals = 68;
+// Up to four occurrences are read along: a lane a depth, 32 of them held in registers, so that one step covers all depths where they agree, and
+// a vote follows where they part.  More of them vote a depth at a time on tokens of which eight depths are requested together: first
+// for the token of the first of them, which a majority ends, then each lane compares its tokens with all of them.
+// Bound by latency and by the fetch of the code, which most warps go through once.  4096 queries on 50 M tokens, max_occ 64, a batch asked
+// again: 15.1 us with votes whose steps are the distinct tokens, one depth after the other; 12.6 with eight occurrences read along,
+// loaded again wherever they part, no look for a majority and four depths requested; 11.5 as it is (10.9 with eight held in registers).
+// Where many occurrences agree for long - 512 queries on groups of 200 thousand tokens - 13.6, 18.3 and 14.4 us (16.2 with eight held).
+constexpr int kWalkFew = 4, kWalkDepths = 8, kWalkVals = 68;
 __device__ __forceinline__ int walk_occurrences(const int32_t* __restrict__ tok, int64_t hi, const int32_t* __restrict__ h, int hl,
                                                 uint32_t e0, uint32_t e1, bool a0, bool a1, int len, int K, int lane, int32_t* s_cur,
                                                 int32_t* s_val) {
@@ -500,6 +502,12 @@ __device__ __forceinline__ int walk_occurrences(const int32_t* __restrict__ tok,
     const int64_t p = int64_t(e) + j;
     return p < hi ? tok[p] : -1;
   };
+  auto of_depth = [](const int32_t (&r)[kWalkDepths], int u) {    // (the loop over the depths is not unrolled: half the code)
+    int32_t t = r[0];
+#pragma unroll
+    for (int x = 1; x < kWalkDepths; ++x) t = u == x ? r[x] : t;
+    return t;
+  };
   const unsigned below = (1u << lane) - 1;
   constexpr int32_t kNone = 0x7fffffff;
   __syncwarp();                         // (s_val may be where e0 and e1 came from)
@@ -508,60 +516,75 @@ __device__ __forceinline__ int walk_occurrences(const int32_t* __restrict__ tok,
     int c = __popc(m0) + __popc(m1);
     if (c == 0) break;
     if (c <= kWalkFew) {
-      const int depth = len + 1 + lane;
+      const int base = len;             // of the 32 depths that the lanes hold
       int32_t x[kWalkFew];
-      unsigned l0 = m0, l1 = m1;
+      unsigned l0 = m0, l1 = m1, left = (1u << c) - 1;
 #pragma unroll
       for (int i = 0; i < kWalkFew; ++i) {
         x[i] = -1;
         if (i >= c) continue;           // (uniform)
         const uint32_t e = __shfl_sync(0xffffffffu, l0 ? e0 : e1, __ffs(l0 ? l0 : l1) - 1);
         if (l0) l0 &= l0 - 1; else l1 &= l1 - 1;
-        if (depth <= K) x[i] = next(e, depth);
+        if (base + 1 + lane <= K) x[i] = next(e, base + 1 + lane);
       }
-      bool same = x[0] >= 0;
+      while (left) {
+        int32_t v = -1;
+        bool same = true;
 #pragma unroll
-      for (int i = 1; i < kWalkFew; ++i) same = same && (i >= c || x[i] == x[0]);
-      const unsigned part = __ballot_sync(0xffffffffu, !same);
-      const int d = part ? __ffs(part) - 1 : 32;
-      if (lane < d) s_cur[len + lane] = x[0];
-      len += d;
-      if (d == 32 || len >= K) continue;
-      // lane d holds the tokens of the depth at which they part or end; lane i votes for the i-th
-      int32_t mine = -1;
-      int votes = 0;
+        for (int i = kWalkFew - 1; i >= 0; --i) if (left >> i & 1u) v = x[i];
 #pragma unroll
-      for (int i = 0; i < kWalkFew; ++i) {
-        x[i] = __shfl_sync(0xffffffffu, x[i], d);
-        if (lane == i) mine = x[i];
+        for (int i = 0; i < kWalkFew; ++i) same = same && (!(left >> i & 1u) || x[i] == v);
+        const unsigned part = __ballot_sync(0xffffffffu, !same || v < 0) & (~0u << (len - base));
+        const int d = part ? __ffs(part) - 1 : 32;
+        if (lane >= len - base && lane < d) s_cur[base + lane] = v;
+        len = base + d;
+        if (d == 32 || len >= K) break;
+        // lane d holds the tokens of the depth at which they part or end; lane i votes for the i-th
+        int32_t mine = -1;
+        int votes = 0;
+        int32_t y[kWalkFew];
+#pragma unroll
+        for (int i = 0; i < kWalkFew; ++i) {
+          y[i] = __shfl_sync(0xffffffffu, x[i], d);
+          if (!(left >> i & 1u)) y[i] = -1;
+          if (lane == i) mine = y[i];
+        }
+#pragma unroll
+        for (int i = 0; i < kWalkFew; ++i) votes += y[i] == mine;
+        if (mine < 0) votes = 0;
+        const int best = __reduce_max_sync(0xffffffffu, votes);
+        const int32_t pick = __reduce_min_sync(0xffffffffu, votes == best ? mine : kNone);
+        left = best ? __ballot_sync(0xffffffffu, votes > 0 && mine == pick) : 0u;
+        if (!left) break;
+        if (lane == 0) s_cur[len] = pick;
+        if (++len >= K || len - base == 32) break;
       }
-#pragma unroll
-      for (int i = 0; i < kWalkFew; ++i) votes += x[i] == mine;
-      if (mine < 0) votes = 0;
-      const int best = __reduce_max_sync(0xffffffffu, votes);
-      if (best == 0) break;
-      const int32_t pick = __reduce_min_sync(0xffffffffu, votes == best ? mine : kNone);
-      const unsigned keep = __ballot_sync(0xffffffffu, votes > 0 && mine == pick);
-      a0 = a0 && (keep >> __popc(m0 & below) & 1u);
-      a1 = a1 && (keep >> (__popc(m0) + __popc(m1 & below)) & 1u);
-      if (lane == 0) s_cur[len] = pick;
-      ++len;
+      if (!left) break;
+      a0 = a0 && (left >> __popc(m0 & below) & 1u);
+      a1 = a1 && (left >> (__popc(m0) + __popc(m1 & below)) & 1u);
       continue;
     }
-    int32_t r0[4], r1[4];
+    int32_t r0[kWalkDepths], r1[kWalkDepths];
 #pragma unroll
-    for (int u = 0; u < 4; ++u) {
+    for (int u = 0; u < kWalkDepths; ++u) {
       r0[u] = a0 && len + 1 + u <= K ? next(e0, len + 1 + u) : -1;
       r1[u] = a1 && len + 1 + u <= K ? next(e1, len + 1 + u) : -1;
     }
 #pragma unroll 1
-    for (int u = 0; u < 4 && len < K; ++u) {
-      const int32_t t0 = u == 0 ? r0[0] : u == 1 ? r0[1] : u == 2 ? r0[2] : r0[3];
-      const int32_t t1 = u == 0 ? r1[0] : u == 1 ? r1[1] : u == 2 ? r1[2] : r1[3];
+    for (int u = 0; u < kWalkDepths && len < K; ++u) {
+      const int32_t t0 = of_depth(r0, u);
+      const int32_t t1 = of_depth(r1, u);
       a0 = a0 && t0 >= 0; a1 = a1 && t1 >= 0;
       m0 = __ballot_sync(0xffffffffu, a0); m1 = __ballot_sync(0xffffffffu, a1);
       c = __popc(m0) + __popc(m1);
-      if (c <= kWalkFew) break;
+      if (c <= 1) break;
+      const int32_t first = __shfl_sync(0xffffffffu, m0 ? t0 : t1, __ffs(m0 ? m0 : m1) - 1);
+      if (2 * (__popc(__ballot_sync(0xffffffffu, a0 && t0 == first)) + __popc(__ballot_sync(0xffffffffu, a1 && t1 == first))) > c) {
+        a0 = a0 && t0 == first; a1 = a1 && t1 == first;
+        if (lane == 0) s_cur[len] = first;
+        ++len;
+        continue;
+      }
       if (a0) s_val[__popc(m0 & below)] = t0;
       if (a1) s_val[__popc(m0) + __popc(m1 & below)] = t1;
       if (lane < 4) s_val[c + lane] = -1;

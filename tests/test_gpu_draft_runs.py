@@ -122,3 +122,26 @@ def test_more_queries_handed_on_than_teams(L, B, min_draft, max_occ):
         L.draft(pool, tails, lens, gids, p, *out)
         for g, w in zip(out, want):
             assert (g.cpu().numpy() == w).all()
+
+
+# A few occurrences that agree up to a depth, with one or several of them parting there (a majority stays, or the smallest of equals): on
+# both sides of what a step reads along, of the depths requested together and of the 32 that a warp's lanes hold; a document ends there too
+@pytest.mark.parametrize("copies", [1, 2, 3, 4, 5, 8, 9, 33, 64])
+def test_occurrences_that_part(L, copies):
+    rng = np.random.default_rng(copies)
+    toks, offs, K = [], [0], 64
+    depths = [1, 2, 8, 9, 16, 31, 32, 33, 34, 63, 64, 65]
+    for d in depths:
+        line = rng.integers(10, 5000, 70).tolist()
+        for c in range(copies):
+            own = list(line)
+            if c % 3 == 1:
+                own[d - 1:] = rng.integers(10, 5000, 71 - d).tolist()
+            if c % 5 == 4:
+                own = own[:d - 1]
+            if c % 4 == 3 and d + 4 < len(own):
+                own[d + 4] = 6000 + c
+            toks += [7, 8] + own + [-1]
+        offs.append(len(toks))
+    tails = np.tile(np.array([[7, 8]], dtype=np.int32), (len(depths), 1))
+    _compare(L, np.array(toks, dtype=np.int32), np.array(offs, dtype=np.int64), tails, np.arange(len(depths)), 2, K=K, max_occ=64, min_draft=1)
