@@ -456,6 +456,23 @@ __device__ __forceinline__ bool is_occurrence(const int32_t* __restrict__ tok, i
   return true;
 }
 
+// The same, and the token at p + j (-1 beyond the group; p >= lo): up to four of the tail's are asked for together with it, for they are
+// mostly of one sector of memory, which with most of an SM's shared memory in use is gone again when it is asked for a second time.
+__device__ __forceinline__ bool occurrence_and_next(const int32_t* __restrict__ tok, int64_t lo, int64_t hi, int64_t p, const int32_t* tail,
+                                                    int n, int j, int32_t& next) {
+  constexpr int kAtOnce = 4;
+  const bool in = p - n + 1 >= lo && p < hi;
+  int32_t w[kAtOnce];
+#pragma unroll
+  for (int x = 0; x < kAtOnce; ++x) w[x] = in && x < n ? tok[p - x] : 0;
+  next = in && p + j < hi ? tok[p + j] : -1;
+  bool ok = in;
+#pragma unroll
+  for (int x = 0; x < kAtOnce; ++x) ok = ok && (x >= n || w[x] == tail[n - 1 - x]);
+  for (int x = kAtOnce; ok && x < n; ++x) ok = tok[p - x] == tail[n - 1 - x];
+  return ok;
+}
+
 // The group's occurrences of the n tail tokens, ascending, behind the n_occ that s_occ[64] already holds, until there are
 // `cap` (more may be counted, 64 are kept).  All lanes of a warp.  start: of their run, if there is one.  off: slots past the home one
 // that are known not to be the key's.
@@ -987,7 +1004,6 @@ __global__ void make_tree_rows_kernel(const int32_t* last, const int32_t* draft,
 constexpr int kBigThreads = 1024;
 constexpr int kBigUnroll = 4;
 constexpr int kBigList = 4096;      // positions: four a thread
-constexpr size_t kBigSmem = 204 * 1024;   // for the histogram and a longer list, as far as the vocabulary leaves room
 
 // A run held in registers by THREADS threads of a CTA (whose barrier is number `bar`), ITEMS positions each: the query's run of suffix
 // length n from `start` on.  Votes go to a histogram over the vocabulary (HIST: all zero before and after), or to a hash table
@@ -997,6 +1013,13 @@ constexpr int kTeams = 4, kTeamThreads = kBigThreads / kTeams, kTeamItems = kTea
 constexpr int kTeamSlots = 2 * kTeamRun, kTeamSlotBits = 12;
 constexpr int kLongItems = 16;
 static_assert(kTeamItems * kTeamThreads == kTeamRun && kTeamSlots == 1 << kTeamSlotBits && kTeamRun < 65536, "");
+// Shared memory for the histogram and a longer list, as far as the vocabulary leaves room, where max_occ does not bound the list; otherwise
+// what the teams' tables take.  A longer list spares passes over the run, and what it takes is lost to the L1 cache, in which the
+// occurrences' next tokens wait for the depths to come.  Groups of 200 thousand tokens: max_occ 500, 512 queries 32.6 us with the longer
+// list, 30.5 without, of min_draft 8 48.2 and 45.3; max_occ 0 286 and 379 (runs of 49 and 109 thousand), but 64 queries of
+// which one has a run of 31 thousand 127 and 107.
+constexpr size_t kHistMost = 200 * 1024, kBigSmem = 204 * 1024, kTeamSmem = size_t(kTeams) * kTeamSlots * sizeof(uint32_t);
+static_assert(kTeamSmem <= kBigSmem && kBigSmem <= kHistMost + kBigList * sizeof(uint32_t), "");
 struct Held {
   __align__(16) uint32_t list[kWalkVals];   // occurrences, then the walk's
   uint32_t end, count;
@@ -1037,17 +1060,12 @@ __device__ __forceinline__ int held_run(const PoolView& pv, const DraftArgs& a, 
   if (!whole && !cut) return n;
   end = whole ? s.end : uint32_t(most) - 1;
   int32_t t[ITEMS];
-#pragma unroll
-  for (int u = 0; u < ITEMS; ++u) {
-    const int64_t p = int64_t(v[u] & ~kRunEnd);
-    const bool in = uint32_t(u * THREADS + tt) <= end && p >= lo;
-    t[u] = in && p + 1 < hi ? pv.tok[p + 1] : -1;
-  }
   bool odd = false;
 #pragma unroll
   for (int u = 0; u < ITEMS; ++u) {
+    t[u] = -1;
     if (uint32_t(u * THREADS + tt) > end) continue;
-    if (is_occurrence(pv.tok, lo, hi, int64_t(v[u] & ~kRunEnd), tn, n)) alive |= 1u << u;
+    if (occurrence_and_next(pv.tok, lo, hi, int64_t(v[u] & ~kRunEnd), tn, n, 1, t[u])) alive |= 1u << u;
     else odd = true;
   }
   if (!whole) {
@@ -1224,8 +1242,8 @@ draft_cta_kernel(PoolView pv, DraftArgs a, int vocab_bound, uint32_t list_cap) {
               const uint32_t idx = base + u * kBigThreads + tid;
               const int64_t p = int64_t(v[u] & ~kRunEnd);
               alive[u] = idx <= end && idx <= cut && int64_t(s_start) + idx < a.n_positions;
-              t[u] = alive[u] && p + j < hi && p >= lo ? pv.tok[p + j] : -1;
-              if (alive[u]) alive[u] = is_occurrence(pv.tok, lo, hi, p, tn, n);
+              t[u] = -1;
+              if (alive[u]) alive[u] = occurrence_and_next(pv.tok, lo, hi, p, tn, n, j, t[u]);
               n_ok += alive[u];
               alive[u] = alive[u] && t[u] >= 0;
               for (int x = 1; x < j && alive[u]; ++x) alive[u] = pv.tok[p + x] == s_cur[x - 1];
@@ -1607,7 +1625,7 @@ LASER_API laser_status laser_draft(const laser_pool* pool, const int32_t* tails,
   const PoolView pv = view_of(pool);
   const bool big = (p->max_occ == 0 || p->max_occ > 64);
   const size_t hist = size_t(pool->vocab_bound) * sizeof(uint32_t);
-  if (big && hist > 200 * 1024) {
+  if (big && hist > kHistMost) {
     set_error("vocabulary bound %d too large for the unlimited-occurrence path", pool->vocab_bound);
     return LASER_ERR_UNSUPPORTED;
   }
@@ -1618,10 +1636,10 @@ LASER_API laser_status laser_draft(const laser_pool* pool, const int32_t* tails,
   LASER_CUDA(launch_overlapped(draft_warp_kernel, dim3(unsigned(ceil_div(B, kDraftWarps))), kDraftWarps * 32, 0, stream, pv, a));
   count_launch();
   if (big) {
-    const size_t smem = std::max(hist + kBigList * sizeof(uint32_t), kBigSmem);
+    const size_t smem = std::max(hist + kBigList * sizeof(uint32_t), p->max_occ > 0 && p->max_occ <= kBigList ? kTeamSmem : kBigSmem);
     const uint32_t list_cap = uint32_t((smem - hist) / sizeof(uint32_t));
-    static_assert(kTeams * kTeamSlots * sizeof(uint32_t) <= kBigSmem, "");
-    LASER_CUDA(cudaFuncSetAttribute(draft_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(smem)));
+    // (the same for all launches: another thread's may come between this and the next line)
+    LASER_CUDA(cudaFuncSetAttribute(draft_cta_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, int(kHistMost + kBigList * sizeof(uint32_t))));
     LASER_CUDA(launch_overlapped(draft_cta_kernel, dim3(unsigned(std::min(B, 148))), kBigThreads, smem, stream, pv, a, pool->vocab_bound, list_cap));
     count_launch();
   }

@@ -145,3 +145,18 @@ def test_occurrences_that_part(L, copies):
         offs.append(len(toks))
     tails = np.tile(np.array([[7, 8]], dtype=np.int32), (len(depths), 1))
     _compare(L, np.array(toks, dtype=np.int32), np.array(offs, dtype=np.int64), tails, np.arange(len(depths)), 2, K=K, max_occ=64, min_draft=1)
+
+
+# max_occ on both sides of what bounds the list of the large-run kernel (4096), on runs that it cuts there and on one that it does not
+@pytest.mark.parametrize("max_occ", [4095, 4096, 4097, 0])
+def test_a_list_at_its_limit(L, max_occ):
+    rng = np.random.default_rng(max_occ)
+    doc = np.full((17000, 5), -1, np.int32)
+    doc[:, 0] = 7
+    doc[:, 1:4] = 10 + np.minimum(rng.integers(0, 3, (17000, 3)), rng.integers(0, 3, (17000, 3)))
+    doc[4090::4, 0] = 8
+    toks = np.concatenate([doc.reshape(-1), np.arange(100, 140, dtype=np.int32)])
+    offs = np.array([0, len(toks)], dtype=np.int64)
+    tails = np.array([[7], [8], [10], [11], [12]], dtype=np.int32)
+    for min_draft in (1, 4):
+        _compare(L, toks, offs, tails, np.zeros(5, dtype=np.int64), 1, K=6, max_occ=max_occ, min_draft=min_draft)
