@@ -379,7 +379,8 @@ laser_status laser_verify_accept(laser_model* m, laser_kv* kv, const int32_t* se
  * a barrier nobody arrives on, for at most limit_cycles clock cycles (1e3 .. 2e9), while a second
  * role of the same kernel drains one bulk copy.  Afterwards laser_check() returns
  * LASER_ERR_TIMEOUT once (and clears it), and the model works as before.
- *   report  dev int32[4] out: [0] the starved wait gave up, [1] the abort flag reached the
+ *   report  dev int32[4] out: [0] the starved wait gave up (and a warp of whose lanes one had given
+ *           up on another wait agreed that it failed), [1] the abort flag reached the
  *           producer role, [2] the producer saw its copy land, [3] cycles the wait took.
  * Asynchronous on `stream`.  Errors: INVALID_ARG. */
 laser_status laser_selftest_wait(laser_model* m, int64_t limit_cycles, int32_t* report, void* stream);

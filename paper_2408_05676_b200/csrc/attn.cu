@@ -203,7 +203,7 @@ attn_paged_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* q, cons
 
   for (int p = pgrp; p < n_pg; p += NPG) {
     const int s = p % ST;
-    if (!mbar_wait(smem_u32(&full_bar[s]), (p / ST) & 1, &abort_flag)) break;
+    if (!mbar_wait_warp(smem_u32(&full_bar[s]), (p / ST) & 1, &abort_flag)) break;
     const uint32_t kbase = tiles + uint32_t(s) * STAGE, vbase = kbase + HALVES * SUB;
     float sc[2][4];
 #pragma unroll

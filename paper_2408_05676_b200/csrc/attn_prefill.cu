@@ -83,7 +83,7 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* q, co
       put_k0 = 0;
       if (!next_prompt(put_first, put_last, put_keys)) { put_keys = 0; return true; }
     }
-    const bool free = mbar_wait(smem_u32(&empty_bar[put_stage]), put_par, &abort_flag);
+    const bool free = mbar_wait_warp(smem_u32(&empty_bar[put_stage]), put_par, &abort_flag);
     if (free && lane == 0) {
       const int32_t* pt = page_table + size_t(s_seq[put_first]) * pages_per_seq;
       const uint32_t bar = smem_u32(&full_bar[put_stage]), dst = tiles + uint32_t(put_stage) * Z::kStage;
@@ -144,7 +144,7 @@ attn_prefill_kernel(const __grid_constant__ CUtensorMap kvmap, const bf16* q, co
     for (int k0 = 0; k0 < keys; k0 += 16 * kPages) {
       const int s = stage;
       if (warp == 0) ok = put();
-      ok = ok && mbar_wait(smem_u32(&full_bar[s]), par, &abort_flag);
+      ok = ok && mbar_wait_warp(smem_u32(&full_bar[s]), par, &abort_flag);
       if (!ok) break;
       if (++stage == kStages) { stage = 0; par ^= 1; }
       if (mine && k0 < my_keys) {

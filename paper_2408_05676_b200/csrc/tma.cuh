@@ -44,6 +44,12 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     if (clock64() - t0 > limit_cycles) { *abort_flag = 1; return false; }
   }
 }
+// The same for all lanes of a warp that goes on with instructions of the whole warp (matrix fragments, shuffles): at the limit one lane may
+// give up where another still sees the phase complete, so the warp takes one verdict.
+__device__ __forceinline__ bool mbar_wait_warp(uint32_t bar, uint32_t parity, volatile int* abort_flag,
+                                               long long limit_cycles = kWaitCycles) {
+  return __all_sync(0xffffffffu, mbar_wait(bar, parity, abort_flag, limit_cycles));
+}
 // The same bounded wait for the two single-thread loops that pace a kernel (the copy producer and the MMA
 // issuer): it polls without suspending, so the thread reacts as soon as the phase completes.
 __device__ __forceinline__ bool mbar_wait_hot(uint32_t bar, uint32_t parity, volatile int* abort_flag,

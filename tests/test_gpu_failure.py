@@ -43,3 +43,13 @@ def test_a_wait_that_runs_out_is_reported_and_the_library_keeps_working(L):
     assert torch.equal(before[0], after[0]) and torch.equal(before[3], after[3]) and torch.equal(before[1, :3], after[1, :3])
     with pytest.raises(L.LaserError):
         L.selftest_wait(m, 10)                    # limits outside [1e3, 2e9] are refused on the host
+
+
+@pytest.mark.parametrize("limit", [1000, 5_000_000])
+def test_a_warp_takes_one_verdict_of_a_wait(L, limit):
+    # one lane's limit runs out, then the barrier completes for the other 31: all of them have to go on as if it had run out
+    cfg = synth.model_cfg("tiny")
+    m = L.model_create(cfg, weights_to(synth.make_weights(cfg, seed=0), "cuda"), max_batch=1)
+    assert L.selftest_wait(m, limit).cpu().numpy()[:3].tolist() == [1, 1, 1]
+    with pytest.raises(L.LaserError):
+        L.check(m)
