@@ -408,7 +408,7 @@ def run_ours(args):
         "roofline": {"kernel": "gemm_tc_kernel (all dense contractions of one verify step)", "bound": "hbm",
                      "achieved": gemm_gbs, "peak": peaks["hbm_gbs"], "peak_source": peaks["source"], "unit": "GB/s",
                      "frac": gemm_gbs / peaks["hbm_gbs"], "traffic": GEMM_DRAM_TRAFFIC_PER_STEP if args.layers == 32 else None,
-                     "traffic_note": "ncu dram read+write summed over the 129 launches of a step (per-launch figures in profiles/gemm_tc_kernel_7b_rows144.md, scaled from a 2-layer capture: per-launch traffic does not depend on the layer count)",
+                     "traffic_note": "ncu dram read+write summed over the 129 launches of a step (scaled from a 2-layer capture: per-launch traffic does not depend on the layer count)",
                      "algorithmic_bytes_per_step": ab["weights"], "ms_per_step": gemm_ms, "launches_per_step": gemm_n // args.steps,
                      "in_pipeline_estimate": {
                          "note": "the event brackets stop consecutive launches from overlapping; scaling the bracketed "

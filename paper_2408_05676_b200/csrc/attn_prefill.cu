@@ -8,7 +8,9 @@
 // behind it: a fifth warp for the copies would leave the four 168 registers a thread instead of 255, and they need more.
 // A warp computes S = Q K^T and O += P V of 32 rows x 32 keys with warp-level MMA, so that a fragment of K or V feeds two row
 // tiles, and the online softmax's shuffles and rescaling are paid once for 32 keys.
-// Bound by the issue of fragment loads and MMAs, and by the CTAs that walk most keys (the host lists those first).  The kernel for
+// Bound by latency - the chain from the score MMA through the softmax to the value MMA, with two warps a scheduler: tensor pipe 41 % busy, issue
+// 35 %, shared memory 31 % - and by the CTAs that walk most keys (the host lists those first).  Head size 128 takes 255 registers,
+// 4 bytes of which are spilled, so there is no room for more in flight.  The kernel for
 // verify steps, which it replaces here, reads a fragment of K and V for 16 rows and takes a page's 16 keys at a time: 7B, prompts of 256 ..
 // 1024 tokens, 61 us a layer for passes of 1024 rows; this one 107 us for passes of 2304 with the chunks as they come, 76 us with those
 // that see most first.
