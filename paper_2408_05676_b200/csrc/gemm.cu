@@ -470,6 +470,11 @@ int pick_splits(int R_pad, int N, int K, int epi) {
 
 }  // namespace
 
+bool gemm_by_pairs(laser_model* m, int R_pad) {
+  GemmState* st = get_state(m);
+  return prepare(st) == LASER_OK && st->pair_fits && R_pad > gemm_pair_rows(m->precise);
+}
+
 laser_status gemm_fused(laser_model* m, const __nv_bfloat16* A, const __nv_bfloat16* W, int R_pad, int N, int K, int epi,
                         const GemmEpilogue& e, cudaStream_t stream) {
   if (R_pad % 16 != 0 || K % 8 != 0 || N % 8 != 0 || (reinterpret_cast<uintptr_t>(A) & 15) || (reinterpret_cast<uintptr_t>(W) & 15)) {
@@ -480,7 +485,7 @@ laser_status gemm_fused(laser_model* m, const __nv_bfloat16* A, const __nv_bfloa
   LASER_TRY(prepare(st));
   const CUtensorMap *tw = nullptr, *ta = nullptr;
   LASER_TRY(tensor_map(st, W, N, K, epi == EPI_SWIGLU ? 64 : 128, &tw));
-  if (st->pair_fits && R_pad > gemm_pair_rows(e.a_lo_off != 0)) {   // many token rows: two SMs per tile (gemm_pair.cu)
+  if (gemm_by_pairs(m, R_pad)) {
     const GemmPairShape sh = gemm_pair_shape(R_pad, N, K, epi, e.a_lo_off != 0);
     LASER_TRY(tensor_map(st, A, m->R_cap, e.a_lo_off ? 2 * K : K, sh.NT / 2, &ta));
     LASER_TRY(gemm_pair_launch(m, sh, *tw, *ta, N, K, epi, e, stream));

@@ -557,6 +557,11 @@ LASER_API laser_status laser_verify_step_tree(laser_model* m, laser_kv* kv, cons
 namespace laser {
 // Passes as large as the workspace are not always the best: what a pass takes goes up in steps, by waves of tiles, and so does what
 // is left for the last.  7B, 10 k prompt tokens in passes of up to 1024 / 1536 / 2304 rows: 133 / 121 / 114 ms.
+// The estimate is that of the contractions on pairs of SMs: a pass of so few rows that another kernel runs it (160, 64 in the precise mode)
+// is not taken but as the only one, and where the device cannot hold the pairs' grid passes are as large as they can be.  Attention
+// grows with the keys that its rows see, whatever pass they are in, and is left out but for its start.  Against passes as large as they can be,
+// timed in turn, prompts of 256 tokens: 13B (3 layers) 90 chunks 3455 -> 3115 us, 73 2718 -> 2622, 250 8913 -> 9122; 7B (4 layers) 320 chunks
+// 11071 -> 10609, 120 4098 -> 4091, 250 8507 -> 8642, precise 90 5701 -> 5520, 76 4814 -> 4876.  Passes of equal size: 7B 320 chunks 11727, 120 4327.
 std::vector<int> prefill_passes(laser_model* m, int n_chunks) {
   const int most = std::min(n_chunks, m->R_cap / kPrefillChunk), d = m->cfg.d_model, f = m->cfg.d_ffn;
   for (int c = int(m->prefill_us.size()); c <= most; ++c) {
@@ -565,12 +570,18 @@ std::vector<int> prefill_passes(laser_model* m, int n_chunks) {
     m->prefill_us.push_back(kEnds + gemm_pair_shape(rows, m->dqkv, d, EPI_QKV, m->precise).us + gemm_pair_shape(rows, d, m->dq, EPI_RESID, m->precise).us +
                             gemm_pair_shape(rows, 2 * f, d, EPI_SWIGLU, m->precise).us + gemm_pair_shape(rows, d, f, EPI_RESID, m->precise).us);
   }
+  auto priced = [&](int c) { return gemm_by_pairs(m, c * kPrefillChunk); };
+  if (n_chunks <= 0 || !priced(most)) {
+    std::vector<int> full;
+    for (int i = 0; i < n_chunks; i += most) full.push_back(std::min(most, n_chunks - i));
+    return full;
+  }
   std::vector<double> us(size_t(n_chunks) + 1, 0.0);     // of the first i chunks
   std::vector<int> last(size_t(n_chunks) + 1, 0);        // their last pass
   for (int i = 1; i <= n_chunks; ++i) {
     us[i] = 1e30;
     for (int c = 1; c <= std::min(i, most); ++c)
-      if (us[i - c] + m->prefill_us[c] < us[i]) { us[i] = us[i - c] + m->prefill_us[c]; last[i] = c; }
+      if ((priced(c) || c == n_chunks) && us[i - c] + m->prefill_us[c] < us[i]) { us[i] = us[i - c] + m->prefill_us[c]; last[i] = c; }
   }
   std::vector<int> passes;
   for (int i = n_chunks; i > 0; i -= last[i]) passes.push_back(last[i]);

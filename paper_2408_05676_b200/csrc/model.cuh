@@ -130,6 +130,8 @@ struct GemmEpilogue {
   int H = 0, Hkv = 0, dh = 0;
 };
 
+// Whether contractions of that many rows run on pairs of SMs (gemm_pair.cu).
+bool gemm_by_pairs(laser_model* m, int R_pad);
 // acc[r][n] = sum_k A[r][k] * W[n][k] (A bf16 [R_pad, K], W bf16 [N, K], both row-major),
 // finished by the epilogue `epi`.  N and K must be multiples of 8.
 laser_status gemm_fused(laser_model* m, const __nv_bfloat16* A, const __nv_bfloat16* W, int R_pad, int N, int K, int epi,
